@@ -35,6 +35,7 @@
 #include <set>
 
 #include "qdec_internal.h"
+#include "gdg_kernel.cuh"
 
 namespace qd {
 namespace {
@@ -499,6 +500,81 @@ bool build_window(const DemHost& d, int W, int F, int k, bool shorten, WindowHos
   std::sort(deg.begin(), deg.end(), std::greater<int>());
   o.short_edges_max = 0;
   for (int c = 0; c < o.n_short; ++c) o.short_edges_max += deg[c];
+  return true;
+}
+
+// The window's graph in slices (see gdg_kernel.cuh): labels by descending
+// degree, ties by window row / column; a check's entries in ascending column
+// label, so that the positions past 31 (checks of 35 entries) fall to columns
+// of the lowest degrees and only their slices look at the second sign word; a
+// column's entries in ascending window row, the order of the sum of Eq. (2).
+bool build_slices(WindowHost& o) {
+  const int nr = o.n_rows, nc = o.n_cols;
+  const int nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
+  auto cdeg = [&](int c) { return o.col_ptr[c + 1] - o.col_ptr[c]; };
+  auto rdeg = [&](int j) { return o.row_ptr[j + 1] - o.row_ptr[j]; };
+  o.s_row.resize(nr);
+  o.s_col.resize(nc);
+  for (int j = 0; j < nr; ++j) o.s_row[j] = (uint16_t)j;
+  for (int c = 0; c < nc; ++c) o.s_col[c] = (uint16_t)c;
+  std::stable_sort(o.s_row.begin(), o.s_row.end(), [&](uint16_t a, uint16_t b) { return rdeg(a) > rdeg(b); });
+  std::stable_sort(o.s_col.begin(), o.s_col.end(), [&](uint16_t a, uint16_t b) { return cdeg(a) > cdeg(b); });
+  std::vector<uint16_t> rlab(nr);
+  for (int l = 0; l < nr; ++l) rlab[o.s_row[l]] = (uint16_t)l;
+  o.max_row_deg = nr ? rdeg(o.s_row[0]) : 0;
+  const int max_col_deg = nc ? cdeg(o.s_col[0]) : 0;
+  if (o.max_row_deg > kMaxRowDeg) {
+    set_error("a detector touches more than " + std::to_string(kMaxRowDeg) + " columns");
+    return false;
+  }
+  o.s_roff.assign(nrs + 1, 0);
+  o.s_coff.assign(ncs + 1, 0);
+  for (int q = 0; q < nrs; ++q) o.s_roff[q + 1] = (uint16_t)(o.s_roff[q] + (rdeg(o.s_row[32 * q]) + 1) / 2);
+  for (int q = 0; q < ncs; ++q) o.s_coff[q + 1] = (uint16_t)(o.s_coff[q] + cdeg(o.s_col[32 * q]));
+  o.row_pairs = o.s_roff[nrs];
+  o.col_cells = o.s_coff[ncs];
+  o.s_rent.assign((size_t)64 * o.row_pairs, 4u * (uint32_t)(32 * ncs));  // the dummy column
+  o.s_cent.assign((size_t)32 * o.col_cells, (uint32_t)(32 * nrs) << 16);  // the dummy check
+  o.s_ref.assign(o.s_rent.size(), 0);
+  o.s_cef.assign(o.s_cent.size(), 0);
+  o.s_llr.assign((size_t)32 * ncs, 0.0f);
+  std::vector<int> fill(nr, 0);
+  std::vector<char> wide(ncs, 0);
+  for (int l = 0; l < nc; ++l) {
+    const int c = o.s_col[l];
+    o.s_llr[l] = o.llr[c];
+    for (int e = o.col_ptr[c]; e < o.col_ptr[c + 1]; ++e) {
+      const int r = rlab[o.col_rows[e]], pos = fill[r]++;
+      const size_t ri = ((size_t)(o.s_roff[r >> 5] + (pos >> 1)) * 32 + (r & 31)) * 2 + (pos & 1);
+      const size_t ci = (size_t)(o.s_coff[l >> 5] + (e - o.col_ptr[c])) * 32 + (l & 31);
+      o.s_rent[ri] = 4u * (uint32_t)l;
+      o.s_ref[ri] = (uint16_t)e;
+      o.s_cent[ci] = ((uint32_t)r << 16) | (uint32_t)pos;
+      o.s_cef[ci] = (uint16_t)e;
+      if (pos >= 32) wide[l >> 5] = 1;
+    }
+  }
+  // a dummy takes its node's first edge's learned weight, so that a weight
+  // touches no node but its own two
+  for (int r = 0; r < nr; ++r)
+    for (int pos = std::max(1, fill[r]); pos < 2 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
+      const size_t r0 = ((size_t)o.s_roff[r >> 5] * 32 + (r & 31)) * 2;
+      o.s_ref[r0 + 64 * (size_t)(pos >> 1) + (pos & 1)] = o.s_ref[r0];
+    }
+  for (int l = 0; l < nc; ++l)
+    for (int u = cdeg(o.s_col[l]); u < o.s_coff[(l >> 5) + 1] - o.s_coff[l >> 5]; ++u) {
+      const size_t c0 = (size_t)o.s_coff[l >> 5] * 32 + (l & 31);
+      o.s_cef[c0 + 32 * (size_t)u] = o.s_cef[c0];
+    }
+  for (int q = 0; q < ncs; ++q)
+    if (wide[q]) o.s_coff[q] |= kWideSlice;
+  // a shortened graph: every slice but the first is no wider than the least
+  // degree of the slice before it, so the widths sum to at most the widest
+  // node plus edges / 32 (check slices rounded up to pairs)
+  const int ns = o.n_short, nss = (ns + 31) / 32, es = o.short_edges_max;
+  const int wr = std::min(o.max_row_deg, ns);
+  o.srow_pairs = std::min(nrs * ((wr + 1) / 2), (wr + es / 32 + nrs) / 2 + 1);
+  o.scol_cells = std::min(nss * max_col_deg, max_col_deg + es / 32);
   return true;
 }
 

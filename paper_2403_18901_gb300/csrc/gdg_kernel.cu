@@ -43,6 +43,7 @@
 
 #include <cfloat>
 #include <cstdint>
+#include <type_traits>
 
 #include "gdg_kernel.cuh"
 #include "qdec_internal.h"
@@ -54,41 +55,210 @@ constexpr unsigned FULL = 0xffffffffu;
 enum { BR_CONVERGED = 0, BR_MAXDEPTH = 1, BR_CONTRADICTION = 2, BR_NOCAND = 3, BR_INTERNAL = 4 };
 constexpr int kNone = 0x7fffffff;
 
-// |x| bounded by c by min / max: for finite x the comparisons' result; a NaN
-// x (only a dead entry of a decision path's check pass) gives +c, so its sign
-// bit is 0 and needs no mask there
-__device__ __forceinline__ float clipf(float x, float c) { return fmaxf(fminf(x, c), -c); }
+// The posterior a decimated VN stores, and that of the dummy column: a check's
+// input from it is +inf whatever its message (finite), so it never is the
+// smallest or second smallest, has sign 0 and no hard decision.
+__device__ __forceinline__ float dead_post() { return CUDART_INF_F; }
 
-// mu_{j->i} from the check's compressed state (see gdg_kernel.cuh).
-__device__ __forceinline__ float c2v_msg(float alpha, float clip, const CNState& c, int e, uint32_t sg) {
-  float m = ((c.ac & 0xFFFFu) == (uint32_t)e) ? c.m2 : c.m1;
-  if (c.ac & (2u << 16)) m = clip;  // single active VN: minimum over the empty set = clip
-  const float mag = __fmul_rn(alpha, m);
-  return ((((c.ac >> 16) & 1u) ^ sg) != 0) ? -mag : mag;
+__device__ __forceinline__ float flip_sign(float x, uint32_t s) {  // s: the sign at bit 31, other bits 0
+  return __uint_as_float(__float_as_uint(x) ^ s);
 }
 
-// Check state as stored.  With learned weights the magnitudes stay unscaled
-// (each edge applies its own weight); for the plain decoder they are stored
-// already multiplied by alpha (alpha * clip for a single active input), the
-// same FP32 products c2v_msg forms, with the parity as their sign, so a
-// message is one select and the edge's own sign.
-// `rows` (the check's CSR range, begin | end << 16) rides along in the
-// record's last word, so the check pass loads it with the state.
+// Eq. (1): mu_{j->i} from the check's record for the edge at position p of
+// its entries (low six bits of e); w: the learned weight.  wide: the position
+// may be past 31.
 template <bool LW>
-__device__ __forceinline__ CNState cn_store(float alpha, float clip, float m1, float m2, int am, uint32_t par,
-                                            bool single, uint32_t rows) {
-  if (LW) return CNState{m1, m2, (uint32_t)am | (par << 16) | ((uint32_t)single << 17), rows};
-  const float s1 = __fmul_rn(alpha, single ? clip : m1);
-  const float s2 = single ? s1 : __fmul_rn(alpha, m2);
-  // the sign parity rides in the sign bits of the two (non-negative) magnitudes
-  return CNState{par ? -s1 : s1, par ? -s2 : s2, (uint32_t)am, rows};
+__device__ __forceinline__ float c2v(const CNState& c, uint32_t e, bool wide, float w) {
+  float m = ((c.am ^ e) & 63u) ? c.m1 : c.m2;
+  uint32_t sg = c.sg;
+  if (wide && (e & 32u)) sg = c.am;
+  m = flip_sign(m, __funnelshift_l(0u, sg, e) & 0x80000000u);  // shift by e mod 32
+  return LW ? __fmul_rn(w, m) : m;
 }
 
+// The inputs a check has seen: two smallest magnitudes, the position of the
+// smallest, the parity of the hard decisions it read (bit 31).  The two
+// smallest and so every message do not depend on the order of the inputs.
+struct CheckAcc {
+  float m1, m2;
+  uint32_t am, hp;
+};
+
+// One input at position u: posterior pv, the previous iteration's record (its
+// argmin position oam, two magnitudes, this edge's sign osg at bit 31).
+// Returns the bits of v, whose sign the caller collects.  The clip of Eq. (3)
+// bounds every magnitude alike, so it is applied to the two smallest at the
+// end.  A posterior is never -0 (its prior is positive and x + y = -0 only for
+// x = y = -0), nor is the difference of two messages, so the sign bit is the
+// comparison with 0, and pv <= 0 is the sign of pv's bits minus one.
+template <bool LW, bool FIRST>
+__device__ __forceinline__ uint32_t check_input(CheckAcc& A, float pv, uint32_t u, uint32_t oam, float om1, float om2,
+                                                uint32_t osg, float w) {
+  float v = pv;
+  if (!FIRST) {
+    float m = flip_sign(u == oam ? om2 : om1, osg & 0x80000000u);
+    if (LW) m = __fmul_rn(w, m);
+    v = __fsub_rn(pv, m);
+    if (LW && pv == CUDART_INF_F) v = pv;  // a dead input stays one under an infinite weighted message
+  }
+  const float a = fabsf(v);
+  A.am = a < A.m1 ? u : A.am;
+  A.m2 = fminf(A.m2, fmaxf(A.m1, a));
+  A.m1 = fminf(A.m1, a);
+  A.hp ^= __float_as_uint(pv) - 1u;
+  return __float_as_uint(v);
+}
+
+// The record of a check from its inputs and the syndrome bit: magnitudes
+// bounded by the clip (an only input gets the clip itself, the minimum over
+// the empty set; the first iteration's inputs are priors, not clipped).
 template <bool LW>
-__device__ __forceinline__ float c2v(float w, float clip, const CNState& c, int e, uint32_t sg) {
-  if (LW) return c2v_msg(w, clip, c, e, sg);
-  const float m = (c.ac == (uint32_t)e) ? c.m2 : c.m1;  // signed by the parity already
-  return sg ? -m : m;
+__device__ __forceinline__ CNState check_record(const CheckAcc& A, uint32_t sg0, uint32_t sg1, uint32_t sbit, bool first,
+                                                float alpha, float clip) {
+  float m1 = A.m1, m2 = A.m2;
+  if (first) {
+    m1 = m1 == CUDART_INF_F ? clip : m1;
+    m2 = m2 == CUDART_INF_F ? clip : m2;
+  } else {
+    m1 = fminf(m1, clip);
+    m2 = fminf(m2, clip);
+  }
+  if (!LW) {
+    m1 = __fmul_rn(alpha, m1);
+    m2 = __fmul_rn(alpha, m2);
+  }
+  const uint32_t par = (uint32_t)(__popc(sg0 ^ sg1) + (int)sbit) << 31;
+  return CNState{flip_sign(m1, par), flip_sign(m2, par), sg0, (sg1 & ~63u) | A.am};
+}
+
+// Learned weights' view of one iteration: its row of w, and the full-window
+// edge of each entry.
+struct LwRow {
+  const float* w;
+  const uint16_t* ef;
+};
+__device__ __forceinline__ float lw_at(const LwRow& r, int i) { return r.w[r.ef[i]]; }
+
+// Check-node update of Eq. (1) of one check by one lane.  ent: the lane's
+// entry pairs, `np` of them, 32 pairs apart (ei: the index of the first entry,
+// for the learned weights' edge ids); post: posteriors; rec: its record, the
+// previous iteration's on entry.  Returns at bit 31 the parity of the hard
+// decisions read, xor the syndrome bit: the test H e = s of the iteration
+// before.  What bounds it: issue, ALU instructions above all (half rate, about
+// 11 of 14 per entry); the posterior gathers' bank conflicts come next.  With
+// a sign byte and an edge id per edge, a NaN test and the clip on every input
+// and ragged rows, 5000 shots of [[144,12,12]] took 450 ms; in slices, with
+// the signs as bits of the record and the clip on the two minima, 354 ms.
+template <bool LW, bool FIRST>
+__device__ __forceinline__ uint32_t check_lane(const uint2* ent, int np, const char* post, CNState* rec, uint32_t sbit,
+                                               float alpha, float clip, const LwRow& lw, int ei) {
+  CNState oc{};
+  if (!FIRST) oc = *rec;
+  const uint32_t oam = oc.am & 63u;
+  uint32_t osg = oc.sg;
+  CheckAcc A{CUDART_INF_F, CUDART_INF_F, 0u, 0u};
+  uint32_t sg0 = 0u, sg1 = 0u;
+  for (int p0 = 0; p0 < np; p0 += 16) {  // 32 positions to a sign word
+    const int p1 = min(np, p0 + 16);
+    uint32_t sg = 0u;
+    for (int p = p0; p < p1; ++p) {
+      const uint2 e = ent[32 * p];
+      const float a = *(const float*)(post + e.x), b = *(const float*)(post + e.y);
+      float wa = 0.0f, wb = 0.0f;
+      if (LW && !FIRST) {
+        wa = lw_at(lw, ei + 64 * p);
+        wb = lw_at(lw, ei + 64 * p + 1);
+      }
+      sg = __funnelshift_l(check_input<LW, FIRST>(A, a, 2 * p, oam, oc.m1, oc.m2, osg, wa), sg, 1);
+      osg += osg;
+      sg = __funnelshift_l(check_input<LW, FIRST>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, osg, wb), sg, 1);
+      osg += osg;
+    }
+    sg = sg << (32 - 2 * (p1 - p0)) % 32;  // the first position to bit 31
+    if (p0 == 0) {
+      sg0 = sg;
+      osg = oc.am;
+    } else {
+      sg1 = sg;
+    }
+  }
+  *rec = check_record<LW>(A, sg0, sg1, sbit, FIRST, alpha, clip);
+  return (A.hp ^ (sbit << 31)) & 0x80000000u;
+}
+
+// The same by TPC neighbouring lanes (entry pairs sub, sub + TPC, ...); every
+// lane of the group ends with the record.
+template <bool LW>
+__device__ __forceinline__ CNState check_group(const uint2* ent, int np, const char* post, const CNState& oc,
+                                               uint32_t sbit, float alpha, float clip, bool first, const LwRow& lw,
+                                               int ei, int sub, int tpc, bool wide, uint32_t& unsat) {
+  const uint32_t oam = oc.am & 63u;
+  CheckAcc A{CUDART_INF_F, CUDART_INF_F, 0u, 0u};
+  uint32_t sg0 = 0u, sg1 = 0u;
+  for (int p = sub; p < np; p += tpc) {
+    const uint2 e = ent[32 * p];
+    const float a = *(const float*)(post + e.x), b = *(const float*)(post + e.y);
+    float wa = 0.0f, wb = 0.0f;
+    if (LW && !first) {
+      wa = lw_at(lw, ei + 64 * p);
+      wb = lw_at(lw, ei + 64 * p + 1);
+    }
+    const uint32_t ow = p < 16 ? oc.sg : oc.am;
+    const int sh = (2 * p) & 31;
+    uint32_t va, vb;
+    if (first) {
+      va = check_input<LW, true>(A, a, 2 * p, oam, oc.m1, oc.m2, 0u, wa);
+      vb = check_input<LW, true>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, 0u, wb);
+    } else {
+      va = check_input<LW, false>(A, a, 2 * p, oam, oc.m1, oc.m2, ow << sh, wa);
+      vb = check_input<LW, false>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, ow << (sh + 1), wb);
+    }
+    const uint32_t s2 = ((va & 0x80000000u) | ((vb & 0x80000000u) >> 1)) >> sh;
+    if (p < 16) sg0 |= s2;
+    else sg1 |= s2;
+  }
+  for (int off = tpc >> 1; off; off >>= 1) {
+    const float x1 = __shfl_xor_sync(FULL, A.m1, off), x2 = __shfl_xor_sync(FULL, A.m2, off);
+    const uint32_t xa = __shfl_xor_sync(FULL, A.am, off);
+    A.hp ^= __shfl_xor_sync(FULL, A.hp, off);
+    sg0 |= __shfl_xor_sync(FULL, sg0, off);
+    if (wide) sg1 |= __shfl_xor_sync(FULL, sg1, off);
+    A.m2 = fminf(fminf(A.m2, x2), fmaxf(A.m1, x1));
+    // equal minima: either position gives the same messages, but every lane of
+    // the group has to take the same one
+    A.am = x1 < A.m1 || (x1 == A.m1 && xa < A.am) ? xa : A.am;
+    A.m1 = fminf(A.m1, x1);
+  }
+  unsat |= (A.hp ^ (sbit << 31)) & 0x80000000u;
+  return check_record<LW>(A, sg0, sg1, sbit, first, alpha, clip);
+}
+
+// Variable-node update of Eq. (2) by one lane: prior + the messages of its
+// checks in ascending check order; `n` places 32 entries apart (a dummy adds
+// +0), at most three records in flight.
+template <bool LW>
+__device__ __forceinline__ float column_sum(float p, const uint32_t* ent, int n, bool wide, const char* cns,
+                                            const LwRow& lw, int ei) {
+  auto msgs = [&](int u, auto cnt) {
+    constexpr int N = decltype(cnt)::value;
+    uint32_t e[N];
+    CNState c[N];
+    float w[N];
+#pragma unroll
+    for (int x = 0; x < N; ++x) e[x] = ent[32 * (u + x)];
+#pragma unroll
+    for (int x = 0; x < N; ++x) {
+      c[x] = *(const CNState*)(cns + (e[x] >> 12));
+      w[x] = LW ? lw_at(lw, ei + 32 * (u + x)) : 0.0f;
+    }
+#pragma unroll
+    for (int x = 0; x < N; ++x) p = __fadd_rn(p, c2v<LW>(c[x], e[x], wide, w[x]));
+  };
+  int u = 0;
+  for (; u + 3 <= n; u += 3) msgs(u, std::integral_constant<int, 3>{});
+  if (u + 2 == n) msgs(u, std::integral_constant<int, 2>{});
+  else if (u + 1 == n) msgs(u, std::integral_constant<int, 1>{});
+  return p;
 }
 
 __device__ __forceinline__ uint32_t bit_of(const uint32_t* w, int j) { return (w[j >> 5] >> (j & 31)) & 1u; }
@@ -171,12 +341,11 @@ __device__ void stage_pieces(Stager& st, const StagePiece* pc, int n) {
   __syncthreads();
 }
 
-// Multiplier of Eq. (1) at iteration t >= 1 for full-window edge ef: alpha, or
-// the learned weight w[min(t, T)][ef].
-__device__ __forceinline__ float edge_weight(const float* wts, int wT, int wE, float alpha, int t, int ef) {
-  if (!wts) return alpha;
-  const int row = t < 1 ? 0 : (t < wT ? t : wT) - 1;  // never a row before the first
-  return wts[(size_t)row * wE + ef];
+// Learned weights of iteration t (1-based): w[min(t, T)], never a row before
+// the first.
+__device__ __forceinline__ const float* weight_row(const float* wts, int wT, int wE, int t) {
+  const int row = t < 1 ? 0 : (t < wT ? t : wT) - 1;
+  return wts + (size_t)row * wE;
 }
 
 // order-preserving map of a float to uint32 (-0 and +0 equal)
@@ -184,40 +353,6 @@ __device__ __forceinline__ uint32_t ordkey(float f) {
   if (f == 0.0f) f = 0.0f;
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ void warp_min2(float& m1, float& m2, int& am) {
-#pragma unroll
-  for (int off = 16; off; off >>= 1) {
-    const float x1 = __shfl_xor_sync(FULL, m1, off);
-    const float x2 = __shfl_xor_sync(FULL, m2, off);
-    const int xa = __shfl_xor_sync(FULL, am, off);
-    if (x1 < m1 || (x1 == m1 && xa < am)) {
-      m2 = fminf(m1, x2);
-      m1 = x1;
-      am = xa;
-    } else {
-      m2 = fminf(m2, x1);
-    }
-  }
-}
-
-// (min1, min2, argmin) and sign parity over aligned groups of tpc lanes
-// (tpc a power of two <= 32); every lane of a group ends with the result.
-__device__ __forceinline__ void group_min2(float& m1, float& m2, int& am, uint32_t& neg, int tpc) {
-  for (int off = tpc >> 1; off; off >>= 1) {
-    const float x1 = __shfl_xor_sync(FULL, m1, off);
-    const float x2 = __shfl_xor_sync(FULL, m2, off);
-    const int xa = __shfl_xor_sync(FULL, am, off);
-    neg ^= __shfl_xor_sync(FULL, neg, off);
-    if (x1 < m1 || (x1 == m1 && xa < am)) {
-      m2 = fminf(m1, x2);
-      m1 = x1;
-      am = xa;
-    } else {
-      m2 = fminf(m2, x1);
-    }
-  }
 }
 
 __host__ __device__ inline int lanes_per_check(int threads, int n_checks) {
@@ -250,25 +385,13 @@ __device__ __forceinline__ void warp_argmin(float& v, int& k) {
   }
 }
 
-// Exclusive scan of a[0..n) in place, by one warp; returns the total.
-__device__ int warp_scan_excl(int* a, int n, int lane) {
-  const int chunk = (n + 31) / 32;
-  const int beg = lane * chunk, end = min(n, beg + chunk);
-  int s = 0;
-  for (int i = beg; i < end; ++i) s += a[i];
-  int incl = s;
+__device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
-    const int y = __shfl_up_sync(FULL, incl, off);
-    if (lane >= off) incl += y;
+    const int y = __shfl_up_sync(FULL, v, off);
+    if (lane >= off) v += y;
   }
-  int run = incl - s;
-  for (int i = beg; i < end; ++i) {
-    const int v = a[i];
-    a[i] = run;
-    run += v;
-  }
-  return __shfl_sync(FULL, incl, 31);
+  return v;
 }
 
 // ---- cooperative groups of threads that run one decision path ----
@@ -410,14 +533,15 @@ struct CtaGrp {  // the whole CTA; every member must call every primitive
   }
 };
 
+// The shortened graph in slices (gdg_kernel.cuh).
 struct ShortG {
-  int nr, ns, rw;
-  const uint16_t *colptr, *colrows, *rowptr;
-  const uint32_t* rowent;  // CSR entry: edge id | (short column << 16)
+  int nr, ns, rw, cw;  // checks, columns, and their slices
+  const uint32_t *rent, *cent;
+  const uint16_t *roff, *coff;
   const float* llr;
   const uint8_t* vdeg;
   const uint32_t* sbits;
-  const uint16_t* efull;  // short edge -> full-window edge (learned weights)
+  const uint16_t *ref, *cef;  // full-window edge of each check / column entry (learned weights)
   const float* wts;
   int wT, wE;
   int rpb;  // window rows per block (block of a column = its first row / rpb)
@@ -428,47 +552,53 @@ struct ShortG {
   const uint16_t* cperm;
   const uint16_t* vperm;
   int ncr;  // window rows [0, ncr) are the ones the window commits
+
+  __device__ __forceinline__ int col_slice(int k) const { return (int)(coff[k >> 5] & (kWideSlice - 1)); }
+  // check label of column k's u-th entry (u < vdeg[k])
+  __device__ __forceinline__ const uint32_t* col_ents(int k) const { return cent + col_slice(k) * 32 + (k & 31); }
 };
 
 struct Slot {
   float *post, *acc;
-  uint8_t *hfl, *sign;
+  uint8_t* hfl;
   int8_t* status;
   CNState* cns;
-  int* deg;
+  uint8_t* deg;  // active VNs per check
   uint32_t *sp, *unsat;
   int8_t* hq;  // ranker only: the last four posteriors as round(2 clamp(x, 63.5)), oldest first
 };
 
 __device__ __forceinline__ Slot make_slot(char* base, const Layout& L) {
-  return Slot{(float*)(base + L.b_post),   (float*)(base + L.b_acc),     (uint8_t*)(base + L.b_hfl),
-              (uint8_t*)(base + L.b_sign), (int8_t*)(base + L.b_status), (CNState*)(base + L.b_cns),
-              (int*)(base + L.b_deg),      (uint32_t*)(base + L.b_sp),
-              (uint32_t*)(base + L.b_unsat), (int8_t*)(base + L.b_hq)};
+  return Slot{(float*)(base + L.b_post),  (float*)(base + L.b_acc),      (uint8_t*)(base + L.b_hfl),
+              (int8_t*)(base + L.b_status), (CNState*)(base + L.b_cns),  (uint8_t*)(base + L.b_deg),
+              (uint32_t*)(base + L.b_sp), (uint32_t*)(base + L.b_unsat), (int8_t*)(base + L.b_hq)};
 }
 
-// Posterior of a decimated VN: a NaN, so the check-node pass recognises a
-// stale edge from the posterior it loads anyway.
-__device__ __forceinline__ float stale() { return __int_as_float(0x7fffffff); }
-
-__device__ __forceinline__ void decimate_atomic(const ShortG& G, const Slot& B, int k, int v) {
+// Fix column k to v while other lanes fix others; returns its degree.
+__device__ __forceinline__ int decimate_atomic(const ShortG& G, const Slot& B, int k, int v) {
   B.status[k] = (int8_t)v;
-  B.post[k] = stale();
-  for (int e = G.colptr[k]; e < G.colptr[k + 1]; ++e) {
-    const int j = G.colrows[e];
-    atomicSub(&B.deg[j], 1);
+  B.post[k] = dead_post();
+  const uint32_t* ce = G.col_ents(k);
+  const int d = G.vdeg[k];
+  for (int u = 0; u < d; ++u) {
+    const int j = (int)(ce[32 * u] >> 16);
+    atomicSub((uint32_t*)B.deg + (j >> 2), 1u << (8 * (j & 3)));  // counts stay >= 0: no borrow
     if (v) atomicXor(&B.sp[j >> 5], 1u << (j & 31));
   }
+  return d;
 }
 
-__device__ __forceinline__ void decimate_one(const ShortG& G, const Slot& B, int k, int v) {
+__device__ __forceinline__ int decimate_one(const ShortG& G, const Slot& B, int k, int v) {
   B.status[k] = (int8_t)v;
-  B.post[k] = stale();
-  for (int e = G.colptr[k]; e < G.colptr[k + 1]; ++e) {
-    const int r = G.colrows[e];
+  B.post[k] = dead_post();
+  const uint32_t* ce = G.col_ents(k);
+  const int d = G.vdeg[k];
+  for (int u = 0; u < d; ++u) {
+    const int r = (int)(ce[32 * u] >> 16);
     B.deg[r] -= 1;
     if (v) B.sp[r >> 5] ^= 1u << (r & 31);
   }
+  return d;
 }
 
 // Peeling (Sec. IV): repeatedly fix the lone active VN of a degree-one check
@@ -476,9 +606,10 @@ __device__ __forceinline__ void decimate_one(const ShortG& G, const Slot& B, int
 // syndrome 1 is a contradiction.  One check at a time, always the lowest-index
 // degree-one check, after testing every check for a contradiction (this order
 // also fixes the partial state of a path killed by a contradiction).
-// Returns #peeled, -1 (contradiction) or -2 (inconsistent degree count).
+// Returns #peeled, -1 (contradiction) or -2 (inconsistent degree count);
+// subtracts the edges of the peeled VNs from rank 0's `act`.
 template <class Grp>
-__device__ int peel(const ShortG& G, const Slot& B, const Grp& g) {
+__device__ int peel(const ShortG& G, const Slot& B, const Grp& g, int& act) {
   int npeel = 0;
   for (int guard = 0; guard <= G.ns + 1; ++guard) {
     bool contra = false;
@@ -496,15 +627,17 @@ __device__ int peel(const ShortG& G, const Slot& B, const Grp& g) {
     if (jc == kNone) return npeel;
     const int j = jc & 0xFFFF;
     int found = kNone;
-    for (int q = G.rowptr[j] + g.rank; q < G.rowptr[j + 1]; q += g.size) {
-      const int i = (int)(G.rowent[q] >> 16);
-      if (B.status[i] == -1) found = i;
+    const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 64 + 2 * (j & 31);
+    const int width = 2 * (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+    for (int u = g.rank; u < width; u += g.size) {
+      const int i = (int)(re[64 * (u >> 1) + (u & 1)] >> 2);
+      if (i < G.ns && B.status[i] == -1) found = i;  // (the dummy column is no VN)
     }
     const int i = (int)g.min_u((unsigned)found);
     if (i == kNone) return -2;
     const int v = (int)bit_of(B.sp, j);
     g.sync();
-    if (g.rank == 0) decimate_one(G, B, i, v);
+    if (g.rank == 0) act -= decimate_one(G, B, i, v);
     g.sync();
     ++npeel;
   }
@@ -561,12 +694,13 @@ __device__ __forceinline__ uint32_t ranker_pair(const ShortG& G, const Slot& B, 
     hi = hv2;
   } else if (tig == 2) {
     int nus = 0;
-    for (int e = G.colptr[k]; e < G.colptr[k + 1]; ++e) nus += bit_of(B.unsat, G.colrows[e]);
+    const uint32_t* ce = G.col_ents(k);
+    for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
     lo = hv3;
     hi = (float)min(nus, 127);
   } else {
     lo = (float)G.vdeg[k];
-    hi = (float)min(G.cperm[G.colrows[G.colptr[k]]] / G.rpb, 255);
+    hi = (float)min(G.cperm[*G.col_ents(k) >> 16] / G.rpb, 255);
   }
   return bf16x2_exact(lo, hi);
 }
@@ -635,7 +769,8 @@ __device__ void dump_candidates(const KParams& P, const ShortG& G, const Slot& B
     if (!ranker_candidate(G, B, k)) continue;
     const uint32_t h4 = *(const uint32_t*)(B.hq + 4 * k);
     int nus = 0;
-    for (int e = G.colptr[k]; e < G.colptr[k + 1]; ++e) nus += bit_of(B.unsat, G.colrows[e]);
+    const uint32_t* ce = G.col_ents(k);
+    for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
     const float L = B.acc[k];
     const int pos = atomicAdd(P.dump_n, 1);
     if (pos >= P.dump_cap) continue;
@@ -647,7 +782,7 @@ __device__ void dump_candidates(const KParams& P, const ShortG& G, const Slot& B
     r.x[4] = (float)(int8_t)(h4 >> 24) * 0.5f;
     r.x[5] = (float)min(nus, 127);
     r.x[6] = (float)G.vdeg[k];
-    r.x[7] = (float)min(G.cperm[G.colrows[G.colptr[k]]] / G.rpb, 255);
+    r.x[7] = (float)min(G.cperm[*G.col_ents(k) >> 16] / G.rpb, 255);
     r.shot = (int32_t)shot;
     r.wcol = G.sel[G.vperm[k]];
     r.depth = (int16_t)D;
@@ -672,22 +807,23 @@ __device__ double path_metric(const ShortG& G, const Slot& B, const Grp& g) {
 
 // H e = s for the current decisions (Eq. (4), decimated VNs through s'):
 // writes every check's unsatisfied bit to B.unsat and returns whether any is
-// unsatisfied.  Checks in natural order, one per lane.
+// unsatisfied.  Checks in label order, one per lane.
 template <class Grp>
 __device__ bool parity_pass(const ShortG& G, const Slot& B, const Grp& g) {
   bool any = false;
-  for (int base = 0; base < G.nr; base += g.size) {
-    const int j = base + g.rank;
-    bool u = false;
-    if (j < G.nr) {
-      uint32_t hp = bit_of(B.sp, j);
-      for (int q = G.rowptr[j]; q < G.rowptr[j + 1]; ++q) hp ^= B.post[G.rowent[q] >> 16] <= 0.0f;  // NaN: decimated
-      u = hp != 0u;
+  for (int s = g.rank >> 5; s < G.rw; s += g.size >> 5) {
+    const int lane = g.rank & 31;
+    uint32_t hp = ((B.sp[s] >> lane) & 1u) << 31;
+    const uint2* ent = (const uint2*)G.rent + (int)G.roff[s] * 32 + lane;
+    const int np = (int)G.roff[s + 1] - (int)G.roff[s];
+    for (int p = 0; p < np; ++p) {
+      const uint2 e = ent[32 * p];
+      hp ^= (__float_as_uint(*(const float*)((const char*)B.post + e.x)) - 1u) ^
+            (__float_as_uint(*(const float*)((const char*)B.post + e.y)) - 1u);
     }
-    const unsigned m = __ballot_sync(FULL, u);
-    const int w0 = base + (g.rank & ~31);
-    if ((g.rank & 31) == 0 && w0 < G.nr) B.unsat[w0 >> 5] = m;
-    any |= u;
+    const unsigned m = __ballot_sync(FULL, (hp >> 31) != 0u);
+    if (lane == 0) B.unsat[s] = m;
+    any |= m != 0u;
   }
   return g.any(any);
 }
@@ -711,7 +847,8 @@ struct PathOut {
 // resume there from a snapshot another path left instead of recomputing the
 // prefix from the root.  A snapshot is a 32-byte header (depth, iterations,
 // iterations since the messages were initialised, the `first` flag, the
-// producing path, the prefix's edge visits) and a copy of the slot.
+// producing path, the active edges, the prefix's edge visits) and a copy of
+// the slot.
 //
 // Preemption (sched): the paths of a shot outnumber the warps, and the main
 // branch is the longest, so a fixed assignment leaves warps idle at the end
@@ -742,7 +879,7 @@ enum { PS_QUEUED = 0, PS_RUNNING = 1, PS_PARKED = 2, PS_DONE = 3 };
 // Snapshot of a path's state after the BP of step D (all lanes of the group).
 template <class Grp>
 __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D, int iters, int tw, bool first,
-                               int producer, long long vs) {
+                               int producer, int act, long long vs) {
   if (g.rank == 0) {
     int* h = (int*)dst;
     __stcg(h, D);
@@ -750,6 +887,7 @@ __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D,
     __stcg(h + 2, tw);
     __stcg(h + 3, first ? 1 : 0);
     __stcg(h + 4, producer);
+    __stcg(h + 5, act);
     __stcg((long long*)(dst + 24), vs);
   }
   const uint4* s4 = (const uint4*)F.slot;
@@ -759,83 +897,50 @@ __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D,
   g.sync();
 }
 
-// Check-node update of Eq. (1) over the active VNs of one decision path, TPC
-// lanes per check (a template parameter, so that the loops and the group
-// reduction are unrolled for it); checks in label order (descending static
-// degree): the lanes of a round loop alike.  Each check also takes the parity
-// of its active VNs' hard decisions (Eq. (4)) from the posteriors it reads:
-// for it >= 2 this pass is the convergence test H e = s of the previous
-// iteration (Sec. II-A).  Returns whether this lane saw an unsatisfied check.
-template <bool LW, int TPC, int FM>
-__device__ __forceinline__ bool check_pass_fm(const KParams& P, const ShortG& G, const Slot& B, int R, int S,
-                                              bool first_rt, int tw, long long& visits) {
-  // FM: 0 the first-iteration flag at run time, 1 / 2 fixed true / false
-  const bool first = FM == 0 ? first_rt : FM == 1;
-  const int nr = G.nr, sub = R & (TPC - 1);
-  const int nr_rounds = (nr + S / TPC - 1) / (S / TPC) * (S / TPC);
-  bool unsat = false;
-  int nvis = 0;  // this pass's active edge visits (added to the 64-bit count once)
-  for (int j0 = R / TPC; j0 < nr_rounds; j0 += S / TPC) {
-    const int j = j0 < nr ? j0 : nr - 1;
-    const int d = j0 < nr ? B.deg[j] : 0;
-    if (TPC == 1 && d == 0) {  // no shuffle partner waits for this lane
-      if (j0 < nr) unsat |= bit_of(B.sp, j) != 0u;
-      continue;
-    }
-    const CNState oc = B.cns[j];
-    float m1 = CUDART_INF_F, m2 = CUDART_INF_F;
-    int am = 0xFFFF;
-    uint32_t neg = 0, hp = 0;
-    // one row entry; the (min1, min2) pair and so every message do not
-    // depend on the order in which a check sees its inputs
-    // (no branch: a NaN input -- the stale message of a decimated VN, or no
-    // entry -- takes part with magnitude +inf and writes nothing)
-    auto take = [&](uint32_t ent, float pv, uint32_t sg) {
-      const bool live = pv == pv;
-      hp ^= pv <= 0.0f;  // false for NaN
-      const int e = (int)(ent & 0xFFFFu);
-      // the previous iteration's multiplier, only when there was one (tw >= 1)
-      const float wprev = (LW && !first) ? edge_weight(G.wts, G.wT, G.wE, P.alpha, tw, G.efull[e]) : P.alpha;
-      const float v = first ? pv : clipf(__fsub_rn(pv, c2v<LW>(wprev, P.clip, oc, e, sg)), P.clip);
-      const float a = live ? fabsf(v) : CUDART_INF_F;
-      am = a < m1 ? e : am;
-      m2 = fminf(m2, fmaxf(m1, a));
-      m1 = fminf(m1, a);
-      const uint32_t sgn = v < 0.0f;  // false for a NaN input: clipf gives +clip, the first pass NaN
-      neg ^= sgn;
-      if (live) B.sign[e] = (uint8_t)sgn;
-    };
-    if (sub == 0) nvis += d;  // the row's active entries (B.deg counts the active VNs of a check)
-    const int qe = d ? (int)(oc.pad >> 16) : 0;
-    for (int q = (d ? (int)(oc.pad & 0xFFFFu) : 0) + 2 * sub; q < qe; q += 2 * TPC) {
-      const bool two = q + 1 < qe;
-      const uint32_t e0 = G.rowent[q], e1 = two ? G.rowent[q + 1] : e0;
-      const float p0 = B.post[e0 >> 16], p1 = two ? B.post[e1 >> 16] : stale();
-      const uint32_t s0 = B.sign[e0 & 0xFFFFu], s1 = B.sign[e1 & 0xFFFFu];
-      take(e0, p0, s0);
-      take(e1, p1, s1);
-    }
-    if (TPC > 1) {
-      group_min2(m1, m2, am, neg, TPC);
-      for (int off = TPC >> 1; off; off >>= 1) hp ^= __shfl_xor_sync(FULL, hp, off);
-    }
-    if (sub == 0 && j0 < nr) unsat |= (hp ^ bit_of(B.sp, j)) != 0u;
-    if (sub == 0 && d > 0)
-      B.cns[j] = cn_store<LW>(P.alpha, P.clip, m1, m2, am, neg ^ bit_of(B.sp, j), d == 1, oc.pad);
+// Check-node update of Eq. (1) over the active VNs of one decision path; a
+// warp takes a slice with one check per lane, a CTA tpc lanes per check.  Each
+// check also takes the parity of its active VNs' hard decisions (Eq. (4)) from
+// the posteriors it reads: for it >= 2 this pass is the convergence test
+// H e = s of the previous iteration (Sec. II-A).  Returns whether this lane saw
+// an unsatisfied check.
+template <bool LW, bool FIRST>
+__device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& G, const Slot& B, int lane, int tw) {
+  LwRow lw{nullptr, G.ref};
+  if (LW && !FIRST) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
+  uint32_t unsat = 0u;
+  int r0 = G.roff[0];
+  for (int s = 0; s < G.rw; ++s) {
+    const int r1 = G.roff[s + 1];
+    unsat |= check_lane<LW, FIRST>((const uint2*)G.rent + r0 * 32 + lane, r1 - r0, (const char*)B.post,
+                                   B.cns + 32 * s + lane, (B.sp[s] >> lane) & 1u, P.alpha, P.clip, lw,
+                                   (r0 * 32 + lane) * 2);
+    r0 = r1;
   }
-  visits += nvis;
-  return unsat;
+  return unsat != 0u;
 }
 
-// One-warp paths (TPC 1) run a copy specialised for the first iteration after
-// the messages were (re)initialised and one for the others.
-template <bool LW, int TPC>
-__device__ __forceinline__ bool check_pass(const KParams& P, const ShortG& G, const Slot& B, int R, int S, bool first,
-                                           int tw, long long& visits) {
-  if (TPC == 1)
-    return first ? check_pass_fm<LW, TPC, 1>(P, G, B, R, S, true, tw, visits)
-                 : check_pass_fm<LW, TPC, 2>(P, G, B, R, S, false, tw, visits);
-  return check_pass_fm<LW, TPC, 0>(P, G, B, R, S, first, tw, visits);
+template <bool LW>
+__device__ __forceinline__ bool check_pass_cta(const KParams& P, const ShortG& G, const Slot& B, int R, int S, int tpc,
+                                               bool first, int tw) {
+  LwRow lw{nullptr, G.ref};
+  if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
+  const int nrp = 32 * G.rw, per = S / tpc, sub = R & (tpc - 1);
+  uint32_t unsat = 0u;
+  for (int b = 0; b < nrp; b += per) {
+    const int j0 = b + R / tpc;
+    const int j = j0 < nrp ? j0 : nrp - 1, s = j >> 5;
+    const int r0 = G.roff[s], np = j0 < nrp ? (int)G.roff[s + 1] - r0 : 0;
+    const uint32_t sbit = (B.sp[s] >> (j & 31)) & 1u;
+    uint32_t u = 0u;
+    const CNState rec =
+        check_group<LW>((const uint2*)G.rent + r0 * 32 + (j & 31), np, (const char*)B.post, B.cns[j], sbit, P.alpha,
+                        P.clip, first, lw, (r0 * 32 + (j & 31)) * 2, sub, tpc, (G.coff[0] & kWideSlice) != 0, u);
+    if (sub == 0 && j0 < nrp) {
+      B.cns[j] = rec;
+      unsat |= u;
+    }
+  }
+  return unsat != 0u;
 }
 
 // One decision path of Alg. 2 on the shortened window, run by group g.
@@ -847,8 +952,6 @@ template <bool LW, class Grp>
 __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id, const Grp& g,
                         const PathOut& out, int dmx, const ForkCtx& F, unsigned* claimed = nullptr) {
   const int nr = G.nr, ns = G.ns, R = g.rank, S = g.size;
-  // one lane per check for a warp; small lane groups per check for a CTA
-  const int tpc = Grp::kWarp ? 1 : path_lanes_per_check(S, nr);
   // Fig. 2: main branch (id 0), tree branches, side branches (split > 0),
   // which keep the main-branch thresholds up to and including their split
   const int split = path_split(P, id);
@@ -858,6 +961,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
   int status = BR_MAXDEPTH, depth = 0, iters = 0;
   int tw = 0;  // iterations since the messages were (re)initialised (learned weights)
   long long visits = 0, inherited = 0;  // executed here / the resumed prefix's (lane 0)
+  int act = 0;  // active edges, summed over the lanes (each subtracts what it decimates)
   double pm = CUDART_INF;
   bool first = true;
   int D0 = 1;  // first depth of this run: resumed runs start at its SELECT-VN
@@ -870,6 +974,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     tw = __ldcg(h + 2);
     first = __ldcg(h + 3) != 0;
     const int producer = __ldcg(h + 4);
+    if (R == 0) act = __ldcg(h + 5);
     if (R == 0) inherited = __ldcg((const long long*)(F.src + 24));
     const uint4* s4 = (const uint4*)(F.src + kSnapHeader);
     uint4* d4 = (uint4*)F.slot;
@@ -888,14 +993,21 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     }
     g.sync();
   } else {
-    for (int k = R; k < ns; k += S) {
-      B.status[k] = -1;
-      B.post[k] = G.llr[k];  // t = 0: mu_{i->j} = Lambda_i (Sec. II-A)
+    const int nrp = 32 * G.rw, nsp = 32 * G.cw;
+    for (int k = R; k <= nsp; k += S) {  // (past ns: no VN; nsp: the dummy column)
+      if (k < nsp) B.status[k] = k < ns ? -1 : 0;
+      B.post[k] = k < ns ? G.llr[k] : dead_post();  // t = 0: mu_{i->j} = Lambda_i (Sec. II-A)
+      if (k < ns) act += G.vdeg[k];
     }
-    for (int j = R; j < nr; j += S) {
-      B.deg[j] = G.rowptr[j + 1] - G.rowptr[j];
-      B.cns[j].pad = (uint32_t)G.rowptr[j] | ((uint32_t)G.rowptr[j + 1] << 16);
+    for (int j = R; j < nrp; j += S) {
+      // active VNs of the check: its entries that are not the dummy column
+      const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 64 + 2 * (j & 31);
+      const int np = (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+      int d = 0;
+      for (int p = 0; p < np; ++p) d += (int)(re[64 * p] < 4u * nsp) + (int)(re[64 * p + 1] < 4u * nsp);
+      B.deg[j] = (uint8_t)d;
     }
+    if (R == 0) B.cns[nrp] = CNState{0.0f, 0.0f, 0u, 0u};  // the dummy check: message +0
     for (int base = 0; base < nr; base += S) {  // the window syndrome by check label
       const int j = base + R;
       const unsigned m = __ballot_sync(FULL, j < nr && bit_of(G.sbits, G.cperm[j]));
@@ -905,7 +1017,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       for (int q = R; q < dmx; q += S) out.st[q] = StepTrace{-2, -1, 0, 0, 0};
     g.sync();
     if (P.peel_init) {
-      const int np = peel(G, B, g);
+      const int np = peel(G, B, g, act);
       if (np < 0) {
         status = np == -1 ? BR_CONTRADICTION : BR_INTERNAL;
         goto done;
@@ -920,13 +1032,12 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // ---- check-node update, Eq. (1), and the previous iteration's H e = s ----
       bool unsat;
       if constexpr (Grp::kWarp) {
-        unsat = check_pass<LW, 1>(P, G, B, R, S, first, tw, visits);
+        unsat = first ? check_pass_warp<LW, true>(P, G, B, R, tw) : check_pass_warp<LW, false>(P, G, B, R, tw);
+        __syncwarp();
       } else {
-        if (tpc == 8) unsat = check_pass<LW, 8>(P, G, B, R, S, first, tw, visits);
-        else if (tpc == 4) unsat = check_pass<LW, 4>(P, G, B, R, S, first, tw, visits);
-        else if (tpc == 2) unsat = check_pass<LW, 2>(P, G, B, R, S, first, tw, visits);
-        else unsat = check_pass<LW, 1>(P, G, B, R, S, first, tw, visits);
+        unsat = check_pass_cta<LW>(P, G, B, R, S, path_lanes_per_check(S, nr), first, tw);
       }
+      visits += act;
       if (!g.any(unsat) && it >= 2) {  // the previous iteration's decisions satisfy H e = s
         status = BR_CONVERGED;
         pm = path_metric(G, B, g);
@@ -935,25 +1046,18 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // ---- variable-node update, Eq. (2)-(3); history of Sec. IV-A ----
       const bool hist = it > ips - 4;
       const bool hist0 = it == ips - 3;
-      // variables in label order (descending degree): the lanes of a round loop alike
-      for (int k = R; k < ns; k += S) {
-        // (a decimated column runs the loop too, without a branch, and stores nothing)
-        const bool act = B.status[k] == -1;
-        float p = G.llr[k];
-        const int eb = G.colptr[k], ee = G.colptr[k + 1];
-        auto msg = [&](int e) {
-          const float wt = LW ? edge_weight(G.wts, G.wT, G.wE, P.alpha, tw + 1, G.efull[e]) : P.alpha;
-          return c2v<LW>(wt, P.clip, B.cns[G.colrows[e]], e, B.sign[e]);
-        };
-        // ascending check order (Eq. (2)); most short columns have degree 1 or 2
-        int e = eb;
-        for (; e + 1 < ee; e += 2) {
-          const float c0 = msg(e), c1 = msg(e + 1);
-          p = __fadd_rn(p, c0);
-          p = __fadd_rn(p, c1);
-        }
-        if (e < ee) p = __fadd_rn(p, msg(e));
-        if (!act) continue;
+      // variables in label order; a decimated column runs the loop too and stores nothing
+      LwRow lw{nullptr, G.cef};
+      if (LW) lw.w = weight_row(G.wts, G.wT, G.wE, tw + 1);
+      for (int k = R; k < 32 * G.cw; k += S) {
+        const int sl = k >> 5;
+        const int cw = G.coff[sl], c0 = cw & (kWideSlice - 1), n = (int)(G.coff[sl + 1] & (kWideSlice - 1)) - c0;
+        const bool wide = (cw & kWideSlice) != 0;
+        const int ei = c0 * 32 + (k & 31);
+        const float p0 = G.llr[k];
+        const float p = wide ? column_sum<LW>(p0, G.cent + ei, n, true, (const char*)B.cns, lw, ei)
+                             : column_sum<LW>(p0, G.cent + ei, n, false, (const char*)B.cns, lw, ei);
+        if (B.status[k] != -1) continue;
         B.post[k] = p;
         if (hist) {
           if (P.rkq || P.dump) B.hq[4 * k + (it - (ips - 3))] = qhist(p);
@@ -989,7 +1093,8 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       int won = 0;
       if (R == 0) won = atomicCAS(&F.flags[n], 0, 1) == 0;
       if (g.any(won != 0)) {
-        write_snapshot(F.pool + (size_t)n * F.stride, F, g, D, iters, tw, first, id, g.sum_ll(visits + inherited));
+        write_snapshot(F.pool + (size_t)n * F.stride, F, g, D, iters, tw, first, id, g.sum_i(act),
+                       g.sum_ll(visits + inherited));
         if (R == 0) atomicExch(&F.flags[n], 2);
       }
     }
@@ -1023,7 +1128,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
         if (claimed) *claimed = cw0;
         // park: this path resumes from its own snapshot after the BP of step D
         const long long own = g.sum_ll(visits);
-        write_snapshot(F.pool + (size_t)(F.n_nodes + id) * F.stride, F, g, D, iters, tw, first, id,
+        write_snapshot(F.pool + (size_t)(F.n_nodes + id) * F.stride, F, g, D, iters, tw, first, id, g.sum_i(act),
                        g.sum_ll(visits + inherited));
         if (R == 0) {
           atomicExch(&F.sched[id], (unsigned)PS_PARKED | ((unsigned)D << 8));
@@ -1048,12 +1153,13 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
         const uint8_t fl = B.hfl[k];
         if (!P.low_err) {
           int nus = 0;
-          for (int e = G.colptr[k]; e < G.colptr[k + 1]; ++e) nus += bit_of(B.unsat, G.colrows[e]);
+          const uint32_t* ce = G.col_ents(k);
+          for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
           int bdec = -1;
           if ((fl & pa_bit) && L < PBd) bdec = 1;
           else if (((fl & 4) && D <= P.pc_max_depth) || ((fl & 8) && nus >= P.n_unsat_min)) bdec = 0;
           if (bdec >= 0) {
-            decimate_atomic(G, B, k, bdec);
+            act -= decimate_atomic(G, B, k, bdec);
             ++nagg;
             continue;
           }
@@ -1100,9 +1206,9 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       } else if (D <= P.k) {
         v = ((id >> (P.k - D)) & 1) ? 1 - f : f;  // b + (-1)^b f
       }
-      if (R == 0) decimate_one(G, B, gsel, v);
+      if (R == 0) act -= decimate_one(G, B, gsel, v);
       g.sync();
-      const int np = peel(G, B, g);
+      const int np = peel(G, B, g, act);
       if (out.st && R == 0)
         out.st[D - 1] = StepTrace{(int16_t)G.vperm[gsel], (int8_t)v, 0, (int16_t)nagg, (int16_t)(np < 0 ? -1 : np)};
       if (np < 0) {
@@ -1226,6 +1332,13 @@ template <bool UG>
 __device__ __forceinline__ char* union_base(const DecodeArgs& A, char* sm) {
   if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
   return sm + A.L.U;
+}
+// The pre-BP scratch: the union region in global memory, else the bytes of the
+// shortened graph and the path slots, which do not exist yet.
+template <bool UG>
+__device__ __forceinline__ char* prebp_base(const DecodeArgs& A, char* sm) {
+  if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
+  return sm + A.L.V;
 }
 
 // One window step of several decoders in one launch (kernel parameter).
@@ -1423,183 +1536,121 @@ __device__ __forceinline__ unsigned cl_map(const void* p, unsigned rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
-__device__ __forceinline__ float cl_ld_f32(unsigned a) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t cl_ld_u32(unsigned a) {
-  uint32_t v;
-  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t cl_ld_u8(unsigned a) {
-  uint16_t v;
-  asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=h"(v) : "r"(a));
-  return v;
-}
 __device__ __forceinline__ void cl_st_f32(unsigned a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 __device__ __forceinline__ void cl_st_u32(unsigned a, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ CNState cl_ld_cns(unsigned a) {
-  CNState c;
-  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(c.m1), "=f"(c.m2), "=r"(c.ac), "=r"(c.pad)
-               : "r"(a));
-  return c;
+__device__ __forceinline__ void cl_st_cns(unsigned a, const CNState& c) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(__float_as_uint(c.m1)),
+               "r"(__float_as_uint(c.m2)), "r"(c.sg), "r"(c.am)
+               : "memory");
+}
+
+// The pre-BP's arrays and graph, all by label.
+struct PreBp {
+  float *post, *key;
+  CNState* cns;
+  const uint32_t* sp;  // the window syndrome
+  const uint32_t *rent, *cent;
+  const uint16_t *roff, *coff;
+  const float* llr;
+};
+
+// One variable of the pre-BP: its posterior, and from iteration tk0 on its
+// ranking key (the running sum of the last four posteriors, Sec. III, padded
+// with the prior when n_pre < 4).
+template <bool LW>
+__device__ __forceinline__ float prebp_column(const KParams& P, const WinDev& W, const PreBp& X, int l, int t) {
+  const int sl = l >> 5;
+  const int cw = X.coff[sl], c0 = cw & (kWideSlice - 1), n = (int)(X.coff[sl + 1] & (kWideSlice - 1)) - c0;
+  const int ei = c0 * 32 + (l & 31);
+  LwRow lw{nullptr, W.s_cef};
+  if (LW) lw.w = weight_row(W.wts, W.wT, W.n_edges, t);
+  if (cw & kWideSlice) return column_sum<LW>(X.llr[l], X.cent + ei, n, true, (const char*)X.cns, lw, ei);
+  return column_sum<LW>(X.llr[l], X.cent + ei, n, false, (const char*)X.cns, lw, ei);
+}
+
+__device__ __forceinline__ float prebp_key(const KParams& P, const PreBp& X, int l, int t, int tk0, float p) {
+  if (t != tk0) return __fadd_rn(X.key[l], p);
+  if (P.n_pre >= 4) return p;
+  const float li = X.llr[l];
+  float s = li;
+  for (int r = 1; r < 4 - P.n_pre; ++r) s = __fadd_rn(s, li);
+  return __fadd_rn(s, p);
 }
 
 // a2 split over the CTAs of a cluster (path mode, one cluster per shot): CTA
 // r owns the r-th slice of the checks and of the variables, runs the check
 // pass of Eq. (1) for its checks and the variable pass of Eq. (2)-(3) for its
 // variables.  A remote load costs a round trip of ~1200 cycles (a cluster
-// barrier ~470), so values travel the cheap way: each CTA pushes its
-// posteriors (and ranking keys) and its "unsatisfied" flag into every CTA's
-// shared memory before the barrier that ends the pass, and the check pass
-// reads them locally; the variable pass requests a variable's check states
-// and signs from their owners in one round trip.  Two cluster barriers per
-// iteration separate the passes, so every value read was written in the pass
-// before, and after the last one no CTA touches another's shared memory.
+// barrier ~470), so values only travel as stores: each CTA pushes the records
+// of its checks, its posteriors (and ranking keys) and its "unsatisfied" flag
+// into every CTA's shared memory before the barrier that ends the pass, and
+// both passes read locally.  Two cluster barriers per iteration separate the
+// passes, so every value read was written in the pass before, and after the
+// last one no CTA touches another's shared memory.
 // The arithmetic of every message and posterior is that of the single-CTA
 // loop; at the end every CTA holds the whole posterior and key.  Returns t as
 // the loop leaves it; conv and t_conv as in the caller.
 template <bool LW>
-__device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const WinDev& Wg, char* sm, char* U,
-                             const uint32_t* sbits, bool& conv, int& t_conv) {
+__device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& X, char* sm, bool& conv, int& t_conv) {
   const KParams& P = A.P;
-  const Layout& L = A.L;
   const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
   const int nr = W.n_rows, nc = W.n_cols;
   const unsigned C = cl_size(), r = cl_rank();
-  float* post = (float*)(U + L.p_post);
-  float* key = (float*)(U + L.p_key);
-  CNState* cns = (CNState*)(U + L.p_cns);
-  uint8_t* sign = (uint8_t*)(U + L.p_sign);
   // flags[8 * parity + c]: CTA c found an unsatisfied check (in the reduction
   // scratch of the path phase, idle until the pre-BP ends)
-  int* flags = (int*)(sm + L.red);
-  // slices; the owner of check j is floor(j / sc) = umulhi(j, ceil(2^32 / sc)), exact for j, sc < 2^16
+  int* flags = (int*)(sm + A.L.red);
   const int sc = (nr + (int)C - 1) / (int)C, sv = (nc + (int)C - 1) / (int)C;
-  const unsigned mc = (unsigned)((0x100000000ull + sc - 1) / sc);
   const int jb = min(nr, (int)r * sc), je = min(nr, jb + sc);
   const int ib = min(nc, (int)r * sv), ie = min(nc, ib + sv);
-  const int tpc = lanes_per_check(NT, max(1, je - jb)), sub = tid & (tpc - 1);
-  const int nrr = (je - jb + NT / tpc - 1) / (NT / tpc) * (NT / tpc);
+  int tpc = 1;  // lanes per check: the most (<= 16) that take the slice in one round
+  while (tpc < 16 && 2 * tpc * max(1, je - jb) <= NT) tpc <<= 1;
+  const int sub = tid & (tpc - 1), per = NT / tpc;
   const int tk0 = P.n_pre - 3 > 1 ? P.n_pre - 3 : 1;
+  const bool rwide = X.roff[1] - X.roff[0] > 16;  // the first slice is the widest
+  cl_sync();  // every CTA of the cluster runs and has set up its arrays
   int t;
   for (t = 1; t <= P.n_pre; ++t) {
-    bool unsat = false;
-    for (int j0 = tid / tpc; j0 < nrr; j0 += NT / tpc) {
-      const bool real = jb + j0 < je;
-      const int j = real ? jb + j0 : je - 1;
-      const int beg = Wg.row_ptr[j], end = real ? Wg.row_ptr[j + 1] : beg;
-      const CNState oc = cns[j];
-      float m1 = CUDART_INF_F, m2 = CUDART_INF_F;
-      int am = 0xFFFF;
-      uint32_t neg = 0, hp = 0;
-      for (int q = beg + 4 * sub; q < end; q += 4 * tpc) {
-        uint32_t ent[4];
-        float pv[4];
-        uint32_t sg[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ent[u] = (q + u < end) ? Wg.row_ent[q + u] : 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const unsigned i = ent[u] >> 16, e = ent[u] & 0xFFFFu;
-          pv[u] = 0.0f;
-          sg[u] = 0u;
-          if (q + u < end) {
-            pv[u] = post[i];  // t = 1: the first VN->CN message (the prior, or the value kept for the column)
-            sg[u] = sign[e];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (q + u >= end) break;
-          const int e = (int)(ent[u] & 0xFFFFu);
-          hp ^= pv[u] <= 0.0f;
-          const float wprev = (LW && t > 1) ? edge_weight(W.wts, W.wT, W.n_edges, P.alpha, t - 1, e) : P.alpha;
-          const float v = (t == 1) ? pv[u] : clipf(__fsub_rn(pv[u], c2v<LW>(wprev, P.clip, oc, e, sg[u])), P.clip);
-          const float a = fabsf(v);
-          am = a < m1 ? e : am;
-          m2 = fminf(m2, fmaxf(m1, a));
-          m1 = fminf(m1, a);
-          const uint32_t sgn = v < 0.0f;
-          neg ^= sgn;
-          sign[e] = (uint8_t)sgn;
-        }
-      }
-      if (tpc > 1) {
-        group_min2(m1, m2, am, neg, tpc);
-        for (int off = tpc >> 1; off; off >>= 1) hp ^= __shfl_xor_sync(FULL, hp, off);
-      }
-      if (sub == 0 && real) {
-        cns[j] = cn_store<LW>(P.alpha, P.clip, m1, m2, am, neg ^ bit_of(sbits, j), end - beg == 1, 0u);
-        unsat |= (hp ^ bit_of(sbits, j)) != 0u;
+    LwRow lw{nullptr, W.s_ref};
+    if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
+    uint32_t unsat = 0u;
+    for (int b = jb; b < je; b += per) {
+      const int j0 = b + tid / tpc;
+      const bool real = j0 < je;
+      const int j = real ? j0 : je - 1, s = j >> 5;
+      const int r0 = X.roff[s], np = real ? (int)X.roff[s + 1] - r0 : 0;
+      uint32_t u = 0u;
+      const CNState rec = check_group<LW>((const uint2*)X.rent + r0 * 32 + (j & 31), np, (const char*)X.post, X.cns[j],
+                                          (X.sp[s] >> (j & 31)) & 1u, P.alpha, P.clip, t == 1, lw,
+                                          (r0 * 32 + (j & 31)) * 2, sub, tpc, rwide, u);
+      if (real) {
+        for (int c = sub; c < (int)C; c += tpc) cl_st_cns(cl_map(&X.cns[j], (unsigned)c), rec);
+        unsat |= u;
       }
     }
-    const int lu = __syncthreads_or(unsat);
+    const int lu = __syncthreads_or(unsat != 0u);
     if (tid < (int)C) cl_st_u32(cl_map(&flags[8 * (t & 1) + (int)r], (unsigned)tid), (uint32_t)lu);
-    cl_sync();  // check states, signs and flags of pass t
+    cl_sync();  // check records and flags of pass t, in every CTA
     const bool any = __any_sync(FULL, lane < (int)C && flags[8 * (t & 1) + lane] != 0);
     if (!any && t >= 2) {  // iteration t-1 satisfies H e = s in every slice
       conv = true;
       t_conv = t - 1;
       break;
     }
-    const bool kacc = t >= tk0;
     for (int i = ib + tid; i < ie; i += NT) {
-      float p = Wg.llr[i];
-      const int eb = Wg.col_ptr[i], ee = Wg.col_ptr[i + 1];
-      // up to six messages requested at once (the column degree of these
-      // windows), then added in ascending check order (Eq. (2))
-      for (int e0 = eb; e0 < ee; e0 += 6) {
-        CNState c[6];
-        uint32_t sg[6];
-#pragma unroll
-        for (int u = 0; u < 6; ++u)
-          if (e0 + u < ee) {
-            const unsigned j = Wg.col_rows[e0 + u], o = __umulhi(j, mc);
-            c[u] = cl_ld_cns(cl_map(&cns[j], o));
-            sg[u] = cl_ld_u8(cl_map(&sign[e0 + u], o));
-          }
-#pragma unroll
-        for (int u = 0; u < 6; ++u)
-          if (e0 + u < ee) {
-            const float wt = LW ? edge_weight(W.wts, W.wT, W.n_edges, P.alpha, t, e0 + u) : P.alpha;
-            p = __fadd_rn(p, c2v<LW>(wt, P.clip, c[u], e0 + u, sg[u]));
-          }
-      }
-      post[i] = p;
+      const float p = prebp_column<LW>(P, W, X, i, t);
       for (unsigned c = 0; c < C; ++c)  // every CTA reads the whole posterior in its check pass
-        if (c != r) cl_st_f32(cl_map(&post[i], c), p);
-      if (kacc) {
-        float kv;
-        if (t == tk0) {
-          if (P.n_pre < 4) {
-            const float li = Wg.llr[i];
-            float s = li;
-            for (int q = 1; q < 4 - P.n_pre; ++q) s = __fadd_rn(s, li);
-            kv = __fadd_rn(s, p);
-          } else {
-            kv = p;
-          }
-        } else {
-          kv = __fadd_rn(key[i], p);
-        }
-        key[i] = kv;
-        for (unsigned c = 0; c < C; ++c)
-          if (c != r) cl_st_f32(cl_map(&key[i], c), kv);
+        cl_st_f32(cl_map(&X.post[i], c), p);
+      if (t >= tk0) {
+        const float kv = prebp_key(P, X, i, t, tk0, p);
+        for (unsigned c = 0; c < C; ++c) cl_st_f32(cl_map(&X.key[i], c), kv);
       }
     }
     cl_sync();  // posteriors (and keys) of pass t, in every CTA
   }
-  // every CTA holds the whole posterior and key: the last variable pass
-  // pushed them before the barrier that ended the loop, and no CTA touches
-  // another's shared memory after it
   return t;
 }
 
@@ -1610,22 +1661,20 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
                               Stager& stg) {
   const KParams& P = A.P;
   const Layout& L = A.L;
-  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nr = W.n_rows, nc = W.n_cols;
+  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
+  const int nr = W.n_rows, nc = W.n_cols, rw = L.rw, ncp = 32 * L.cw, nrp = 32 * rw;
   uint32_t* sbits = (uint32_t*)(sm + L.sbits);
   uint32_t* cbits = (uint32_t*)(sm + L.cbits);
-  uint16_t* sel = (uint16_t*)(sm + L.sel);
-  char* U = union_base<UG>(A, sm);
+  char* U = prebp_base<UG>(A, sm);
   float* post = (float*)(U + L.p_post);
   float* key = (float*)(U + L.p_key);
   CNState* cns = (CNState*)(U + L.p_cns);
-  uint8_t* sign = (uint8_t*)(U + L.p_sign);
   uint32_t* parb = (uint32_t*)(U + L.p_par);
-  unsigned long long* sortb = (unsigned long long*)(U + L.p_sort);
+  uint32_t* spre = parb + rw;  // the window syndrome by check label
 
   // ---- a1: window syndrome ----
   const uint32_t* dp = A.det + (size_t)shot * A.det_words;
-  for (int x = tid; x < L.rw; x += NT) {
+  for (int x = tid; x < rw; x += NT) {
     const int b0 = W.row0 + 32 * x;
     const uint32_t lo = dp[b0 >> 5];
     const uint32_t hi = ((b0 >> 5) + 1 < A.det_words) ? dp[(b0 >> 5) + 1] : 0u;
@@ -1638,242 +1687,166 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   for (int x = tid; x < L.cw; x += NT) cbits[x] = 0;
   __syncthreads();
 
-  // the window graph in shared memory for the pre-BP loop when the union
-  // region has room (shot mode); the ranking and shortening below read W
-  WinDev Wg = W;
+  // the window graph in shared memory for the pre-BP loop when there is room
+  PreBp X{post, key, cns, spre, W.s_rent, W.s_cent, W.s_roff, W.s_coff, W.s_llr};
   if (L.pre_stage) {
-    uint16_t* cp = (uint16_t*)(U + L.q_colptr);
-    uint16_t* cr = (uint16_t*)(U + L.q_colrows);
-    uint16_t* rp = (uint16_t*)(U + L.q_rowptr);
-    uint32_t* re = (uint32_t*)(U + L.q_rowent);
-    float* ll = (float*)(U + L.q_llr);
-    uint16_t* vp = (uint16_t*)(U + L.q_vperm);
-    const StagePiece pc[6] = {{cp, W.col_ptr, al16(2u * (nc + 1))},       {cr, W.col_rows, al16(2u * W.n_edges)},
-                              {rp, W.row_ptr, al16(2u * (nr + 1))},       {re, W.row_ent, al16(4u * W.n_edges)},
-                              {ll, W.llr, al16(4u * nc)},                 {vp, W.vperm, al16(2u * nc)}};
-    stage_pieces(stg, pc, 6);
-    Wg.col_ptr = cp;
-    Wg.col_rows = cr;
-    Wg.row_ptr = rp;
-    Wg.row_ent = re;
-    Wg.llr = ll;
-    Wg.vperm = vp;
+    const StagePiece pc[5] = {{U + L.q_rent, W.s_rent, 256u * W.row_pairs},
+                              {U + L.q_cent, W.s_cent, 128u * W.col_cells},
+                              {U + L.q_roff, W.s_roff, al16(2u * (rw + 1))},
+                              {U + L.q_coff, W.s_coff, al16(2u * (L.cw + 1))},
+                              {U + L.q_sllr, W.s_llr, 4u * ncp}};
+    stage_pieces(stg, pc, 5);
+    X.rent = (const uint32_t*)(U + L.q_rent);
+    X.cent = (const uint32_t*)(U + L.q_cent);
+    X.roff = (const uint16_t*)(U + L.q_roff);
+    X.coff = (const uint16_t*)(U + L.q_coff);
+    X.llr = (const float*)(U + L.q_sllr);
+  }
+  for (int s = warp; s < rw; s += nw) {
+    const int j = 32 * s + lane;
+    const unsigned m = __ballot_sync(FULL, j < nr && bit_of(sbits, W.s_row[j]));
+    if (lane == 0) spre[s] = m;
+  }
+  if (tid == 0) {
+    post[ncp] = dead_post();                    // the dummy column
+    cns[nrp] = CNState{0.0f, 0.0f, 0u, 0u};     // the dummy check: message +0
   }
 
   // ---- a2: pre-BP on the full window ----
-  const int tpc_pre = WIDE ? lanes_per_check(NT, nr) : 1, sub_pre = tid & (tpc_pre - 1);
-  const int nr_rounds = (nr + NT / tpc_pre - 1) / (NT / tpc_pre) * (NT / tpc_pre);
   bool conv = false;
   int t = 0;
   const int tk0 = P.n_pre - 3 > 1 ? P.n_pre - 3 : 1;
   if (P.n_pre == 0) {
-    uint32_t* pb = parb;
-    for (int x = tid; x < L.rw; x += NT) pb[x] = 0;
-    __syncthreads();
-    for (int i = tid; i < nc; i += NT) {
-      const float li = Wg.llr[i];
-      post[i] = li;
-      key[i] = __fadd_rn(__fadd_rn(__fadd_rn(li, li), li), li);
-      if (li <= 0.0f)
-        for (int e = Wg.col_ptr[i]; e < Wg.col_ptr[i + 1]; ++e) {
-          const int j = Wg.col_rows[e];
-          atomicXor(&pb[j >> 5], 1u << (j & 31));
-        }
+    for (int l = tid; l < nc; l += NT) {
+      const float li = X.llr[l];
+      post[l] = li;
+      key[l] = __fadd_rn(__fadd_rn(__fadd_rn(li, li), li), li);
     }
     __syncthreads();
-    bool ok = true;
-    for (int x = 0; x < L.rw; ++x) ok &= (pb[x] == sbits[x]);
-    conv = ok;
-  }
-  if (P.n_pre > 0) {
+  } else {
     // the first VN->CN messages of the pre-BP: the prior, or (message reuse)
     // what the previous window's output path kept for the same DEM column
     const float* kept = (A.keep && A.prev) ? A.keep + (size_t)shot * A.keep_ld : nullptr;
-    for (int i = tid; i < nc; i += NT) {
-      float v = Wg.llr[i];
+    for (int l = tid; l < nc; l += NT) {
+      float v = X.llr[l];
       if (kept) {
-        const int pc = A.prev[i];
+        const int pc = A.prev[W.s_col[l]];
         if (pc >= 0) {
           const float x = kept[pc];
           if (x == x) v = x;
         }
       }
-      post[i] = v;
+      post[l] = v;
     }
     __syncthreads();
   }
   int t_conv = 0;
   if (WIDE && !UG && P.n_pre > 0 && cl_size() > 1 && nr >= 2 * (int)cl_size() && nc >= 2 * (int)cl_size()) {
-    t = prebp_cluster<LW>(A, W, Wg, sm, U, sbits, conv, t_conv);
+    t = prebp_cluster<LW>(A, W, X, sm, conv, t_conv);
   } else {
-  for (t = 1; t <= P.n_pre; ++t) {
-    // check nodes; each check also takes the parity of the hard decisions it
-    // reads, so for t >= 2 the pass is the convergence test of iteration t-1
-    bool unsat = false;
-    for (int j0 = tid / tpc_pre; j0 < nr_rounds; j0 += NT / tpc_pre) {
-      const int j = j0 < nr ? j0 : nr - 1;
-      const int beg = Wg.row_ptr[j], end = j0 < nr ? Wg.row_ptr[j + 1] : beg;
-      const CNState oc = cns[j];
-      float m1 = CUDART_INF_F, m2 = CUDART_INF_F;
-      int am = 0xFFFF;
-      uint32_t neg = 0, hp = 0;
-      for (int q = beg + 4 * sub_pre; q < end; q += 4 * tpc_pre) {
-        uint32_t ent[4];
-        float pv[4];
-        uint32_t sg[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ent[u] = (q + u < end) ? Wg.row_ent[q + u] : 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = (int)(ent[u] >> 16), e = (int)(ent[u] & 0xFFFFu);
-          pv[u] = post[i];  // t = 1: the first VN->CN message (the prior, or the value kept for the column)
-          sg[u] = sign[e];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (q + u >= end) break;
-          const int e = (int)(ent[u] & 0xFFFFu);
-          hp ^= pv[u] <= 0.0f;
-          const float wprev = (LW && t > 1) ? edge_weight(W.wts, W.wT, W.n_edges, P.alpha, t - 1, e) : P.alpha;
-          const float v = (t == 1) ? pv[u] : clipf(__fsub_rn(pv[u], c2v<LW>(wprev, P.clip, oc, e, sg[u])), P.clip);
-          const float a = fabsf(v);
-          am = a < m1 ? e : am;
-          m2 = fminf(m2, fmaxf(m1, a));
-          m1 = fminf(m1, a);
-          const uint32_t sgn = v < 0.0f;
-          neg ^= sgn;
-          sign[e] = (uint8_t)sgn;
-        }
+    for (t = 1; t <= P.n_pre; ++t) {
+      // check nodes; each check also takes the parity of the hard decisions it
+      // reads, so for t >= 2 the pass is the convergence test of iteration t-1
+      LwRow lw{nullptr, W.s_ref};
+      if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
+      uint32_t unsat = 0u;
+      for (int s = warp; s < rw; s += nw) {
+        const int r0 = X.roff[s], np = (int)X.roff[s + 1] - r0;
+        const uint2* ent = (const uint2*)X.rent + r0 * 32 + lane;
+        const uint32_t sbit = (spre[s] >> lane) & 1u;
+        CNState* rec = cns + 32 * s + lane;
+        const int ei = (r0 * 32 + lane) * 2;
+        if (t == 1) unsat |= check_lane<LW, true>(ent, np, (const char*)post, rec, sbit, P.alpha, P.clip, lw, ei);
+        else unsat |= check_lane<LW, false>(ent, np, (const char*)post, rec, sbit, P.alpha, P.clip, lw, ei);
       }
-      if (tpc_pre > 1) {
-        group_min2(m1, m2, am, neg, tpc_pre);
-        for (int off = tpc_pre >> 1; off; off >>= 1) hp ^= __shfl_xor_sync(FULL, hp, off);
+      if (!__syncthreads_or(unsat != 0u) && t >= 2) {  // iteration t-1 satisfies H e = s
+        conv = true;
+        t_conv = t - 1;
+        break;
       }
-      if (sub_pre == 0 && j0 < nr) {
-        cns[j] = cn_store<LW>(P.alpha, P.clip, m1, m2, am, neg ^ bit_of(sbits, j), end - beg == 1, 0u);
-        unsat |= (hp ^ bit_of(sbits, j)) != 0u;
+      for (int l = tid; l < nc; l += NT) {
+        const float p = prebp_column<LW>(P, W, X, l, t);
+        post[l] = p;
+        if (t >= tk0) key[l] = prebp_key(P, X, l, t, tk0, p);
       }
+      __syncthreads();
     }
-    if (!__syncthreads_or(unsat) && t >= 2) {  // iteration t-1 satisfies H e = s
-      conv = true;
-      t_conv = t - 1;
-      break;
-    }
-    const bool kacc = t >= tk0;
-    for (int i0 = tid; i0 < nc; i0 += NT) {
-      const int i = Wg.vperm[i0];  // descending degree: the lanes of a round loop alike
-      float p = Wg.llr[i];
-      const int eb = Wg.col_ptr[i], ee = Wg.col_ptr[i + 1];
-      // up to six messages requested at once, then added in ascending check
-      // order (Eq. (2))
-      for (int e0 = eb; e0 < ee; e0 += 6) {
-        CNState c[6];
-        uint32_t sg[6];
-#pragma unroll
-        for (int u = 0; u < 6; ++u)
-          if (e0 + u < ee) {
-            c[u] = cns[Wg.col_rows[e0 + u]];
-            sg[u] = sign[e0 + u];
-          }
-#pragma unroll
-        for (int u = 0; u < 6; ++u)
-          if (e0 + u < ee) {
-            const float wt = LW ? edge_weight(W.wts, W.wT, W.n_edges, P.alpha, t, e0 + u) : P.alpha;
-            p = __fadd_rn(p, c2v<LW>(wt, P.clip, c[u], e0 + u, sg[u]));
-          }
-      }
-      post[i] = p;
-      if (kacc) {
-        float kv;
-        if (t == tk0) {
-          if (P.n_pre < 4) {
-            const float li = Wg.llr[i];
-            float s = li;
-            for (int r = 1; r < 4 - P.n_pre; ++r) s = __fadd_rn(s, li);
-            kv = __fadd_rn(s, p);
-          } else {
-            kv = p;
-          }
-        } else {
-          kv = __fadd_rn(key[i], p);
-        }
-        key[i] = kv;
-      }
-    }
-    __syncthreads();
   }
-  }
-  if (!conv && P.n_pre > 0) {  // the convergence test of the last iteration
+  if (!conv) {  // the convergence test of the last iteration (or of the priors)
     bool unsat = false;
-    for (int j = tid; j < nr; j += NT) {
-      uint32_t hp = bit_of(sbits, j);
-      for (int q = Wg.row_ptr[j]; q < Wg.row_ptr[j + 1]; ++q) hp ^= post[Wg.row_ent[q] >> 16] <= 0.0f;
-      unsat |= hp != 0u;
+    for (int s = warp; s < rw; s += nw) {
+      uint32_t hp = ((spre[s] >> lane) & 1u) << 31;
+      const uint2* ent = (const uint2*)X.rent + (int)X.roff[s] * 32 + lane;
+      const int np = (int)X.roff[s + 1] - (int)X.roff[s];
+      for (int p = 0; p < np; ++p) {
+        const uint2 e = ent[32 * p];
+        hp ^= (__float_as_uint(*(const float*)((const char*)post + e.x)) - 1u) ^
+              (__float_as_uint(*(const float*)((const char*)post + e.y)) - 1u);
+      }
+      unsat |= (hp >> 31) != 0u;
     }
     if (!__syncthreads_or(unsat)) {
       conv = true;
       t_conv = P.n_pre;
     }
   }
-  if (conv && P.n_pre > 0) t = t_conv;
-  *t_run_out = conv ? (P.n_pre == 0 ? 0 : t) : P.n_pre;
+  *t_run_out = conv ? t_conv : P.n_pre;
   if (conv) {
-    for (int base = warp * 32; base < nc; base += NT) {
-      const int i = base + lane;
-      const bool one = i < nc && post[i] <= 0.0f;
-      const unsigned m = __ballot_sync(FULL, one);
-      if (lane == 0) cbits[base >> 5] = m;
-    }
+    for (int l = tid; l < nc; l += NT)
+      if (post[l] <= 0.0f) {
+        const int c = W.s_col[l];
+        atomicOr(&cbits[c >> 5], 1u << (c & 31));
+      }
     __syncthreads();
     return true;
   }
 
   // ---- a3: rank by the four-iteration sum, keep the first n_short ----
-  const int n_short = W.n_short;
-  for (int i = tid; i < L.sortn; i += NT)
-    sortb[i] = i < nc ? (((unsigned long long)ordkey(key[i]) << 32) | (unsigned)i) : ~0ull;
+  const int n_short = W.n_short, nsp = 32 * L.sw;
+  unsigned long long* sortb = (unsigned long long*)(U + L.p_sort);
+  for (int l = tid; l < L.sortn; l += NT)  // ties by window column
+    sortb[l] = l < nc ? (((unsigned long long)ordkey(key[l]) << 32) | ((unsigned)W.s_col[l] << 16) | (unsigned)l) : ~0ull;
   __syncthreads();
   block_sort_u64(sortb, L.sortn);
-  for (int k = tid; k < n_short; k += NT) sel[k] = (uint16_t)(sortb[k] & 0xFFFFu);
-  __syncthreads();
-  // ---- shortened matrix in shared memory, numbered in processing order ----
-  // Columns and checks get labels by descending degree (ties by rank / row),
-  // so the lanes of a round loop alike and touch neighbouring words; vperm
-  // and cperm map a label back to the ranked column and the window row, which
-  // decide every tie.  A column's checks stay in ascending window row (the
-  // order of the sum of Eq. (2)).
-  uint16_t* scp = (uint16_t*)(sm + L.s_colptr);
-  uint16_t* scr = (uint16_t*)(sm + L.s_colrows);
-  uint16_t* srp = (uint16_t*)(sm + L.s_rowptr);
-  uint32_t* sre = (uint32_t*)(sm + L.s_rowent);
+  // (from here on the pre-BP's arrays are dead: the shortened graph takes their place)
+  uint16_t* sel = (uint16_t*)(sm + L.sel);
+  uint32_t* rent = (uint32_t*)(sm + L.s_rent);
+  uint32_t* cent = (uint32_t*)(sm + L.s_cent);
+  uint16_t* roff = (uint16_t*)(sm + L.s_roff);
+  uint16_t* coff = (uint16_t*)(sm + L.s_coff);
   float* sllr = (float*)(sm + L.s_llr);
   uint8_t* svd = (uint8_t*)(sm + L.s_vdeg);
-  uint16_t* sef = (uint16_t*)(sm + L.s_efull);
+  uint16_t* sref = (uint16_t*)(sm + L.s_ref);
+  uint16_t* scef = (uint16_t*)(sm + L.s_cef);
   uint16_t* cperm = (uint16_t*)(sm + L.s_cperm);
   uint16_t* vperm = (uint16_t*)(sm + L.s_vperm);
   int* rc = (int*)(sm + L.rowcnt);
-  int* tmp = (int*)sortb;  // the sort buffer is free now
-  for (int k = tid; k < n_short; k += NT) {
-    const int c = sel[k];
-    tmp[k] = W.col_ptr[c + 1] - W.col_ptr[c];
-  }
-  for (int j = tid; j <= nr; j += NT) rc[j] = 0;
+  for (int k = tid; k < n_short; k += NT) sel[k] = (uint16_t)(sortb[k] >> 16);
+  for (int j = tid; j < nrp; j += NT) rc[j] = 0;
   __syncthreads();
-  for (int k = tid; k < n_short; k += NT) {  // rows of the shortened matrix
-    const int c = sel[k];
-    for (int e = W.col_ptr[c]; e < W.col_ptr[c + 1]; ++e) atomicAdd(&rc[W.col_rows[e]], 1);
+  // ---- shortened matrix in shared memory, numbered in processing order ----
+  // Columns and checks get labels by descending degree (ties by rank / row),
+  // so the lanes of a round loop alike; vperm and cperm map a label back to
+  // the ranked column and the window row, which decide every tie.  A column's
+  // checks stay in ascending window row (the order of the sum of Eq. (2)).
+  int* deg = (int*)sortb;            // the sort buffer is free now: degree by rank, then
+  int* cinv = deg + up32(n_short);   // window row -> label (no room past the keys: see below)
+  for (int k = tid; k < n_short; k += NT) {
+    const int c = sel[k], e0 = W.col_ptr[c], e1 = W.col_ptr[c + 1];
+    deg[k] = e1 - e0;
+    for (int e = e0; e < e1; ++e) atomicAdd(&rc[W.col_rows[e]], 1);  // rows of the shortened matrix
   }
+  __syncthreads();
   for (int k = tid; k < n_short; k += NT) {  // rank by counting; no sort needed at these sizes
-    const int dk = tmp[k];
+    const int dk = deg[k];
     int r = 0;
     for (int i = 0; i < n_short; ++i) {
-      const int di = tmp[i];
+      const int di = deg[i];
       r += (di > dk) || (di == dk && i < k);
     }
     vperm[r] = (uint16_t)k;
+    svd[r] = (uint8_t)dk;
   }
-  __syncthreads();
-  uint16_t* cinv = srp;  // window row -> label, until the row pointers are built
   for (int j = tid; j < nr; j += NT) {
     const int dj = rc[j];
     int r = 0;
@@ -1882,57 +1855,78 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
       r += (di > dj) || (di == dj && i < j);
     }
     cperm[r] = (uint16_t)j;
-    cinv[j] = (uint16_t)r;
-  }
-  for (int k = tid; k < n_short; k += NT) {
-    const int kr = vperm[k];
-    svd[k] = (uint8_t)tmp[kr];
-    sllr[k] = W.llr[sel[kr]];
   }
   __syncthreads();
-  for (int k = tid; k < n_short; k += NT) tmp[k] = svd[k];
-  __syncthreads();
+  // slice starts (a slice is as wide as its first node), one warp each
   if (warp == 0) {
-    const int tot = warp_scan_excl(tmp, n_short, lane);
-    if (lane == 0) tmp[n_short] = tot;
+    int run = 0;
+    for (int b = 0; b < rw; b += 32) {
+      const int s = b + lane;
+      int v = s < rw ? (rc[cperm[32 * s]] + 1) >> 1 : 0;
+      v = warp_incl_scan(v, lane);
+      if (s < rw) roff[s + 1] = (uint16_t)(run + v);
+      run += __shfl_sync(FULL, v, 31);
+    }
+    if (lane == 0) roff[0] = 0;
+  }
+  if (warp == (nw > 1 ? 1 : 0)) {
+    // (a check past 32 entries is rare in a shortened graph: one flag for all)
+    const uint16_t flag = rc[cperm[0]] > 32 ? kWideSlice : (uint16_t)0;
+    int run = 0;
+    for (int b = 0; b < L.sw; b += 32) {
+      const int s = b + lane;
+      int v = s < L.sw ? (int)svd[32 * s] : 0;
+      v = warp_incl_scan(v, lane);
+      if (s < L.sw) coff[s + 1] = (uint16_t)((run + v) | flag);
+      run += __shfl_sync(FULL, v, 31);
+    }
+    if (lane == 0) coff[0] = flag;
   }
   __syncthreads();
-  for (int k = tid; k <= n_short; k += NT) scp[k] = (uint16_t)tmp[k];
+  // every place a dummy, then the edges
+  {
+    const int np = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
+    for (int x = tid; x < 64 * np; x += NT) rent[x] = 4u * (unsigned)nsp;
+    for (int x = tid; x < 32 * ncell; x += NT) cent[x] = (unsigned)nrp << 16;
+    if (LW) {
+      for (int x = tid; x < 64 * np; x += NT) sref[x] = 0;
+      for (int x = tid; x < 32 * ncell; x += NT) scef[x] = 0;
+    }
+    for (int l = tid; l < nr; l += NT) cinv[cperm[l]] = l;
+    for (int k = n_short + tid; k < nsp; k += NT) sllr[k] = 0.0f;
+  }
+  __syncthreads();
+  for (int j = tid; j < nrp; j += NT) rc[j] = 0;
+  __syncthreads();
   for (int k = tid; k < n_short; k += NT) {
-    const int c = sel[vperm[k]];
-    int o = tmp[k];
-    for (int e = W.col_ptr[c]; e < W.col_ptr[c + 1]; ++e, ++o) {
-      scr[o] = cinv[W.col_rows[e]];
-      if (LW) sef[o] = (uint16_t)e;  // the shortened edge keeps its full-window edge's weights
+    const int c = sel[vperm[k]], e0 = W.col_ptr[c], d = svd[k];
+    sllr[k] = W.llr[c];
+    const int ci = (coff[k >> 5] & (kWideSlice - 1)) * 32 + (k & 31);
+    for (int u = 0; u < d; ++u) {
+      const int r = cinv[W.col_rows[e0 + u]];
+      const int pos = atomicAdd(&rc[r], 1);
+      const int ri = (roff[r >> 5] + (pos >> 1)) * 64 + 2 * (r & 31) + (pos & 1);
+      rent[ri] = 4u * (unsigned)k;
+      cent[ci + 32 * u] = ((unsigned)r << 16) | (unsigned)pos;
+      if (LW) {  // the shortened edge keeps its full-window edge's weights
+        sref[ri] = (uint16_t)(e0 + u);
+        scef[ci + 32 * u] = (uint16_t)(e0 + u);
+      }
     }
+    if (LW)  // a dummy takes its column's first edge's weight (a check's dummies are dead inputs)
+      for (int u = d; u < (int)(coff[(k >> 5) + 1] & (kWideSlice - 1)) - (coff[k >> 5] & (kWideSlice - 1)); ++u)
+        scef[ci + 32 * u] = (uint16_t)e0;
   }
-  for (int j = tid; j <= nr; j += NT) rc[j] = 0;
-  __syncthreads();
-  for (int k = tid; k < n_short; k += NT)
-    for (int e = scp[k]; e < scp[k + 1]; ++e) atomicAdd(&rc[scr[e]], 1);
-  __syncthreads();
-  if (warp == 0) {
-    const int tot = warp_scan_excl(rc, nr, lane);
-    if (lane == 0) rc[nr] = tot;
-  }
-  __syncthreads();
-  for (int j = tid; j <= nr; j += NT) srp[j] = (uint16_t)rc[j];
-  __syncthreads();
-  for (int k = tid; k < n_short; k += NT)
-    for (int e = scp[k]; e < scp[k + 1]; ++e) {
-      const int pos = atomicAdd(&rc[scr[e]], 1);
-      sre[pos] = (uint32_t)e | ((uint32_t)k << 16);
-    }
   __syncthreads();
   return false;
 }
 
 __device__ __forceinline__ ShortG short_graph(char* sm, const Layout& L, const WinDev& W, int ns) {
-  return ShortG{W.n_rows, ns, L.rw,
-                (const uint16_t*)(sm + L.s_colptr), (const uint16_t*)(sm + L.s_colrows),
-                (const uint16_t*)(sm + L.s_rowptr), (const uint32_t*)(sm + L.s_rowent),
-                (const float*)(sm + L.s_llr),       (const uint8_t*)(sm + L.s_vdeg),
-                (const uint32_t*)(sm + L.sbits),    (const uint16_t*)(sm + L.s_efull),
+  return ShortG{W.n_rows, ns, L.rw, L.sw,
+                (const uint32_t*)(sm + L.s_rent), (const uint32_t*)(sm + L.s_cent),
+                (const uint16_t*)(sm + L.s_roff), (const uint16_t*)(sm + L.s_coff),
+                (const float*)(sm + L.s_llr),     (const uint8_t*)(sm + L.s_vdeg),
+                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(sm + L.s_ref), (const uint16_t*)(sm + L.s_cef),
                 W.wts, W.wT, W.n_edges, W.rows_per_block, (const uint16_t*)(sm + L.sel),
                 (const uint16_t*)(sm + L.s_cperm), (const uint16_t*)(sm + L.s_vperm), W.n_commit_rows};
 }
@@ -1994,7 +1988,7 @@ __device__ void keep_for_next(const DecodeArgs& A, char* sm, long long shot, con
   const int tid = threadIdx.x, NT = blockDim.x, nc = A.W.n_cols;
   float* out = A.keep + (size_t)shot * A.keep_ld;
   if (!kp) {
-    for (int c = tid; c < nc; c += NT) out[c] = post[c];
+    for (int l = tid; l < nc; l += NT) out[A.W.s_col[l]] = post[l];
     return;
   }
   const uint16_t* sel = (const uint16_t*)(sm + A.L.sel);
@@ -2149,7 +2143,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
     }
     __syncthreads();
   } else if (A.keep) {
-    keep_for_next(A, sm, shot, nullptr, 0, (const float*)(union_base<UG>(A, sm) + L.p_post));
+    keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<UG>(A, sm) + L.p_post));
   }
   write_outputs(A, sm, shot, conv, winner, n_short, t_run, tr);
 }
@@ -2215,32 +2209,13 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   int* misc = (int*)(sm + L.misc);
   char* tr = A.trace ? A.trace + (size_t)shot * A.tr_bytes : nullptr;
   Stager stg = stager_init((char*)(misc + 8), &A.counters[4]);
-  // stage the window graph in shared memory (one CTA per SM in this mode)
-  WinDev W = A.W;
-  if (L.g_bytes) {
-    const WinDev& G = A.W;
-    uint16_t* cp = (uint16_t*)(sm + L.g_colptr);
-    uint16_t* cr = (uint16_t*)(sm + L.g_colrows);
-    uint16_t* rp = (uint16_t*)(sm + L.g_rowptr);
-    uint32_t* re = (uint32_t*)(sm + L.g_rowent);
-    float* ll = (float*)(sm + L.g_llr);
-    const StagePiece pc[5] = {{cp, G.col_ptr, al16(2u * (G.n_cols + 1))}, {cr, G.col_rows, al16(2u * G.n_edges)},
-                              {rp, G.row_ptr, al16(2u * (G.n_rows + 1))}, {re, G.row_ent, al16(4u * G.n_edges)},
-                              {ll, G.llr, al16(4u * G.n_cols)}};
-    stage_pieces(stg, pc, 5);
-    W.col_ptr = cp;
-    W.col_rows = cr;
-    W.row_ptr = rp;
-    W.row_ent = re;
-    W.llr = ll;
-  }
   int t_run = 0;
-  const bool conv = window_prefix<LW, true, false>(A, W, sm, shot, &t_run, stg);
+  const bool conv = window_prefix<LW, true, false>(A, A.W, sm, shot, &t_run, stg);
   if (id >= nb) return;  // a CTA that only shared the pre-BP of its cluster
   if (conv) {
     if (id == 0) {
       write_outputs(A, sm, shot, true, -1, 0, t_run, tr);
-      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(union_base<false>(A, sm) + L.p_post));
+      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<false>(A, sm) + L.p_post));
     }
     return;
   }

@@ -5,11 +5,22 @@
 // which only depends on the check's two smallest |mu| (min1, min2), the edge
 // holding min1 (amin), the sign parity of all its inputs xor s_j, and the sign
 // of the receiving edge's own input.  The kernel keeps exactly that per check
-// (one 16-byte record) plus one sign byte per edge, instead of two FP32
+// in one 16-byte record (the signs as one bit per edge), instead of two FP32
 // messages per edge.  The VN->CN message of Eq. (3) is recomputed where it is
 // needed as clip(Lambda_i^(t) - mu_{j->i}), the same FP32 operations the
 // explicit form performs, so every value is bit-identical to it.  All FP32
 // operations are __fadd_rn / __fsub_rn / __fmul_rn (never contracted).
+//
+// Graph format.  Checks and columns are numbered by descending degree, and the
+// entries of 32 consecutive ones (a slice, one per lane of a warp) are stored
+// lane by lane, entry u of every lane side by side, each slice as wide as its
+// first node's degree (check slices rounded up to an even width).  A warp
+// walks a slice with conflict-free loads, one trip count for all lanes and no
+// bounds test: the places past a node's degree hold a dummy whose value
+// changes nothing (a column with posterior +inf, a check record with message
+// +0).
+//   check entry:  byte offset 4 * column of the column's posterior
+//   column entry: check << 16 | position of the edge among the check's entries
 #pragma once
 #include <cstddef>
 #include <cstdint>
@@ -94,8 +105,14 @@ struct WinDev {
   // alpha at iteration t (counted from message initialisation); NULL = alpha
   const float* wts;
   int wT;
-  const uint16_t* vperm;  // pre-BP processing order of the columns (descending degree)
   int n_commit_rows;      // rows [0, n_commit_rows) are the ones the window commits
+  // the graph in slices (see the top of the file), checks and columns by label
+  int row_pairs, col_cells;    // slice totals: check-entry pairs, column entries, both per lane
+  const uint32_t *s_rent, *s_cent;   // [2 * 32 * row_pairs], [32 * col_cells]
+  const uint16_t *s_roff, *s_coff;   // slice starts, in pairs / in entries per lane
+  const float* s_llr;                // priors by column label
+  const uint16_t *s_row, *s_col;     // label -> window row / window column
+  const uint16_t *s_ref, *s_cef;     // full-window edge of each check / column entry (learned weights)
 };
 
 // Shot mode's plan for resuming decision paths from snapshots of shared
@@ -137,16 +154,22 @@ struct WmsGraph {
   float clip;
 };
 
-// Compressed state of one check node: two smallest |input| and the edge
-// holding the smallest (ac).  Plain decoder: the magnitudes multiplied by
-// alpha (alpha * clip twice when exactly one input is active), each negated
-// when the sign parity xor s_j is 1, and ac = the edge.  Learned weights: the
-// magnitudes unscaled, ac = edge | parity << 16 | (exactly one active input)
-// << 17.
+// Compressed state of one check node: its two smallest |input| (bounded by the
+// clip), each negated when the sign parity xor s_j is 1 and, in the plain
+// decoder, multiplied by alpha; sg: the inputs' signs, position p at bit 31 - p
+// (p < 32); am: the position of the smallest input (low six bits) and the
+// signs of positions 32 .. 57, position p at bit 63 - p.
 struct __align__(16) CNState {
   float m1, m2;
-  uint32_t ac, pad;
+  uint32_t sg, am;
 };
+// Most entries a check may have.  A detector of these codes' circuits touches
+// at most 35 columns: the fault classes of a round are the same for every
+// choice of A and B (three terms each), and coinciding terms only merge them.
+constexpr int kMaxRowDeg = 58;
+// Flag of a column slice's start (s_coff) when some edge of it has a position
+// past 31 and its sign is in the second word.
+constexpr uint16_t kWideSlice = 0x8000;
 
 struct BranchTrace {
   int32_t status, depth, iters, pad;
@@ -161,6 +184,14 @@ struct StepTrace {
 // Result of one decision path in the path-per-CTA launch (global scratch).
 __host__ __device__ inline size_t path_result_bytes(int sw) { return (16 + 4 * (size_t)sw + 15) & ~(size_t)15; }
 
+// Sizes of a window's graph in slices, and bounds on those of its shortened
+// graphs.
+struct SliceDims {
+  int row_pairs, col_cells;    // the window's, as WinDev
+  int srow_pairs, scol_cells;  // the shortened graph's, at most
+};
+__host__ __device__ inline unsigned up32(unsigned x) { return (x + 31u) & ~31u; }
+
 // Shared-memory layout of one CTA (byte offsets), identical on host and device.
 struct Layout {
   // persistent
@@ -169,7 +200,7 @@ struct Layout {
   // window graph staged in shared memory (path mode only; 0 bytes otherwise)
   unsigned g_colptr, g_colrows, g_rowptr, g_rowent, g_llr, g_bytes;
   unsigned U;  // start of the union region
-  // pre-BP (relative to U)
+  // pre-BP (relative to U; make_slice_layout: to V)
   unsigned p_post, p_key, p_cns, p_sign, p_par, p_sort, p_end;
   // the window graph staged for the pre-BP loop in otherwise idle union bytes
   // (from p_sort on; overwritten by the sort that follows); pre_stage = 0: none
@@ -178,10 +209,104 @@ struct Layout {
   unsigned b_post, b_acc, b_hfl, b_status, b_sign, b_cns, b_deg, b_sp, b_unsat, b_hq, b_size;
   unsigned total;
   int rw, cw, sw, sortn, nslots;
+  // slices: the shortened graph (s_rent .. s_coff; s_ref / s_cef with learned
+  // weights) and the staged window graph (q_rent .. q_llr)
+  unsigned s_rent, s_cent, s_roff, s_coff, s_ref, s_cef;
+  unsigned q_rent, q_cent, q_roff, q_coff, q_sllr;
+  // The pre-BP's arrays start at V, where the shortened graph and the path
+  // slots begin: neither exists before the pre-BP has ended.
+  unsigned V;
 };
 
 __host__ __device__ inline unsigned al16(unsigned x) { return (x + 15u) & ~15u; }
 
+// Layout of the decode kernels.  The pre-BP scratch (and the staged window
+// graph: stage = 1) shares its bytes with the shortened graph and the path
+// slots that follow it; only the ranking's sort buffer, read while the
+// shortened graph is being written, lies past that graph (and past the keys it
+// is filled from).  stage = 2: the staged graph lies past everything else, so
+// that the ranking and the shortening can read it too.  ub_glob: the union is
+// addressed from its own base (global memory), the shortened graph stays in
+// shared memory.
+__host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, int nc, int ns, int nb, int nslots,
+                                                    int stage, bool ranker, bool lw, bool ub_glob) {
+  Layout L{};
+  L.rw = (nr + 31) / 32;
+  L.cw = (nc + 31) / 32;
+  L.sw = (ns + 31) / 32;
+  L.nslots = nslots;
+  int sn = 1;
+  while (sn < nc) sn <<= 1;
+  L.sortn = sn;
+  const unsigned nrp = up32(nr), ncp = up32(nc), nsp = up32(ns);
+  unsigned o = 0;
+  L.sbits = o; o = al16(o + 4u * L.rw);
+  L.cbits = o; o = al16(o + 4u * L.cw);
+  L.res_status = o; o = al16(o + 4u * nb);
+  L.res_pm = o; o = al16(o + 8u * nb);
+  L.res_ebits = o; o = al16(o + 4u * L.sw * nb);
+  L.red = o; o = al16(o + 16u * 32);
+  L.misc = o; o = al16(o + 64u);
+  L.V = o;
+  L.sel = o; o = al16(o + 2u * ns);
+  L.s_rent = o; o = al16(o + 256u * D.srow_pairs);
+  L.s_cent = o; o = al16(o + 128u * D.scol_cells);
+  L.s_roff = o; o = al16(o + 2u * (L.rw + 1));
+  L.s_coff = o; o = al16(o + 2u * (L.sw + 1));
+  L.s_llr = o; o = al16(o + 4u * nsp);
+  L.s_vdeg = o; o = al16(o + nsp);
+  L.s_ref = o; o = al16(o + (lw ? 128u * D.srow_pairs : 0u));
+  L.s_cef = o; o = al16(o + (lw ? 64u * D.scol_cells : 0u));
+  L.s_cperm = o; o = al16(o + 2u * nr);
+  L.s_vperm = o; o = al16(o + 2u * ns);
+  L.rowcnt = o; o = al16(o + 4u * (nrp + 1));
+  L.U = o;
+  const unsigned p0 = ub_glob ? 0u : L.V;  // where the pre-BP scratch starts, as an absolute offset
+  unsigned u = 0;                          // relative to it
+  L.p_post = u; u = al16(u + 4u * (ncp + 1));
+  L.p_key = u; u = al16(u + 4u * ncp);
+  L.p_cns = u; u = al16(u + 16u * (nrp + 1));
+  L.p_par = u; u = al16(u + 8u * L.rw);
+  const unsigned own = u;
+  unsigned srt = al16(L.p_key + 4u * ncp);
+  if (!ub_glob && srt < L.U - L.V) srt = L.U - L.V;
+  if (ub_glob) srt = own;
+  L.p_sort = srt;
+  // the keys, later the shortening's scratch: the columns' degrees and the checks' labels
+  const unsigned sb = 8u * sn > 4u * (nsp + nrp) ? 8u * sn : 4u * (nsp + nrp);
+  L.p_end = own > srt + sb ? own : srt + sb;
+  unsigned b = 0;
+  L.b_post = b; b = al16(b + 4u * (nsp + 1));
+  L.b_acc = b; b = al16(b + 4u * ns);
+  L.b_hfl = b; b = al16(b + 1u * ns);
+  L.b_status = b; b = al16(b + 1u * nsp);
+  L.b_cns = b; b = al16(b + 16u * (nrp + 1));
+  L.b_deg = b; b = al16(b + nrp);
+  L.b_sp = b; b = al16(b + 4u * L.rw);
+  L.b_unsat = b; b = al16(b + 4u * L.rw);
+  L.b_hq = b; b = al16(b + (ranker ? 4u * ns : 0u));
+  L.b_size = b;
+  const unsigned slots = b * (unsigned)nslots;
+  unsigned end = ub_glob ? (slots > L.p_end ? slots : L.p_end)
+                         : (L.U + slots > p0 + L.p_end ? L.U + slots : p0 + L.p_end);
+  if (stage) {
+    const unsigned q0 = stage == 2 ? al16(end) - p0 : own;
+    unsigned q = q0;
+    L.q_rent = q; q = al16(q + 256u * D.row_pairs);
+    L.q_cent = q; q = al16(q + 128u * D.col_cells);
+    L.q_roff = q; q = al16(q + 2u * (L.rw + 1));
+    L.q_coff = q; q = al16(q + 2u * (L.cw + 1));
+    L.q_sllr = q; q = al16(q + 4u * ncp);
+    L.pre_stage = 1u;
+    if (p0 + q > end) end = p0 + q;
+  }
+  L.total = ub_glob ? L.U + end : end;
+  return L;
+}
+
+// The layout with one sign byte per edge and plain CSC / CSR arrays, kept as
+// the reference the layout checks state their invariants on; the decode
+// kernels take make_slice_layout.
 // lw: the shortened edges' full-window edge ids (s_efull) are kept, which
 // only learned weights read
 __host__ __device__ inline Layout make_layout(int nr, int nc, int ne, int ns, int es, int nb,

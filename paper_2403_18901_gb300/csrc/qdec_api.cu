@@ -253,6 +253,10 @@ ForkPlan fork_plan(const qd::KParams& P, int dmx, int wave) {
   return F;
 }
 
+qd::SliceDims slice_dims(const qd::WindowHost& h) {
+  return qd::SliceDims{h.row_pairs, h.col_cells, h.srow_pairs, h.scol_cells};
+}
+
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   struct Conf {
     qd::Layout L, Lp, Lg;
@@ -267,28 +271,29 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     Conf& c = cf[w];
     c.pcl = 1;
     const auto& h = dec->wins[w].h;
-    auto lay = [&](int slots, bool stage) {
-      return qd::make_layout(h.n_rows, h.n_cols, h.n_edges, h.n_short, h.short_edges_max, nb, slots, stage, hist,
-                             dec->lw_on);
+    auto lay = [&](int slots, int stage, bool glob = false) {
+      return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, slots, stage, hist, dec->lw_on,
+                                   glob);
     };
     // the most resident decision-path warps per SM (slots per CTA x CTAs per
-    // SM); ties to more slots per CTA
-    int best = 0;
+    // SM); ties to more slots per CTA, then to staging the window graph
+    int best = 0, stage = 0;
     c.shot_warps = 1;
-    for (int sw = kShotWarps; sw >= 1; --sw) {
-      const qd::Layout Ls = lay(sw, false);
-      if (Ls.total > (unsigned)optin) continue;
-      int blocks = 0;
-      QD_CK(qd::decode_occupancy(0, 32 * sw, Ls.total, &blocks));
-      if (sw * blocks > best) {
-        best = sw * blocks;
-        c.shot_warps = sw;
+    for (int sw = kShotWarps; sw >= 1; --sw)
+      for (int sg = 1; sg >= 0; --sg) {
+        const qd::Layout Ls = lay(sw, sg);
+        if (Ls.total > (unsigned)optin) continue;
+        int blocks = 0;
+        QD_CK(qd::decode_occupancy(0, 32 * sw, Ls.total, &blocks));
+        if (sw * blocks > best) {
+          best = sw * blocks;
+          c.shot_warps = sw;
+          stage = sg;
+        }
       }
-    }
     // the union region in global memory: eight path slots, shared memory for
     // the persistent part only, no pre-BP staging (its copies need shared memory)
-    c.Lg = lay(kShotWarps, false);
-    c.Lg.pre_stage = 0;
+    c.Lg = lay(kShotWarps, 0, true);
     if (c.Lg.U > (unsigned)optin) {
       set_error(std::string(who) + ": window " + std::to_string(w) + " needs " + std::to_string(c.Lg.U) +
                 " B of shared memory even with its path state in global memory (limit " +
@@ -298,11 +303,11 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     int bg = 0;
     QD_CK(qd::decode_occupancy(3, 32 * kShotWarps, c.Lg.U, &bg));
     c.grid_g = std::max(1, bg);
-    c.L = lay(c.shot_warps, false);
+    c.L = lay(c.shot_warps, stage);
     c.fits = c.L.total <= (unsigned)optin;
     if (!c.fits) c.L = c.Lg;  // shot mode streams the path state through L2 / HBM
-    c.Lp = lay(1, true);
-    if (c.Lp.total > (unsigned)optin) c.Lp = lay(1, false);
+    c.Lp = lay(1, 1);
+    if (c.Lp.total > (unsigned)optin) c.Lp = lay(1, 0);
     c.path_fits = c.Lp.total <= (unsigned)optin;
     // path mode: the largest cluster (8, 4 or 2 CTAs, at most the number of
     // paths) that can be resident, its CTAs splitting the pre-BP of a shot
@@ -625,34 +630,32 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     dec->corr_words = std::max(dec->corr_words, (h.n_cols + 31) / 32);
     dec->ns_max = std::max(dec->ns_max, h.n_short);
     dec->sw_max = std::max(dec->sw_max, (h.n_short + 31) / 32);
-    // graph arrays in one allocation
-    // every array starts on a 16-byte boundary and is padded to a multiple of
-    // 16 bytes, as the kernels' bulk (TMA) copies into shared memory require
-    auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-    size_t o_cp = 0, o_cr = a16(o_cp + 2 * h.col_ptr.size()), o_rp = a16(o_cr + 2 * h.col_rows.size()),
-           o_re = a16(o_rp + 2 * h.row_ptr.size()), o_ll = a16(o_re + 4 * h.row_ent.size()),
-           o_vp = a16(o_ll + 4 * h.llr.size()), tot = a16(o_vp + 2 * (size_t)h.n_cols);
-    // pre-BP processing order of the variables: descending degree, ties by index
-    std::vector<uint16_t> vperm(h.n_cols);
-    for (int c = 0; c < h.n_cols; ++c) vperm[c] = (uint16_t)c;
-    std::stable_sort(vperm.begin(), vperm.end(), [&](uint16_t a, uint16_t b) {
-      return h.col_ptr[a + 1] - h.col_ptr[a] > h.col_ptr[b + 1] - h.col_ptr[b];
-    });
-    std::vector<char> blob(tot);
-    memcpy(blob.data() + o_vp, vperm.data(), 2 * vperm.size());
-    memcpy(blob.data() + o_cp, h.col_ptr.data(), 2 * h.col_ptr.size());
-    memcpy(blob.data() + o_cr, h.col_rows.data(), 2 * h.col_rows.size());
-    memcpy(blob.data() + o_rp, h.row_ptr.data(), 2 * h.row_ptr.size());
-    memcpy(blob.data() + o_re, h.row_ent.data(), 4 * h.row_ent.size());
-    memcpy(blob.data() + o_ll, h.llr.data(), 4 * h.llr.size());
-    QD_CK(cudaMalloc(&g.d_graph, tot));
-    QD_CK(cudaMemcpy(g.d_graph, blob.data(), tot, cudaMemcpyHostToDevice));
+    if (!qd::build_slices(g.h)) return QD_EUNSUPPORTED;
+    // graph arrays in one allocation: every array starts on a 16-byte boundary
+    // and is padded to a multiple of 16 bytes, as the kernels' bulk (TMA)
+    // copies into shared memory require
+    std::vector<char> blob;
+    auto put = [&](const auto& v) {
+      const size_t o = blob.size(), n = v.size() * sizeof(v[0]);
+      blob.resize((o + n + 15) & ~(size_t)15);
+      if (n) memcpy(blob.data() + o, v.data(), n);
+      return o;
+    };
+    const size_t o_cp = put(h.col_ptr), o_cr = put(h.col_rows), o_rp = put(h.row_ptr), o_re = put(h.row_ent),
+                 o_ll = put(h.llr), s_re = put(h.s_rent), s_ce = put(h.s_cent), s_ro = put(h.s_roff),
+                 s_co = put(h.s_coff), s_ll = put(h.s_llr), s_rw = put(h.s_row), s_cl = put(h.s_col),
+                 s_rf = put(h.s_ref), s_cf = put(h.s_cef);
+    QD_CK(cudaMalloc(&g.d_graph, std::max<size_t>(blob.size(), 16)));
+    QD_CK(cudaMemcpy(g.d_graph, blob.data(), blob.size(), cudaMemcpyHostToDevice));
     char* b = (char*)g.d_graph;
     g.dv = qd::WinDev{h.n_rows, h.n_cols, h.n_edges, h.row0, h.n_short, h.short_edges_max, h.n_rows / h.n_blocks,
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
                       (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0,
-                      (const uint16_t*)(b + o_vp),
-                      h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks))};
+                      h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks)),
+                      h.row_pairs, h.col_cells, (const uint32_t*)(b + s_re), (const uint32_t*)(b + s_ce),
+                      (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
+                      (const uint16_t*)(b + s_rw), (const uint16_t*)(b + s_cl), (const uint16_t*)(b + s_rf),
+                      (const uint16_t*)(b + s_cf)};
     // committed columns: their full detector sets and observables
     std::vector<int> cc_ptr(1, 0), cc_det;
     std::vector<uint32_t> cc_obs;
@@ -1141,10 +1144,14 @@ qd_status batch_plan(qd_batch* b, int j, int warps, size_t budget) {
     if (j >= (int)d->wins.size()) continue;
     const auto& h = d->wins[j].h;
     int s = warps;
-    for (; s >= 1; --s) {
-      S.L[i] = qd::make_layout(h.n_rows, h.n_cols, h.n_edges, h.n_short, h.short_edges_max, d->kp.nb, s, false,
-                               d->hist_on, d->lw_on);
-      if (qd::al16(S.L[i].total) + 32 <= budget) break;
+    for (; s >= 1; --s) {  // as many slots as fit; the window graph staged when that costs none
+      bool fits = false;
+      for (int sg = 1; sg >= 0 && !fits; --sg) {
+        S.L[i] = qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, d->kp.nb, s, sg, d->hist_on,
+                                       d->lw_on, false);
+        fits = qd::al16(S.L[i].total) + 32 <= budget;
+      }
+      if (fits) break;
     }
     if (s < 1) {
       set_error("qd_batch: member " + std::to_string(i) + " window " + std::to_string(j) + " needs " +

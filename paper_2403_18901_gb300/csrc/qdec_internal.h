@@ -24,6 +24,13 @@ struct WindowHost {
   std::vector<uint16_t> row_ptr;            // CSR row pointers
   std::vector<uint32_t> row_ent;            // CSR entries: CSC edge id | (window column << 16)
   std::vector<float> llr;
+  // the graph in slices (gdg_kernel.cuh), checks and columns by label
+  int row_pairs = 0, col_cells = 0;    // slice totals
+  int srow_pairs = 0, scol_cells = 0;  // bounds on those of a shortened graph
+  int max_row_deg = 0;
+  std::vector<uint32_t> s_rent, s_cent;
+  std::vector<uint16_t> s_roff, s_coff, s_row, s_col, s_ref, s_cef;
+  std::vector<float> s_llr;
 };
 
 struct DemHost {
@@ -52,6 +59,9 @@ bool build_dem_code_capacity(const qd_bb_code& code, double p_data, double p_syn
 int n_windows(const DemHost& d, int W, int F);
 // merge: the H_1 merge of Sec. III (0 none, 1 equal restrictions, 2 identity)
 bool build_window(const DemHost& d, int W, int F, int k, bool shorten, WindowHost& out, int merge = 0);
+
+// The graph in slices (s_* of WindowHost) and the bounds for its shortened graphs.
+bool build_slices(WindowHost& o);
 
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max);
 cudaError_t set_decode_smem(size_t bytes);

@@ -1,0 +1,187 @@
+// Host check of the sliced window graphs (build_slices) and of the decode
+// kernels' shared-memory layout (make_slice_layout), built with g++ by
+// tests/test_slices_host.py.
+//
+// usage: slice_check l m a0x a0y .. b2x b2y rounds W F merge shorten trials
+// For every window: each edge is stored once per side and the two sides agree
+// on its position; every other place is a dummy; a column's checks ascend in
+// window row; the flag of a wide slice is set where a position passes 31.
+// For random shortened graphs (and the one of the highest degrees) the slices
+// stay within the bounds.  Layout regions are 16-byte aligned and disjoint
+// where they live together.  Prints "ok" or the first violation.
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include <string>
+
+#include "../paper_2403_18901_gb300/csrc/qdec_internal.h"
+#include "../paper_2403_18901_gb300/csrc/gdg_kernel.cuh"
+
+namespace qd {
+std::string last;
+void set_error(const std::string& m) { last = m; }
+}  // namespace qd
+
+namespace {
+#define REQ(c, ...)                \
+  do {                             \
+    if (!(c)) {                    \
+      std::printf(__VA_ARGS__);    \
+      std::printf(" [%s]\n", #c);  \
+      return false;                \
+    }                              \
+  } while (0)
+
+bool check_graph(const qd::WindowHost& h) {
+  const int nr = h.n_rows, nc = h.n_cols, nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
+  REQ((int)h.s_roff.size() == nrs + 1 && (int)h.s_coff.size() == ncs + 1, "offsets");
+  const unsigned low = qd::kWideSlice - 1;
+  size_t real = 0, dummies = 0;
+  std::vector<int> seen(h.n_edges, 0);
+  for (int l = 0; l < nc; ++l) {
+    const int c = h.s_col[l], d = h.col_ptr[c + 1] - h.col_ptr[c], c0 = h.s_coff[l >> 5] & low;
+    const int w = (int)(h.s_coff[(l >> 5) + 1] & low) - c0;
+    REQ(d <= w, "column %d wider than its slice", l);
+    REQ(h.s_llr[l] == h.llr[c], "prior of column %d", l);
+    for (int u = 0; u < w; ++u) {
+      const uint32_t e = h.s_cent[(size_t)(c0 + u) * 32 + (l & 31)];
+      if (u >= d) {
+        REQ(e == (uint32_t)(32 * nrs) << 16, "column %d: place %d is no dummy", l, u);
+        continue;
+      }
+      const int r = (int)(e >> 16), pos = (int)(e & 0xFFFF), fe = h.s_cef[(size_t)(c0 + u) * 32 + (l & 31)];
+      REQ(r < nr && pos < qd::kMaxRowDeg, "column %d entry %d", l, u);
+      REQ(fe == h.col_ptr[c] + u && h.col_rows[fe] == h.s_row[r], "column %d entry %d: edge", l, u);
+      seen[fe]++;
+      const size_t ri = ((size_t)(h.s_roff[r >> 5] + (pos >> 1)) * 32 + (r & 31)) * 2 + (pos & 1);
+      REQ((pos >> 1) < h.s_roff[(r >> 5) + 1] - h.s_roff[r >> 5], "check %d position %d", r, pos);
+      REQ(h.s_rent[ri] == 4u * (uint32_t)l && h.s_ref[ri] == fe, "check %d position %d: other side", r, pos);
+      REQ(pos < 32 || (h.s_coff[l >> 5] & qd::kWideSlice), "column %d: slice not flagged", l);
+    }
+  }
+  for (int e = 0; e < h.n_edges; ++e) REQ(seen[e] == 1, "edge %d stored %d times", e, seen[e]);
+  for (size_t i = 0; i < h.s_rent.size(); ++i) (h.s_rent[i] < 4u * (uint32_t)nc ? real : dummies)++;
+  for (uint32_t x : h.s_rent)
+    REQ(x < 4u * (uint32_t)nc || x == 4u * (uint32_t)(32 * ncs), "check entry is neither a column nor the dummy");
+  REQ((int)real == h.n_edges && real + dummies == (size_t)64 * h.row_pairs, "check entries");
+  return true;
+}
+
+// the slices a shortened graph of these window columns takes
+bool check_short(const qd::WindowHost& h, const std::vector<int>& cols) {
+  std::vector<int> cd, rd(h.n_rows, 0);
+  for (int c : cols) {
+    cd.push_back(h.col_ptr[c + 1] - h.col_ptr[c]);
+    for (int e = h.col_ptr[c]; e < h.col_ptr[c + 1]; ++e) rd[h.col_rows[e]]++;
+  }
+  std::sort(cd.rbegin(), cd.rend());
+  std::sort(rd.rbegin(), rd.rend());
+  int cells = 0, pairs = 0;
+  for (size_t i = 0; i < cd.size(); i += 32) cells += cd[i];
+  for (size_t i = 0; i < rd.size(); i += 32) pairs += (rd[i] + 1) / 2;
+  REQ(cells <= h.scol_cells, "column slices %d > %d", cells, h.scol_cells);
+  REQ(pairs <= h.srow_pairs, "check slices %d > %d", pairs, h.srow_pairs);
+  return true;
+}
+
+struct Region {
+  const char* name;
+  unsigned off, bytes;
+};
+bool disjoint(std::vector<Region> rs, unsigned lo, unsigned hi, const char* part) {
+  std::sort(rs.begin(), rs.end(), [](const Region& a, const Region& b) { return a.off < b.off; });
+  unsigned end = lo;
+  for (const Region& r : rs) {
+    REQ(r.off % 16u == 0, "%s.%s at %u", part, r.name, r.off);
+    if (!r.bytes) continue;
+    REQ(r.off >= end, "%s.%s at %u overlaps (ends %u)", part, r.name, r.off, end);
+    end = r.off + r.bytes;
+    REQ(end <= hi, "%s.%s ends at %u past %u", part, r.name, end, hi);
+  }
+  return true;
+}
+
+bool check_layout(const qd::WindowHost& h, int nb, int nslots, int stage, bool ranker, bool lw, bool glob) {
+  const qd::SliceDims D{h.row_pairs, h.col_cells, h.srow_pairs, h.scol_cells};
+  const int nr = h.n_rows, nc = h.n_cols, ns = h.n_short;
+  const qd::Layout L = qd::make_slice_layout(D, nr, nc, ns, nb, nslots, stage, ranker, lw, glob);
+  const unsigned nrp = qd::up32(nr), ncp = qd::up32(nc), nsp = qd::up32(ns), rw = L.rw;
+  REQ(L.total % 16u == 0 && L.U % 16u == 0 && L.V % 16u == 0 && L.b_size % 16u == 0, "alignment");
+  const std::vector<Region> keep = {{"sbits", L.sbits, 4u * rw}, {"cbits", L.cbits, 4u * L.cw},
+                                    {"res_status", L.res_status, 4u * nb}, {"res_pm", L.res_pm, 8u * nb},
+                                    {"res_ebits", L.res_ebits, 4u * L.sw * nb}, {"red", L.red, 512u},
+                                    {"misc", L.misc, 64u}};
+  if (!disjoint(keep, 0, L.V, "persistent")) return false;
+  std::vector<Region> sg = {{"sel", L.sel, 2u * ns}, {"rent", L.s_rent, 256u * D.srow_pairs},
+                            {"cent", L.s_cent, 128u * D.scol_cells}, {"roff", L.s_roff, 2u * (rw + 1)},
+                            {"coff", L.s_coff, 2u * (L.sw + 1u)}, {"llr", L.s_llr, 4u * nsp},
+                            {"vdeg", L.s_vdeg, nsp}, {"ref", L.s_ref, lw ? 128u * D.srow_pairs : 0u},
+                            {"cef", L.s_cef, lw ? 64u * D.scol_cells : 0u}, {"cperm", L.s_cperm, 2u * nr},
+                            {"vperm", L.s_vperm, 2u * ns}, {"rowcnt", L.rowcnt, 4u * (nrp + 1)}};
+  if (!disjoint(sg, L.V, L.U, "shortened graph")) return false;
+  const unsigned base = glob ? 0u : L.V, hi = glob ? L.total - L.U : L.total;
+  std::vector<Region> pre = {{"post", L.p_post + base, 4u * (ncp + 1)}, {"key", L.p_key + base, 4u * ncp},
+                             {"cns", L.p_cns + base, 16u * (nrp + 1)}, {"par", L.p_par + base, 8u * rw}};
+  std::vector<Region> st;
+  if (L.pre_stage)
+    st = {{"q_rent", L.q_rent + base, 256u * D.row_pairs}, {"q_cent", L.q_cent + base, 128u * D.col_cells},
+          {"q_roff", L.q_roff + base, 2u * (rw + 1)},      {"q_coff", L.q_coff + base, 2u * (L.cw + 1u)},
+          {"q_llr", L.q_sllr + base, 4u * ncp}};
+  pre.insert(pre.end(), st.begin(), st.end());
+  if (!disjoint(pre, base, hi, "pre-BP")) return false;
+  // the sort: filled from the keys; then read while the shortened graph is written
+  const unsigned need = std::max(8u * (unsigned)L.sortn, 4u * (nsp + nrp));
+  REQ(L.sortn >= nc && !(L.sortn & (L.sortn - 1)), "sort size");
+  std::vector<Region> rank = {{"key", L.p_key + base, 4u * ncp}, {"sort", L.p_sort + base, need}};
+  if (stage == 2) rank.insert(rank.end(), st.begin(), st.end());
+  if (!disjoint(rank, base, hi, "ranking")) return false;
+  if (!glob) {
+    sg.push_back({"sort", L.p_sort + base, need});
+    if (stage == 2) sg.insert(sg.end(), st.begin(), st.end());
+    if (!disjoint(sg, L.V, hi, "shortening")) return false;
+  }
+  const std::vector<Region> slot = {{"post", L.b_post, 4u * (nsp + 1)}, {"acc", L.b_acc, 4u * ns},
+                                    {"hfl", L.b_hfl, 1u * ns}, {"status", L.b_status, nsp},
+                                    {"cns", L.b_cns, 16u * (nrp + 1)}, {"deg", L.b_deg, nrp}, {"sp", L.b_sp, 4u * rw},
+                                    {"unsat", L.b_unsat, 4u * rw}, {"hq", L.b_hq, ranker ? 4u * ns : 0u}};
+  if (!disjoint(slot, 0, L.b_size, "slot")) return false;
+  REQ((glob ? 0u : L.U) + L.b_size * (unsigned)nslots <= hi, "slots past the end");
+  return true;
+}
+}  // namespace
+
+int main(int argc, char** argv) {
+  if (argc != 21) return 2;
+  int x[20];
+  for (int i = 0; i < 20; ++i) x[i] = std::atoi(argv[i + 1]);
+  qd_bb_code code{x[0], x[1], {x[2], x[4], x[6]}, {x[3], x[5], x[7]}, {x[8], x[10], x[12]}, {x[9], x[11], x[13]}};
+  const int rounds = x[14], W = x[15], F = x[16], merge = x[17], shorten = x[18], trials = x[19];
+  qd::DemHost d;
+  const bool ok = rounds > 0 ? qd::build_dem_host(code, qd_noise{0.003, rounds}, d)
+                             : qd::build_dem_code_capacity(code, 0.04, 0.001, d);
+  if (!ok) return std::printf("dem: %s\n", qd::last.c_str()), 1;
+  std::mt19937 rng(5);
+  for (int k = 0; k < qd::n_windows(d, W, F); ++k) {
+    qd::WindowHost h;
+    if (!qd::build_window(d, W, F, k, shorten != 0, h, merge) || !qd::build_slices(h))
+      return std::printf("window %d: %s\n", k, qd::last.c_str()), 1;
+    if (h.n_cols == 0) continue;
+    if (!check_graph(h)) return 1;
+    std::vector<int> cols(h.n_cols);
+    for (int c = 0; c < h.n_cols; ++c) cols[c] = h.s_col[c];  // the highest degrees first
+    for (int t = 0; t < trials; ++t) {
+      if (!check_short(h, std::vector<int>(cols.begin(), cols.begin() + h.n_short))) return 1;
+      std::shuffle(cols.begin(), cols.end(), rng);
+      if (t & 1)  // the columns of few checks, so that those checks are as heavy as they get
+        std::stable_sort(cols.begin(), cols.end(),
+                         [&](int a, int b) { return h.col_rows[h.col_ptr[a]] < h.col_rows[h.col_ptr[b]]; });
+    }
+    for (int nb : {1, 22, 47})
+      for (int slots : {1, 3, 8})
+        for (int m = 0; m < 24; ++m)
+          if (!check_layout(h, nb, slots, m >> 3, m & 1, m & 2, m & 4)) return 1;
+  }
+  std::printf("ok\n");
+  return 0;
+}
