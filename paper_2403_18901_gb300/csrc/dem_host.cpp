@@ -529,11 +529,11 @@ bool build_slices(WindowHost& o) {
   }
   o.s_roff.assign(nrs + 1, 0);
   o.s_coff.assign(ncs + 1, 0);
-  for (int q = 0; q < nrs; ++q) o.s_roff[q + 1] = (uint16_t)(o.s_roff[q] + (rdeg(o.s_row[32 * q]) + 1) / 2);
+  for (int q = 0; q < nrs; ++q) o.s_roff[q + 1] = (uint16_t)(o.s_roff[q] + (rdeg(o.s_row[32 * q]) + 3) / 4);
   for (int q = 0; q < ncs; ++q) o.s_coff[q + 1] = (uint16_t)(o.s_coff[q] + cdeg(o.s_col[32 * q]));
-  o.row_pairs = o.s_roff[nrs];
+  o.row_quads = o.s_roff[nrs];
   o.col_cells = o.s_coff[ncs];
-  o.s_rent.assign((size_t)64 * o.row_pairs, 4u * (uint32_t)(32 * ncs));  // the dummy column
+  o.s_rent.assign((size_t)128 * o.row_quads, 4u * (uint32_t)(32 * ncs));  // the dummy column
   o.s_cent.assign((size_t)32 * o.col_cells, (uint32_t)(32 * nrs) << 16);  // the dummy check
   o.s_ref.assign(o.s_rent.size(), 0);
   o.s_cef.assign(o.s_cent.size(), 0);
@@ -545,7 +545,7 @@ bool build_slices(WindowHost& o) {
     o.s_llr[l] = o.llr[c];
     for (int e = o.col_ptr[c]; e < o.col_ptr[c + 1]; ++e) {
       const int r = rlab[o.col_rows[e]], pos = fill[r]++;
-      const size_t ri = ((size_t)(o.s_roff[r >> 5] + (pos >> 1)) * 32 + (r & 31)) * 2 + (pos & 1);
+      const size_t ri = ((size_t)(o.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
       const size_t ci = (size_t)(o.s_coff[l >> 5] + (e - o.col_ptr[c])) * 32 + (l & 31);
       o.s_rent[ri] = 4u * (uint32_t)l;
       o.s_ref[ri] = (uint16_t)e;
@@ -557,23 +557,29 @@ bool build_slices(WindowHost& o) {
   // a dummy takes its node's first edge's learned weight, so that a weight
   // touches no node but its own two
   for (int r = 0; r < nr; ++r)
-    for (int pos = std::max(1, fill[r]); pos < 2 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
-      const size_t r0 = ((size_t)o.s_roff[r >> 5] * 32 + (r & 31)) * 2;
-      o.s_ref[r0 + 64 * (size_t)(pos >> 1) + (pos & 1)] = o.s_ref[r0];
+    for (int pos = std::max(1, fill[r]); pos < 4 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
+      const size_t r0 = ((size_t)o.s_roff[r >> 5] * 32 + (r & 31)) * 4;
+      o.s_ref[r0 + 128 * (size_t)(pos >> 2) + (pos & 3)] = o.s_ref[r0];
     }
   for (int l = 0; l < nc; ++l)
     for (int u = cdeg(o.s_col[l]); u < o.s_coff[(l >> 5) + 1] - o.s_coff[l >> 5]; ++u) {
       const size_t c0 = (size_t)o.s_coff[l >> 5] * 32 + (l & 31);
       o.s_cef[c0 + 32 * (size_t)u] = o.s_cef[c0];
     }
+  for (int q = 0; q < ncs; ++q) {
+    const int w = o.s_coff[q + 1] - o.s_coff[q];
+    for (int x = 0; x < 4; ++x)
+      if (w >= 4 - x) o.cls[x] = q + 1;
+    if (wide[q] && w >= 3) o.wide3 = 1;
+  }
   for (int q = 0; q < ncs; ++q)
     if (wide[q]) o.s_coff[q] |= kWideSlice;
   // a shortened graph: every slice but the first is no wider than the least
   // degree of the slice before it, so the widths sum to at most the widest
-  // node plus edges / 32 (check slices rounded up to pairs)
+  // node plus edges / 32 (check slices rounded up to fours)
   const int ns = o.n_short, nss = (ns + 31) / 32, es = o.short_edges_max;
   const int wr = std::min(o.max_row_deg, ns);
-  o.srow_pairs = std::min(nrs * ((wr + 1) / 2), (wr + es / 32 + nrs) / 2 + 1);
+  o.srow_quads = std::min(nrs * ((wr + 3) / 4), (wr + es / 32 + 3 * nrs) / 4 + 1);
   o.scol_cells = std::min(nss * max_col_deg, max_col_deg + es / 32);
   return true;
 }

@@ -85,22 +85,22 @@ struct CheckAcc {
 };
 
 // One input at position u: posterior pv, the previous iteration's record (its
-// argmin position oam, two magnitudes, this edge's sign osg at bit 31).
-// Returns the bits of v, whose sign the caller collects.  The clip of Eq. (3)
-// bounds every magnitude alike, so it is applied to the two smallest at the
-// end.  A posterior is never -0 (its prior is positive and x + y = -0 only for
+// argmin position oam, two magnitudes, this edge's sign osg at bit 31); before
+// the first iteration that record is zero, and so is the message.  Returns the
+// bits of v, whose sign the caller collects.  The clip of Eq. (3) bounds every
+// magnitude alike, so it is applied to the two smallest at the end.  A
+// posterior is never -0 (its prior is positive and x + y = -0 only for
 // x = y = -0), nor is the difference of two messages, so the sign bit is the
 // comparison with 0, and pv <= 0 is the sign of pv's bits minus one.
-template <bool LW, bool FIRST>
+template <bool LW>
 __device__ __forceinline__ uint32_t check_input(CheckAcc& A, float pv, uint32_t u, uint32_t oam, float om1, float om2,
-                                                uint32_t osg, float w) {
-  float v = pv;
-  if (!FIRST) {
-    float m = flip_sign(u == oam ? om2 : om1, osg & 0x80000000u);
-    if (LW) m = __fmul_rn(w, m);
-    v = __fsub_rn(pv, m);
-    if (LW && pv == CUDART_INF_F) v = pv;  // a dead input stays one under an infinite weighted message
-  }
+                                                uint32_t osg, float w, bool first) {
+  float m = flip_sign(u == oam ? om2 : om1, osg & 0x80000000u);
+  if (LW) m = __fmul_rn(w, m);
+  float v = __fsub_rn(pv, m);
+  // (an infinite weight: no message before the first iteration, and a dead
+  // input stays one)
+  if (LW && (first || pv == CUDART_INF_F)) v = pv;
   const float a = fabsf(v);
   A.am = a < A.m1 ? u : A.am;
   A.m2 = fminf(A.m2, fmaxf(A.m1, a));
@@ -109,20 +109,29 @@ __device__ __forceinline__ uint32_t check_input(CheckAcc& A, float pv, uint32_t 
   return __float_as_uint(v);
 }
 
+// Four inputs at positions u .. u + 3; osg: the old signs, position u at bit
+// 31.  The new signs are shifted into sg, one bit each.
+template <bool LW>
+__device__ __forceinline__ void check_four(CheckAcc& A, const uint4& e, const char* post, uint32_t u, uint32_t oam,
+                                           float om1, float om2, uint32_t osg, const float (&w)[4], bool first,
+                                           uint32_t& sg) {
+  const float p0 = *(const float*)(post + e.x), p1 = *(const float*)(post + e.y);
+  const float p2 = *(const float*)(post + e.z), p3 = *(const float*)(post + e.w);
+  sg = __funnelshift_l(check_input<LW>(A, p0, u, oam, om1, om2, osg, w[0], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p1, u + 1, oam, om1, om2, osg << 1, w[1], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p2, u + 2, oam, om1, om2, osg << 2, w[2], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p3, u + 3, oam, om1, om2, osg << 3, w[3], first), sg, 1);
+}
+
 // The record of a check from its inputs and the syndrome bit: magnitudes
 // bounded by the clip (an only input gets the clip itself, the minimum over
 // the empty set; the first iteration's inputs are priors, not clipped).
 template <bool LW>
 __device__ __forceinline__ CNState check_record(const CheckAcc& A, uint32_t sg0, uint32_t sg1, uint32_t sbit, bool first,
                                                 float alpha, float clip) {
-  float m1 = A.m1, m2 = A.m2;
-  if (first) {
-    m1 = m1 == CUDART_INF_F ? clip : m1;
-    m2 = m2 == CUDART_INF_F ? clip : m2;
-  } else {
-    m1 = fminf(m1, clip);
-    m2 = fminf(m2, clip);
-  }
+  const float lim = first ? FLT_MAX : clip;
+  float m1 = A.m1 == CUDART_INF_F ? clip : fminf(A.m1, lim);
+  float m2 = A.m2 == CUDART_INF_F ? clip : fminf(A.m2, lim);
   if (!LW) {
     m1 = __fmul_rn(alpha, m1);
     m2 = __fmul_rn(alpha, m2);
@@ -138,84 +147,71 @@ struct LwRow {
   const uint16_t* ef;
 };
 __device__ __forceinline__ float lw_at(const LwRow& r, int i) { return r.w[r.ef[i]]; }
+template <bool LW>
+__device__ __forceinline__ void lw_four(const LwRow& r, int i, bool first, float (&w)[4]) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x) w[x] = LW && !first ? lw_at(r, i + x) : 0.0f;
+}
 
 // Check-node update of Eq. (1) of one check by one lane.  ent: the lane's
-// entry pairs, `np` of them, 32 pairs apart (ei: the index of the first entry,
-// for the learned weights' edge ids); post: posteriors; rec: its record, the
-// previous iteration's on entry.  Returns at bit 31 the parity of the hard
-// decisions read, xor the syndrome bit: the test H e = s of the iteration
-// before.  What bounds it: issue, ALU instructions above all (half rate, about
-// 11 of 14 per entry); the posterior gathers' bank conflicts come next.  With
-// a sign byte and an edge id per edge, a NaN test and the clip on every input
-// and ragged rows, 5000 shots of [[144,12,12]] took 450 ms; in slices, with
-// the signs as bits of the record and the clip on the two minima, 354 ms.
-template <bool LW, bool FIRST>
-__device__ __forceinline__ uint32_t check_lane(const uint2* ent, int np, const char* post, CNState* rec, uint32_t sbit,
-                                               float alpha, float clip, const LwRow& lw, int ei) {
-  CNState oc{};
-  if (!FIRST) oc = *rec;
+// entries, four at a time, `nq` times, 32 lanes apart (ei: the index of the
+// first entry, for the learned weights' edge ids); post: posteriors; rec: its
+// record, the previous iteration's on entry.  Returns at bit 31 the parity of
+// the hard decisions read, xor the syndrome bit: the test H e = s of the
+// iteration before.  What bounds it: issue, ALU instructions above all (half
+// rate, about 11 of 14 per entry), and the latency of entry and posterior
+// loads, which four entries at a time overlap; the posterior gathers' bank
+// conflicts come next.  With a sign byte and an edge id per edge, a NaN test
+// and the clip on every input and ragged rows, 5000 shots of [[144,12,12]]
+// took 450 ms; in slices, with the signs as bits of the record and the clip on
+// the two minima, 354 ms.
+template <bool LW>
+__device__ __forceinline__ uint32_t check_lane(const uint4* ent, int nq, const char* post, CNState* rec, uint32_t sbit,
+                                               float alpha, float clip, const LwRow& lw, int ei, bool first) {
+  CNState oc = *rec;
+  if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
   const uint32_t oam = oc.am & 63u;
   uint32_t osg = oc.sg;
   CheckAcc A{CUDART_INF_F, CUDART_INF_F, 0u, 0u};
   uint32_t sg0 = 0u, sg1 = 0u;
-  for (int p0 = 0; p0 < np; p0 += 16) {  // 32 positions to a sign word
-    const int p1 = min(np, p0 + 16);
+  for (int q0 = 0; q0 < nq; q0 += 8) {  // 32 positions to a sign word
+    const int q1 = min(nq, q0 + 8);
     uint32_t sg = 0u;
-    for (int p = p0; p < p1; ++p) {
-      const uint2 e = ent[32 * p];
-      const float a = *(const float*)(post + e.x), b = *(const float*)(post + e.y);
-      float wa = 0.0f, wb = 0.0f;
-      if (LW && !FIRST) {
-        wa = lw_at(lw, ei + 64 * p);
-        wb = lw_at(lw, ei + 64 * p + 1);
-      }
-      sg = __funnelshift_l(check_input<LW, FIRST>(A, a, 2 * p, oam, oc.m1, oc.m2, osg, wa), sg, 1);
-      osg += osg;
-      sg = __funnelshift_l(check_input<LW, FIRST>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, osg, wb), sg, 1);
-      osg += osg;
+#pragma unroll 1
+    for (int q = q0; q < q1; ++q) {
+      float w[4];
+      lw_four<LW>(lw, ei + 128 * q, first, w);
+      check_four<LW>(A, ent[32 * q], post, 4 * q, oam, oc.m1, oc.m2, osg, w, first, sg);
+      osg <<= 4;
     }
-    sg = sg << (32 - 2 * (p1 - p0)) % 32;  // the first position to bit 31
-    if (p0 == 0) {
-      sg0 = sg;
-      osg = oc.am;
-    } else {
-      sg1 = sg;
-    }
+    sg <<= (32 - 4 * (q1 - q0)) & 31;  // the first position to bit 31
+    if (q0 == 0) sg0 = sg;
+    else sg1 = sg;
+    osg = oc.am;
   }
-  *rec = check_record<LW>(A, sg0, sg1, sbit, FIRST, alpha, clip);
+  *rec = check_record<LW>(A, sg0, sg1, sbit, first, alpha, clip);
   return (A.hp ^ (sbit << 31)) & 0x80000000u;
 }
 
-// The same by TPC neighbouring lanes (entry pairs sub, sub + TPC, ...); every
-// lane of the group ends with the record.
+// The same by tpc neighbouring lanes (fours sub, sub + tpc, ...); every lane
+// of the group ends with the record.
 template <bool LW>
-__device__ __forceinline__ CNState check_group(const uint2* ent, int np, const char* post, const CNState& oc,
-                                               uint32_t sbit, float alpha, float clip, bool first, const LwRow& lw,
-                                               int ei, int sub, int tpc, bool wide, uint32_t& unsat) {
+__device__ __forceinline__ CNState check_group(const uint4* ent, int nq, const char* post, CNState oc, uint32_t sbit,
+                                               float alpha, float clip, bool first, const LwRow& lw, int ei, int sub,
+                                               int tpc, bool wide, uint32_t& unsat) {
+  if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
   const uint32_t oam = oc.am & 63u;
   CheckAcc A{CUDART_INF_F, CUDART_INF_F, 0u, 0u};
   uint32_t sg0 = 0u, sg1 = 0u;
-  for (int p = sub; p < np; p += tpc) {
-    const uint2 e = ent[32 * p];
-    const float a = *(const float*)(post + e.x), b = *(const float*)(post + e.y);
-    float wa = 0.0f, wb = 0.0f;
-    if (LW && !first) {
-      wa = lw_at(lw, ei + 64 * p);
-      wb = lw_at(lw, ei + 64 * p + 1);
-    }
-    const uint32_t ow = p < 16 ? oc.sg : oc.am;
-    const int sh = (2 * p) & 31;
-    uint32_t va, vb;
-    if (first) {
-      va = check_input<LW, true>(A, a, 2 * p, oam, oc.m1, oc.m2, 0u, wa);
-      vb = check_input<LW, true>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, 0u, wb);
-    } else {
-      va = check_input<LW, false>(A, a, 2 * p, oam, oc.m1, oc.m2, ow << sh, wa);
-      vb = check_input<LW, false>(A, b, 2 * p + 1, oam, oc.m1, oc.m2, ow << (sh + 1), wb);
-    }
-    const uint32_t s2 = ((va & 0x80000000u) | ((vb & 0x80000000u) >> 1)) >> sh;
-    if (p < 16) sg0 |= s2;
-    else sg1 |= s2;
+#pragma unroll 1
+  for (int q = sub; q < nq; q += tpc) {
+    float w[4];
+    lw_four<LW>(lw, ei + 128 * q, first, w);
+    const int sh = (4 * q) & 31;
+    uint32_t sg = 0u;
+    check_four<LW>(A, ent[32 * q], post, 4 * q, oam, oc.m1, oc.m2, (q < 8 ? oc.sg : oc.am) << sh, w, first, sg);
+    if (q < 8) sg0 |= sg << (28 - sh);
+    else sg1 |= sg << (28 - sh);
   }
   for (int off = tpc >> 1; off; off >>= 1) {
     const float x1 = __shfl_xor_sync(FULL, A.m1, off), x2 = __shfl_xor_sync(FULL, A.m2, off);
@@ -233,32 +229,123 @@ __device__ __forceinline__ CNState check_group(const uint2* ent, int np, const c
   return check_record<LW>(A, sg0, sg1, sbit, first, alpha, clip);
 }
 
-// Variable-node update of Eq. (2) by one lane: prior + the messages of its
-// checks in ascending check order; `n` places 32 entries apart (a dummy adds
-// +0), at most three records in flight.
-template <bool LW>
-__device__ __forceinline__ float column_sum(float p, const uint32_t* ent, int n, bool wide, const char* cns,
-                                            const LwRow& lw, int ei) {
-  auto msgs = [&](int u, auto cnt) {
-    constexpr int N = decltype(cnt)::value;
-    uint32_t e[N];
-    CNState c[N];
-    float w[N];
+// The parity of a check's hard decisions, at bit 31.
+__device__ __forceinline__ uint32_t check_parity(const uint4* ent, int nq, const char* post) {
+  uint32_t hp = 0u;
+  for (int q = 0; q < nq; ++q) {
+    const uint4 e = ent[32 * q];
+    const uint32_t a = *(const uint32_t*)(post + e.x), b = *(const uint32_t*)(post + e.y);
+    const uint32_t c = *(const uint32_t*)(post + e.z), d = *(const uint32_t*)(post + e.w);
+    hp ^= ((a - 1u) ^ (b - 1u)) ^ ((c - 1u) ^ (d - 1u));
+  }
+  return hp & 0x80000000u;
+}
+
+// What the variable pass walks: this lane's view of the column slices.
+struct ColView {
+  ColClasses K;
+  const uint32_t* cent;
+  const uint16_t* coff;
+  const float* llr;
+  const int8_t* status;  // nullptr: every column is active
+  const char* cns;
+  LwRow lw;
+  int lane, st;  // the group takes every st-th slice
+};
+
+// The first slice s, s - st, ... of the group at or past end.
+__device__ __forceinline__ int back_to(int s, int end, int st) {
+  while (s - st >= end) s -= st;
+  return s;
+}
+
+// Variable-node update of Eq. (2), one column per lane: prior + the messages
+// of its checks in ascending check order (a dummy adds +0).  M slices of N
+// entries each at once, so that M * N record gathers are in flight: the pass
+// is a chain of shared-memory round trips (entry, record) ahead of a few
+// instructions, and with one slice after another it took 1.75 times the check
+// pass although it issues fewer instructions.  Slices past `end` repeat the
+// first and store nothing: one copy of the code serves every remainder (a copy
+// for each cost more in instruction fetches than the repeated loads do).
+// put(s, p): the posterior of this lane's column of slice s.
+template <bool LW, bool WIDE, int N, int M, class Put>
+__device__ __forceinline__ void column_group(const ColView& V, int s, int end, int cell, int stride, Put put) {
+  uint32_t e[M][N];
+  CNState c[M][N];
+  float p[M], w[M][N];
+  int act[M];
 #pragma unroll
-    for (int x = 0; x < N; ++x) e[x] = ent[32 * (u + x)];
+  for (int m = 0; m < M; ++m) {
+    const bool in = m == 0 || s + m * V.st < end;
+    const int k = 32 * (in ? s + m * V.st : s) + V.lane, ei = 32 * (in ? cell + m * stride : cell) + V.lane;
+    act[m] = V.status ? (int)V.status[k] : -1;
+    if (!in) act[m] = 0;
+    p[m] = V.llr[k];
 #pragma unroll
     for (int x = 0; x < N; ++x) {
-      c[x] = *(const CNState*)(cns + (e[x] >> 12));
-      w[x] = LW ? lw_at(lw, ei + 32 * (u + x)) : 0.0f;
+      e[m][x] = V.cent[ei + 32 * x];
+      w[m][x] = LW ? lw_at(V.lw, ei + 32 * x) : 0.0f;
     }
+  }
 #pragma unroll
-    for (int x = 0; x < N; ++x) p = __fadd_rn(p, c2v<LW>(c[x], e[x], wide, w[x]));
-  };
-  int u = 0;
-  for (; u + 3 <= n; u += 3) msgs(u, std::integral_constant<int, 3>{});
-  if (u + 2 == n) msgs(u, std::integral_constant<int, 2>{});
-  else if (u + 1 == n) msgs(u, std::integral_constant<int, 1>{});
-  return p;
+  for (int m = 0; m < M; ++m)
+#pragma unroll
+    for (int x = 0; x < N; ++x) c[m][x] = *(const CNState*)(V.cns + (e[m][x] >> 12));
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+#pragma unroll
+    for (int x = 0; x < N; ++x) p[m] = __fadd_rn(p[m], c2v<LW>(c[m][x], e[m][x], WIDE, w[m][x]));
+    if (act[m] == -1) put(s + m * V.st, p[m]);
+  }
+}
+
+// The variable pass over column slices first, first + st, ...  WIDE: columns
+// of degree one and two may have edges at positions past 31; wide: so may the
+// others (then, and for widths past three, one slice at a time).
+template <bool LW, bool WIDE, class Put>
+__device__ __forceinline__ void column_pass(const ColView& V, int first, bool wide, Put put) {
+  constexpr int kLow = kWideSlice - 1;
+  int s = first;
+#pragma unroll 1
+  for (const int end = wide ? V.K.n1 : V.K.n4; s < end; s += V.st) {
+    int c0 = V.coff[s] & kLow;
+    const int c1 = V.coff[s + 1] & kLow, k = 32 * s + V.lane;
+    float p = V.llr[k];
+    auto more = [&](auto cnt) {
+      constexpr int N = decltype(cnt)::value;
+      uint32_t e[N];
+      CNState c[N];
+#pragma unroll
+      for (int x = 0; x < N; ++x) e[x] = V.cent[32 * (c0 + x) + V.lane];
+#pragma unroll
+      for (int x = 0; x < N; ++x) c[x] = *(const CNState*)(V.cns + (e[x] >> 12));
+#pragma unroll
+      for (int x = 0; x < N; ++x)
+        p = __fadd_rn(p, c2v<LW>(c[x], e[x], true, LW ? lw_at(V.lw, 32 * (c0 + x) + V.lane) : 0.0f));
+      c0 += N;
+    };
+    while (c0 + 3 <= c1) more(std::integral_constant<int, 3>{});
+    while (c0 < c1) more(std::integral_constant<int, 1>{});
+    if (!V.status || V.status[k] == -1) put(s, p);
+  }
+  if (wide) return;
+  {
+    const int b = V.coff[V.K.n4] & kLow;
+#pragma unroll 1
+    for (; s < V.K.n3; s += 2 * V.st) column_group<LW, false, 3, 2>(V, s, V.K.n3, b + 3 * (s - V.K.n4), 3 * V.st, put);
+    s = back_to(s, V.K.n3, V.st);
+  }
+  {
+    const int b = V.coff[V.K.n3] & kLow;
+#pragma unroll 1
+    for (; s < V.K.n2; s += 2 * V.st) column_group<LW, WIDE, 2, 2>(V, s, V.K.n2, b + 2 * (s - V.K.n3), 2 * V.st, put);
+    s = back_to(s, V.K.n2, V.st);
+  }
+  {
+    const int b = V.coff[V.K.n2] & kLow;
+#pragma unroll 1
+    for (; s < V.K.n1; s += 4 * V.st) column_group<LW, WIDE, 1, 4>(V, s, V.K.n1, b + (s - V.K.n2), V.st, put);
+  }
 }
 
 __device__ __forceinline__ uint32_t bit_of(const uint32_t* w, int j) { return (w[j >> 5] >> (j & 31)) & 1u; }
@@ -542,6 +629,7 @@ struct ShortG {
   const uint8_t* vdeg;
   const uint32_t* sbits;
   const uint16_t *ref, *cef;  // full-window edge of each check / column entry (learned weights)
+  const ColClasses* cls;
   const float* wts;
   int wT, wE;
   int rpb;  // window rows per block (block of a column = its first row / rpb)
@@ -627,10 +715,10 @@ __device__ int peel(const ShortG& G, const Slot& B, const Grp& g, int& act) {
     if (jc == kNone) return npeel;
     const int j = jc & 0xFFFF;
     int found = kNone;
-    const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 64 + 2 * (j & 31);
-    const int width = 2 * (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+    const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 128 + 4 * (j & 31);
+    const int width = 4 * (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
     for (int u = g.rank; u < width; u += g.size) {
-      const int i = (int)(re[64 * (u >> 1) + (u & 1)] >> 2);
+      const int i = (int)(re[128 * (u >> 2) + (u & 3)] >> 2);
       if (i < G.ns && B.status[i] == -1) found = i;  // (the dummy column is no VN)
     }
     const int i = (int)g.min_u((unsigned)found);
@@ -813,14 +901,9 @@ __device__ bool parity_pass(const ShortG& G, const Slot& B, const Grp& g) {
   bool any = false;
   for (int s = g.rank >> 5; s < G.rw; s += g.size >> 5) {
     const int lane = g.rank & 31;
-    uint32_t hp = ((B.sp[s] >> lane) & 1u) << 31;
-    const uint2* ent = (const uint2*)G.rent + (int)G.roff[s] * 32 + lane;
-    const int np = (int)G.roff[s + 1] - (int)G.roff[s];
-    for (int p = 0; p < np; ++p) {
-      const uint2 e = ent[32 * p];
-      hp ^= (__float_as_uint(*(const float*)((const char*)B.post + e.x)) - 1u) ^
-            (__float_as_uint(*(const float*)((const char*)B.post + e.y)) - 1u);
-    }
+    const uint32_t hp = (((B.sp[s] >> lane) & 1u) << 31) ^
+                        check_parity((const uint4*)G.rent + (int)G.roff[s] * 32 + lane,
+                                     (int)G.roff[s + 1] - (int)G.roff[s], (const char*)B.post);
     const unsigned m = __ballot_sync(FULL, (hp >> 31) != 0u);
     if (lane == 0) B.unsat[s] = m;
     any |= m != 0u;
@@ -903,17 +986,23 @@ __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D,
 // the posteriors it reads: for it >= 2 this pass is the convergence test
 // H e = s of the previous iteration (Sec. II-A).  Returns whether this lane saw
 // an unsatisfied check.
-template <bool LW, bool FIRST>
-__device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& G, const Slot& B, int lane, int tw) {
+template <bool LW>
+__device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& G, const Slot& B, int lane, bool first,
+                                                int tw) {
   LwRow lw{nullptr, G.ref};
-  if (LW && !FIRST) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
+  if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
   uint32_t unsat = 0u;
   int r0 = G.roff[0];
+#pragma unroll 1
   for (int s = 0; s < G.rw; ++s) {
     const int r1 = G.roff[s + 1];
-    unsat |= check_lane<LW, FIRST>((const uint2*)G.rent + r0 * 32 + lane, r1 - r0, (const char*)B.post,
-                                   B.cns + 32 * s + lane, (B.sp[s] >> lane) & 1u, P.alpha, P.clip, lw,
-                                   (r0 * 32 + lane) * 2);
+    const uint32_t sw = B.sp[s];
+    if (r1 == r0) {  // checks without columns: unsatisfied when their syndrome bit is set
+      unsat |= sw;
+      continue;
+    }
+    unsat |= check_lane<LW>((const uint4*)G.rent + r0 * 32 + lane, r1 - r0, (const char*)B.post, B.cns + 32 * s + lane,
+                            (sw >> lane) & 1u, P.alpha, P.clip, lw, (r0 * 32 + lane) * 4, first);
     r0 = r1;
   }
   return unsat != 0u;
@@ -929,12 +1018,12 @@ __device__ __forceinline__ bool check_pass_cta(const KParams& P, const ShortG& G
   for (int b = 0; b < nrp; b += per) {
     const int j0 = b + R / tpc;
     const int j = j0 < nrp ? j0 : nrp - 1, s = j >> 5;
-    const int r0 = G.roff[s], np = j0 < nrp ? (int)G.roff[s + 1] - r0 : 0;
+    const int r0 = G.roff[s], nq = j0 < nrp ? (int)G.roff[s + 1] - r0 : 0;
     const uint32_t sbit = (B.sp[s] >> (j & 31)) & 1u;
     uint32_t u = 0u;
     const CNState rec =
-        check_group<LW>((const uint2*)G.rent + r0 * 32 + (j & 31), np, (const char*)B.post, B.cns[j], sbit, P.alpha,
-                        P.clip, first, lw, (r0 * 32 + (j & 31)) * 2, sub, tpc, (G.coff[0] & kWideSlice) != 0, u);
+        check_group<LW>((const uint4*)G.rent + r0 * 32 + (j & 31), nq, (const char*)B.post, B.cns[j], sbit, P.alpha,
+                        P.clip, first, lw, (r0 * 32 + (j & 31)) * 4, sub, tpc, (G.coff[0] & kWideSlice) != 0, u);
     if (sub == 0 && j0 < nrp) {
       B.cns[j] = rec;
       unsat |= u;
@@ -1001,10 +1090,14 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     }
     for (int j = R; j < nrp; j += S) {
       // active VNs of the check: its entries that are not the dummy column
-      const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 64 + 2 * (j & 31);
-      const int np = (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+      const uint4* re = (const uint4*)G.rent + (int)G.roff[j >> 5] * 32 + (j & 31);
+      const int nq = (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+      const uint32_t dum = 4u * nsp;
       int d = 0;
-      for (int p = 0; p < np; ++p) d += (int)(re[64 * p] < 4u * nsp) + (int)(re[64 * p + 1] < 4u * nsp);
+      for (int q = 0; q < nq; ++q) {
+        const uint4 e = re[32 * q];
+        d += (int)(e.x < dum) + (int)(e.y < dum) + (int)(e.z < dum) + (int)(e.w < dum);
+      }
       B.deg[j] = (uint8_t)d;
     }
     if (R == 0) B.cns[nrp] = CNState{0.0f, 0.0f, 0u, 0u};  // the dummy check: message +0
@@ -1032,7 +1125,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // ---- check-node update, Eq. (1), and the previous iteration's H e = s ----
       bool unsat;
       if constexpr (Grp::kWarp) {
-        unsat = first ? check_pass_warp<LW, true>(P, G, B, R, tw) : check_pass_warp<LW, false>(P, G, B, R, tw);
+        unsat = check_pass_warp<LW>(P, G, B, R, first, tw);
         __syncwarp();
       } else {
         unsat = check_pass_cta<LW>(P, G, B, R, S, path_lanes_per_check(S, nr), first, tw);
@@ -1049,17 +1142,17 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // variables in label order; a decimated column runs the loop too and stores nothing
       LwRow lw{nullptr, G.cef};
       if (LW) lw.w = weight_row(G.wts, G.wT, G.wE, tw + 1);
-      for (int k = R; k < 32 * G.cw; k += S) {
-        const int sl = k >> 5;
-        const int cw = G.coff[sl], c0 = cw & (kWideSlice - 1), n = (int)(G.coff[sl + 1] & (kWideSlice - 1)) - c0;
-        const bool wide = (cw & kWideSlice) != 0;
-        const int ei = c0 * 32 + (k & 31);
-        const float p0 = G.llr[k];
-        const float p = wide ? column_sum<LW>(p0, G.cent + ei, n, true, (const char*)B.cns, lw, ei)
-                             : column_sum<LW>(p0, G.cent + ei, n, false, (const char*)B.cns, lw, ei);
-        if (B.status[k] != -1) continue;
-        B.post[k] = p;
-        if (hist) {
+      const bool wide = (G.coff[0] & kWideSlice) != 0;
+      const int lane = R & 31;
+      const ColView V{*G.cls, G.cent, G.coff, G.llr, B.status, (const char*)B.cns, lw, lane, S >> 5};
+      column_pass<LW, false>(V, R >> 5, wide, [&](int s, float p) { B.post[32 * s + lane] = p; });
+      // the history of Sec. IV-A, for the columns a decimation step looks at:
+      // SELECT-VN's and Alg. 3's candidates have degree three or more
+      if (hist)
+        for (int s = R >> 5; s < V.K.n3; s += V.st) {
+          const int k = 32 * s + lane;
+          if (B.status[k] != -1) continue;
+          const float p = B.post[k];
           if (P.rkq || P.dump) B.hq[4 * k + (it - (ips - 3))] = qhist(p);
           // both P_A tests of Alg. 3 (main branch: bit 1, other branches: bit 4),
           // so that the step's BP does not depend on the path
@@ -1073,7 +1166,6 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
             B.hfl[k] &= f;
           }
         }
-      }
       g.sync();
       ++iters;
       ++tw;
@@ -1558,18 +1650,14 @@ struct PreBp {
   const float* llr;
 };
 
-// One variable of the pre-BP: its posterior, and from iteration tk0 on its
-// ranking key (the running sum of the last four posteriors, Sec. III, padded
-// with the prior when n_pre < 4).
-template <bool LW>
-__device__ __forceinline__ float prebp_column(const KParams& P, const WinDev& W, const PreBp& X, int l, int t) {
-  const int sl = l >> 5;
-  const int cw = X.coff[sl], c0 = cw & (kWideSlice - 1), n = (int)(X.coff[sl + 1] & (kWideSlice - 1)) - c0;
-  const int ei = c0 * 32 + (l & 31);
+// The pre-BP's variable pass (Eq. (2)) over the column slices first, first + st, ...
+template <bool LW, class Put>
+__device__ __forceinline__ void prebp_columns(const WinDev& W, const PreBp& X, int t, int first, int st, int lane,
+                                              Put put) {
   LwRow lw{nullptr, W.s_cef};
   if (LW) lw.w = weight_row(W.wts, W.wT, W.n_edges, t);
-  if (cw & kWideSlice) return column_sum<LW>(X.llr[l], X.cent + ei, n, true, (const char*)X.cns, lw, ei);
-  return column_sum<LW>(X.llr[l], X.cent + ei, n, false, (const char*)X.cns, lw, ei);
+  const ColView V{W.cls, X.cent, X.coff, X.llr, nullptr, (const char*)X.cns, lw, lane, st};
+  column_pass<LW, true>(V, first, W.wide3 != 0, put);
 }
 
 __device__ __forceinline__ float prebp_key(const KParams& P, const PreBp& X, int l, int t, int tk0, float p) {
@@ -1610,7 +1698,7 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
   while (tpc < 16 && 2 * tpc * max(1, je - jb) <= NT) tpc <<= 1;
   const int sub = tid & (tpc - 1), per = NT / tpc;
   const int tk0 = P.n_pre - 3 > 1 ? P.n_pre - 3 : 1;
-  const bool rwide = X.roff[1] - X.roff[0] > 16;  // the first slice is the widest
+  const bool rwide = X.roff[1] - X.roff[0] > 8;  // the first slice is the widest
   cl_sync();  // every CTA of the cluster runs and has set up its arrays
   int t;
   for (t = 1; t <= P.n_pre; ++t) {
@@ -1621,11 +1709,11 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       const int j0 = b + tid / tpc;
       const bool real = j0 < je;
       const int j = real ? j0 : je - 1, s = j >> 5;
-      const int r0 = X.roff[s], np = real ? (int)X.roff[s + 1] - r0 : 0;
+      const int r0 = X.roff[s], nq = real ? (int)X.roff[s + 1] - r0 : 0;
       uint32_t u = 0u;
-      const CNState rec = check_group<LW>((const uint2*)X.rent + r0 * 32 + (j & 31), np, (const char*)X.post, X.cns[j],
+      const CNState rec = check_group<LW>((const uint4*)X.rent + r0 * 32 + (j & 31), nq, (const char*)X.post, X.cns[j],
                                           (X.sp[s] >> (j & 31)) & 1u, P.alpha, P.clip, t == 1, lw,
-                                          (r0 * 32 + (j & 31)) * 2, sub, tpc, rwide, u);
+                                          (r0 * 32 + (j & 31)) * 4, sub, tpc, rwide, u);
       if (real) {
         for (int c = sub; c < (int)C; c += tpc) cl_st_cns(cl_map(&X.cns[j], (unsigned)c), rec);
         unsat |= u;
@@ -1640,8 +1728,17 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       t_conv = t - 1;
       break;
     }
+    LwRow lc{nullptr, W.s_cef};
+    if (LW) lc.w = weight_row(W.wts, W.wT, W.n_edges, t);
     for (int i = ib + tid; i < ie; i += NT) {
-      const float p = prebp_column<LW>(P, W, X, i, t);
+      const int q = i >> 5, c0 = X.coff[q] & (kWideSlice - 1), n = (int)(X.coff[q + 1] & (kWideSlice - 1)) - c0;
+      const int ei = c0 * 32 + (i & 31);
+      float p = X.llr[i];
+      for (int u = 0; u < n; ++u) {
+        const uint32_t e = X.cent[ei + 32 * u];
+        p = __fadd_rn(p, c2v<LW>(*(const CNState*)((const char*)X.cns + (e >> 12)), e, true,
+                                 LW ? lw_at(lc, ei + 32 * u) : 0.0f));
+      }
       for (unsigned c = 0; c < C; ++c)  // every CTA reads the whole posterior in its check pass
         cl_st_f32(cl_map(&X.post[i], c), p);
       if (t >= tk0) {
@@ -1690,7 +1787,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   // the window graph in shared memory for the pre-BP loop when there is room
   PreBp X{post, key, cns, spre, W.s_rent, W.s_cent, W.s_roff, W.s_coff, W.s_llr};
   if (L.pre_stage) {
-    const StagePiece pc[5] = {{U + L.q_rent, W.s_rent, 256u * W.row_pairs},
+    const StagePiece pc[5] = {{U + L.q_rent, W.s_rent, 512u * W.row_quads},
                               {U + L.q_cent, W.s_cent, 128u * W.col_cells},
                               {U + L.q_roff, W.s_roff, al16(2u * (rw + 1))},
                               {U + L.q_coff, W.s_coff, al16(2u * (L.cw + 1))},
@@ -1751,38 +1848,30 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
       if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
       uint32_t unsat = 0u;
       for (int s = warp; s < rw; s += nw) {
-        const int r0 = X.roff[s], np = (int)X.roff[s + 1] - r0;
-        const uint2* ent = (const uint2*)X.rent + r0 * 32 + lane;
-        const uint32_t sbit = (spre[s] >> lane) & 1u;
-        CNState* rec = cns + 32 * s + lane;
-        const int ei = (r0 * 32 + lane) * 2;
-        if (t == 1) unsat |= check_lane<LW, true>(ent, np, (const char*)post, rec, sbit, P.alpha, P.clip, lw, ei);
-        else unsat |= check_lane<LW, false>(ent, np, (const char*)post, rec, sbit, P.alpha, P.clip, lw, ei);
+        const int r0 = X.roff[s], nq = (int)X.roff[s + 1] - r0;
+        unsat |= check_lane<LW>((const uint4*)X.rent + r0 * 32 + lane, nq, (const char*)post, cns + 32 * s + lane,
+                                (spre[s] >> lane) & 1u, P.alpha, P.clip, lw, (r0 * 32 + lane) * 4, t == 1);
       }
       if (!__syncthreads_or(unsat != 0u) && t >= 2) {  // iteration t-1 satisfies H e = s
         conv = true;
         t_conv = t - 1;
         break;
       }
-      for (int l = tid; l < nc; l += NT) {
-        const float p = prebp_column<LW>(P, W, X, l, t);
+      auto put = [&](int s, float p) {
+        const int l = 32 * s + lane;
         post[l] = p;
         if (t >= tk0) key[l] = prebp_key(P, X, l, t, tk0, p);
-      }
+      };
+      prebp_columns<LW>(W, X, t, warp, nw, lane, put);
       __syncthreads();
     }
   }
   if (!conv) {  // the convergence test of the last iteration (or of the priors)
     bool unsat = false;
     for (int s = warp; s < rw; s += nw) {
-      uint32_t hp = ((spre[s] >> lane) & 1u) << 31;
-      const uint2* ent = (const uint2*)X.rent + (int)X.roff[s] * 32 + lane;
-      const int np = (int)X.roff[s + 1] - (int)X.roff[s];
-      for (int p = 0; p < np; ++p) {
-        const uint2 e = ent[32 * p];
-        hp ^= (__float_as_uint(*(const float*)((const char*)post + e.x)) - 1u) ^
-              (__float_as_uint(*(const float*)((const char*)post + e.y)) - 1u);
-      }
+      const uint32_t hp = (((spre[s] >> lane) & 1u) << 31) ^
+                          check_parity((const uint4*)X.rent + (int)X.roff[s] * 32 + lane,
+                                       (int)X.roff[s + 1] - (int)X.roff[s], (const char*)post);
       unsat |= (hp >> 31) != 0u;
     }
     if (!__syncthreads_or(unsat)) {
@@ -1862,7 +1951,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     int run = 0;
     for (int b = 0; b < rw; b += 32) {
       const int s = b + lane;
-      int v = s < rw ? (rc[cperm[32 * s]] + 1) >> 1 : 0;
+      int v = s < rw ? (rc[cperm[32 * s]] + 3) >> 2 : 0;
       v = warp_incl_scan(v, lane);
       if (s < rw) roff[s + 1] = (uint16_t)(run + v);
       run += __shfl_sync(FULL, v, 31);
@@ -1881,15 +1970,20 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
       run += __shfl_sync(FULL, v, 31);
     }
     if (lane == 0) coff[0] = flag;
+    if (lane < 4) {  // slices at least 4 - lane wide
+      int n = 0;
+      while (n < L.sw && svd[32 * n] >= 4 - lane) ++n;
+      ((int*)(sm + L.s_cls))[lane] = n;
+    }
   }
   __syncthreads();
   // every place a dummy, then the edges
   {
-    const int np = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
-    for (int x = tid; x < 64 * np; x += NT) rent[x] = 4u * (unsigned)nsp;
+    const int nq = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
+    for (int x = tid; x < 128 * nq; x += NT) rent[x] = 4u * (unsigned)nsp;
     for (int x = tid; x < 32 * ncell; x += NT) cent[x] = (unsigned)nrp << 16;
     if (LW) {
-      for (int x = tid; x < 64 * np; x += NT) sref[x] = 0;
+      for (int x = tid; x < 128 * nq; x += NT) sref[x] = 0;
       for (int x = tid; x < 32 * ncell; x += NT) scef[x] = 0;
     }
     for (int l = tid; l < nr; l += NT) cinv[cperm[l]] = l;
@@ -1905,7 +1999,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     for (int u = 0; u < d; ++u) {
       const int r = cinv[W.col_rows[e0 + u]];
       const int pos = atomicAdd(&rc[r], 1);
-      const int ri = (roff[r >> 5] + (pos >> 1)) * 64 + 2 * (r & 31) + (pos & 1);
+      const int ri = (roff[r >> 5] + (pos >> 2)) * 128 + 4 * (r & 31) + (pos & 3);
       rent[ri] = 4u * (unsigned)k;
       cent[ci + 32 * u] = ((unsigned)r << 16) | (unsigned)pos;
       if (LW) {  // the shortened edge keeps its full-window edge's weights
@@ -1927,7 +2021,7 @@ __device__ __forceinline__ ShortG short_graph(char* sm, const Layout& L, const W
                 (const uint16_t*)(sm + L.s_roff), (const uint16_t*)(sm + L.s_coff),
                 (const float*)(sm + L.s_llr),     (const uint8_t*)(sm + L.s_vdeg),
                 (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(sm + L.s_ref), (const uint16_t*)(sm + L.s_cef),
-                W.wts, W.wT, W.n_edges, W.rows_per_block, (const uint16_t*)(sm + L.sel),
+                (const ColClasses*)(sm + L.s_cls), W.wts, W.wT, W.n_edges, W.rows_per_block, (const uint16_t*)(sm + L.sel),
                 (const uint16_t*)(sm + L.s_cperm), (const uint16_t*)(sm + L.s_vperm), W.n_commit_rows};
 }
 

@@ -13,8 +13,9 @@
 //
 // Graph format.  Checks and columns are numbered by descending degree, and the
 // entries of 32 consecutive ones (a slice, one per lane of a warp) are stored
-// lane by lane, entry u of every lane side by side, each slice as wide as its
-// first node's degree (check slices rounded up to an even width).  A warp
+// lane by lane, entry u of every lane side by side (a check's four at a time),
+// each slice as wide as its first node's degree (check slices rounded up to a
+// multiple of four).  A warp
 // walks a slice with conflict-free loads, one trip count for all lanes and no
 // bounds test: the places past a node's degree hold a dummy whose value
 // changes nothing (a column with posterior +inf, a check record with message
@@ -95,6 +96,12 @@ __host__ __device__ inline int path_at(const KParams& P, int pos) {
   return pos - nside;
 }
 
+// Column slices by width: [0, n4) at least four wide, [n4, n3) three, [n3, n2)
+// two, [n2, n1) one.
+struct ColClasses {
+  int n4, n3, n2, n1;
+};
+
 // One window's Tanner graph in global memory (read-only for all shots).
 struct WinDev {
   int n_rows, n_cols, n_edges, row0, n_short, es_max, rows_per_block;
@@ -107,11 +114,13 @@ struct WinDev {
   int wT;
   int n_commit_rows;      // rows [0, n_commit_rows) are the ones the window commits
   // the graph in slices (see the top of the file), checks and columns by label
-  int row_pairs, col_cells;    // slice totals: check-entry pairs, column entries, both per lane
-  const uint32_t *s_rent, *s_cent;   // [2 * 32 * row_pairs], [32 * col_cells]
-  const uint16_t *s_roff, *s_coff;   // slice starts, in pairs / in entries per lane
+  int row_quads, col_cells;    // slice totals per lane: check entries in fours, column entries
+  const uint32_t *s_rent, *s_cent;   // [4 * 32 * row_quads], [32 * col_cells]
+  const uint16_t *s_roff, *s_coff;   // slice starts, in fours / in entries per lane
   const float* s_llr;                // priors by column label
   const uint16_t *s_row, *s_col;     // label -> window row / window column
+  ColClasses cls;
+  int wide3;  // some column of degree three or more has an edge at a position past 31
   const uint16_t *s_ref, *s_cef;     // full-window edge of each check / column entry (learned weights)
 };
 
@@ -187,8 +196,8 @@ __host__ __device__ inline size_t path_result_bytes(int sw) { return (16 + 4 * (
 // Sizes of a window's graph in slices, and bounds on those of its shortened
 // graphs.
 struct SliceDims {
-  int row_pairs, col_cells;    // the window's, as WinDev
-  int srow_pairs, scol_cells;  // the shortened graph's, at most
+  int row_quads, col_cells;    // the window's, as WinDev
+  int srow_quads, scol_cells;  // the shortened graph's, at most
 };
 __host__ __device__ inline unsigned up32(unsigned x) { return (x + 31u) & ~31u; }
 
@@ -211,7 +220,7 @@ struct Layout {
   int rw, cw, sw, sortn, nslots;
   // slices: the shortened graph (s_rent .. s_coff; s_ref / s_cef with learned
   // weights) and the staged window graph (q_rent .. q_llr)
-  unsigned s_rent, s_cent, s_roff, s_coff, s_ref, s_cef;
+  unsigned s_rent, s_cent, s_roff, s_coff, s_ref, s_cef, s_cls;
   unsigned q_rent, q_cent, q_roff, q_coff, q_sllr;
   // The pre-BP's arrays start at V, where the shortened graph and the path
   // slots begin: neither exists before the pre-BP has ended.
@@ -249,13 +258,14 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.misc = o; o = al16(o + 64u);
   L.V = o;
   L.sel = o; o = al16(o + 2u * ns);
-  L.s_rent = o; o = al16(o + 256u * D.srow_pairs);
+  L.s_rent = o; o = al16(o + 512u * D.srow_quads);
   L.s_cent = o; o = al16(o + 128u * D.scol_cells);
   L.s_roff = o; o = al16(o + 2u * (L.rw + 1));
   L.s_coff = o; o = al16(o + 2u * (L.sw + 1));
+  L.s_cls = o; o = al16(o + 16u);
   L.s_llr = o; o = al16(o + 4u * nsp);
   L.s_vdeg = o; o = al16(o + nsp);
-  L.s_ref = o; o = al16(o + (lw ? 128u * D.srow_pairs : 0u));
+  L.s_ref = o; o = al16(o + (lw ? 256u * D.srow_quads : 0u));
   L.s_cef = o; o = al16(o + (lw ? 64u * D.scol_cells : 0u));
   L.s_cperm = o; o = al16(o + 2u * nr);
   L.s_vperm = o; o = al16(o + 2u * ns);
@@ -292,7 +302,7 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   if (stage) {
     const unsigned q0 = stage == 2 ? al16(end) - p0 : own;
     unsigned q = q0;
-    L.q_rent = q; q = al16(q + 256u * D.row_pairs);
+    L.q_rent = q; q = al16(q + 512u * D.row_quads);
     L.q_cent = q; q = al16(q + 128u * D.col_cells);
     L.q_roff = q; q = al16(q + 2u * (L.rw + 1));
     L.q_coff = q; q = al16(q + 2u * (L.cw + 1));

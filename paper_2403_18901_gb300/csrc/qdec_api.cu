@@ -254,7 +254,7 @@ ForkPlan fork_plan(const qd::KParams& P, int dmx, int wave) {
 }
 
 qd::SliceDims slice_dims(const qd::WindowHost& h) {
-  return qd::SliceDims{h.row_pairs, h.col_cells, h.srow_pairs, h.scol_cells};
+  return qd::SliceDims{h.row_quads, h.col_cells, h.srow_quads, h.scol_cells};
 }
 
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
@@ -652,9 +652,10 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
                       (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0,
                       h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks)),
-                      h.row_pairs, h.col_cells, (const uint32_t*)(b + s_re), (const uint32_t*)(b + s_ce),
+                      h.row_quads, h.col_cells, (const uint32_t*)(b + s_re), (const uint32_t*)(b + s_ce),
                       (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
-                      (const uint16_t*)(b + s_rw), (const uint16_t*)(b + s_cl), (const uint16_t*)(b + s_rf),
+                      (const uint16_t*)(b + s_rw), (const uint16_t*)(b + s_cl),
+                      qd::ColClasses{h.cls[0], h.cls[1], h.cls[2], h.cls[3]}, h.wide3, (const uint16_t*)(b + s_rf),
                       (const uint16_t*)(b + s_cf)};
     // committed columns: their full detector sets and observables
     std::vector<int> cc_ptr(1, 0), cc_det;

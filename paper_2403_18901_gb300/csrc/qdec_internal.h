@@ -25,9 +25,10 @@ struct WindowHost {
   std::vector<uint32_t> row_ent;            // CSR entries: CSC edge id | (window column << 16)
   std::vector<float> llr;
   // the graph in slices (gdg_kernel.cuh), checks and columns by label
-  int row_pairs = 0, col_cells = 0;    // slice totals
-  int srow_pairs = 0, scol_cells = 0;  // bounds on those of a shortened graph
+  int row_quads = 0, col_cells = 0;    // slice totals
+  int srow_quads = 0, scol_cells = 0;  // bounds on those of a shortened graph
   int max_row_deg = 0;
+  int cls[4] = {0, 0, 0, 0}, wide3 = 0;  // ColClasses; an edge of a column of degree >= 3 past position 31
   std::vector<uint32_t> s_rent, s_cent;
   std::vector<uint16_t> s_roff, s_coff, s_row, s_col, s_ref, s_cef;
   std::vector<float> s_llr;

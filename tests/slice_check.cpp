@@ -37,6 +37,11 @@ bool check_graph(const qd::WindowHost& h) {
   const int nr = h.n_rows, nc = h.n_cols, nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
   REQ((int)h.s_roff.size() == nrs + 1 && (int)h.s_coff.size() == ncs + 1, "offsets");
   const unsigned low = qd::kWideSlice - 1;
+  for (int q = 0; q < ncs; ++q) {
+    const int w = (int)(h.s_coff[q + 1] & low) - (int)(h.s_coff[q] & low);
+    for (int x = 0; x < 4; ++x) REQ((w >= 4 - x) == (q < h.cls[x]), "slice %d of width %d: class %d", q, w, x);
+    REQ(w < 3 || !(h.s_coff[q] & qd::kWideSlice) || h.wide3, "slice %d: wide", q);
+  }
   size_t real = 0, dummies = 0;
   std::vector<int> seen(h.n_edges, 0);
   for (int l = 0; l < nc; ++l) {
@@ -54,8 +59,8 @@ bool check_graph(const qd::WindowHost& h) {
       REQ(r < nr && pos < qd::kMaxRowDeg, "column %d entry %d", l, u);
       REQ(fe == h.col_ptr[c] + u && h.col_rows[fe] == h.s_row[r], "column %d entry %d: edge", l, u);
       seen[fe]++;
-      const size_t ri = ((size_t)(h.s_roff[r >> 5] + (pos >> 1)) * 32 + (r & 31)) * 2 + (pos & 1);
-      REQ((pos >> 1) < h.s_roff[(r >> 5) + 1] - h.s_roff[r >> 5], "check %d position %d", r, pos);
+      const size_t ri = ((size_t)(h.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
+      REQ((pos >> 2) < h.s_roff[(r >> 5) + 1] - h.s_roff[r >> 5], "check %d position %d", r, pos);
       REQ(h.s_rent[ri] == 4u * (uint32_t)l && h.s_ref[ri] == fe, "check %d position %d: other side", r, pos);
       REQ(pos < 32 || (h.s_coff[l >> 5] & qd::kWideSlice), "column %d: slice not flagged", l);
     }
@@ -64,7 +69,7 @@ bool check_graph(const qd::WindowHost& h) {
   for (size_t i = 0; i < h.s_rent.size(); ++i) (h.s_rent[i] < 4u * (uint32_t)nc ? real : dummies)++;
   for (uint32_t x : h.s_rent)
     REQ(x < 4u * (uint32_t)nc || x == 4u * (uint32_t)(32 * ncs), "check entry is neither a column nor the dummy");
-  REQ((int)real == h.n_edges && real + dummies == (size_t)64 * h.row_pairs, "check entries");
+  REQ((int)real == h.n_edges && real + dummies == (size_t)128 * h.row_quads, "check entries");
   return true;
 }
 
@@ -77,11 +82,11 @@ bool check_short(const qd::WindowHost& h, const std::vector<int>& cols) {
   }
   std::sort(cd.rbegin(), cd.rend());
   std::sort(rd.rbegin(), rd.rend());
-  int cells = 0, pairs = 0;
+  int cells = 0, quads = 0;
   for (size_t i = 0; i < cd.size(); i += 32) cells += cd[i];
-  for (size_t i = 0; i < rd.size(); i += 32) pairs += (rd[i] + 1) / 2;
+  for (size_t i = 0; i < rd.size(); i += 32) quads += (rd[i] + 3) / 4;
   REQ(cells <= h.scol_cells, "column slices %d > %d", cells, h.scol_cells);
-  REQ(pairs <= h.srow_pairs, "check slices %d > %d", pairs, h.srow_pairs);
+  REQ(quads <= h.srow_quads, "check slices %d > %d", quads, h.srow_quads);
   return true;
 }
 
@@ -103,7 +108,7 @@ bool disjoint(std::vector<Region> rs, unsigned lo, unsigned hi, const char* part
 }
 
 bool check_layout(const qd::WindowHost& h, int nb, int nslots, int stage, bool ranker, bool lw, bool glob) {
-  const qd::SliceDims D{h.row_pairs, h.col_cells, h.srow_pairs, h.scol_cells};
+  const qd::SliceDims D{h.row_quads, h.col_cells, h.srow_quads, h.scol_cells};
   const int nr = h.n_rows, nc = h.n_cols, ns = h.n_short;
   const qd::Layout L = qd::make_slice_layout(D, nr, nc, ns, nb, nslots, stage, ranker, lw, glob);
   const unsigned nrp = qd::up32(nr), ncp = qd::up32(nc), nsp = qd::up32(ns), rw = L.rw;
@@ -113,10 +118,10 @@ bool check_layout(const qd::WindowHost& h, int nb, int nslots, int stage, bool r
                                     {"res_ebits", L.res_ebits, 4u * L.sw * nb}, {"red", L.red, 512u},
                                     {"misc", L.misc, 64u}};
   if (!disjoint(keep, 0, L.V, "persistent")) return false;
-  std::vector<Region> sg = {{"sel", L.sel, 2u * ns}, {"rent", L.s_rent, 256u * D.srow_pairs},
+  std::vector<Region> sg = {{"sel", L.sel, 2u * ns}, {"rent", L.s_rent, 512u * D.srow_quads},
                             {"cent", L.s_cent, 128u * D.scol_cells}, {"roff", L.s_roff, 2u * (rw + 1)},
-                            {"coff", L.s_coff, 2u * (L.sw + 1u)}, {"llr", L.s_llr, 4u * nsp},
-                            {"vdeg", L.s_vdeg, nsp}, {"ref", L.s_ref, lw ? 128u * D.srow_pairs : 0u},
+                            {"coff", L.s_coff, 2u * (L.sw + 1u)}, {"cls", L.s_cls, 16u}, {"llr", L.s_llr, 4u * nsp},
+                            {"vdeg", L.s_vdeg, nsp}, {"ref", L.s_ref, lw ? 256u * D.srow_quads : 0u},
                             {"cef", L.s_cef, lw ? 64u * D.scol_cells : 0u}, {"cperm", L.s_cperm, 2u * nr},
                             {"vperm", L.s_vperm, 2u * ns}, {"rowcnt", L.rowcnt, 4u * (nrp + 1)}};
   if (!disjoint(sg, L.V, L.U, "shortened graph")) return false;
@@ -125,7 +130,7 @@ bool check_layout(const qd::WindowHost& h, int nb, int nslots, int stage, bool r
                              {"cns", L.p_cns + base, 16u * (nrp + 1)}, {"par", L.p_par + base, 8u * rw}};
   std::vector<Region> st;
   if (L.pre_stage)
-    st = {{"q_rent", L.q_rent + base, 256u * D.row_pairs}, {"q_cent", L.q_cent + base, 128u * D.col_cells},
+    st = {{"q_rent", L.q_rent + base, 512u * D.row_quads}, {"q_cent", L.q_cent + base, 128u * D.col_cells},
           {"q_roff", L.q_roff + base, 2u * (rw + 1)},      {"q_coff", L.q_coff + base, 2u * (L.cw + 1u)},
           {"q_llr", L.q_sllr + base, 4u * ncp}};
   pre.insert(pre.end(), st.begin(), st.end());
