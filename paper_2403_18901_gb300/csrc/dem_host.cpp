@@ -533,7 +533,7 @@ bool build_slices(WindowHost& o) {
   for (int q = 0; q < ncs; ++q) o.s_coff[q + 1] = (uint16_t)(o.s_coff[q] + cdeg(o.s_col[32 * q]));
   o.row_quads = o.s_roff[nrs];
   o.col_cells = o.s_coff[ncs];
-  o.s_rent.assign((size_t)128 * o.row_quads, 4u * (uint32_t)(32 * ncs));  // the dummy column
+  o.s_rent.assign((size_t)128 * o.row_quads, (uint16_t)(32 * ncs));  // the dummy column
   o.s_cent.assign((size_t)32 * o.col_cells, (uint32_t)(32 * nrs) << 16);  // the dummy check
   o.s_ref.assign(o.s_rent.size(), 0);
   o.s_cef.assign(o.s_cent.size(), 0);
@@ -547,7 +547,7 @@ bool build_slices(WindowHost& o) {
       const int r = rlab[o.col_rows[e]], pos = fill[r]++;
       const size_t ri = ((size_t)(o.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
       const size_t ci = (size_t)(o.s_coff[l >> 5] + (e - o.col_ptr[c])) * 32 + (l & 31);
-      o.s_rent[ri] = 4u * (uint32_t)l;
+      o.s_rent[ri] = (uint16_t)l;
       o.s_ref[ri] = (uint16_t)e;
       o.s_cent[ci] = ((uint32_t)r << 16) | (uint32_t)pos;
       o.s_cef[ci] = (uint16_t)e;

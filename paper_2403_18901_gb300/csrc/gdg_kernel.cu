@@ -109,18 +109,33 @@ __device__ __forceinline__ uint32_t check_input(CheckAcc& A, float pv, uint32_t 
   return __float_as_uint(v);
 }
 
+// The columns of four check entries.  The window graph keeps 16-bit column
+// labels (it is staged in shared memory whole, and twice the bytes would cost
+// resident CTAs); a shortened graph keeps byte offsets, one instruction less
+// per entry.
+__device__ __forceinline__ void four_posts(const uint2& e, const char* post, float (&p)[4]) {
+  const float* f = (const float*)post;
+  p[0] = f[e.x & 0xFFFFu];
+  p[1] = f[e.x >> 16];
+  p[2] = f[e.y & 0xFFFFu];
+  p[3] = f[e.y >> 16];
+}
+__device__ __forceinline__ void four_posts(const uint4& e, const char* post, float (&p)[4]) {
+  p[0] = *(const float*)(post + e.x);
+  p[1] = *(const float*)(post + e.y);
+  p[2] = *(const float*)(post + e.z);
+  p[3] = *(const float*)(post + e.w);
+}
+
 // Four inputs at positions u .. u + 3; osg: the old signs, position u at bit
 // 31.  The new signs are shifted into sg, one bit each.
 template <bool LW>
-__device__ __forceinline__ void check_four(CheckAcc& A, const uint4& e, const char* post, uint32_t u, uint32_t oam,
-                                           float om1, float om2, uint32_t osg, const float (&w)[4], bool first,
-                                           uint32_t& sg) {
-  const float p0 = *(const float*)(post + e.x), p1 = *(const float*)(post + e.y);
-  const float p2 = *(const float*)(post + e.z), p3 = *(const float*)(post + e.w);
-  sg = __funnelshift_l(check_input<LW>(A, p0, u, oam, om1, om2, osg, w[0], first), sg, 1);
-  sg = __funnelshift_l(check_input<LW>(A, p1, u + 1, oam, om1, om2, osg << 1, w[1], first), sg, 1);
-  sg = __funnelshift_l(check_input<LW>(A, p2, u + 2, oam, om1, om2, osg << 2, w[2], first), sg, 1);
-  sg = __funnelshift_l(check_input<LW>(A, p3, u + 3, oam, om1, om2, osg << 3, w[3], first), sg, 1);
+__device__ __forceinline__ void check_four(CheckAcc& A, const float (&p)[4], uint32_t u, uint32_t oam, float om1,
+                                           float om2, uint32_t osg, const float (&w)[4], bool first, uint32_t& sg) {
+  sg = __funnelshift_l(check_input<LW>(A, p[0], u, oam, om1, om2, osg, w[0], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p[1], u + 1, oam, om1, om2, osg << 1, w[1], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p[2], u + 2, oam, om1, om2, osg << 2, w[2], first), sg, 1);
+  sg = __funnelshift_l(check_input<LW>(A, p[3], u + 3, oam, om1, om2, osg << 3, w[3], first), sg, 1);
 }
 
 // The record of a check from its inputs and the syndrome bit: magnitudes
@@ -165,8 +180,8 @@ __device__ __forceinline__ void lw_four(const LwRow& r, int i, bool first, float
 // and the clip on every input and ragged rows, 5000 shots of [[144,12,12]]
 // took 450 ms; in slices, with the signs as bits of the record and the clip on
 // the two minima, 354 ms.
-template <bool LW>
-__device__ __forceinline__ uint32_t check_lane(const uint4* ent, int nq, const char* post, CNState* rec, uint32_t sbit,
+template <bool LW, class E>
+__device__ __forceinline__ uint32_t check_lane(const E* ent, int nq, const char* post, CNState* rec, uint32_t sbit,
                                                float alpha, float clip, const LwRow& lw, int ei, bool first) {
   CNState oc = *rec;
   if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
@@ -174,6 +189,7 @@ __device__ __forceinline__ uint32_t check_lane(const uint4* ent, int nq, const c
   uint32_t osg = oc.sg;
   CheckAcc A{CUDART_INF_F, CUDART_INF_F, 0u, 0u};
   uint32_t sg0 = 0u, sg1 = 0u;
+#pragma unroll 1
   for (int q0 = 0; q0 < nq; q0 += 8) {  // 32 positions to a sign word
     const int q1 = min(nq, q0 + 8);
     uint32_t sg = 0u;
@@ -181,7 +197,9 @@ __device__ __forceinline__ uint32_t check_lane(const uint4* ent, int nq, const c
     for (int q = q0; q < q1; ++q) {
       float w[4];
       lw_four<LW>(lw, ei + 128 * q, first, w);
-      check_four<LW>(A, ent[32 * q], post, 4 * q, oam, oc.m1, oc.m2, osg, w, first, sg);
+      float p[4];
+      four_posts(ent[32 * q], post, p);
+      check_four<LW>(A, p, 4 * q, oam, oc.m1, oc.m2, osg, w, first, sg);
       osg <<= 4;
     }
     sg <<= (32 - 4 * (q1 - q0)) & 31;  // the first position to bit 31
@@ -195,8 +213,8 @@ __device__ __forceinline__ uint32_t check_lane(const uint4* ent, int nq, const c
 
 // The same by tpc neighbouring lanes (fours sub, sub + tpc, ...); every lane
 // of the group ends with the record.
-template <bool LW>
-__device__ __forceinline__ CNState check_group(const uint4* ent, int nq, const char* post, CNState oc, uint32_t sbit,
+template <bool LW, class E>
+__device__ __forceinline__ CNState check_group(const E* ent, int nq, const char* post, CNState oc, uint32_t sbit,
                                                float alpha, float clip, bool first, const LwRow& lw, int ei, int sub,
                                                int tpc, bool wide, uint32_t& unsat) {
   if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
@@ -209,10 +227,13 @@ __device__ __forceinline__ CNState check_group(const uint4* ent, int nq, const c
     lw_four<LW>(lw, ei + 128 * q, first, w);
     const int sh = (4 * q) & 31;
     uint32_t sg = 0u;
-    check_four<LW>(A, ent[32 * q], post, 4 * q, oam, oc.m1, oc.m2, (q < 8 ? oc.sg : oc.am) << sh, w, first, sg);
+    float p[4];
+    four_posts(ent[32 * q], post, p);
+    check_four<LW>(A, p, 4 * q, oam, oc.m1, oc.m2, (q < 8 ? oc.sg : oc.am) << sh, w, first, sg);
     if (q < 8) sg0 |= sg << (28 - sh);
     else sg1 |= sg << (28 - sh);
   }
+#pragma unroll 1
   for (int off = tpc >> 1; off; off >>= 1) {
     const float x1 = __shfl_xor_sync(FULL, A.m1, off), x2 = __shfl_xor_sync(FULL, A.m2, off);
     const uint32_t xa = __shfl_xor_sync(FULL, A.am, off);
@@ -230,13 +251,15 @@ __device__ __forceinline__ CNState check_group(const uint4* ent, int nq, const c
 }
 
 // The parity of a check's hard decisions, at bit 31.
-__device__ __forceinline__ uint32_t check_parity(const uint4* ent, int nq, const char* post) {
+template <class E>
+__device__ __forceinline__ uint32_t check_parity(const E* ent, int nq, const char* post) {
   uint32_t hp = 0u;
+#pragma unroll 1
   for (int q = 0; q < nq; ++q) {
-    const uint4 e = ent[32 * q];
-    const uint32_t a = *(const uint32_t*)(post + e.x), b = *(const uint32_t*)(post + e.y);
-    const uint32_t c = *(const uint32_t*)(post + e.z), d = *(const uint32_t*)(post + e.w);
-    hp ^= ((a - 1u) ^ (b - 1u)) ^ ((c - 1u) ^ (d - 1u));
+    float p[4];
+    four_posts(ent[32 * q], post, p);
+    hp ^= ((__float_as_uint(p[0]) - 1u) ^ (__float_as_uint(p[1]) - 1u)) ^
+          ((__float_as_uint(p[2]) - 1u) ^ (__float_as_uint(p[3]) - 1u));
   }
   return hp & 0x80000000u;
 }
@@ -255,6 +278,7 @@ struct ColView {
 
 // The first slice s, s - st, ... of the group at or past end.
 __device__ __forceinline__ int back_to(int s, int end, int st) {
+#pragma unroll 1
   while (s - st >= end) s -= st;
   return s;
 }
@@ -324,7 +348,9 @@ __device__ __forceinline__ void column_pass(const ColView& V, int first, bool wi
         p = __fadd_rn(p, c2v<LW>(c[x], e[x], true, LW ? lw_at(V.lw, 32 * (c0 + x) + V.lane) : 0.0f));
       c0 += N;
     };
+#pragma unroll 1
     while (c0 + 3 <= c1) more(std::integral_constant<int, 3>{});
+#pragma unroll 1
     while (c0 < c1) more(std::integral_constant<int, 1>{});
     if (!V.status || V.status[k] == -1) put(s, p);
   }
@@ -385,9 +411,11 @@ struct StagePiece {
 // thread waiting with a bound of ~2^31 cycles.  Pieces that are not 16-byte
 // aligned in address and size, an empty list, or a wait that ran out (counted
 // in *err; the bulk path then stays off for this CTA) use plain loads.
-__device__ void stage_pieces(Stager& st, const StagePiece* pc, int n) {
+template <int n>
+__device__ __forceinline__ void stage_pieces(Stager& st, const StagePiece (&pc)[n]) {
   bool aligned = true;
   unsigned tot = 0;
+#pragma unroll
   for (int i = 0; i < n; ++i) {
     aligned = aligned && (((smem_u32(pc[i].dst) | (unsigned)(uintptr_t)pc[i].src | pc[i].bytes) & 15u) == 0u);
     tot += pc[i].bytes;
@@ -398,6 +426,7 @@ __device__ void stage_pieces(Stager& st, const StagePiece* pc, int n) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(st.bar)), "r"(tot)
                    : "memory");
+#pragma unroll
       for (int i = 0; i < n; ++i)
         if (pc[i].bytes)
           asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -407,6 +436,7 @@ __device__ void stage_pieces(Stager& st, const StagePiece* pc, int n) {
     }
     unsigned ok = 0;
     const long long t0 = clock64();
+#pragma unroll 1
     while (!ok && clock64() - t0 < (1ll << 31)) {
       asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
                    : "=r"(ok)
@@ -420,9 +450,11 @@ __device__ void stage_pieces(Stager& st, const StagePiece* pc, int n) {
       atomicAdd((unsigned long long*)st.err, 1ull);
     }
   }
+#pragma unroll
   for (int i = 0; i < n; ++i) {
     const uint16_t* s16 = (const uint16_t*)pc[i].src;
     uint16_t* d16 = (uint16_t*)pc[i].dst;
+#pragma unroll 1
     for (unsigned x = threadIdx.x; x < pc[i].bytes / 2; x += blockDim.x) d16[x] = s16[x];
   }
   __syncthreads();
@@ -444,6 +476,7 @@ __device__ __forceinline__ uint32_t ordkey(float f) {
 
 __host__ __device__ inline int lanes_per_check(int threads, int n_checks) {
   int t = 1;
+#pragma unroll 1
   while (t < 8 && 2 * t * n_checks <= threads) t <<= 1;
   return t;
 }
@@ -455,6 +488,7 @@ __host__ __device__ inline int lanes_per_check(int threads, int n_checks) {
 // 512 threads: 1.18 / 1.02 / 1.19 ms per window with 2 / 4 / 8 lanes).
 __host__ __device__ inline int path_lanes_per_check(int threads, int n_checks) {
   int t = 1;
+#pragma unroll 1
   while (t < 8 && 2 * (threads / (2 * t)) >= n_checks) t <<= 1;
   return t;
 }
@@ -519,111 +553,77 @@ struct CtaGrp {  // the whole CTA; every member must call every primitive
   __device__ void sync() const { __syncthreads(); }
   __device__ bool all(bool p) const { return __syncthreads_and(p) != 0; }
   __device__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
-  __device__ unsigned min_u(unsigned v) const {
-    v = __reduce_min_sync(FULL, v);
-    unsigned* r = (unsigned*)red;
+  // Reductions: each warp's result through shared memory, then every warp
+  // reduces the (at most 32) results again, one per lane: a loop over them
+  // would be as many shared-memory round trips in a row.
+  template <class T>
+  __device__ T exchange(T v, T none) const {
+    T* r = (T*)red;
     __syncthreads();
     if ((rank & 31) == 0) r[rank >> 5] = v;
     __syncthreads();
-    unsigned m = r[0];
-    for (int i = 1; i < (size >> 5); ++i) m = min(m, r[i]);
-    return m;
+    return (rank & 31) < (size >> 5) ? r[rank & 31] : none;
+  }
+  __device__ unsigned min_u(unsigned v) const {
+    return __reduce_min_sync(FULL, exchange(__reduce_min_sync(FULL, v), 0xFFFFFFFFu));
   }
   __device__ int sum_i(int v) const {
-    v = (int)__reduce_add_sync(FULL, (unsigned)v);
-    int* r = (int*)red;
-    __syncthreads();
-    if ((rank & 31) == 0) r[rank >> 5] = v;
-    __syncthreads();
-    int s = 0;
-    for (int i = 0; i < (size >> 5); ++i) s += r[i];
-    return s;
+    return (int)__reduce_add_sync(FULL, exchange(__reduce_add_sync(FULL, (unsigned)v), 0u));
   }
-  __device__ long long sum_ll(long long v) const {
+  template <class T>
+  __device__ T sum(T v) const {
 #pragma unroll
     for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-    long long* r = (long long*)red;
-    __syncthreads();
-    if ((rank & 31) == 0) r[rank >> 5] = v;
-    __syncthreads();
-    long long s = 0;
-    for (int i = 0; i < (size >> 5); ++i) s += r[i];
-    return s;
-  }
-  __device__ double sum_d(double v) const {
+    v = exchange(v, (T)0);
 #pragma unroll
     for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-    double* r = (double*)red;
-    __syncthreads();
-    if ((rank & 31) == 0) r[rank >> 5] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int i = 0; i < (size >> 5); ++i) s += r[i];
-    return s;
+    return v;
   }
+  __device__ long long sum_ll(long long v) const { return sum(v); }
+  __device__ double sum_d(double v) const { return sum(v); }
   __device__ void argmin(float& v, int& k) const {
     warp_argmin(v, k);
-    float* rv = (float*)red;
-    int* rk = (int*)(red + 4 * 32);
-    __syncthreads();
-    if ((rank & 31) == 0) {
-      rv[rank >> 5] = v;
-      rk[rank >> 5] = k;
-    }
-    __syncthreads();
-    v = rv[0];
-    k = rk[0];
-    for (int i = 1; i < (size >> 5); ++i)
-      if (rv[i] < v || (rv[i] == v && rk[i] < k)) {
-        v = rv[i];
-        k = rk[i];
-      }
+    const unsigned long long x =
+        exchange(((unsigned long long)__float_as_uint(v) << 32) | (unsigned)k,
+                 ((unsigned long long)__float_as_uint(CUDART_INF_F) << 32) | (unsigned)kNone);
+    v = __uint_as_float((unsigned)(x >> 32));
+    k = (int)(unsigned)x;
+    warp_argmin(v, k);
   }
-  // SELECT-VN's reductions in one exchange (two barriers instead of seven):
-  // two lexicographic argmins and a count, for at most 16 warps (the
-  // path-mode CTA); every thread's shared-memory writes are visible after it
+  // SELECT-VN's reductions in one exchange: two lexicographic argmins and a
+  // count, for at most 16 warps (the path-mode CTA); every thread's
+  // shared-memory writes are visible after it
   __device__ void select_reduce(float& bv, int& bk, float& tv, int& tk, int& n) const {
     warp_argmin(bv, bk);
     warp_argmin(tv, tk);
     n = (int)__reduce_add_sync(FULL, (unsigned)n);
-    float* r_bv = (float*)red;
-    int* r_bk = (int*)(red + 64);
-    float* r_tv = (float*)(red + 128);
-    int* r_tk = (int*)(red + 192);
+    uint4* r = (uint4*)red;
     int* r_n = (int*)(red + 256);
+    const int lane = rank & 31;
     __syncthreads();
-    if ((rank & 31) == 0) {
-      const int w = rank >> 5;
-      r_bv[w] = bv;
-      r_bk[w] = bk;
-      r_tv[w] = tv;
-      r_tk[w] = tk;
-      r_n[w] = n;
+    if (lane == 0) {
+      r[rank >> 5] = make_uint4(__float_as_uint(bv), (unsigned)bk, __float_as_uint(tv), (unsigned)tk);
+      r_n[rank >> 5] = n;
     }
     __syncthreads();
-    bv = r_bv[0];
-    bk = r_bk[0];
-    tv = r_tv[0];
-    tk = r_tk[0];
-    n = r_n[0];
-    for (int i = 1; i < (size >> 5); ++i) {
-      if (r_bv[i] < bv || (r_bv[i] == bv && r_bk[i] < bk)) {
-        bv = r_bv[i];
-        bk = r_bk[i];
-      }
-      if (r_tv[i] < tv || (r_tv[i] == tv && r_tk[i] < tk)) {
-        tv = r_tv[i];
-        tk = r_tk[i];
-      }
-      n += r_n[i];
-    }
+    const bool in = lane < (size >> 5);
+    const uint4 x = in ? r[lane] : make_uint4(__float_as_uint(CUDART_INF_F), (unsigned)kNone,
+                                              __float_as_uint(CUDART_INF_F), (unsigned)kNone);
+    bv = __uint_as_float(x.x);
+    bk = (int)x.y;
+    tv = __uint_as_float(x.z);
+    tk = (int)x.w;
+    warp_argmin(bv, bk);
+    warp_argmin(tv, tk);
+    n = (int)__reduce_add_sync(FULL, in ? (unsigned)r_n[lane] : 0u);
   }
 };
 
 // The shortened graph in slices (gdg_kernel.cuh).
 struct ShortG {
   int nr, ns, rw, cw;  // checks, columns, and their slices
-  const uint32_t *rent, *cent;
+  int rwz;             // non-empty check slices
+  const uint32_t *rent, *cent;  // rent: byte offsets of the columns' posteriors
   const uint16_t *roff, *coff;
   const float* llr;
   const uint8_t* vdeg;
@@ -656,10 +656,10 @@ struct Slot {
   int8_t* hq;  // ranker only: the last four posteriors as round(2 clamp(x, 63.5)), oldest first
 };
 
-__device__ __forceinline__ Slot make_slot(char* base, const Layout& L) {
-  return Slot{(float*)(base + L.b_post),  (float*)(base + L.b_acc),      (uint8_t*)(base + L.b_hfl),
-              (int8_t*)(base + L.b_status), (CNState*)(base + L.b_cns),  (uint8_t*)(base + L.b_deg),
-              (uint32_t*)(base + L.b_sp), (uint32_t*)(base + L.b_unsat), (int8_t*)(base + L.b_hq)};
+__device__ __forceinline__ Slot make_slot(char* base, const SlotPlan& S) {
+  return Slot{(float*)base,                 (float*)(base + S.b_acc),      (uint8_t*)(base + S.b_hfl),
+              (int8_t*)(base + S.b_status), (CNState*)(base + S.b_cns),    (uint8_t*)(base + S.b_deg),
+              (uint32_t*)(base + S.b_sp),   (uint32_t*)(base + S.b_unsat), (int8_t*)(base + S.b_hq)};
 }
 
 // Fix column k to v while other lanes fix others; returns its degree.
@@ -668,6 +668,7 @@ __device__ __forceinline__ int decimate_atomic(const ShortG& G, const Slot& B, i
   B.post[k] = dead_post();
   const uint32_t* ce = G.col_ents(k);
   const int d = G.vdeg[k];
+#pragma unroll 1
   for (int u = 0; u < d; ++u) {
     const int j = (int)(ce[32 * u] >> 16);
     atomicSub((uint32_t*)B.deg + (j >> 2), 1u << (8 * (j & 3)));  // counts stay >= 0: no borrow
@@ -681,6 +682,7 @@ __device__ __forceinline__ int decimate_one(const ShortG& G, const Slot& B, int 
   B.post[k] = dead_post();
   const uint32_t* ce = G.col_ents(k);
   const int d = G.vdeg[k];
+#pragma unroll 1
   for (int u = 0; u < d; ++u) {
     const int r = (int)(ce[32 * u] >> 16);
     B.deg[r] -= 1;
@@ -699,9 +701,11 @@ __device__ __forceinline__ int decimate_one(const ShortG& G, const Slot& B, int 
 template <class Grp>
 __device__ int peel(const ShortG& G, const Slot& B, const Grp& g, int& act) {
   int npeel = 0;
+#pragma unroll 1
   for (int guard = 0; guard <= G.ns + 1; ++guard) {
     bool contra = false;
     int cand = kNone;  // (window row << 16) | label of the lowest degree-one check
+#pragma unroll 1
     for (int j = g.rank; j < G.nr; j += g.size) {
       const int d = B.deg[j];
       if (d == 0) {
@@ -717,6 +721,7 @@ __device__ int peel(const ShortG& G, const Slot& B, const Grp& g, int& act) {
     int found = kNone;
     const uint32_t* re = G.rent + (int)G.roff[j >> 5] * 128 + 4 * (j & 31);
     const int width = 4 * (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+#pragma unroll 1
     for (int u = g.rank; u < width; u += g.size) {
       const int i = (int)(re[128 * (u >> 2) + (u & 3)] >> 2);
       if (i < G.ns && B.status[i] == -1) found = i;  // (the dummy column is no VN)
@@ -783,6 +788,7 @@ __device__ __forceinline__ uint32_t ranker_pair(const ShortG& G, const Slot& B, 
   } else if (tig == 2) {
     int nus = 0;
     const uint32_t* ce = G.col_ents(k);
+#pragma unroll 1
     for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
     lo = hv3;
     hi = (float)min(nus, 127);
@@ -806,6 +812,7 @@ __device__ void ranker_select(const KParams& P, const ShortG& G, const Slot& B, 
   const float b2 = P.rkq[640];
   nv = CUDART_INF_F;
   nk = kNone;
+#pragma unroll 1
   for (int t0 = 16 * wid; t0 < G.ns; t0 += 16 * nw) {
     const int r0 = t0 + gi, r1 = r0 + 8;
     const bool c0 = ranker_candidate(G, B, r0), c1 = ranker_candidate(G, B, r1);
@@ -853,11 +860,13 @@ __device__ void ranker_select(const KParams& P, const ShortG& G, const Slot& B, 
 template <class Grp>
 __device__ void dump_candidates(const KParams& P, const ShortG& G, const Slot& B, const Grp& g, long long shot, int D,
                                 int gsel) {
+#pragma unroll 1
   for (int k = g.rank; k < G.ns; k += g.size) {
     if (!ranker_candidate(G, B, k)) continue;
     const uint32_t h4 = *(const uint32_t*)(B.hq + 4 * k);
     int nus = 0;
     const uint32_t* ce = G.col_ents(k);
+#pragma unroll 1
     for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
     const float L = B.acc[k];
     const int pos = atomicAdd(P.dump_n, 1);
@@ -886,6 +895,7 @@ __device__ void dump_candidates(const KParams& P, const ShortG& G, const Slot& B
 template <class Grp>
 __device__ double path_metric(const ShortG& G, const Slot& B, const Grp& g) {
   double s = 0.0;
+#pragma unroll 1
   for (int k = g.rank; k < G.ns; k += g.size) {
     const int st8 = B.status[k];
     if (st8 == 1 || (st8 == -1 && B.post[k] <= 0.0f)) s += (double)G.llr[k];
@@ -899,9 +909,16 @@ __device__ double path_metric(const ShortG& G, const Slot& B, const Grp& g) {
 template <class Grp>
 __device__ bool parity_pass(const ShortG& G, const Slot& B, const Grp& g) {
   bool any = false;
+#pragma unroll 1
   for (int s = g.rank >> 5; s < G.rw; s += g.size >> 5) {
     const int lane = g.rank & 31;
-    const uint32_t hp = (((B.sp[s] >> lane) & 1u) << 31) ^
+    const uint32_t sw = B.sp[s];
+    if (s >= G.rwz) {  // checks without columns
+      if (lane == 0) B.unsat[s] = sw;
+      any |= sw != 0u;
+      continue;
+    }
+    const uint32_t hp = (((sw >> lane) & 1u) << 31) ^
                         check_parity((const uint4*)G.rent + (int)G.roff[s] * 32 + lane,
                                      (int)G.roff[s + 1] - (int)G.roff[s], (const char*)B.post);
     const unsigned m = __ballot_sync(FULL, (hp >> 31) != 0u);
@@ -975,6 +992,7 @@ __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D,
   }
   const uint4* s4 = (const uint4*)F.slot;
   uint4* d4 = (uint4*)(dst + kSnapHeader);
+#pragma unroll 1
   for (unsigned x = g.rank; x < F.slot_bytes / 16u; x += g.size) __stcg(d4 + x, s4[x]);
   __threadfence();  // the snapshot and this path's decision records before its flag
   g.sync();
@@ -992,19 +1010,17 @@ __device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& 
   LwRow lw{nullptr, G.ref};
   if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
   uint32_t unsat = 0u;
-  int r0 = G.roff[0];
+  int r0 = 0;
 #pragma unroll 1
-  for (int s = 0; s < G.rw; ++s) {
+  for (int s = 0; s < G.rwz; ++s) {
     const int r1 = G.roff[s + 1];
-    const uint32_t sw = B.sp[s];
-    if (r1 == r0) {  // checks without columns: unsatisfied when their syndrome bit is set
-      unsat |= sw;
-      continue;
-    }
     unsat |= check_lane<LW>((const uint4*)G.rent + r0 * 32 + lane, r1 - r0, (const char*)B.post, B.cns + 32 * s + lane,
-                            (sw >> lane) & 1u, P.alpha, P.clip, lw, (r0 * 32 + lane) * 4, first);
+                            (B.sp[s] >> lane) & 1u, P.alpha, P.clip, lw, (r0 * 32 + lane) * 4, first);
     r0 = r1;
   }
+  // checks without columns are unsatisfied when their syndrome bit is set
+#pragma unroll 1
+  for (int s = G.rwz + lane; s < G.rw; s += 32) unsat |= B.sp[s];
   return unsat != 0u;
 }
 
@@ -1013,8 +1029,11 @@ __device__ __forceinline__ bool check_pass_cta(const KParams& P, const ShortG& G
                                                bool first, int tw) {
   LwRow lw{nullptr, G.ref};
   if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
-  const int nrp = 32 * G.rw, per = S / tpc, sub = R & (tpc - 1);
+  const int nrp = 32 * G.rwz, per = S / tpc, sub = R & (tpc - 1);
   uint32_t unsat = 0u;
+#pragma unroll 1
+  for (int s = G.rwz + R; s < G.rw; s += S) unsat |= B.sp[s];  // checks without columns
+#pragma unroll 1
   for (int b = 0; b < nrp; b += per) {
     const int j0 = b + R / tpc;
     const int j = j0 < nrp ? j0 : nrp - 1, s = j >> 5;
@@ -1067,10 +1086,12 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     if (R == 0) inherited = __ldcg((const long long*)(F.src + 24));
     const uint4* s4 = (const uint4*)(F.src + kSnapHeader);
     uint4* d4 = (uint4*)F.slot;
+#pragma unroll 1
     for (unsigned x = R; x < F.slot_bytes / 16u; x += S) d4[x] = __ldcg(s4 + x);
     // a path resumed from its own parking snapshot keeps its records
     if (out.st && producer != id) {  // the decision records of the shared prefix are the producer's
       const StepTrace* ps = F.st0 + (size_t)producer * dmx;
+#pragma unroll 1
       for (int q = R; q < dmx; q += S) {
         StepTrace r{-2, -1, 0, 0, 0};
         if (q < D0 - 1) {
@@ -1083,30 +1104,37 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     g.sync();
   } else {
     const int nrp = 32 * G.rw, nsp = 32 * G.cw;
+#pragma unroll 1
     for (int k = R; k <= nsp; k += S) {  // (past ns: no VN; nsp: the dummy column)
       if (k < nsp) B.status[k] = k < ns ? -1 : 0;
       B.post[k] = k < ns ? G.llr[k] : dead_post();  // t = 0: mu_{i->j} = Lambda_i (Sec. II-A)
       if (k < ns) act += G.vdeg[k];
     }
+#pragma unroll 1
     for (int j = R; j < nrp; j += S) {
       // active VNs of the check: its entries that are not the dummy column
-      const uint4* re = (const uint4*)G.rent + (int)G.roff[j >> 5] * 32 + (j & 31);
-      const int nq = (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
-      const uint32_t dum = 4u * nsp;
       int d = 0;
-      for (int q = 0; q < nq; ++q) {
-        const uint4 e = re[32 * q];
-        d += (int)(e.x < dum) + (int)(e.y < dum) + (int)(e.z < dum) + (int)(e.w < dum);
+      if (j < 32 * G.rwz) {
+        const uint4* re = (const uint4*)G.rent + (int)G.roff[j >> 5] * 32 + (j & 31);
+        const int nq = (int)(G.roff[(j >> 5) + 1] - G.roff[j >> 5]);
+        const uint32_t dum = 4u * nsp;
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+          const uint4 e = re[32 * q];
+          d += (int)(e.x < dum) + (int)(e.y < dum) + (int)(e.z < dum) + (int)(e.w < dum);
+        }
       }
       B.deg[j] = (uint8_t)d;
     }
-    if (R == 0) B.cns[nrp] = CNState{0.0f, 0.0f, 0u, 0u};  // the dummy check: message +0
+    if (R == 0) B.cns[32 * G.rwz] = CNState{0.0f, 0.0f, 0u, 0u};  // the dummy check: message +0
+#pragma unroll 1
     for (int base = 0; base < nr; base += S) {  // the window syndrome by check label
       const int j = base + R;
       const unsigned m = __ballot_sync(FULL, j < nr && bit_of(G.sbits, G.cperm[j]));
       if ((R & 31) == 0 && base + R < nr) B.sp[(base + R) >> 5] = m;
     }
     if (out.st)
+#pragma unroll 1
       for (int q = R; q < dmx; q += S) out.st[q] = StepTrace{-2, -1, 0, 0, 0};
     g.sync();
     if (P.peel_init) {
@@ -1117,10 +1145,12 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       }
     }
   }
+#pragma unroll 1
   for (int D = D0; D <= dmax; ++D) {
     depth = D;
     if (!(F.src && D == D0)) {  // (a resumed run's snapshot holds its first step's BP)
     const int ips = (D == 1 && P.ips1 > 0) ? P.ips1 : P.ips;  // the first step may have its own length
+#pragma unroll 1
     for (int it = 1; it <= ips; ++it) {
       // ---- check-node update, Eq. (1), and the previous iteration's H e = s ----
       bool unsat;
@@ -1128,7 +1158,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
         unsat = check_pass_warp<LW>(P, G, B, R, first, tw);
         __syncwarp();
       } else {
-        unsat = check_pass_cta<LW>(P, G, B, R, S, path_lanes_per_check(S, nr), first, tw);
+        unsat = check_pass_cta<LW>(P, G, B, R, S, path_lanes_per_check(S, 32 * G.rwz), first, tw);
       }
       visits += act;
       if (!g.any(unsat) && it >= 2) {  // the previous iteration's decisions satisfy H e = s
@@ -1149,6 +1179,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // the history of Sec. IV-A, for the columns a decimation step looks at:
       // SELECT-VN's and Alg. 3's candidates have degree three or more
       if (hist)
+#pragma unroll 1
         for (int s = R >> 5; s < V.K.n3; s += V.st) {
           const int k = 32 * s + lane;
           if (B.status[k] != -1) continue;
@@ -1198,6 +1229,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       unsigned cw = 0;
       if (R == 0) {
         int best = dmax - D + 2;  // more than one step more than this path's dmax - D + 1
+#pragma unroll 1
         for (int p = 0; p < P.nb; ++p) {
           const unsigned w = *(volatile unsigned*)&F.sched[p];
           int at = 0;
@@ -1239,6 +1271,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // ranked column (the oracle's index order) whatever the label order
       float bL = CUDART_INF_F, tL = CUDART_INF_F;
       int bk = kNone, tk = kNone, nagg = 0;
+#pragma unroll 1
       for (int k = R; k < ns; k += S) {
         if (B.status[k] != -1 || G.vdeg[k] <= 2) continue;
         const float L = B.acc[k];
@@ -1246,6 +1279,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
         if (!P.low_err) {
           int nus = 0;
           const uint32_t* ce = G.col_ents(k);
+#pragma unroll 1
           for (int u = 0; u < G.vdeg[k]; ++u) nus += bit_of(B.unsat, (int)(ce[32 * u] >> 16));
           int bdec = -1;
           if ((fl & pa_bit) && L < PBd) bdec = 1;
@@ -1308,6 +1342,7 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
         goto done;
       }
       if (D == d_reinit) {  // mu_{i->j} = Lambda_i again: the next pass reads the priors
+#pragma unroll 1
         for (int k = R; k < ns; k += S)
           if (B.status[k] == -1) B.post[k] = G.llr[k];
         tw = 0;
@@ -1318,8 +1353,10 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
   }
 done:
   // the estimate by ranked column (bit vperm[k] for label k)
+#pragma unroll 1
   for (int x = R; x < (ns + 31) >> 5; x += S) out.ebits[x] = 0u;
   g.sync();
+#pragma unroll 1
   for (int k = R; k < ns; k += S) {
     const int s8 = B.status[k];
     const int kr = G.vperm[k];
@@ -1336,6 +1373,7 @@ done:
     parity_pass(G, B, g);
     g.sync();
     long long nu = 0;
+#pragma unroll 1
     for (int j = R; j < G.nr; j += S)
       if (bit_of(B.unsat, j)) nu += (P.fallback == 2 && G.cperm[j] < G.ncr) ? (long long)G.nr + 2 : 1;
     fkey = (double)g.sum_ll(nu);
@@ -1344,6 +1382,7 @@ done:
   // window's output path (converged, path 0, or any path under a fallback
   // rule): the final posterior of each active column, +-clip for a decimated one
   if (out.keep && (status == BR_CONVERGED || id == 0 || P.fallback))
+#pragma unroll 1
     for (int k = R; k < ns; k += S) {
       const int s8 = B.status[k];
       out.keep[k] = s8 == -1 ? B.post[k] : (s8 ? -P.clip : P.clip);
@@ -1421,9 +1460,9 @@ struct DecodeArgs {
 // UG (a template parameter, so that shared-memory kernels keep shared-memory
 // instructions for every union access): the region lives in global memory.
 template <bool UG>
-__device__ __forceinline__ char* union_base(const DecodeArgs& A, char* sm) {
+__device__ __forceinline__ char* union_base(const DecodeArgs& A, char* sm, const SlotPlan& S) {
   if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
-  return sm + A.L.U;
+  return sm + S.U;
 }
 // The pre-BP scratch: the union region in global memory, else the bytes of the
 // shortened graph and the path slots, which do not exist yet.
@@ -1489,6 +1528,7 @@ __device__ __forceinline__ void reg_stage(unsigned long long (&v)[8], int base, 
 // the stages of block size kk with strides j0 >= j >= 1 (j0 < 256) of one
 // register segment whose first key has global index base
 __device__ __forceinline__ void seg_stages(unsigned long long (&v)[8], int base, int lane, int kk, int j0) {
+#pragma unroll 1
   for (int j = j0; j > 0; j >>= 1) {
     if (j == 128) {
       reg_stage<4>(v, base, lane, kk);
@@ -1513,6 +1553,7 @@ __device__ __forceinline__ void seg_stages(unsigned long long (&v)[8], int base,
 template <int M>
 __device__ __forceinline__ void smem_stages(unsigned long long* s, int n, int kk, int j) {
   const int b1 = __ffs(j) - 1;
+#pragma unroll 1
   for (int g = threadIdx.x; g < (n >> M); g += blockDim.x) {
     int base = g;
 #pragma unroll
@@ -1553,8 +1594,11 @@ __device__ __forceinline__ void smem_stages(unsigned long long* s, int n, int kk
 __device__ void block_sort_u64(unsigned long long* s, int n) {
   const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
   if (n < 256) {  // tiny windows: the plain network
+#pragma unroll 1
     for (int kk = 2; kk <= n; kk <<= 1)
+#pragma unroll 1
       for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+#pragma unroll 1
         for (int i = tid; i < n; i += NT) {
           const int ixj = i ^ jj;
           if (ixj > i) {
@@ -1570,18 +1614,22 @@ __device__ void block_sort_u64(unsigned long long* s, int n) {
     return;
   }
   // every block size up to 256 inside the segments
+#pragma unroll 1
   for (int sg = warp; sg < (n >> 8); sg += nw) {
     const int base = sg << 8;
     unsigned long long v[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) v[r] = s[base + 32 * r + lane];
+#pragma unroll 1
     for (int kk = 2; kk <= 256; kk <<= 1) seg_stages(v, base, lane, kk, kk >> 1);
 #pragma unroll
     for (int r = 0; r < 8; ++r) s[base + 32 * r + lane] = v[r];
   }
   __syncthreads();
+#pragma unroll 1
   for (int kk = 512; kk <= n; kk <<= 1) {
     int j = kk >> 1;
+#pragma unroll 1
     for (; j >= 256 * 4; j >>= 3) {  // three stages, all of stride >= 256
       smem_stages<3>(s, n, kk, j);
       __syncthreads();
@@ -1593,6 +1641,7 @@ __device__ void block_sort_u64(unsigned long long* s, int n) {
       smem_stages<1>(s, n, kk, j);
       __syncthreads();
     }
+#pragma unroll 1
     for (int sg = warp; sg < (n >> 8); sg += nw) {
       const int base = sg << 8;
       unsigned long long v[8];
@@ -1645,7 +1694,8 @@ struct PreBp {
   float *post, *key;
   CNState* cns;
   const uint32_t* sp;  // the window syndrome
-  const uint32_t *rent, *cent;
+  const uint16_t* rent;
+  const uint32_t* cent;
   const uint16_t *roff, *coff;
   const float* llr;
 };
@@ -1665,6 +1715,7 @@ __device__ __forceinline__ float prebp_key(const KParams& P, const PreBp& X, int
   if (P.n_pre >= 4) return p;
   const float li = X.llr[l];
   float s = li;
+#pragma unroll 1
   for (int r = 1; r < 4 - P.n_pre; ++r) s = __fadd_rn(s, li);
   return __fadd_rn(s, p);
 }
@@ -1711,7 +1762,7 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       const int j = real ? j0 : je - 1, s = j >> 5;
       const int r0 = X.roff[s], nq = real ? (int)X.roff[s + 1] - r0 : 0;
       uint32_t u = 0u;
-      const CNState rec = check_group<LW>((const uint4*)X.rent + r0 * 32 + (j & 31), nq, (const char*)X.post, X.cns[j],
+      const CNState rec = check_group<LW>((const uint2*)X.rent + r0 * 32 + (j & 31), nq, (const char*)X.post, X.cns[j],
                                           (X.sp[s] >> (j & 31)) & 1u, P.alpha, P.clip, t == 1, lw,
                                           (r0 * 32 + (j & 31)) * 4, sub, tpc, rwide, u);
       if (real) {
@@ -1734,6 +1785,7 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       const int q = i >> 5, c0 = X.coff[q] & (kWideSlice - 1), n = (int)(X.coff[q + 1] & (kWideSlice - 1)) - c0;
       const int ei = c0 * 32 + (i & 31);
       float p = X.llr[i];
+#pragma unroll 3
       for (int u = 0; u < n; ++u) {
         const uint32_t e = X.cent[ei + 32 * u];
         p = __fadd_rn(p, c2v<LW>(*(const CNState*)((const char*)X.cns + (e >> 12)), e, true,
@@ -1771,6 +1823,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
 
   // ---- a1: window syndrome ----
   const uint32_t* dp = A.det + (size_t)shot * A.det_words;
+#pragma unroll 1
   for (int x = tid; x < rw; x += NT) {
     const int b0 = W.row0 + 32 * x;
     const uint32_t lo = dp[b0 >> 5];
@@ -1781,24 +1834,29 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     if (rem < 32) v &= (1u << rem) - 1u;
     sbits[x] = v;
   }
+#pragma unroll 1
   for (int x = tid; x < L.cw; x += NT) cbits[x] = 0;
   __syncthreads();
 
   // the window graph in shared memory for the pre-BP loop when there is room
   PreBp X{post, key, cns, spre, W.s_rent, W.s_cent, W.s_roff, W.s_coff, W.s_llr};
-  if (L.pre_stage) {
-    const StagePiece pc[5] = {{U + L.q_rent, W.s_rent, 512u * W.row_quads},
-                              {U + L.q_cent, W.s_cent, 128u * W.col_cells},
-                              {U + L.q_roff, W.s_roff, al16(2u * (rw + 1))},
-                              {U + L.q_coff, W.s_coff, al16(2u * (L.cw + 1))},
-                              {U + L.q_sllr, W.s_llr, 4u * ncp}};
-    stage_pieces(stg, pc, 5);
-    X.rent = (const uint32_t*)(U + L.q_rent);
-    X.cent = (const uint32_t*)(U + L.q_cent);
-    X.roff = (const uint16_t*)(U + L.q_roff);
-    X.coff = (const uint16_t*)(U + L.q_coff);
-    X.llr = (const float*)(U + L.q_sllr);
+  if (L.pre_stage) {  // (an array that is not staged has no bytes)
+    const unsigned sg = L.pre_stage;
+    const StagePiece pc[5] = {{U + L.q_rent, W.s_rent, sg & kStageRent ? 256u * W.row_quads : 0u},
+                              {U + L.q_cent, W.s_cent, sg & kStageCent ? 128u * W.col_cells : 0u},
+                              {U + L.q_roff, W.s_roff, sg & kStageOff ? al16(2u * (rw + 1)) : 0u},
+                              {U + L.q_coff, W.s_coff, sg & kStageOff ? al16(2u * (L.cw + 1)) : 0u},
+                              {U + L.q_sllr, W.s_llr, sg & kStageLlr ? 4u * ncp : 0u}};
+    stage_pieces(stg, pc);
+    if (sg & kStageRent) X.rent = (const uint16_t*)(U + L.q_rent);
+    if (sg & kStageCent) X.cent = (const uint32_t*)(U + L.q_cent);
+    if (sg & kStageLlr) X.llr = (const float*)(U + L.q_sllr);
+    if (sg & kStageOff) {
+      X.roff = (const uint16_t*)(U + L.q_roff);
+      X.coff = (const uint16_t*)(U + L.q_coff);
+    }
   }
+#pragma unroll 1
   for (int s = warp; s < rw; s += nw) {
     const int j = 32 * s + lane;
     const unsigned m = __ballot_sync(FULL, j < nr && bit_of(sbits, W.s_row[j]));
@@ -1814,6 +1872,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   int t = 0;
   const int tk0 = P.n_pre - 3 > 1 ? P.n_pre - 3 : 1;
   if (P.n_pre == 0) {
+#pragma unroll 1
     for (int l = tid; l < nc; l += NT) {
       const float li = X.llr[l];
       post[l] = li;
@@ -1824,6 +1883,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     // the first VN->CN messages of the pre-BP: the prior, or (message reuse)
     // what the previous window's output path kept for the same DEM column
     const float* kept = (A.keep && A.prev) ? A.keep + (size_t)shot * A.keep_ld : nullptr;
+#pragma unroll 1
     for (int l = tid; l < nc; l += NT) {
       float v = X.llr[l];
       if (kept) {
@@ -1841,15 +1901,17 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   if (WIDE && !UG && P.n_pre > 0 && cl_size() > 1 && nr >= 2 * (int)cl_size() && nc >= 2 * (int)cl_size()) {
     t = prebp_cluster<LW>(A, W, X, sm, conv, t_conv);
   } else {
+#pragma unroll 1
     for (t = 1; t <= P.n_pre; ++t) {
       // check nodes; each check also takes the parity of the hard decisions it
       // reads, so for t >= 2 the pass is the convergence test of iteration t-1
       LwRow lw{nullptr, W.s_ref};
       if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
       uint32_t unsat = 0u;
+#pragma unroll 1
       for (int s = warp; s < rw; s += nw) {
         const int r0 = X.roff[s], nq = (int)X.roff[s + 1] - r0;
-        unsat |= check_lane<LW>((const uint4*)X.rent + r0 * 32 + lane, nq, (const char*)post, cns + 32 * s + lane,
+        unsat |= check_lane<LW>((const uint2*)X.rent + r0 * 32 + lane, nq, (const char*)post, cns + 32 * s + lane,
                                 (spre[s] >> lane) & 1u, P.alpha, P.clip, lw, (r0 * 32 + lane) * 4, t == 1);
       }
       if (!__syncthreads_or(unsat != 0u) && t >= 2) {  // iteration t-1 satisfies H e = s
@@ -1868,9 +1930,10 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   }
   if (!conv) {  // the convergence test of the last iteration (or of the priors)
     bool unsat = false;
+#pragma unroll 1
     for (int s = warp; s < rw; s += nw) {
       const uint32_t hp = (((spre[s] >> lane) & 1u) << 31) ^
-                          check_parity((const uint4*)X.rent + (int)X.roff[s] * 32 + lane,
+                          check_parity((const uint2*)X.rent + (int)X.roff[s] * 32 + lane,
                                        (int)X.roff[s + 1] - (int)X.roff[s], (const char*)post);
       unsat |= (hp >> 31) != 0u;
     }
@@ -1881,6 +1944,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   }
   *t_run_out = conv ? t_conv : P.n_pre;
   if (conv) {
+#pragma unroll 1
     for (int l = tid; l < nc; l += NT)
       if (post[l] <= 0.0f) {
         const int c = W.s_col[l];
@@ -1893,24 +1957,28 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   // ---- a3: rank by the four-iteration sum, keep the first n_short ----
   const int n_short = W.n_short, nsp = 32 * L.sw;
   unsigned long long* sortb = (unsigned long long*)(U + L.p_sort);
+#pragma unroll 1
   for (int l = tid; l < L.sortn; l += NT)  // ties by window column
     sortb[l] = l < nc ? (((unsigned long long)ordkey(key[l]) << 32) | ((unsigned)W.s_col[l] << 16) | (unsigned)l) : ~0ull;
   __syncthreads();
   block_sort_u64(sortb, L.sortn);
   // (from here on the pre-BP's arrays are dead: the shortened graph takes their place)
   uint16_t* sel = (uint16_t*)(sm + L.sel);
-  uint32_t* rent = (uint32_t*)(sm + L.s_rent);
-  uint32_t* cent = (uint32_t*)(sm + L.s_cent);
   uint16_t* roff = (uint16_t*)(sm + L.s_roff);
   uint16_t* coff = (uint16_t*)(sm + L.s_coff);
   float* sllr = (float*)(sm + L.s_llr);
   uint8_t* svd = (uint8_t*)(sm + L.s_vdeg);
-  uint16_t* sref = (uint16_t*)(sm + L.s_ref);
-  uint16_t* scef = (uint16_t*)(sm + L.s_cef);
   uint16_t* cperm = (uint16_t*)(sm + L.s_cperm);
   uint16_t* vperm = (uint16_t*)(sm + L.s_vperm);
-  int* rc = (int*)(sm + L.rowcnt);
+#pragma unroll 1
   for (int k = tid; k < n_short; k += NT) sel[k] = (uint16_t)(sortb[k] >> 16);
+  __syncthreads();
+  // sort keys of the labels, (degree, lowest index first), by rank and by row;
+  // zero in the padding
+  unsigned* ckey = (unsigned*)(U + L.p_scr);
+  unsigned* rkey = ckey + nsp;
+  int* rc = (int*)(rkey + nrp);  // degree by window row, later entries placed by label
+#pragma unroll 1
   for (int j = tid; j < nrp; j += NT) rc[j] = 0;
   __syncthreads();
   // ---- shortened matrix in shared memory, numbered in processing order ----
@@ -1918,37 +1986,46 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   // so the lanes of a round loop alike; vperm and cperm map a label back to
   // the ranked column and the window row, which decide every tie.  A column's
   // checks stay in ascending window row (the order of the sum of Eq. (2)).
-  int* deg = (int*)sortb;            // the sort buffer is free now: degree by rank, then
-  int* cinv = deg + up32(n_short);   // window row -> label (no room past the keys: see below)
+#pragma unroll 1
+  for (int k = tid; k < nsp; k += NT) {
+    unsigned d = 0;
+    if (k < n_short) {
+      const int c = sel[k], e0 = W.col_ptr[c];
+      d = W.col_ptr[c + 1] - e0;
+#pragma unroll 1
+      for (unsigned u = 0; u < d; ++u) atomicAdd(&rc[W.col_rows[e0 + u]], 1);  // rows of the shortened matrix
+    }
+    ckey[k] = k < n_short ? (d << 16) | (0xFFFFu - (unsigned)k) : 0u;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int j = tid; j < nrp; j += NT) rkey[j] = j < nr ? ((unsigned)rc[j] << 16) | (0xFFFFu - (unsigned)j) : 0u;
+  // a label is the number of larger keys; no sort needed at these sizes
+  auto above = [](const unsigned* key, int n, unsigned k) {
+    int r = 0;
+#pragma unroll 2
+    for (int i = 0; i < n; i += 4) {
+      const uint4 x = *(const uint4*)(key + i);
+      r += (x.x > k) + (x.y > k) + (x.z > k) + (x.w > k);
+    }
+    return r;
+  };
+#pragma unroll 1
   for (int k = tid; k < n_short; k += NT) {
-    const int c = sel[k], e0 = W.col_ptr[c], e1 = W.col_ptr[c + 1];
-    deg[k] = e1 - e0;
-    for (int e = e0; e < e1; ++e) atomicAdd(&rc[W.col_rows[e]], 1);  // rows of the shortened matrix
-  }
-  __syncthreads();
-  for (int k = tid; k < n_short; k += NT) {  // rank by counting; no sort needed at these sizes
-    const int dk = deg[k];
-    int r = 0;
-    for (int i = 0; i < n_short; ++i) {
-      const int di = deg[i];
-      r += (di > dk) || (di == dk && i < k);
-    }
+    const unsigned key_k = ckey[k];
+    const int r = above(ckey, nsp, key_k);
     vperm[r] = (uint16_t)k;
-    svd[r] = (uint8_t)dk;
-  }
-  for (int j = tid; j < nr; j += NT) {
-    const int dj = rc[j];
-    int r = 0;
-    for (int i = 0; i < nr; ++i) {
-      const int di = rc[i];
-      r += (di > dj) || (di == dj && i < j);
-    }
-    cperm[r] = (uint16_t)j;
+    svd[r] = (uint8_t)(key_k >> 16);
   }
   __syncthreads();
+#pragma unroll 1
+  for (int j = tid; j < nr; j += NT) cperm[above(rkey, nrp, rkey[j])] = (uint16_t)j;
+  __syncthreads();
+  int* cinv = (int*)rkey;  // window row -> label, once the keys have been read
   // slice starts (a slice is as wide as its first node), one warp each
   if (warp == 0) {
     int run = 0;
+#pragma unroll 1
     for (int b = 0; b < rw; b += 32) {
       const int s = b + lane;
       int v = s < rw ? (rc[cperm[32 * s]] + 3) >> 2 : 0;
@@ -1962,6 +2039,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     // (a check past 32 entries is rare in a shortened graph: one flag for all)
     const uint16_t flag = rc[cperm[0]] > 32 ? kWideSlice : (uint16_t)0;
     int run = 0;
+#pragma unroll 1
     for (int b = 0; b < L.sw; b += 32) {
       const int s = b + lane;
       int v = s < L.sw ? (int)svd[32 * s] : 0;
@@ -1972,30 +2050,54 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     if (lane == 0) coff[0] = flag;
     if (lane < 4) {  // slices at least 4 - lane wide
       int n = 0;
+#pragma unroll 1
       while (n < L.sw && svd[32 * n] >= 4 - lane) ++n;
       ((int*)(sm + L.s_cls))[lane] = n;
     }
   }
   __syncthreads();
+  // the shot's own layout
+  SlotPlan S;
+  {
+    int rwz = 0;
+#pragma unroll 1
+    while (rwz < rw && roff[rwz + 1] > roff[rwz]) ++rwz;
+    S = slot_plan(L, roff[rw], coff[L.sw] & (kWideSlice - 1), rwz, ((const int*)(sm + L.s_cls))[1],
+                  UG ? (unsigned)A.ubytes : L.total, UG, nw);
+    if (tid == 0) *(SlotPlan*)(sm + L.plan) = S;
+  }
+  uint32_t* rent = (uint32_t*)(sm + S.rent);
+  uint32_t* cent = (uint32_t*)(sm + S.cent);
+  uint16_t* sref = (uint16_t*)(sm + S.ref);
+  uint16_t* scef = (uint16_t*)(sm + S.cef);
   // every place a dummy, then the edges
   {
     const int nq = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
+#pragma unroll 1
     for (int x = tid; x < 128 * nq; x += NT) rent[x] = 4u * (unsigned)nsp;
-    for (int x = tid; x < 32 * ncell; x += NT) cent[x] = (unsigned)nrp << 16;
+#pragma unroll 1
+    for (int x = tid; x < 32 * ncell; x += NT) cent[x] = (unsigned)(32 * S.rwz) << 16;
     if (LW) {
+#pragma unroll 1
       for (int x = tid; x < 128 * nq; x += NT) sref[x] = 0;
+#pragma unroll 1
       for (int x = tid; x < 32 * ncell; x += NT) scef[x] = 0;
     }
+#pragma unroll 1
     for (int l = tid; l < nr; l += NT) cinv[cperm[l]] = l;
+#pragma unroll 1
     for (int k = n_short + tid; k < nsp; k += NT) sllr[k] = 0.0f;
   }
   __syncthreads();
+#pragma unroll 1
   for (int j = tid; j < nrp; j += NT) rc[j] = 0;
   __syncthreads();
+#pragma unroll 1
   for (int k = tid; k < n_short; k += NT) {
     const int c = sel[vperm[k]], e0 = W.col_ptr[c], d = svd[k];
     sllr[k] = W.llr[c];
     const int ci = (coff[k >> 5] & (kWideSlice - 1)) * 32 + (k & 31);
+#pragma unroll 1
     for (int u = 0; u < d; ++u) {
       const int r = cinv[W.col_rows[e0 + u]];
       const int pos = atomicAdd(&rc[r], 1);
@@ -2008,6 +2110,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
       }
     }
     if (LW)  // a dummy takes its column's first edge's weight (a check's dummies are dead inputs)
+#pragma unroll 1
       for (int u = d; u < (int)(coff[(k >> 5) + 1] & (kWideSlice - 1)) - (coff[k >> 5] & (kWideSlice - 1)); ++u)
         scef[ci + 32 * u] = (uint16_t)e0;
   }
@@ -2015,13 +2118,14 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   return false;
 }
 
-__device__ __forceinline__ ShortG short_graph(char* sm, const Layout& L, const WinDev& W, int ns) {
-  return ShortG{W.n_rows, ns, L.rw, L.sw,
-                (const uint32_t*)(sm + L.s_rent), (const uint32_t*)(sm + L.s_cent),
+__device__ __forceinline__ ShortG short_graph(char* sm, const Layout& L, const SlotPlan& S, const WinDev& W, int ns) {
+  return ShortG{W.n_rows, ns, L.rw, L.sw, S.rwz,
+                (const uint32_t*)(sm + S.rent),   (const uint32_t*)(sm + S.cent),
                 (const uint16_t*)(sm + L.s_roff), (const uint16_t*)(sm + L.s_coff),
                 (const float*)(sm + L.s_llr),     (const uint8_t*)(sm + L.s_vdeg),
-                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(sm + L.s_ref), (const uint16_t*)(sm + L.s_cef),
-                (const ColClasses*)(sm + L.s_cls), W.wts, W.wT, W.n_edges, W.rows_per_block, (const uint16_t*)(sm + L.sel),
+                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(sm + S.ref), (const uint16_t*)(sm + S.cef),
+                (const ColClasses*)(sm + L.s_cls), W.wts, W.wT, W.n_edges, W.rows_per_block,
+                (const uint16_t*)(sm + L.sel),
                 (const uint16_t*)(sm + L.s_cperm), (const uint16_t*)(sm + L.s_vperm), W.n_commit_rows};
 }
 
@@ -2044,6 +2148,7 @@ __device__ __forceinline__ PathOut trace_out(const DecodeArgs& A, char* tr, int 
 __device__ __forceinline__ int fallback_path(const KParams& P, const double* pm) {
   int fb = 0;
   if (P.fallback)
+#pragma unroll 1
     for (int id = 1; id < P.nb; ++id)
       if (pm[id] < pm[fb]) fb = id;
   return fb;
@@ -2055,8 +2160,10 @@ __device__ void write_outputs(const DecodeArgs& A, char* sm, long long shot, boo
   const int tid = threadIdx.x, NT = blockDim.x;
   const uint32_t* cbits = (const uint32_t*)(sm + L.cbits);
   uint32_t* co = A.corr + (size_t)shot * A.corr_words;
+#pragma unroll 1
   for (int x = tid; x < A.corr_words; x += NT) co[x] = x < L.cw ? cbits[x] : 0u;
   if (tr && !conv)
+#pragma unroll 1
     for (int k = tid; k < n_short; k += NT)
       ((uint16_t*)(tr + trace_off_sel(A.P.nb, A.dmx, A.ns_max)))[k] = ((const uint16_t*)(sm + L.sel))[k];
   if (tid == 0) {
@@ -2082,13 +2189,16 @@ __device__ void keep_for_next(const DecodeArgs& A, char* sm, long long shot, con
   const int tid = threadIdx.x, NT = blockDim.x, nc = A.W.n_cols;
   float* out = A.keep + (size_t)shot * A.keep_ld;
   if (!kp) {
+#pragma unroll 1
     for (int l = tid; l < nc; l += NT) out[A.W.s_col[l]] = post[l];
     return;
   }
   const uint16_t* sel = (const uint16_t*)(sm + A.L.sel);
   const uint16_t* vperm = (const uint16_t*)(sm + A.L.s_vperm);
+#pragma unroll 1
   for (int c = tid; c < nc; c += NT) out[c] = CUDART_NAN_F;
   __syncthreads();
+#pragma unroll 1
   for (int k = tid; k < n_short; k += NT) out[sel[vperm[k]]] = __ldcg(kp + k);
 }
 
@@ -2111,11 +2221,12 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
   int winner = -1;
   const int n_short = conv ? 0 : A.W.n_short;
   if (!conv) {
-    // warps beyond the layout's path slots (batched launches) sit out the paths
-    if (warp < L.nslots) {
-      const ShortG G = short_graph(sm, L, A.W, n_short);
-      char* slot = union_base<UG>(A, sm) + (size_t)warp * L.b_size;
-      const Slot B = make_slot(slot, L);
+    // warps beyond the shot's path slots sit out the paths
+    const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
+    if (warp < S.nslots) {
+      const ShortG G = short_graph(sm, L, S, A.W, n_short);
+      char* slot = union_base<UG>(A, sm, S) + (size_t)warp * S.b_size;
+      const Slot B = make_slot(slot, S);
       const WarpGrp g{lane};
       // snapshots of shared prefixes, when planned and this CTA has a pool
       // shared prefixes and preemption, when planned and this CTA has a pool
@@ -2126,7 +2237,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
       F.pool = fork ? A.F.pool + (size_t)blockIdx.x * A.F.cta_bytes : nullptr;
       F.stride = kSnapHeader + L.b_size;
       F.slot = slot;
-      F.slot_bytes = L.b_size;
+      F.slot_bytes = S.b_size;
       F.st0 = tr ? (const StepTrace*)(tr + trace_off_st(nb)) : nullptr;
       F.sched = (fork && A.F.sched) ? (unsigned*)(sm + L.red) + kMaxForkNodes : nullptr;
       F.fnode = A.F.fnode;
@@ -2134,6 +2245,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
       F.n_nodes = A.F.n_nodes;
       int next = -1;  // the path taken at a preemption point
       unsigned next_w = 0;
+#pragma unroll 1
       while (true) {
         int id = -1;
         unsigned w0 = PS_QUEUED;  // the taken path's state word: queued or parked after step D
@@ -2142,6 +2254,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
           w0 = next_w;
           next = -1;
         } else {
+#pragma unroll 1
           while (true) {  // the next queued path that no preemption took
             int pos = 0;
             if (lane == 0) pos = atomicAdd(&misc[2], 1);
@@ -2159,9 +2272,11 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
             int c = -1;
             unsigned cw = 0;
             if (lane == 0)
+#pragma unroll 1
               for (int tries = 0; tries < 4 * nb; ++tries) {
                 c = -1;
                 int best = 0;
+#pragma unroll 1
                 for (int p = 0; p < nb; ++p) {
                   const unsigned w = *(volatile unsigned*)&F.sched[p];
                   if ((w & 3u) != PS_PARKED) continue;
@@ -2198,6 +2313,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
           int node = -1;
           if (lane == 0) {
             const int dm = path_dmax(A.P, id, path_split(A.P, id));
+#pragma unroll 1
             for (int D = dm; D >= 1 && node < 0; --D) {
               const int n = F.chain[D - 1];
               if (n >= 0 && *(volatile int*)&F.flags[n] == 2) node = n;
@@ -2217,6 +2333,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
     if (tid == 0) {
       int best = -1;
       double bp = CUDART_INF;
+#pragma unroll 1
       for (int id = 0; id < A.P.nb; ++id)
         if (res_status[id] == BR_CONVERGED && res_pm[id] < bp) {
           bp = res_pm[id];
@@ -2229,6 +2346,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
     winner = misc[1];
     const int outp = misc[4];
     const uint32_t* eb = res_e + (size_t)outp * L.sw;
+#pragma unroll 1
     for (int k = tid; k < n_short; k += blockDim.x)
       if ((eb[k >> 5] >> (k & 31)) & 1u) atomicOr(&cbits[sel[k] >> 5], 1u << (sel[k] & 31));
     if (A.keep) {
@@ -2242,11 +2360,13 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
   write_outputs(A, sm, shot, conv, winner, n_short, t_run, tr);
 }
 
-template <bool LW, bool UG>
-__global__ void __launch_bounds__(256, 2) decode_shot_kernel(DecodeArgs A) {
+// CTAS: CTAs per SM (register budget), see configure_layouts.
+template <bool LW, bool UG, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) decode_shot_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
   int* misc = (int*)(sm + A.L.misc);
   Stager stg = stager_init((char*)(misc + 8), &A.counters[4]);
+#pragma unroll 1
   while (true) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -2273,6 +2393,7 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
   extern __shared__ __align__(16) char sm[];
   int* q = (int*)(sm + B.q_off);
   Stager stg = stager_init((char*)(q + 4), &B.seg[0].counters[4]);
+#pragma unroll 1
   while (true) {
     __syncthreads();
     if (threadIdx.x == 0) q[0] = atomicAdd(B.work, 1);
@@ -2280,6 +2401,7 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
     const long long g = q[0];
     if (g >= B.seg_end[B.n_seg - 1]) break;
     int m = 0;
+#pragma unroll 1
     while (g >= B.seg_end[m]) ++m;
     const DecodeArgs& A = B.seg[m];
     const long long shot = g - (m ? B.seg_end[m - 1] : 0);
@@ -2314,8 +2436,9 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
     return;
   }
   const int n_short = A.W.n_short;
-  const ShortG G = short_graph(sm, L, A.W, n_short);
-  const Slot B = make_slot(union_base<false>(A, sm), L);
+  const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
+  const ShortG G = short_graph(sm, L, S, A.W, n_short);
+  const Slot B = make_slot(union_base<false>(A, sm, S), S);
   const CtaGrp g{tid, (int)blockDim.x, sm + L.red};
   const size_t rb = path_result_bytes(A.sw_max);
   char* mine = A.path_res + ((size_t)shot * nb + id) * rb;
@@ -2335,6 +2458,7 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   if (tid == 0) {
     int best = -1, fb = 0;
     double bp = CUDART_INF, bk = CUDART_INF;
+#pragma unroll 1
     for (int q = 0; q < nb; ++q) {
       const char* r = A.path_res + ((size_t)shot * nb + q) * rb;
       const int st = __ldcg((const int*)r);
@@ -2358,6 +2482,7 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   const uint32_t* eb = (const uint32_t*)(A.path_res + ((size_t)shot * nb + outp) * rb + 16);
   uint32_t* cbits = (uint32_t*)(sm + L.cbits);
   const uint16_t* sel = (const uint16_t*)(sm + L.sel);
+#pragma unroll 1
   for (int k = tid; k < n_short; k += blockDim.x)
     if ((__ldcg(&eb[k >> 5]) >> (k & 31)) & 1u) atomicOr(&cbits[sel[k] >> 5], 1u << (sel[k] & 31));
   if (A.keep) keep_for_next(A, sm, shot, A.kpath + ((size_t)shot * nb + outp) * A.ns_max, n_short);
@@ -2388,6 +2513,7 @@ __global__ void sample_kernel(int n_cols, const uint32_t* __restrict__ thr, cons
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const long long s = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
   uint32_t* row = srow + (size_t)wib * det_words;
+#pragma unroll 1
   for (int x = lane; x < det_words; x += 32) row[x] = 0;
   __syncwarp();
   uint32_t ob = 0;
@@ -2395,6 +2521,7 @@ __global__ void sample_kernel(int n_cols, const uint32_t* __restrict__ thr, cons
     const unsigned long long shot = off + (unsigned long long)s;
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const int ng = (n_cols + 3) >> 2;
+#pragma unroll 1
     for (int g = lane; g < ng; g += 32) {
       const uint4 u = philox4x32_10(make_uint4((uint32_t)g, (uint32_t)shot, (uint32_t)(shot >> 32), 0u), key);
       const uint32_t uu[4] = {u.x, u.y, u.z, u.w};
@@ -2402,6 +2529,7 @@ __global__ void sample_kernel(int n_cols, const uint32_t* __restrict__ thr, cons
       for (int r = 0; r < 4; ++r) {
         const int c = 4 * g + r;
         if (c < n_cols && uu[r] < thr[c]) {
+#pragma unroll 1
           for (int e = cptr[c]; e < cptr[c + 1]; ++e) {
             const int d = cdet[e];
             atomicXor(&row[d >> 5], 1u << (d & 31));
@@ -2414,6 +2542,7 @@ __global__ void sample_kernel(int n_cols, const uint32_t* __restrict__ thr, cons
   __syncwarp();
   ob = __reduce_xor_sync(FULL, ob);
   if (s < n) {
+#pragma unroll 1
     for (int x = lane; x < det_words; x += 32) det[(size_t)s * det_words + x] = row[x];
     if (lane == 0) obs[s] = ob;
   }
@@ -2425,14 +2554,17 @@ __device__ void commit_one(const CommitArgs& C, long long s) {
   uint32_t* d = C.det + (size_t)s * C.det_words;
   uint32_t ob = 0;
   const int nw = (C.n_commit + 31) >> 5;
+#pragma unroll 1
   for (int x = 0; x < nw; ++x) {
     uint32_t m = c[x];
     const int rem = C.n_commit - 32 * x;
     if (rem < 32) m &= (1u << rem) - 1u;
+#pragma unroll 1
     while (m) {
       const int b = __ffs(m) - 1;
       m &= m - 1;
       const int col = 32 * x + b;
+#pragma unroll 1
       for (int e = C.cptr[col]; e < C.cptr[col + 1]; ++e) {
         const int q = C.cdet[e];
         d[q >> 5] ^= 1u << (q & 31);
@@ -2442,6 +2574,7 @@ __device__ void commit_one(const CommitArgs& C, long long s) {
   }
   C.obs_pred[s] ^= ob;
   uint32_t bad = 0;
+#pragma unroll 1
   for (int q = C.b0; q < C.b1;) {
     const int wq = q >> 5, lo = q & 31;
     const int hiq = min(C.b1, (wq + 1) * 32);
@@ -2465,6 +2598,7 @@ __global__ void commit_batch_kernel(const __grid_constant__ CommitBatch B) {
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= B.seg_end[B.n_seg - 1]) return;
   int m = 0;
+#pragma unroll 1
   while (g >= B.seg_end[m]) ++m;
   commit_one(B.seg[m], g - (m ? B.seg_end[m - 1] : 0));
 }
@@ -2490,24 +2624,14 @@ __global__ void evaluate_kernel(const uint32_t* __restrict__ pred, const uint32_
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max) { return dev::trace_bytes(nb, dmx, ns_max); }
 
 cudaError_t set_decode_smem(size_t bytes) {
-  const int b = (int)bytes;
-  cudaError_t e =
-      cudaFuncSetAttribute(dev::decode_shot_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_shot_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_shot_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_shot_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_path_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_path_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_batch_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dev::decode_batch_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  return e;
+  const void* f[] = {(const void*)dev::decode_shot_kernel<false, false, 2>, (const void*)dev::decode_shot_kernel<true, false, 2>,
+                     (const void*)dev::decode_shot_kernel<false, true, 2>,  (const void*)dev::decode_shot_kernel<true, true, 2>,
+                     (const void*)dev::decode_shot_kernel<false, false, 3>, (const void*)dev::decode_path_kernel<false>,
+                     (const void*)dev::decode_path_kernel<true>,            (const void*)dev::decode_batch_kernel<false>,
+                     (const void*)dev::decode_batch_kernel<true>};
+  for (const void* k : f)
+    if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) return e;
+  return cudaSuccess;
 }
 
 cudaError_t batch_occupancy(int threads, size_t smem, int* blocks) {
@@ -2556,12 +2680,14 @@ cudaError_t launch_commit_batch(cudaStream_t st, const BatchMember* m, int n) {
   return cudaGetLastError();
 }
 
-cudaError_t decode_occupancy(int mode, int threads, size_t smem, int* blocks) {
+cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* blocks) {
   if (mode == 1)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_path_kernel<false>, threads, smem);
   if (mode == 3)  // shot mode with the union region in global memory
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, true>, threads, smem);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, true, 2>, threads, smem);
+  if (ctas >= 3)
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 3>, threads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 2>, threads, smem);
 }
 
 cudaError_t path_cluster_occupancy(int threads, size_t smem, int cluster, int* clusters) {
@@ -2579,7 +2705,7 @@ cudaError_t path_cluster_occupancy(int threads, size_t smem, int cluster, int* c
   return cudaOccupancyMaxActiveClusters(clusters, dev::decode_path_kernel<false>, &cfg);
 }
 
-cudaError_t launch_decode(int mode, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
+cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
                           const WinDev& W, const Layout& L, const uint32_t* det, int det_words, long long n,
                           uint32_t* corr, int corr_words, int32_t* status, char* trace, size_t tr_bytes, int dmx,
                           int ns_max, int* work, long long* counters, char* path_res, int* arrive, int sw_max,
@@ -2612,11 +2738,13 @@ cudaError_t launch_decode(int mode, int grid, int threads, size_t smem, cudaStre
     return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<false>, A);
   } else {
     if (uglob) {
-      if (lw) dev::decode_shot_kernel<true, true><<<grid, threads, smem, st>>>(A);
-      else dev::decode_shot_kernel<false, true><<<grid, threads, smem, st>>>(A);
+      if (lw) dev::decode_shot_kernel<true, true, 2><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, true, 2><<<grid, threads, smem, st>>>(A);
+    } else if (ctas >= 3 && !lw) {
+      dev::decode_shot_kernel<false, false, 3><<<grid, threads, smem, st>>>(A);
     } else {
-      if (lw) dev::decode_shot_kernel<true, false><<<grid, threads, smem, st>>>(A);
-      else dev::decode_shot_kernel<false, false><<<grid, threads, smem, st>>>(A);
+      if (lw) dev::decode_shot_kernel<true, false, 2><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, false, 2><<<grid, threads, smem, st>>>(A);
     }
   }
   return cudaGetLastError();

@@ -20,7 +20,7 @@
 // bounds test: the places past a node's degree hold a dummy whose value
 // changes nothing (a column with posterior +inf, a check record with message
 // +0).
-//   check entry:  byte offset 4 * column of the column's posterior
+//   check entry:  the column, or (shortened graph) its posterior's byte offset
 //   column entry: check << 16 | position of the edge among the check's entries
 #pragma once
 #include <cstddef>
@@ -115,7 +115,8 @@ struct WinDev {
   int n_commit_rows;      // rows [0, n_commit_rows) are the ones the window commits
   // the graph in slices (see the top of the file), checks and columns by label
   int row_quads, col_cells;    // slice totals per lane: check entries in fours, column entries
-  const uint32_t *s_rent, *s_cent;   // [4 * 32 * row_quads], [32 * col_cells]
+  const uint16_t* s_rent;  // [4 * 32 * row_quads]
+  const uint32_t* s_cent;  // [32 * col_cells]
   const uint16_t *s_roff, *s_coff;   // slice starts, in fours / in entries per lane
   const float* s_llr;                // priors by column label
   const uint16_t *s_row, *s_col;     // label -> window row / window column
@@ -199,6 +200,7 @@ struct SliceDims {
   int row_quads, col_cells;    // the window's, as WinDev
   int srow_quads, scol_cells;  // the shortened graph's, at most
 };
+__host__ __device__ inline unsigned al16(unsigned x) { return (x + 15u) & ~15u; }
 __host__ __device__ inline unsigned up32(unsigned x) { return (x + 31u) & ~31u; }
 
 // Shared-memory layout of one CTA (byte offsets), identical on host and device.
@@ -212,41 +214,89 @@ struct Layout {
   // pre-BP (relative to U; make_slice_layout: to V)
   unsigned p_post, p_key, p_cns, p_sign, p_par, p_sort, p_end;
   // the window graph staged for the pre-BP loop in otherwise idle union bytes
-  // (from p_sort on; overwritten by the sort that follows); pre_stage = 0: none
+  // (overwritten by the sort that follows); pre_stage = 0: none
   unsigned pre_stage, q_colptr, q_colrows, q_rowptr, q_rowent, q_llr, q_vperm;
   // one path slot (relative to the slot base)
   unsigned b_post, b_acc, b_hfl, b_status, b_sign, b_cns, b_deg, b_sp, b_unsat, b_hq, b_size;
   unsigned total;
   int rw, cw, sw, sortn, nslots;
-  // slices: the shortened graph (s_rent .. s_coff; s_ref / s_cef with learned
-  // weights) and the staged window graph (q_rent .. q_llr)
-  unsigned s_rent, s_cent, s_roff, s_coff, s_ref, s_cef, s_cls;
+  // slices: the shortened graph's fixed arrays, and where its entries and the
+  // path slots start (s_dyn; laid out per shot, see SlotPlan; U: the slots'
+  // start at the latest); the staged window graph (q_rent .. q_sllr; pre_stage
+  // has a bit for each array that is staged)
+  unsigned s_roff, s_coff, s_cls, s_dyn, plan, p_scr;
   unsigned q_rent, q_cent, q_roff, q_coff, q_sllr;
   // The pre-BP's arrays start at V, where the shortened graph and the path
   // slots begin: neither exists before the pre-BP has ended.
   unsigned V;
+  unsigned hist, lwe;  // bytes of quantised history per column of degree >= 3; 1: learned weights' edge ids
+};
+enum { kStageRent = 1, kStageCent = 2, kStageLlr = 4, kStageOff = 8 };
+
+// A shot's part of the layout: the entries of its shortened graph, then its
+// path slots, sized by the graph the shot has (its non-empty check slices,
+// its columns of degree three or more), not by the largest there could be:
+// 671 edges against a bound of 2304 for [[144,12,12]] (3,1) windows.
+struct SlotPlan {
+  unsigned rent, cent, ref, cef, U;
+  unsigned b_acc, b_hfl, b_status, b_cns, b_deg, b_sp, b_unsat, b_hq, b_size;
+  int nslots, rwz;  // path slots that fit; non-empty check slices
 };
 
-__host__ __device__ inline unsigned al16(unsigned x) { return (x + 15u) & ~15u; }
 
-// Layout of the decode kernels.  The pre-BP scratch (and the staged window
-// graph: stage = 1) shares its bytes with the shortened graph and the path
-// slots that follow it; only the ranking's sort buffer, read while the
-// shortened graph is being written, lies past that graph (and past the keys it
-// is filled from).  stage = 2: the staged graph lies past everything else, so
-// that the ranking and the shortening can read it too.  ub_glob: the union is
-// addressed from its own base (global memory), the shortened graph stays in
-// shared memory.
-__host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, int nc, int ns, int nb, int nslots,
-                                                    int stage, bool ranker, bool lw, bool ub_glob) {
+// nq, ncell: the shortened graph's check entries in fours and column entries
+// (per lane); rwz, n3: its non-empty check slices, its column slices of width
+// three or more; end: the bytes there are (glob: of the union region, which
+// then holds only the slots); the slots' number is at most `most`.
+__host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell, int rwz, int n3, unsigned end,
+                                              bool glob, int most) {
+  SlotPlan S{};
+  const unsigned nsp = 32u * L.sw;
+  unsigned o = L.s_dyn;
+  S.rent = o; o = al16(o + 512u * nq);
+  S.cent = o; o = al16(o + 128u * ncell);
+  S.ref = o; o = al16(o + (L.lwe ? 256u * nq : 0u));
+  S.cef = o; o = al16(o + (L.lwe ? 64u * ncell : 0u));
+  S.U = o;
+  unsigned b = al16(4u * (nsp + 1));  // posteriors and the dummy column's
+  S.b_acc = b; b += 128u * n3;
+  S.b_hfl = b; b += 32u * n3;
+  S.b_status = b; b = al16(b + nsp);
+  S.b_cns = b; b += 16u * (32u * rwz + 1);
+  S.b_deg = b; b = al16(b + 32u * L.rw);
+  S.b_sp = b; b = al16(b + 4u * L.rw);
+  S.b_unsat = b; b = al16(b + 4u * L.rw);
+  S.b_hq = b; b = al16(b + 32u * L.hist * n3);
+  S.b_size = b;
+  const unsigned room = glob ? end : (end > S.U ? end - S.U : 0u);
+  const int n = (int)(room / b);
+  S.nslots = n < most ? n : most;
+  S.rwz = rwz;
+  return S;
+}
+
+// Layout of the decode kernels for a CTA with `budget` bytes of shared memory.
+// The pre-BP scratch and as much of the window graph as fits beside it share
+// their bytes with the shortened graph and the path slots that follow.  The
+// ranking's sort buffer lies past the keys it is filled from and past the
+// shortened graph's fixed arrays, which are written from it; the shortening's
+// scratch (p_scr), in use while the entries are written, past the graph at its
+// largest.
+// total: what the window needs at least (one slot), or with what is staged;
+// past the budget the window does not fit.  ub_glob: pre-BP scratch and slots
+// live in a region of global memory (eight slots), the shortened graph stays
+// in shared memory, total - U is the region's size.
+__host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, int nc, int ns, int nb, unsigned budget,
+                                                    bool ranker, bool lw, bool ub_glob) {
   Layout L{};
   L.rw = (nr + 31) / 32;
   L.cw = (nc + 31) / 32;
   L.sw = (ns + 31) / 32;
-  L.nslots = nslots;
   int sn = 1;
   while (sn < nc) sn <<= 1;
   L.sortn = sn;
+  L.hist = ranker ? 4u : 0u;
+  L.lwe = lw ? 1u : 0u;
   const unsigned nrp = up32(nr), ncp = up32(nc), nsp = up32(ns);
   unsigned o = 0;
   L.sbits = o; o = al16(o + 4u * L.rw);
@@ -256,22 +306,21 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.res_ebits = o; o = al16(o + 4u * L.sw * nb);
   L.red = o; o = al16(o + 16u * 32);
   L.misc = o; o = al16(o + 64u);
+  L.plan = o; o = al16(o + (unsigned)sizeof(SlotPlan));
   L.V = o;
   L.sel = o; o = al16(o + 2u * ns);
-  L.s_rent = o; o = al16(o + 512u * D.srow_quads);
-  L.s_cent = o; o = al16(o + 128u * D.scol_cells);
   L.s_roff = o; o = al16(o + 2u * (L.rw + 1));
   L.s_coff = o; o = al16(o + 2u * (L.sw + 1));
   L.s_cls = o; o = al16(o + 16u);
   L.s_llr = o; o = al16(o + 4u * nsp);
   L.s_vdeg = o; o = al16(o + nsp);
-  L.s_ref = o; o = al16(o + (lw ? 256u * D.srow_quads : 0u));
-  L.s_cef = o; o = al16(o + (lw ? 64u * D.scol_cells : 0u));
   L.s_cperm = o; o = al16(o + 2u * nr);
   L.s_vperm = o; o = al16(o + 2u * ns);
-  L.rowcnt = o; o = al16(o + 4u * (nrp + 1));
-  L.U = o;
-  const unsigned p0 = ub_glob ? 0u : L.V;  // where the pre-BP scratch starts, as an absolute offset
+  L.s_dyn = o;
+  const SlotPlan S = slot_plan(L, D.srow_quads, D.scol_cells, L.rw, L.sw, 0u, ub_glob, 0);  // the largest
+  L.U = S.U;
+  L.b_size = S.b_size;
+  const unsigned p0 = ub_glob ? 0u : L.V;  // where the pre-BP scratch starts
   unsigned u = 0;                          // relative to it
   L.p_post = u; u = al16(u + 4u * (ncp + 1));
   L.p_key = u; u = al16(u + 4u * ncp);
@@ -279,38 +328,38 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.p_par = u; u = al16(u + 8u * L.rw);
   const unsigned own = u;
   unsigned srt = al16(L.p_key + 4u * ncp);
-  if (!ub_glob && srt < L.U - L.V) srt = L.U - L.V;
+  if (!ub_glob && srt < L.s_dyn - L.V) srt = L.s_dyn - L.V;
   if (ub_glob) srt = own;
   L.p_sort = srt;
-  // the keys, later the shortening's scratch: the columns' degrees and the checks' labels
-  const unsigned sb = 8u * sn > 4u * (nsp + nrp) ? 8u * sn : 4u * (nsp + nrp);
-  L.p_end = own > srt + sb ? own : srt + sb;
-  unsigned b = 0;
-  L.b_post = b; b = al16(b + 4u * (nsp + 1));
-  L.b_acc = b; b = al16(b + 4u * ns);
-  L.b_hfl = b; b = al16(b + 1u * ns);
-  L.b_status = b; b = al16(b + 1u * nsp);
-  L.b_cns = b; b = al16(b + 16u * (nrp + 1));
-  L.b_deg = b; b = al16(b + nrp);
-  L.b_sp = b; b = al16(b + 4u * L.rw);
-  L.b_unsat = b; b = al16(b + 4u * L.rw);
-  L.b_hq = b; b = al16(b + (ranker ? 4u * ns : 0u));
-  L.b_size = b;
-  const unsigned slots = b * (unsigned)nslots;
-  unsigned end = ub_glob ? (slots > L.p_end ? slots : L.p_end)
-                         : (L.U + slots > p0 + L.p_end ? L.U + slots : p0 + L.p_end);
-  if (stage) {
-    const unsigned q0 = stage == 2 ? al16(end) - p0 : own;
-    unsigned q = q0;
-    L.q_rent = q; q = al16(q + 512u * D.row_quads);
-    L.q_cent = q; q = al16(q + 128u * D.col_cells);
+  const unsigned sort_end = al16(srt + 8u * sn);
+  // degrees by rank, check labels, check degrees
+  L.p_scr = ub_glob ? srt : L.U - L.V;
+  const unsigned scr_end = al16(L.p_scr + 4u * (nsp + 2u * nrp));
+  L.p_end = own > sort_end ? own : sort_end;
+  if (scr_end > L.p_end) L.p_end = scr_end;
+  if (ub_glob) {
+    L.total = L.U + (8u * L.b_size > L.p_end ? 8u * L.b_size : L.p_end);
+    return L;
+  }
+  unsigned end = L.U + L.b_size > p0 + L.p_end ? L.U + L.b_size : p0 + L.p_end;
+  const unsigned lim = budget > end ? budget : end;
+  unsigned q = own;
+  auto put = [&](unsigned& at, unsigned bytes, unsigned bit) {
+    if (p0 + q + bytes > lim) return;
+    at = q;
+    q = al16(q + bytes);
+    L.pre_stage |= bit;
+  };
+  if (p0 + q + al16(2u * (L.rw + 1)) + al16(2u * (L.cw + 1)) <= lim) {
     L.q_roff = q; q = al16(q + 2u * (L.rw + 1));
     L.q_coff = q; q = al16(q + 2u * (L.cw + 1));
-    L.q_sllr = q; q = al16(q + 4u * ncp);
-    L.pre_stage = 1u;
-    if (p0 + q > end) end = p0 + q;
+    L.pre_stage |= kStageOff;
   }
-  L.total = ub_glob ? L.U + end : end;
+  put(L.q_cent, 128u * D.col_cells, kStageCent);
+  put(L.q_rent, 256u * D.row_quads, kStageRent);
+  put(L.q_sllr, 4u * ncp, kStageLlr);
+  if (p0 + q > end) end = p0 + q;
+  L.total = end;
   return L;
 }
 

@@ -58,6 +58,10 @@ namespace {
 // kShotWarps warps, one warp per decision path, as many as fit in shared
 // memory) and path mode (one CTA of kPathThreads threads per (shot, path)).
 constexpr int kShotWarps = 8;
+// CTAs per SM at most: three take 80 registers a thread.  5000 shots of
+// [[144,12,12]] run 4 % faster so than with two and 128 registers (the paper
+// preset 5 %); with learned weights or a ranker 3 and 6 % slower.
+constexpr int kShotCtas = 3;
 constexpr int kPathThreads = 512;
 constexpr long long kPathModeMaxShots = 64;
 constexpr int kCounters = 8;
@@ -73,6 +77,8 @@ struct WinGpu {
   uint32_t* d_ccobs = nullptr;
   int grid_per_sm = 1;
   int shot_warps = kShotWarps;
+  int wave = 1;  // path slots of a typical shot
+  int ctas = 2;  // CTAs per SM planned
   uint32_t* d_wthr = nullptr;  // window-local sampling thresholds (on first use)
   // union region in global memory (windows too large for shared memory, or
   // launch mode 3): layout, CTAs per SM, and whether the shared-memory
@@ -124,7 +130,7 @@ struct qd_decoder {
   char* d_path_res = nullptr;
   int* d_arrive = nullptr;
   size_t trace_bytes = 0, smem_max = 0;
-  int smem_optin = 0;
+  int smem_optin = 0, smem_sm = 0, smem_reserved = 0;  // dynamic per CTA at most, per SM, taken by each CTA
   bool hist_on = false;  // layouts hold the quantised history (ranker or dump)
   bool lw_on = false;    // layouts keep the shortened edges' full-window ids (learned weights)
   void* d_ranker = nullptr;  // grid-rounded parameters (644 floats), then the 256 B fragments
@@ -257,10 +263,29 @@ qd::SliceDims slice_dims(const qd::WindowHost& h) {
   return qd::SliceDims{h.row_quads, h.col_cells, h.srow_quads, h.scol_cells};
 }
 
+// Dynamic shared memory of one of n CTAs per SM.
+unsigned smem_budget(const qd_decoder* dec, int n) {
+  return (unsigned)std::max(0, std::min(dec->smem_optin, dec->smem_sm / n - dec->smem_reserved)) & ~15u;
+}
+
+// Path slots of a typical shot within L.total: shortened graphs hold fewer and
+// thinner columns than the window's mean (the ranking keeps likely faults;
+// measured 671 to 750 edges for the 432 columns of [[144,12,12]] (3,1)
+// windows, half the mean), their check slices are about half full, two thirds
+// of them non-empty, and half of the columns have degree three or more.
+int typical_slots(const qd::Layout& L, const qd::WindowHost& h, int most) {
+  const double edges = 0.67 * h.n_edges / std::max(1, h.n_cols) * h.n_short;
+  const int nq = std::min(h.srow_quads, (int)(2.0 * edges / 128) + 1);
+  const int cells = std::min(h.scol_cells, (int)(1.4 * edges / 32) + 1);
+  const qd::SlotPlan S =
+      qd::slot_plan(L, nq, cells, std::max(1, (2 * L.rw + 2) / 3), std::max(1, (L.sw + 1) / 2), L.total, false, most);
+  return std::max(1, S.nslots);
+}
+
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   struct Conf {
     qd::Layout L, Lp, Lg;
-    int shot_warps, grid_per_sm, grid_g, pcl;
+    int shot_warps, wave, ctas, grid_per_sm, grid_g, pcl;
     bool fits, path_fits;
   };
   const int optin = dec->smem_optin;
@@ -271,29 +296,36 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     Conf& c = cf[w];
     c.pcl = 1;
     const auto& h = dec->wins[w].h;
-    auto lay = [&](int slots, int stage, bool glob = false) {
-      return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, slots, stage, hist, dec->lw_on,
-                                   glob);
+    auto lay = [&](unsigned budget, bool glob = false) {
+      return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob);
     };
-    // the most resident decision-path warps per SM (slots per CTA x CTAs per
-    // SM); ties to more slots per CTA, then to staging the window graph
-    int best = 0, stage = 0;
-    c.shot_warps = 1;
-    for (int sw = kShotWarps; sw >= 1; --sw)
-      for (int sg = 1; sg >= 0; --sg) {
-        const qd::Layout Ls = lay(sw, sg);
-        if (Ls.total > (unsigned)optin) continue;
-        int blocks = 0;
-        QD_CK(qd::decode_occupancy(0, 32 * sw, Ls.total, &blocks));
-        if (sw * blocks > best) {
-          best = sw * blocks;
-          c.shot_warps = sw;
-          stage = sg;
-        }
+    // CTAs per SM: the most resident decision-path warps (CTAs x slots a
+    // typical shot gets); ties to fewer CTAs, which have room to stage more of
+    // the window graph
+    int best = 0;
+    c.fits = false;
+    c.ctas = 2;
+    c.shot_warps = kShotWarps;
+    c.wave = 1;
+    for (int n = 1; n <= (dec->lw_on || hist ? 2 : kShotCtas); ++n) {
+      const unsigned budget = smem_budget(dec, n);
+      qd::Layout Ls = lay(budget);
+      if (Ls.total > budget) continue;
+      Ls.total = budget;  // the slots take what the budget holds
+      int blocks = 0;
+      QD_CK(qd::decode_occupancy(0, n, 32 * kShotWarps, Ls.total, &blocks));
+      const int sl = typical_slots(Ls, h, kShotWarps);
+      if (std::min(blocks, n) * sl > best) {
+        best = std::min(blocks, n) * sl;
+        c.L = Ls;
+        c.fits = true;
+        c.ctas = n;
+        c.wave = sl;
       }
+    }
     // the union region in global memory: eight path slots, shared memory for
     // the persistent part only, no pre-BP staging (its copies need shared memory)
-    c.Lg = lay(kShotWarps, 0, true);
+    c.Lg = lay(0, true);
     if (c.Lg.U > (unsigned)optin) {
       set_error(std::string(who) + ": window " + std::to_string(w) + " needs " + std::to_string(c.Lg.U) +
                 " B of shared memory even with its path state in global memory (limit " +
@@ -301,13 +333,13 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       return QD_EUNSUPPORTED;
     }
     int bg = 0;
-    QD_CK(qd::decode_occupancy(3, 32 * kShotWarps, c.Lg.U, &bg));
+    QD_CK(qd::decode_occupancy(3, 2, 32 * kShotWarps, c.Lg.U, &bg));
     c.grid_g = std::max(1, bg);
-    c.L = lay(c.shot_warps, stage);
-    c.fits = c.L.total <= (unsigned)optin;
-    if (!c.fits) c.L = c.Lg;  // shot mode streams the path state through L2 / HBM
-    c.Lp = lay(1, 1);
-    if (c.Lp.total > (unsigned)optin) c.Lp = lay(1, 0);
+    if (!c.fits) {  // shot mode streams the path state through L2 / HBM
+      c.L = c.Lg;
+      c.wave = kShotWarps;
+    }
+    c.Lp = lay((unsigned)optin);
     c.path_fits = c.Lp.total <= (unsigned)optin;
     // path mode: the largest cluster (8, 4 or 2 CTAs, at most the number of
     // paths) that can be resident, its CTAs splitting the pre-BP of a shot
@@ -326,7 +358,7 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     }
     smem_max = std::max<size_t>(smem_max, std::max(c.fits ? c.L.total : c.Lg.U, c.path_fits ? c.Lp.total : 0u));
     int blocks = 0;
-    QD_CK(qd::decode_occupancy(c.fits ? 0 : 3, 32 * (c.fits ? c.shot_warps : kShotWarps), c.fits ? c.L.total : c.Lg.U,
+    QD_CK(qd::decode_occupancy(c.fits ? 0 : 3, c.ctas, 32 * c.shot_warps, c.fits ? c.L.total : c.Lg.U,
                                &blocks));
     c.grid_per_sm = std::max(1, blocks);
   }
@@ -339,16 +371,18 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     g.fits = cf[w].fits;
     g.path_fits = cf[w].path_fits;
     g.pcl = cf[w].pcl;
-    g.shot_warps = cf[w].fits ? cf[w].shot_warps : kShotWarps;
+    g.shot_warps = cf[w].shot_warps;
+    g.wave = cf[w].wave;
+    g.ctas = cf[w].ctas;
     g.grid_per_sm = cf[w].grid_per_sm;
   }
   QD_CK_ST(ensure_uscratch(dec, dec->launch_mode == 3));
-  // shot mode's snapshot plans (one per window: the first wave is its slot
-  // count) and one snapshot pool per resident CTA
+  // shot mode's snapshot plans (one per window: the first wave is a typical
+  // shot's slot count) and one snapshot pool per resident CTA
   size_t cta_bytes = 0;
   int ctas = 0;
   for (WinGpu& g : dec->wins) {
-    const ForkPlan F = fork_plan(dec->kp, dec->dmx, std::max(1, g.L.nslots));
+    const ForkPlan F = fork_plan(dec->kp, dec->dmx, g.wave);
     g.fork_on = F.on;
     g.fork_nodes = F.n_nodes;
     if (!F.on) continue;
@@ -652,7 +686,7 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
                       (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0,
                       h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks)),
-                      h.row_quads, h.col_cells, (const uint32_t*)(b + s_re), (const uint32_t*)(b + s_ce),
+                      h.row_quads, h.col_cells, (const uint16_t*)(b + s_re), (const uint32_t*)(b + s_ce),
                       (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
                       (const uint16_t*)(b + s_rw), (const uint16_t*)(b + s_cl),
                       qd::ColClasses{h.cls[0], h.cls[1], h.cls[2], h.cls[3]}, h.wide3, (const uint16_t*)(b + s_rf),
@@ -671,6 +705,8 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     QD_CK(upload(&g.d_ccobs, cc_obs));
   }
   dec->smem_optin = optin;
+  QD_CK(cudaDeviceGetAttribute(&dec->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+  QD_CK(cudaDeviceGetAttribute(&dec->smem_reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
   // the kernels' dynamic shared-memory allowance is the device limit, so
   // decoders of different sizes coexist (the launch asks for what it needs)
   QD_CK(qd::set_decode_smem((size_t)optin));
@@ -805,7 +841,7 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   if (global) {
     QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
     const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * g.grid_g);
-    QD_CK(qd::launch_decode(0, (int)grid, 32 * kShotWarps, g.Lg.U, st, dec->kp, g.dv, g.Lg, det_bits, dw, n_shots,
+    QD_CK(qd::launch_decode(0, 2, (int)grid, 32 * kShotWarps, g.Lg.U, st, dec->kp, g.dv, g.Lg, det_bits, dw, n_shots,
                             win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes, dec->dmx,
                             dec->ns_max, dec->d_work + k, dec->d_counters, nullptr, nullptr, dec->sw_max,
                             dec->d_uscratch, g.Lg.total - g.Lg.U, 1, 1, &fk, &ru));
@@ -813,7 +849,7 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   }
   if (path_mode) {
     const int cps = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
-    QD_CK(qd::launch_decode(1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
+    QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
                             dw, n_shots, win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes,
                             dec->dmx, dec->ns_max, nullptr, dec->d_counters, dec->d_path_res, dec->d_arrive,
                             dec->sw_max, nullptr, 0, cps, g.pcl, nullptr, &ru));
@@ -821,7 +857,7 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   }
   QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
   const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * g.grid_per_sm);
-  QD_CK(qd::launch_decode(0, (int)grid, 32 * g.shot_warps, g.L.total, st, dec->kp, g.dv, g.L, det_bits, dw,
+  QD_CK(qd::launch_decode(0, g.ctas, (int)grid, 32 * g.shot_warps, g.L.total, st, dec->kp, g.dv, g.L, det_bits, dw,
                           n_shots, win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes,
                           dec->dmx, dec->ns_max, dec->d_work + k, dec->d_counters, nullptr, nullptr, dec->sw_max,
                           nullptr, 0, 1, 1, &fk, &ru));
@@ -1093,7 +1129,7 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
       path_mode = false;
     if (path_mode) {
       const int cps = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
-      QD_CK(qd::launch_decode(1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
+      QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
                               dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0, dec->dmx, dec->ns_max, nullptr,
                               dec->d_counters, dec->d_path_res, dec->d_arrive, dec->sw_max, nullptr, 0, cps, g.pcl,
                               nullptr, &ru));
@@ -1104,7 +1140,7 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
       const qd::Layout& L = global ? g.Lg : g.L;
       const long long grid =
           std::min<long long>(n_shots, (long long)dec->sm_count * (global ? g.grid_g : g.grid_per_sm));
-      QD_CK(qd::launch_decode(0, (int)grid, 32 * (global ? kShotWarps : g.shot_warps), global ? L.U : L.total, st,
+      QD_CK(qd::launch_decode(0, g.ctas, (int)grid, 32 * (global ? kShotWarps : g.shot_warps), global ? L.U : L.total, st,
                               dec->kp, g.dv, L, det_bits, dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0,
                               dec->dmx, dec->ns_max, work, dec->d_counters, nullptr, nullptr, dec->sw_max,
                               global ? dec->d_uscratch : nullptr, global ? L.total - L.U : 0, 1, 1, &fk, &ru));
@@ -1144,22 +1180,16 @@ qd_status batch_plan(qd_batch* b, int j, int warps, size_t budget) {
     const qd_decoder* d = b->mem[i];
     if (j >= (int)d->wins.size()) continue;
     const auto& h = d->wins[j].h;
-    int s = warps;
-    for (; s >= 1; --s) {  // as many slots as fit; the window graph staged when that costs none
-      bool fits = false;
-      for (int sg = 1; sg >= 0 && !fits; --sg) {
-        S.L[i] = qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, d->kp.nb, s, sg, d->hist_on,
-                                       d->lw_on, false);
-        fits = qd::al16(S.L[i].total) + 32 <= budget;
-      }
-      if (fits) break;
-    }
-    if (s < 1) {
+    const unsigned room = budget > 64 ? (unsigned)(budget - 32) & ~15u : 0u;
+    S.L[i] = qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, d->kp.nb, room, d->hist_on, d->lw_on,
+                                   false);
+    if (S.L[i].total > room) {
       set_error("qd_batch: member " + std::to_string(i) + " window " + std::to_string(j) + " needs " +
                 std::to_string(S.L[i].total + 32) + " B of shared memory with one path slot (budget " +
                 std::to_string(budget) + ")");
       return QD_EUNSUPPORTED;
     }
+    S.L[i].total = room;  // its slots take what the budget holds
     mx = std::max(mx, S.L[i].total);
   }
   S.q_off = qd::al16(mx);

@@ -29,8 +29,8 @@ struct WindowHost {
   int srow_quads = 0, scol_cells = 0;  // bounds on those of a shortened graph
   int max_row_deg = 0;
   int cls[4] = {0, 0, 0, 0}, wide3 = 0;  // ColClasses; an edge of a column of degree >= 3 past position 31
-  std::vector<uint32_t> s_rent, s_cent;
-  std::vector<uint16_t> s_roff, s_coff, s_row, s_col, s_ref, s_cef;
+  std::vector<uint32_t> s_cent;
+  std::vector<uint16_t> s_rent, s_roff, s_coff, s_row, s_col, s_ref, s_cef;
   std::vector<float> s_llr;
 };
 
@@ -67,9 +67,10 @@ bool build_slices(WindowHost& o);
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max);
 cudaError_t set_decode_smem(size_t bytes);
 // CTAs per SM of the decode kernel: mode 0 shot mode, 1 path mode, 3 shot
-// mode with the union region in global memory.
-cudaError_t decode_occupancy(int mode, int threads, size_t smem, int* blocks);
-cudaError_t launch_decode(int mode, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
+// mode with the union region in global memory; ctas: the CTAs per SM the kernel
+// is compiled for (2, or 3 with fewer registers).
+cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* blocks);
+cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
                           const WinDev& W, const Layout& L, const uint32_t* det, int det_words, long long n,
                           uint32_t* corr, int corr_words, int32_t* status, char* trace, size_t tr_bytes, int dmx,
                           int ns_max, int* work, long long* counters, char* path_res, int* arrive, int sw_max,

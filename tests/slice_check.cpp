@@ -61,32 +61,15 @@ bool check_graph(const qd::WindowHost& h) {
       seen[fe]++;
       const size_t ri = ((size_t)(h.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
       REQ((pos >> 2) < h.s_roff[(r >> 5) + 1] - h.s_roff[r >> 5], "check %d position %d", r, pos);
-      REQ(h.s_rent[ri] == 4u * (uint32_t)l && h.s_ref[ri] == fe, "check %d position %d: other side", r, pos);
+      REQ(h.s_rent[ri] == l && h.s_ref[ri] == fe, "check %d position %d: other side", r, pos);
       REQ(pos < 32 || (h.s_coff[l >> 5] & qd::kWideSlice), "column %d: slice not flagged", l);
     }
   }
   for (int e = 0; e < h.n_edges; ++e) REQ(seen[e] == 1, "edge %d stored %d times", e, seen[e]);
-  for (size_t i = 0; i < h.s_rent.size(); ++i) (h.s_rent[i] < 4u * (uint32_t)nc ? real : dummies)++;
-  for (uint32_t x : h.s_rent)
-    REQ(x < 4u * (uint32_t)nc || x == 4u * (uint32_t)(32 * ncs), "check entry is neither a column nor the dummy");
+  for (size_t i = 0; i < h.s_rent.size(); ++i) (h.s_rent[i] < nc ? real : dummies)++;
+  for (int x : h.s_rent)
+    REQ(x < nc || x == 32 * ncs, "check entry is neither a column nor the dummy");
   REQ((int)real == h.n_edges && real + dummies == (size_t)128 * h.row_quads, "check entries");
-  return true;
-}
-
-// the slices a shortened graph of these window columns takes
-bool check_short(const qd::WindowHost& h, const std::vector<int>& cols) {
-  std::vector<int> cd, rd(h.n_rows, 0);
-  for (int c : cols) {
-    cd.push_back(h.col_ptr[c + 1] - h.col_ptr[c]);
-    for (int e = h.col_ptr[c]; e < h.col_ptr[c + 1]; ++e) rd[h.col_rows[e]]++;
-  }
-  std::sort(cd.rbegin(), cd.rend());
-  std::sort(rd.rbegin(), rd.rend());
-  int cells = 0, quads = 0;
-  for (size_t i = 0; i < cd.size(); i += 32) cells += cd[i];
-  for (size_t i = 0; i < rd.size(); i += 32) quads += (rd[i] + 3) / 4;
-  REQ(cells <= h.scol_cells, "column slices %d > %d", cells, h.scol_cells);
-  REQ(quads <= h.srow_quads, "check slices %d > %d", quads, h.srow_quads);
   return true;
 }
 
@@ -107,51 +90,91 @@ bool disjoint(std::vector<Region> rs, unsigned lo, unsigned hi, const char* part
   return true;
 }
 
-bool check_layout(const qd::WindowHost& h, int nb, int nslots, int stage, bool ranker, bool lw, bool glob) {
+// the slices a shortened graph of these window columns takes
+bool check_short(const qd::WindowHost& h, const std::vector<int>& cols) {
+  std::vector<int> cd, rd(h.n_rows, 0);
+  for (int c : cols) {
+    cd.push_back(h.col_ptr[c + 1] - h.col_ptr[c]);
+    for (int e = h.col_ptr[c]; e < h.col_ptr[c + 1]; ++e) rd[h.col_rows[e]]++;
+  }
+  std::sort(cd.rbegin(), cd.rend());
+  std::sort(rd.rbegin(), rd.rend());
+  int cells = 0, quads = 0;
+  for (size_t i = 0; i < cd.size(); i += 32) cells += cd[i];
+  for (size_t i = 0; i < rd.size(); i += 32) quads += (rd[i] + 3) / 4;
+  REQ(cells <= h.scol_cells, "column slices %d > %d", cells, h.scol_cells);
+  REQ(quads <= h.srow_quads, "check slices %d > %d", quads, h.srow_quads);
+  int rwz = 0, n3 = 0;
+  while (32 * rwz < h.n_rows && rd[32 * rwz] > 0) ++rwz;
+  while (32 * n3 < (int)cd.size() && cd[32 * n3] >= 3) ++n3;
+  for (int m = 0; m < 24; ++m) {  // the shot's own layout
+    const qd::SliceDims D{h.row_quads, h.col_cells, h.srow_quads, h.scol_cells};
+    const unsigned budget = m & 8 ? 76000u : 232000u;
+    const bool ranker = m & 1, lw = m & 2, glob = m & 4;
+    qd::Layout L = qd::make_slice_layout(D, h.n_rows, h.n_cols, h.n_short, 22, budget, ranker, lw, glob);
+    if (!glob && m >= 16 && L.total < budget) L.total = budget;
+    const unsigned end = glob ? L.total - L.U : L.total;
+    const qd::SlotPlan S = qd::slot_plan(L, quads, cells, rwz, n3, end, glob, 8);
+    const unsigned nsp = qd::up32(h.n_short), rw = L.rw;
+    const std::vector<Region> ent = {{"rent", S.rent, 512u * quads}, {"cent", S.cent, 128u * cells},
+                                     {"ref", S.ref, lw ? 256u * quads : 0u}, {"cef", S.cef, lw ? 64u * cells : 0u}};
+    if (!disjoint(ent, L.s_dyn, S.U, "entries")) return false;
+    REQ(S.U <= L.U && S.b_size <= L.b_size, "plan larger than its bound");
+    const std::vector<Region> slot = {{"post", 0, 4u * (nsp + 1)}, {"acc", S.b_acc, 128u * n3},
+                                      {"hfl", S.b_hfl, 32u * n3}, {"status", S.b_status, nsp},
+                                      {"cns", S.b_cns, 16u * (32u * rwz + 1)}, {"deg", S.b_deg, 32u * rw},
+                                      {"sp", S.b_sp, 4u * rw}, {"unsat", S.b_unsat, 4u * rw},
+                                      {"hq", S.b_hq, ranker ? 128u * n3 : 0u}};
+    if (!disjoint(slot, 0, S.b_size, "slot")) return false;
+    REQ(S.b_size % 16u == 0 && S.nslots >= 1 && S.nslots <= 8, "%d slots", S.nslots);
+    REQ((glob ? 0u : S.U) + S.b_size * (unsigned)S.nslots <= end, "slots past the end");
+    REQ(!glob || S.nslots == 8, "%d slots in global memory", S.nslots);
+  }
+  return true;
+}
+
+bool check_layout(const qd::WindowHost& h, int nb, unsigned budget, bool ranker, bool lw, bool glob) {
   const qd::SliceDims D{h.row_quads, h.col_cells, h.srow_quads, h.scol_cells};
   const int nr = h.n_rows, nc = h.n_cols, ns = h.n_short;
-  const qd::Layout L = qd::make_slice_layout(D, nr, nc, ns, nb, nslots, stage, ranker, lw, glob);
+  const qd::Layout L = qd::make_slice_layout(D, nr, nc, ns, nb, budget, ranker, lw, glob);
   const unsigned nrp = qd::up32(nr), ncp = qd::up32(nc), nsp = qd::up32(ns), rw = L.rw;
   REQ(L.total % 16u == 0 && L.U % 16u == 0 && L.V % 16u == 0 && L.b_size % 16u == 0, "alignment");
   const std::vector<Region> keep = {{"sbits", L.sbits, 4u * rw}, {"cbits", L.cbits, 4u * L.cw},
                                     {"res_status", L.res_status, 4u * nb}, {"res_pm", L.res_pm, 8u * nb},
                                     {"res_ebits", L.res_ebits, 4u * L.sw * nb}, {"red", L.red, 512u},
-                                    {"misc", L.misc, 64u}};
+                                    {"misc", L.misc, 64u}, {"plan", L.plan, (unsigned)sizeof(qd::SlotPlan)}};
   if (!disjoint(keep, 0, L.V, "persistent")) return false;
-  std::vector<Region> sg = {{"sel", L.sel, 2u * ns}, {"rent", L.s_rent, 512u * D.srow_quads},
-                            {"cent", L.s_cent, 128u * D.scol_cells}, {"roff", L.s_roff, 2u * (rw + 1)},
+  std::vector<Region> sg = {{"sel", L.sel, 2u * ns}, {"roff", L.s_roff, 2u * (rw + 1)},
                             {"coff", L.s_coff, 2u * (L.sw + 1u)}, {"cls", L.s_cls, 16u}, {"llr", L.s_llr, 4u * nsp},
-                            {"vdeg", L.s_vdeg, nsp}, {"ref", L.s_ref, lw ? 256u * D.srow_quads : 0u},
-                            {"cef", L.s_cef, lw ? 64u * D.scol_cells : 0u}, {"cperm", L.s_cperm, 2u * nr},
-                            {"vperm", L.s_vperm, 2u * ns}, {"rowcnt", L.rowcnt, 4u * (nrp + 1)}};
-  if (!disjoint(sg, L.V, L.U, "shortened graph")) return false;
+                            {"vdeg", L.s_vdeg, nsp}, {"cperm", L.s_cperm, 2u * nr}, {"vperm", L.s_vperm, 2u * ns}};
+  if (!disjoint(sg, L.V, L.s_dyn, "shortened graph")) return false;
+  sg.push_back({"entries", L.s_dyn, L.U - L.s_dyn});
   const unsigned base = glob ? 0u : L.V, hi = glob ? L.total - L.U : L.total;
   std::vector<Region> pre = {{"post", L.p_post + base, 4u * (ncp + 1)}, {"key", L.p_key + base, 4u * ncp},
                              {"cns", L.p_cns + base, 16u * (nrp + 1)}, {"par", L.p_par + base, 8u * rw}};
-  std::vector<Region> st;
-  if (L.pre_stage)
-    st = {{"q_rent", L.q_rent + base, 512u * D.row_quads}, {"q_cent", L.q_cent + base, 128u * D.col_cells},
-          {"q_roff", L.q_roff + base, 2u * (rw + 1)},      {"q_coff", L.q_coff + base, 2u * (L.cw + 1u)},
-          {"q_llr", L.q_sllr + base, 4u * ncp}};
-  pre.insert(pre.end(), st.begin(), st.end());
+  if (L.pre_stage & qd::kStageRent) pre.push_back({"q_rent", L.q_rent + base, 256u * D.row_quads});
+  if (L.pre_stage & qd::kStageCent) pre.push_back({"q_cent", L.q_cent + base, 128u * D.col_cells});
+  if (L.pre_stage & qd::kStageLlr) pre.push_back({"q_llr", L.q_sllr + base, 4u * ncp});
+  if (L.pre_stage & qd::kStageOff) {
+    pre.push_back({"q_roff", L.q_roff + base, 2u * (rw + 1)});
+    pre.push_back({"q_coff", L.q_coff + base, 2u * (L.cw + 1u)});
+  }
+  REQ(!glob || !L.pre_stage, "staging for a union in global memory");
+  REQ(budget < 230000u || glob || L.total > 200000u || L.pre_stage == 15u, "a roomy budget stages everything");
   if (!disjoint(pre, base, hi, "pre-BP")) return false;
   // the sort: filled from the keys; then read while the shortened graph is written
-  const unsigned need = std::max(8u * (unsigned)L.sortn, 4u * (nsp + nrp));
+  const unsigned need = 8u * (unsigned)L.sortn, scr = 4u * (nsp + 2u * nrp);
   REQ(L.sortn >= nc && !(L.sortn & (L.sortn - 1)), "sort size");
-  std::vector<Region> rank = {{"key", L.p_key + base, 4u * ncp}, {"sort", L.p_sort + base, need}};
-  if (stage == 2) rank.insert(rank.end(), st.begin(), st.end());
-  if (!disjoint(rank, base, hi, "ranking")) return false;
+  if (!disjoint({{"key", L.p_key + base, 4u * ncp}, {"sort", L.p_sort + base, need}}, base, hi, "ranking")) return false;
+  if (!disjoint({{"scratch", L.p_scr + base, scr}}, base, hi, "scratch")) return false;
   if (!glob) {
-    sg.push_back({"sort", L.p_sort + base, need});
-    if (stage == 2) sg.insert(sg.end(), st.begin(), st.end());
+    std::vector<Region> a(sg.begin(), sg.end() - 1);
+    a.push_back({"sort", L.p_sort + base, need});
+    if (!disjoint(a, L.V, hi, "selection")) return false;
+    sg.push_back({"scratch", L.p_scr + base, scr});
     if (!disjoint(sg, L.V, hi, "shortening")) return false;
   }
-  const std::vector<Region> slot = {{"post", L.b_post, 4u * (nsp + 1)}, {"acc", L.b_acc, 4u * ns},
-                                    {"hfl", L.b_hfl, 1u * ns}, {"status", L.b_status, nsp},
-                                    {"cns", L.b_cns, 16u * (nrp + 1)}, {"deg", L.b_deg, nrp}, {"sp", L.b_sp, 4u * rw},
-                                    {"unsat", L.b_unsat, 4u * rw}, {"hq", L.b_hq, ranker ? 4u * ns : 0u}};
-  if (!disjoint(slot, 0, L.b_size, "slot")) return false;
-  REQ((glob ? 0u : L.U) + L.b_size * (unsigned)nslots <= hi, "slots past the end");
+  REQ((glob ? 0u : L.U) + L.b_size * (glob ? 8u : 1u) <= hi, "slots past the end");
   return true;
 }
 }  // namespace
@@ -183,9 +206,9 @@ int main(int argc, char** argv) {
                          [&](int a, int b) { return h.col_rows[h.col_ptr[a]] < h.col_rows[h.col_ptr[b]]; });
     }
     for (int nb : {1, 22, 47})
-      for (int slots : {1, 3, 8})
-        for (int m = 0; m < 24; ++m)
-          if (!check_layout(h, nb, slots, m >> 3, m & 1, m & 2, m & 4)) return 1;
+      for (unsigned budget : {0u, 76000u, 115000u, 232000u})
+        for (int m = 0; m < 8; ++m)
+          if (!check_layout(h, nb, budget, m & 1, m & 2, m & 4)) return 1;
   }
   std::printf("ok\n");
   return 0;
