@@ -584,4 +584,45 @@ bool build_slices(WindowHost& o) {
   return true;
 }
 
+WmsHost build_wms(const WindowHost& h) {
+  WmsHost o;
+  const int nr = h.n_rows, nc = h.n_cols, nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
+  std::vector<uint16_t> clab(nc), rlab(nr);
+  for (int l = 0; l < nc; ++l) clab[h.s_col[l]] = (uint16_t)l;
+  for (int l = 0; l < nr; ++l) rlab[h.s_row[l]] = (uint16_t)l;
+  o.row.assign(32 * nrs, 0);
+  std::copy(h.s_row.begin(), h.s_row.end(), o.row.begin());
+  o.col = h.s_col;
+  o.coff.resize(ncs + 1);
+  for (int q = 0; q <= ncs; ++q) o.coff[q] = (uint16_t)(h.s_coff[q] & (kWideSlice - 1));
+  o.roff.assign(nrs + 1, 0);
+  for (int q = 0; q < nrs; ++q) {
+    const int j = h.s_row[32 * q];
+    o.roff[q + 1] = (uint16_t)(o.roff[q] + h.row_ptr[j + 1] - h.row_ptr[j]);
+  }
+  const size_t nre = (size_t)32 * o.roff[nrs], cells = (size_t)32 * h.col_cells;
+  o.rcell.assign(nre, (uint16_t)cells);  // the dummy cell, column and check
+  o.rcol.assign(nre, (uint16_t)(32 * ncs));
+  o.reid.assign(nre, 0);
+  o.cent.assign(cells, (uint32_t)(32 * nrs) << 16);
+  o.ceid.assign(cells, 0);
+  for (int l = 0; l < nc; ++l)  // a dummy takes its column's first edge's weight
+    for (int u = 0; u < o.coff[(l >> 5) + 1] - o.coff[l >> 5]; ++u)
+      o.ceid[(size_t)(o.coff[l >> 5] + u) * 32 + (l & 31)] = h.col_ptr[h.s_col[l]];
+  for (int j = 0; j < nr; ++j) {
+    const int r = rlab[j];
+    for (int q = h.row_ptr[j]; q < h.row_ptr[j + 1]; ++q) {
+      const int e = (int)(h.row_ent[q] & 0xFFFF), c = (int)(h.row_ent[q] >> 16), l = clab[c], pos = q - h.row_ptr[j];
+      const size_t ri = (size_t)(o.roff[r >> 5] + pos) * 32 + (r & 31);
+      const size_t ci = (size_t)(o.coff[l >> 5] + (e - h.col_ptr[c])) * 32 + (l & 31);
+      o.rcell[ri] = (uint16_t)ci;
+      o.rcol[ri] = (uint16_t)l;
+      o.reid[ri] = (uint16_t)e;
+      o.cent[ci] = ((uint32_t)r << 16) | (uint32_t)pos;
+      o.ceid[ci] = (uint16_t)e;
+    }
+  }
+  return o;
+}
+
 }  // namespace qd

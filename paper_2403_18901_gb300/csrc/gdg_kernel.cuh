@@ -164,6 +164,21 @@ struct WmsGraph {
   float clip;
 };
 
+// The same in slices for the training kernel (labels of WinDev; every check's
+// entries in ascending edge order, which decides ties and the order of the
+// loss's products; check slices exactly as wide as their first check).
+struct WmsSlices {
+  int nr, nc, ne, rw, T;
+  int nrs, ncs, col_cells;       // check and column slices, column entries per lane
+  const uint16_t *roff, *coff;   // slice starts, in entries per lane
+  const uint16_t *rcell, *rcol, *reid;  // check entry: the edge's column cell, column label, edge id
+  const uint32_t* cent;          // column entry: check label << 16 | position
+  const uint16_t* ceid;          // its edge id
+  const float* llr;              // by column label
+  const uint16_t *row, *col;     // label -> window row (0 for the padding), window column
+  float clip;
+};
+
 // Compressed state of one check node: its two smallest |input| (bounded by the
 // clip), each negated when the sign parity xor s_j is 1 and, in the plain
 // decoder, multiplied by alpha; sg: the inputs' signs, position p at bit 31 - p
@@ -176,7 +191,7 @@ struct __align__(16) CNState {
 // Most entries a check may have.  A detector of these codes' circuits touches
 // at most 35 columns: the fault classes of a round are the same for every
 // choice of A and B (three terms each), and coinciding terms only merge them.
-constexpr int kMaxRowDeg = 58;
+constexpr int kMaxRowDeg = 51;
 // Flag of a column slice's start (s_coff) when some edge of it has a position
 // past 31 and its sign is in the second word.
 constexpr uint16_t kWideSlice = 0x8000;

@@ -13,16 +13,30 @@
 //   P(check j odd) = (1 - prod_{i in N(j)} tanh(post_i / 2)) / 2,
 //   loss = mean_j BCE(P_j, s_j),
 // since 1 - 2 sigma(-x) = tanh(x / 2).
-// Backward: the adjoint of the unrolled iterations, recomputed segment by
-// segment from checkpoints of v2c every `ckpt` iterations.  A min-sum check
-// sends each edge the magnitude of one other edge (the smallest, or the second
-// smallest for the edge holding the smallest), so its gradient flows to at
-// most two inputs; derivatives of sign() and of a saturated clip are zero.
-// FP32 throughout; tanhf / logf are CUDA's.
+// Backward: the adjoint of the unrolled iterations.  A min-sum check sends each
+// edge the magnitude of one other edge (the smallest, or the second smallest
+// for the edge holding the smallest), so its gradient flows to at most two
+// inputs; derivatives of sign() and of a saturated clip are zero.  Everything
+// the adjoint of iteration t needs of the forward pass is in the checks'
+// records of iterations t and t + 1: the two smallest magnitudes and their
+// positions and the messages' signs; an input is within the clip exactly when
+// its magnitude is below it.  So the forward pass keeps 16 bytes per check and
+// iteration in global scratch and nothing is computed twice.  The gradient
+// into the inputs of an iteration is non-zero at two edges per check only:
+// those are scattered to the columns, and an edge whose column got nothing has
+// no weight gradient (but in the last iteration, where every column has one).
+// FP32 throughout (the loss is summed in FP64); tanhf / logf are CUDA's.
+//
+// What bounds it: issue and latency of the checks' serial passes over their 35
+// inputs; 40 KB of shared memory a CTA for [[144,12,12]] (3,1) windows keeps
+// four CTAs of 8 warps on an SM.  With the messages of both directions and
+// their gradients in shared memory (123 KB, one CTA per SM), checkpoints and
+// two recomputations, 1024 samples of 25 iterations took 10.0 ms.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "gdg_kernel.cuh"
 
@@ -30,236 +44,252 @@ namespace qd {
 
 namespace lrn {
 
+constexpr unsigned FULL = 0xffffffffu;
 __device__ __forceinline__ float clipf(float x, float c) { return x > c ? c : (x < -c ? -c : x); }
 
-struct CheckMins {
+// A check's record of one iteration: its two smallest |v2c|; sg, pw: the signs
+// of the messages it sends, position p at bit 31 - p of sg (p < 32) or bit
+// 63 - p of pw; pw also holds (bit 12) whether the inputs' own signs are those
+// inverted, and the positions of the two smallest inputs (bits 11..6 the
+// second, 5..0 the first).
+struct __align__(16) WRec {
   float m1, m2;
-  int e1, e2;
-  uint32_t neg;
+  uint32_t sg, pw;
 };
-
-// two smallest |v| over the check's edges and their edge ids, sign parity
-__device__ __forceinline__ CheckMins check_mins(const WmsGraph& G, const float* v, int j) {
-  CheckMins c{CUDART_INF_F, CUDART_INF_F, -1, -1, 0u};
-  for (int q = G.row_ptr[j]; q < G.row_ptr[j + 1]; ++q) {
-    const int e = (int)(G.row_ent[q] & 0xFFFFu);
-    const float x = v[e];
-    const float a = fabsf(x);
-    if (a < c.m1) {
-      c.m2 = c.m1;
-      c.e2 = c.e1;
-      c.m1 = a;
-      c.e1 = e;
-    } else if (a < c.m2) {
-      c.m2 = a;
-      c.e2 = e;
-    }
-    c.neg ^= (x < 0.0f);
-  }
-  return c;
+__device__ __forceinline__ uint32_t rec_sign(const WRec& r, int p) {  // of position p's message, at bit 31
+  return ((p < 32 ? r.sg : r.pw) << (p & 31)) & 0x80000000u;
+}
+__device__ __forceinline__ float with_sign(float x, uint32_t s) {
+  return __uint_as_float(__float_as_uint(x) ^ s);
 }
 
-struct Smem {
-  float *v2c, *c2v, *gv, *post, *gpost, *tmp;
-  uint32_t* sb;
-};
-
-// one flooding iteration t (1-based) of weighted min-sum; v2c -> c2v, post, v2c
-__device__ void wms_iteration(const WmsGraph& G, const float* w, const Smem& S, int t) {
-  const int tid = threadIdx.x, NT = blockDim.x;
-  const float* wt = w + (size_t)(t - 1) * G.ne;
-  for (int j = tid; j < G.nr; j += NT) {
-    const CheckMins c = check_mins(G, S.v2c, j);
-    const uint32_t sj = (S.sb[j >> 5] >> (j & 31)) & 1u;
-    for (int q = G.row_ptr[j]; q < G.row_ptr[j + 1]; ++q) {
-      const int e = (int)(G.row_ent[q] & 0xFFFFu);
-      const float m = (e == c.e1) ? c.m2 : c.m1;
-      const uint32_t sg = c.neg ^ (S.v2c[e] < 0.0f) ^ sj;
-      const float mag = __fmul_rn(wt[e], m);
-      S.c2v[e] = sg ? -mag : mag;
+// Check pass of one check by one lane: the record of its inputs v2c.
+__device__ __forceinline__ WRec check_forward(const uint16_t* cell, int n, const float* v2c, uint32_t sj) {
+  float m1 = CUDART_INF_F, m2 = CUDART_INF_F;
+  uint32_t p1 = 0u, p2 = 0u, sg[2] = {0u, 0u};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {  // 32 positions to a word
+    const int u0 = 32 * h, u1 = min(n, u0 + 32);
+    uint32_t s = 0u;
+#pragma unroll 4
+    for (int u = u0; u < u1; ++u) {
+      const float x = v2c[cell[32 * u]];  // (a dummy is +inf)
+      const float a = fabsf(x);
+      const bool l1 = a < m1, l2 = a < m2;  // the first of equal magnitudes stays
+      p2 = l1 ? p1 : (l2 ? (uint32_t)u : p2);
+      p1 = l1 ? (uint32_t)u : p1;
+      m2 = fminf(m2, fmaxf(m1, a));
+      m1 = fminf(m1, a);
+      s = s + s + (x < 0.0f ? 1u : 0u);
     }
+    if (u1 > u0) sg[h] = s << ((32 - (u1 - u0)) & 31);
   }
-  __syncthreads();
-  for (int i = tid; i < G.nc; i += NT) {
-    float p = G.llr[i];
-    for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) p = __fadd_rn(p, S.c2v[e]);
-    S.post[i] = p;
-    for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) S.v2c[e] = clipf(__fsub_rn(p, S.c2v[e]), G.clip);
-  }
-  __syncthreads();
+  const uint32_t par = (__popc(sg[0]) + __popc(sg[1]) + sj) & 1u;
+  const uint32_t all = 0u - par;  // message sign = parity xor s_j xor the own sign
+  return WRec{m1, m2, sg[0] ^ all, ((sg[1] ^ all) & 0xFFFFE000u) | (par << 12) | (p2 << 6) | p1};
 }
 
-// soft-syndrome BCE of the posteriors in S.post; writes dLoss/dpost to S.gpost
-// (scaled by 1/nr) and returns the loss (thread 0)
-__device__ float soft_syndrome_loss(const WmsGraph& G, const Smem& S, bool want_grad) {
-  const int tid = threadIdx.x, NT = blockDim.x;
-  __shared__ float red[32];
-  float lsum = 0.0f;
-  // per check: product of tanh(post/2) over its variables; per-edge exclusive products in tmp
-  for (int j = tid; j < G.nr; j += NT) {
-    const int qb = G.row_ptr[j], qe = G.row_ptr[j + 1];
-    float prod = 1.0f;
-    for (int q = qb; q < qe; ++q) {
-      const int i = (int)(G.row_ent[q] >> 16);
-      const int e = (int)(G.row_ent[q] & 0xFFFFu);
-      S.tmp[e] = prod;  // prefix product (exclusive)
-      prod *= tanhf(0.5f * S.post[i]);
-    }
-    const uint32_t sj = (S.sb[j >> 5] >> (j & 31)) & 1u;
-    float P = 0.5f * (1.0f - prod);
-    const float eps = 1e-7f;
-    const bool clamped = P < eps || P > 1.0f - eps;
-    P = fminf(fmaxf(P, eps), 1.0f - eps);
-    lsum += sj ? -logf(P) : -logf(1.0f - P);
-    if (want_grad) {
-      // dL/dprod = dL/dP * dP/dprod, with dP/dprod = -1/2
-      const float dP = clamped ? 0.0f : (sj ? -1.0f / P : 1.0f / (1.0f - P)) / (float)G.nr;
-      const float dprod = -0.5f * dP;
-      float suf = 1.0f;
-      for (int q = qe - 1; q >= qb; --q) {
-        const int i = (int)(G.row_ent[q] >> 16);
-        const int e = (int)(G.row_ent[q] & 0xFFFFu);
-        const float th = tanhf(0.5f * S.post[i]);
-        S.tmp[e] = dprod * S.tmp[e] * suf * 0.5f * (1.0f - th * th);  // contribution to dL/dpost_i
-        suf *= th;
-      }
-    }
-  }
-  __syncthreads();
-  if (want_grad)
-    for (int i = tid; i < G.nc; i += NT) {
-      float g = 0.0f;
-      for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) g += S.tmp[e];
-      S.gpost[i] = g;
-    }
-  // block sum of the loss
-  for (int off = 16; off; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-  if ((tid & 31) == 0) red[tid >> 5] = lsum;
-  __syncthreads();
-  float tot = 0.0f;
-  if (tid == 0)
-    for (int x = 0; x < (NT >> 5); ++x) tot += red[x];
-  __syncthreads();
-  return tot / (float)G.nr;
+// Message of Eq. (1) with weight w for the edge at position p.
+__device__ __forceinline__ float message(const WRec& r, uint32_t p, float w) {
+  const float m = (r.pw & 63u) == p ? r.m2 : r.m1;
+  return with_sign(__fmul_rn(w, m), rec_sign(r, (int)p));
 }
 
-__global__ void __launch_bounds__(256) wms_kernel(WmsGraph G, const float* __restrict__ w,
-                                                  const uint32_t* __restrict__ synd, long long n,
-                                                  int backward, float grad_scale, float* __restrict__ grad_w,
-                                                  float* __restrict__ loss_out, float* __restrict__ post_out,
-                                                  float* __restrict__ scratch, size_t scratch_per_cta,
-                                                  int* __restrict__ work) {
+// v2c by cell and its dummy, or the adjoint's three buffers by column
+__host__ __device__ inline int wms_v2c_floats(int col_cells, int ncs) {
+  const int a = 32 * col_cells + 32, b = 3 * (32 * ncs + 32);
+  return a > b ? a : b;
+}
+
+__global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const float* __restrict__ w,
+                                                     const uint32_t* __restrict__ synd, long long n, int backward,
+                                                     float grad_scale, float* __restrict__ grad_w,
+                                                     float* __restrict__ loss_out, float* __restrict__ post_out,
+                                                     WRec* __restrict__ scratch, int* __restrict__ work) {
   extern __shared__ __align__(16) char smem[];
-  const int tid = threadIdx.x, NT = blockDim.x;
-  Smem S;
-  S.v2c = (float*)smem;
-  S.c2v = S.v2c + G.ne;
-  S.gv = S.c2v + G.ne;
-  S.tmp = S.gv + G.ne;
-  S.post = S.tmp + G.ne;
-  S.gpost = S.post + G.nc;
-  S.sb = (uint32_t*)(S.gpost + G.nc);
-  __shared__ long long sh_sample;
-  float* ck = scratch + (size_t)blockIdx.x * scratch_per_cta;  // checkpoints [nseg][ne]
-  const int nseg = (G.T + G.ckpt - 1) / G.ckpt;
-  float* segbuf = ck + (size_t)nseg * G.ne;  // inputs of a segment's iterations [ckpt][ne]
+  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
+  const int nrp = 32 * G.nrs, ncp = 32 * G.ncs, cells = 32 * G.col_cells;
+  float* v2c = (float*)smem;                       // by column cell; [cells] = +inf
+  float* post = v2c + wms_v2c_floats(G.col_cells, G.ncs);  // by column label
+  WRec* rec = (WRec*)(post + ncp);                 // this iteration's, [nrp] = zero (the dummy check)
+  uint32_t* sb = (uint32_t*)(rec + nrp + 1);       // window syndrome by row
+  double* red = (double*)(sb + ((G.rw + 3) & ~3));  // [32]
+  // the adjoint's column gradients: three buffers in v2c's place, [ncp] the dummy column's
+  auto gp = [&](int t) { return v2c + (t % 3) * (ncp + 32); };
+  int* sh_sample = (int*)(red + 32);
+  WRec* hist = scratch + (size_t)blockIdx.x * G.T * nrp;  // records by iteration
   while (true) {
     __syncthreads();
-    if (tid == 0) sh_sample = atomicAdd(work, 1);
+    if (tid == 0) *sh_sample = atomicAdd(work, 1);
     __syncthreads();
-    const long long s = sh_sample;
-    if (s >= n) break;
-    for (int x = tid; x < G.rw; x += NT) S.sb[x] = synd[(size_t)s * G.rw + x];
-    for (int i = tid; i < G.nc; i += NT)
-      for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) S.v2c[e] = G.llr[i];  // t = 0
-    __syncthreads();
-    // ---- forward with checkpoints ----
-    for (int t = 1; t <= G.T; ++t) {
-      if (backward && (t - 1) % G.ckpt == 0) {
-        float* dst = ck + (size_t)((t - 1) / G.ckpt) * G.ne;
-        for (int e = tid; e < G.ne; e += NT) dst[e] = S.v2c[e];
-      }
-      wms_iteration(G, w, S, t);
+    const long long smp = *sh_sample;
+    if (smp >= n) break;
+    for (int x = tid; x < G.rw; x += NT) sb[x] = synd[(size_t)smp * G.rw + x];
+    for (int s = warp; s < G.ncs; s += nw) {  // t = 0: v2c = Lambda
+      const float l = G.llr[32 * s + lane];
+      for (int c = G.coff[s]; c < G.coff[s + 1]; ++c) v2c[32 * c + lane] = l;
     }
-    const float L = soft_syndrome_loss(G, S, backward != 0);
-    if (tid == 0 && loss_out) loss_out[s] = L;
-    if (post_out)
-      for (int i = tid; i < G.nc; i += NT) post_out[(size_t)s * G.nc + i] = S.post[i];
-    if (!backward) continue;
-    // ---- adjoint, segment by segment ----
-    for (int e = tid; e < G.ne; e += NT) S.gv[e] = 0.0f;  // v2c^(T) does not enter the loss
+    if (tid == 0) {
+      v2c[cells] = CUDART_INF_F;
+      rec[nrp] = WRec{0.0f, 0.0f, 0u, 0u};
+    }
     __syncthreads();
-    for (int seg = nseg - 1; seg >= 0; --seg) {
-      const int t0 = seg * G.ckpt, t1 = min(G.T, t0 + G.ckpt);
-      // recompute the segment, keeping each iteration's input messages
-      for (int e = tid; e < G.ne; e += NT) S.v2c[e] = ck[(size_t)seg * G.ne + e];
-      __syncthreads();
-      for (int t = t0 + 1; t <= t1; ++t) {
-        float* dst = segbuf + (size_t)(t - t0 - 1) * G.ne;
-        for (int e = tid; e < G.ne; e += NT) dst[e] = S.v2c[e];
-        __syncthreads();
-        if (t < t1) wms_iteration(G, w, S, t);
+    // ---- forward ----
+    for (int t = 1; t <= G.T; ++t) {
+      for (int s = warp; s < G.nrs; s += nw) {
+        const int r0 = G.roff[s], l = 32 * s + lane;
+        const int j = G.row[l];  // window row (0 for the padding, whose inputs are dummies)
+        const WRec r = check_forward(G.rcell + 32 * r0 + lane, G.roff[s + 1] - r0, v2c, (sb[j >> 5] >> (j & 31)) & 1u);
+        rec[l] = r;
+        if (backward) hist[(size_t)(t - 1) * nrp + l] = r;
       }
-      for (int t = t1; t > t0; --t) {
-        const float* vin = segbuf + (size_t)(t - t0 - 1) * G.ne;  // v2c^(t-1)
-        const float* wt = w + (size_t)(t - 1) * G.ne;
-        // recompute c2v^(t), post^(t) from vin
-        for (int e = tid; e < G.ne; e += NT) S.v2c[e] = vin[e];
-        __syncthreads();
-        for (int j = tid; j < G.nr; j += NT) {
-          const CheckMins c = check_mins(G, S.v2c, j);
-          const uint32_t sj = (S.sb[j >> 5] >> (j & 31)) & 1u;
-          for (int q = G.row_ptr[j]; q < G.row_ptr[j + 1]; ++q) {
-            const int e = (int)(G.row_ent[q] & 0xFFFFu);
-            const float m = (e == c.e1) ? c.m2 : c.m1;
-            const uint32_t sg = c.neg ^ (S.v2c[e] < 0.0f) ^ sj;
-            const float mag = __fmul_rn(wt[e], m);
-            S.c2v[e] = sg ? -mag : mag;
+      __syncthreads();
+      const float* wt = w + (size_t)(t - 1) * G.ne;
+      for (int s = warp; s < G.ncs; s += nw) {
+        const int c0 = G.coff[s], d = G.coff[s + 1] - c0;
+        float p = G.llr[32 * s + lane];
+        auto column = [&](auto cnt) {  // the messages stay in registers
+          constexpr int N = decltype(cnt)::value;
+          float m[N];
+#pragma unroll
+          for (int u = 0; u < N; ++u) {
+            const int c = 32 * (c0 + u) + lane;
+            const uint32_t e = G.cent[c];
+            m[u] = message(rec[e >> 16], e & 0xFFFFu, wt[G.ceid[c]]);
           }
+#pragma unroll
+          for (int u = 0; u < N; ++u) p = __fadd_rn(p, m[u]);  // ascending check order
+#pragma unroll
+          for (int u = 0; u < N; ++u) v2c[32 * (c0 + u) + lane] = clipf(__fsub_rn(p, m[u]), G.clip);
+        };
+        switch (d) {
+          case 1: column(std::integral_constant<int, 1>{}); break;
+          case 2: column(std::integral_constant<int, 2>{}); break;
+          case 3: column(std::integral_constant<int, 3>{}); break;
+          case 4: column(std::integral_constant<int, 4>{}); break;
+          case 5: column(std::integral_constant<int, 5>{}); break;
+          case 6: column(std::integral_constant<int, 6>{}); break;
+          default:
+            for (int pass = 0; pass < 2; ++pass)
+              for (int u = 0; u < d; ++u) {
+                const int c = 32 * (c0 + u) + lane;
+                const uint32_t e = G.cent[c];
+                const float m = message(rec[e >> 16], e & 0xFFFFu, wt[G.ceid[c]]);
+                if (pass == 0) p = __fadd_rn(p, m);
+                else v2c[c] = clipf(__fsub_rn(p, m), G.clip);
+              }
         }
-        __syncthreads();
-        // VN adjoint: v2c^(t)[e] = clip(post - c2v[e]), post = Lambda + sum c2v
-        for (int i = tid; i < G.nc; i += NT) {
-          float p = G.llr[i];
-          for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) p = __fadd_rn(p, S.c2v[e]);
-          float gp = (t == G.T) ? S.gpost[i] : 0.0f;
-          for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) {
-            const float x = __fsub_rn(p, S.c2v[e]);
-            if (x > -G.clip && x < G.clip) gp += S.gv[e];
-          }
-          for (int e = G.col_ptr[i]; e < G.col_ptr[i + 1]; ++e) {
-            const float x = __fsub_rn(p, S.c2v[e]);
-            const float pass = (x > -G.clip && x < G.clip) ? S.gv[e] : 0.0f;
-            S.tmp[e] = gp - pass;  // dL/dc2v[e]
-          }
+        if (t == G.T) post[32 * s + lane] = p;
+      }
+      __syncthreads();
+    }
+    if (post_out)
+      for (int l = tid; l < G.nc; l += NT) post_out[(size_t)smp * G.nc + G.col[l]] = post[l];
+    // ---- soft-syndrome BCE; dLoss/dpost by edge in v2c's place ----
+    __syncthreads();
+    for (int l = tid; l < ncp; l += NT) post[l] = tanhf(0.5f * post[l]);
+    __syncthreads();
+    double lsum = 0.0;
+    for (int s = warp; s < G.nrs; s += nw) {
+      const int r0 = G.roff[s], d = G.roff[s + 1] - r0, l = 32 * s + lane;
+      if (l >= G.nr) continue;
+      const uint16_t *cell = G.rcell + 32 * r0 + lane, *col = G.rcol + 32 * r0 + lane;
+      float prod = 1.0f;
+      for (int u = 0; u < d; ++u) {
+        if (col[32 * u] >= G.nc) break;  // (dummies come last)
+        v2c[cell[32 * u]] = prod;        // prefix product (exclusive)
+        prod *= post[col[32 * u]];
+      }
+      const int j = G.row[l];
+      const uint32_t sj = (sb[j >> 5] >> (j & 31)) & 1u;
+      float P = 0.5f * (1.0f - prod);
+      const float eps = 1e-7f;
+      const bool clamped = P < eps || P > 1.0f - eps;
+      P = fminf(fmaxf(P, eps), 1.0f - eps);
+      lsum += (double)(sj ? -logf(P) : -logf(1.0f - P));
+      if (backward) {
+        // dL/dprod = dL/dP * dP/dprod, with dP/dprod = -1/2
+        const float dP = clamped ? 0.0f : (sj ? -1.0f / P : 1.0f / (1.0f - P)) / (float)G.nr;
+        const float dprod = -0.5f * dP;
+        float suf = 1.0f;
+        for (int u = d - 1; u >= 0; --u) {
+          if (col[32 * u] >= G.nc) continue;
+          const float th = post[col[32 * u]];
+          const int c = cell[32 * u];
+          v2c[c] = dprod * v2c[c] * suf * 0.5f * (1.0f - th * th);  // contribution to dL/dpost_i
+          suf *= th;
         }
-        __syncthreads();
-        // CN adjoint: weight gradient and routing to the argmin inputs
-        for (int j = tid; j < G.nr; j += NT) {
-          const CheckMins c = check_mins(G, S.v2c, j);
-          const uint32_t sj = (S.sb[j >> 5] >> (j & 31)) & 1u;
-          float g1 = 0.0f, g2 = 0.0f;  // into |v2c[e1]| and |v2c[e2]|
-          for (int q = G.row_ptr[j]; q < G.row_ptr[j + 1]; ++q) {
-            const int e = (int)(G.row_ent[q] & 0xFFFFu);
-            const bool own = (e == c.e1);
-            const float m = own ? c.m2 : c.m1;
-            const uint32_t sg = c.neg ^ (S.v2c[e] < 0.0f) ^ sj;
-            const float sgn = sg ? -1.0f : 1.0f;
-            const float gc = S.tmp[e];
-            atomicAdd(&grad_w[(size_t)(t - 1) * G.ne + e], grad_scale * gc * sgn * m);
-            const float gm = gc * sgn * wt[e];
-            if (own) g2 += gm;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1) lsum += __shfl_xor_sync(FULL, lsum, off);
+    if (lane == 0) red[warp] = lsum;
+    __syncthreads();
+    if (tid == 0 && loss_out) {
+      double tot = 0.0;
+      for (int x = 0; x < nw; ++x) tot += red[x];
+      loss_out[smp] = (float)(tot / (double)G.nr);
+    }
+    if (!backward) continue;
+    for (int s = warp; s < G.ncs; s += nw) {  // dL/dpost (its contributions sit in v2c's place)
+      float g = 0.0f;
+      for (int c = G.coff[s]; c < G.coff[s + 1]; ++c)
+        if ((int)(G.cent[32 * c + lane] >> 16) < nrp) g += v2c[32 * c + lane];
+      post[32 * s + lane] = g;
+    }
+    __syncthreads();
+    // buffer T mod 3 takes dL/dpost, the others are zero
+    for (int l = tid; l < ncp + 32; l += NT) {
+      gp(G.T)[l] = l < ncp ? post[l] : 0.0f;
+      gp(G.T + 1)[l] = 0.0f;
+      gp(G.T + 2)[l] = 0.0f;
+    }
+    // ---- adjoint: iteration t reads buffer t mod 3, the gradient into its
+    // posteriors, and leaves each check's two input gradients in its record's
+    // place: gA, gB; the columns; the positions and whether the clip passes ----
+    for (int t = G.T; t >= 1; --t) {
+      float* cur = gp(t);
+      if (t < G.T)
+        for (int s = warp; s < G.nrs; s += nw) {
+          const WRec a = rec[32 * s + lane];
+          if (a.pw & 0x1000u) atomicAdd(&cur[a.sg & 0xFFFFu], a.m1);
+          if (a.pw & 0x2000u) atomicAdd(&cur[a.sg >> 16], a.m2);
+        }
+      __syncthreads();
+      float* old = gp(t + 1);  // read in the iteration before, next written two iterations on
+      for (int l = tid; l < ncp; l += NT) old[l] = 0.0f;
+      const float* wt = w + (size_t)(t - 1) * G.ne;
+      float* gw = grad_w + (size_t)(t - 1) * G.ne;
+      for (int s = warp; s < G.nrs; s += nw) {
+        const int r0 = G.roff[s], d = G.roff[s + 1] - r0, l = 32 * s + lane;
+        const uint16_t *col = G.rcol + 32 * r0 + lane, *eid = G.reid + 32 * r0 + lane;
+        const WRec r = hist[(size_t)(t - 1) * nrp + l];
+        WRec a{0.0f, 0.0f, 0u, 0u};
+        if (t < G.T) a = rec[l];
+        const int q1 = a.pw & 0x1000u ? (int)(a.pw & 63u) : -1, q2 = a.pw & 0x2000u ? (int)((a.pw >> 6) & 63u) : -1;
+        const int p1 = (int)(r.pw & 63u), p2 = (int)((r.pw >> 6) & 63u);
+        float g1 = 0.0f, g2 = 0.0f;  // into |v2c| at p1 and p2
+#pragma unroll 4
+        for (int u = 0; u < d; ++u) {
+          float gc = cur[col[32 * u]];  // dL/dc2v: the column's less the edge's own
+          if (u == q1) gc -= a.m1;
+          if (u == q2) gc -= a.m2;
+          if (gc != 0.0f) {
+            const int e = eid[32 * u];
+            const uint32_t sg = rec_sign(r, u);
+            atomicAdd(&gw[e], with_sign(grad_scale * gc, sg) * (u == p1 ? r.m2 : r.m1));
+            const float gm = with_sign(gc, sg) * wt[e];
+            if (u == p1) g2 += gm;
             else g1 += gm;
           }
-          for (int q = G.row_ptr[j]; q < G.row_ptr[j + 1]; ++q) {
-            const int e = (int)(G.row_ent[q] & 0xFFFFu);
-            float g = 0.0f;
-            if (e == c.e1) g = g1 * (S.v2c[e] < 0.0f ? -1.0f : 1.0f);
-            else if (e == c.e2) g = g2 * (S.v2c[e] < 0.0f ? -1.0f : 1.0f);
-            S.gv[e] = g;  // dL/dv2c^(t-1)[e]
-          }
         }
-        __syncthreads();
+        // gradient into the inputs at p1 and p2: times their own signs
+        const uint32_t par = (r.pw << 19) & 0x80000000u;
+        a.m1 = with_sign(g1, rec_sign(r, p1) ^ par);
+        a.m2 = with_sign(g2, rec_sign(r, p2) ^ par);
+        a.sg = (uint32_t)col[32 * min(p1, max(d - 1, 0))] | ((uint32_t)col[32 * min(p2, max(d - 1, 0))] << 16);
+        a.pw = (r.pw & 0xFFFu) | (r.m1 < G.clip ? 0x1000u : 0u) | (r.m2 < G.clip ? 0x2000u : 0u);
+        rec[l] = a;
       }
     }
   }
@@ -347,12 +377,14 @@ __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, 
 
 }  // namespace lrn
 
-size_t wms_smem_bytes(int ne, int nc, int rw) { return sizeof(float) * (4 * (size_t)ne + 2 * (size_t)nc) + 4 * (size_t)rw; }
+size_t wms_window_bytes(int ne, int nc, int rw) { return sizeof(float) * (4 * (size_t)ne + 2 * (size_t)nc) + 4 * (size_t)rw; }
 
-size_t wms_scratch_per_cta(int ne, int T, int ckpt) {
-  const int nseg = (T + ckpt - 1) / ckpt;
-  return (size_t)(nseg + ckpt) * ne;  // floats
+size_t wms_smem_bytes(const WmsSlices& G) {
+  return sizeof(float) * ((size_t)lrn::wms_v2c_floats(G.col_cells, G.ncs) + 32 * G.ncs) +
+         sizeof(lrn::WRec) * (32 * (size_t)G.nrs + 1) + 4 * (size_t)((G.rw + 3) & ~3) + 32 * sizeof(double) + 16;
 }
+
+size_t wms_scratch_per_cta(const WmsSlices& G) { return sizeof(lrn::WRec) * 32 * (size_t)G.nrs * G.T; }
 
 cudaError_t wms_set_smem(size_t bytes) {
   return cudaFuncSetAttribute(lrn::wms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -362,11 +394,11 @@ cudaError_t wms_occupancy(size_t smem, int* blocks) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, lrn::wms_kernel, 256, smem);
 }
 
-cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsGraph& G, const float* w, const uint32_t* synd,
+cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsSlices& G, const float* w, const uint32_t* synd,
                        long long n, int backward, float grad_scale, float* grad_w, float* loss, float* post,
-                       float* scratch, size_t scratch_per_cta, int* work) {
-  lrn::wms_kernel<<<grid, 256, smem, st>>>(G, w, synd, n, backward, grad_scale, grad_w, loss, post, scratch,
-                                           scratch_per_cta, work);
+                       char* scratch, int* work) {
+  lrn::wms_kernel<<<grid, 256, smem, st>>>(G, w, synd, n, backward, grad_scale, grad_w, loss, post,
+                                           (lrn::WRec*)scratch, work);
   return cudaGetLastError();
 }
 

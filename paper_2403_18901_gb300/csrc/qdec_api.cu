@@ -71,7 +71,7 @@ struct WinGpu {
   qd::WinDev dv{};
   qd::Layout L{};   // shot mode
   qd::Layout Lp{};  // path mode
-  void* d_graph = nullptr;
+  char* d_graph = nullptr;
   int* d_ccptr = nullptr;  // committed columns: CSR of their global detector ids
   int* d_ccdet = nullptr;
   uint32_t* d_ccobs = nullptr;
@@ -106,12 +106,32 @@ cudaError_t upload(T** dst, const std::vector<T>& v) {
   return e;
 }
 
+// Arrays in one allocation: every array starts on a 16-byte boundary and is
+// padded to a multiple of 16 bytes, as the kernels' bulk (TMA) copies into
+// shared memory require.
+struct Blob {
+  std::vector<char> bytes;
+  template <class T>
+  size_t put(const std::vector<T>& v) {
+    const size_t o = bytes.size(), n = v.size() * sizeof(T);
+    bytes.resize((o + n + 15) & ~(size_t)15);
+    if (n) memcpy(bytes.data() + o, v.data(), n);
+    return o;
+  }
+  cudaError_t upload(char** dst) const {
+    const cudaError_t e = cudaMalloc((void**)dst, std::max<size_t>(bytes.size(), 16));
+    return e != cudaSuccess ? e : cudaMemcpy(*dst, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+  }
+};
+
 qd_status ensure_device(const qd_dem* d) {
   if (d->d_thr) return QD_OK;
   QD_CK(upload(&d->d_cptr, d->h.col_ptr));
   QD_CK(upload(&d->d_cdet, d->h.col_dets));
   QD_CK(upload(&d->d_cobs, d->h.col_obs));
-  QD_CK(upload(&d->d_thr, d->h.col_thr));
+  std::vector<uint32_t> thr(d->h.col_thr);  // in fours, the last ones padded with columns that never fire
+  thr.resize((thr.size() + 3) & ~(size_t)3, 0u);
+  QD_CK(upload(&d->d_thr, thr));
   return QD_OK;
 }
 
@@ -665,23 +685,14 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     dec->ns_max = std::max(dec->ns_max, h.n_short);
     dec->sw_max = std::max(dec->sw_max, (h.n_short + 31) / 32);
     if (!qd::build_slices(g.h)) return QD_EUNSUPPORTED;
-    // graph arrays in one allocation: every array starts on a 16-byte boundary
-    // and is padded to a multiple of 16 bytes, as the kernels' bulk (TMA)
-    // copies into shared memory require
-    std::vector<char> blob;
-    auto put = [&](const auto& v) {
-      const size_t o = blob.size(), n = v.size() * sizeof(v[0]);
-      blob.resize((o + n + 15) & ~(size_t)15);
-      if (n) memcpy(blob.data() + o, v.data(), n);
-      return o;
-    };
+    Blob blob;
+    auto put = [&](const auto& v) { return blob.put(v); };
     const size_t o_cp = put(h.col_ptr), o_cr = put(h.col_rows), o_rp = put(h.row_ptr), o_re = put(h.row_ent),
                  o_ll = put(h.llr), s_re = put(h.s_rent), s_ce = put(h.s_cent), s_ro = put(h.s_roff),
                  s_co = put(h.s_coff), s_ll = put(h.s_llr), s_rw = put(h.s_row), s_cl = put(h.s_col),
                  s_rf = put(h.s_ref), s_cf = put(h.s_cef);
-    QD_CK(cudaMalloc(&g.d_graph, std::max<size_t>(blob.size(), 16)));
-    QD_CK(cudaMemcpy(g.d_graph, blob.data(), blob.size(), cudaMemcpyHostToDevice));
-    char* b = (char*)g.d_graph;
+    QD_CK(blob.upload(&g.d_graph));
+    char* b = g.d_graph;
     g.dv = qd::WinDev{h.n_rows, h.n_cols, h.n_edges, h.row0, h.n_short, h.short_edges_max, h.n_rows / h.n_blocks,
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
                       (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0,
@@ -1419,10 +1430,11 @@ qd_status qd_batch_autotune(qd_batch* b, int step, uint32_t* const* det_bits, co
 // Learned weighted min-sum: training on window samples.
 struct qd_wms {
   qd::WmsGraph G{};
+  qd::WmsSlices S{};
   int k = 0;
   uint32_t* d_thr = nullptr;
-  float* d_scratch = nullptr;
-  size_t scratch_per_cta = 0;
+  char* d_graph = nullptr;    // the arrays of S
+  char* d_scratch = nullptr;  // check records by iteration, per CTA
   int* d_work = nullptr;
   int grid = 0;
   size_t smem = 0;
@@ -1443,20 +1455,30 @@ qd_status qd_wms_create(const qd_decoder* dec, int k, int T, int ckpt, qd_wms** 
   std::vector<uint32_t> thr(g.h.n_cols);
   for (int c = 0; c < g.h.n_cols; ++c) thr[c] = dec->dem->h.col_thr[g.h.gcols[c]];
   QD_CK(upload(&m->d_thr, thr));
-  m->smem = qd::wms_smem_bytes(m->G.ne, m->G.nc, m->G.rw);
   int optin = 0, dev = 0;
   QD_CK(cudaGetDevice(&dev));
   QD_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (m->smem > (size_t)optin) {
+  if (qd::wms_window_bytes(m->G.ne, m->G.nc, m->G.rw) > (size_t)optin) {
     set_error("qd_wms_create: window too large for shared memory");
     return QD_EUNSUPPORTED;
   }
-  QD_CK(qd::wms_set_smem(m->smem));
+  const qd::WmsHost H = qd::build_wms(g.h);
+  Blob b;
+  const size_t o_ro = b.put(H.roff), o_co = b.put(H.coff), o_rc = b.put(H.rcell), o_rl = b.put(H.rcol),
+               o_re = b.put(H.reid), o_ce = b.put(H.cent), o_ei = b.put(H.ceid), o_ll = b.put(g.h.s_llr),
+               o_rw = b.put(H.row), o_cl = b.put(H.col);
+  QD_CK(b.upload(&m->d_graph));
+  auto u16 = [&](size_t o) { return (const uint16_t*)(m->d_graph + o); };
+  m->S = qd::WmsSlices{m->G.nr, m->G.nc, m->G.ne, m->G.rw, T, (int)H.roff.size() - 1, (int)H.coff.size() - 1,
+                       g.h.col_cells, u16(o_ro), u16(o_co), u16(o_rc), u16(o_rl), u16(o_re),
+                       (const uint32_t*)(m->d_graph + o_ce), u16(o_ei), (const float*)(m->d_graph + o_ll), u16(o_rw),
+                       u16(o_cl), dec->P.clip};
+  m->smem = qd::wms_smem_bytes(m->S);
+  QD_CK(qd::wms_set_smem((size_t)optin));  // the device limit: contexts of different sizes coexist
   int blocks = 0;
   QD_CK(qd::wms_occupancy(m->smem, &blocks));
   m->grid = dec->sm_count * std::max(1, blocks);
-  m->scratch_per_cta = qd::wms_scratch_per_cta(m->G.ne, T, ckpt);
-  QD_CK(cudaMalloc(&m->d_scratch, sizeof(float) * m->scratch_per_cta * m->grid));
+  QD_CK(cudaMalloc(&m->d_scratch, qd::wms_scratch_per_cta(m->S) * m->grid));
   QD_CK(cudaMalloc(&m->d_work, sizeof(int)));
   *out = m.release();
   return QD_OK;
@@ -1465,6 +1487,7 @@ qd_status qd_wms_create(const qd_decoder* dec, int k, int T, int ckpt, qd_wms** 
 qd_status qd_wms_destroy(qd_wms* m) {
   if (!m) return QD_OK;
   cudaFree(m->d_thr);
+  cudaFree(m->d_graph);
   cudaFree(m->d_scratch);
   cudaFree(m->d_work);
   delete m;
@@ -1496,8 +1519,8 @@ static qd_status wms_run(qd_wms* m, const float* w, const uint32_t* synd, int64_
   cudaStream_t st = (cudaStream_t)stream;
   QD_CK(cudaMemsetAsync(m->d_work, 0, sizeof(int), st));
   const int grid = (int)std::min<long long>(n, m->grid);
-  QD_CK(qd::launch_wms(st, grid, m->smem, m->G, w, synd, n, backward, scale, grad_w, loss, post, m->d_scratch,
-                       m->scratch_per_cta, m->d_work));
+  QD_CK(qd::launch_wms(st, grid, m->smem, m->S, w, synd, n, backward, scale, grad_w, loss, post, m->d_scratch,
+                       m->d_work));
   return QD_OK;
 }
 

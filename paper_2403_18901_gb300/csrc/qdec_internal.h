@@ -49,6 +49,7 @@ struct KParams;
 struct WinDev;
 struct Layout;
 struct WmsGraph;
+struct WmsSlices;
 struct RankRec;
 struct ForkDev;
 struct ReuseDev;
@@ -60,6 +61,13 @@ bool build_dem_code_capacity(const qd_bb_code& code, double p_data, double p_syn
 int n_windows(const DemHost& d, int W, int F);
 // merge: the H_1 merge of Sec. III (0 none, 1 equal restrictions, 2 identity)
 bool build_window(const DemHost& d, int W, int F, int k, bool shorten, WindowHost& out, int merge = 0);
+
+// The training kernel's arrays (WmsSlices) of a window whose slices are built.
+struct WmsHost {
+  std::vector<uint16_t> roff, coff, rcell, rcol, reid, ceid, row, col;
+  std::vector<uint32_t> cent;
+};
+WmsHost build_wms(const WindowHost& h);
 
 // The graph in slices (s_* of WindowHost) and the bounds for its shortened graphs.
 bool build_slices(WindowHost& o);
@@ -111,13 +119,16 @@ cudaError_t launch_commit(cudaStream_t st, int n_commit, const int* cptr, const 
 cudaError_t launch_evaluate(cudaStream_t st, const uint32_t* pred, const uint32_t* obs,
                             const uint32_t* resid, long long n, uint32_t* fail, long long* n_fail);
 
-size_t wms_smem_bytes(int ne, int nc, int rw);
-size_t wms_scratch_per_cta(int ne, int T, int ckpt);
+// A window trains when this many bytes fit a CTA's shared memory (messages and
+// gradients of both directions; the kernel itself takes less, wms_smem_bytes).
+size_t wms_window_bytes(int ne, int nc, int rw);
+size_t wms_smem_bytes(const WmsSlices& G);
+size_t wms_scratch_per_cta(const WmsSlices& G);  // bytes
 cudaError_t wms_set_smem(size_t bytes);
 cudaError_t wms_occupancy(size_t smem, int* blocks);
-cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsGraph& G, const float* w, const uint32_t* synd,
+cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsSlices& G, const float* w, const uint32_t* synd,
                        long long n, int backward, float grad_scale, float* grad_w, float* loss, float* post,
-                       float* scratch, size_t scratch_per_cta, int* work);
+                       char* scratch, int* work);
 cudaError_t launch_wms_sample(cudaStream_t st, const WmsGraph& G, const uint32_t* thr, unsigned long long seed,
                               unsigned long long off, long long n, unsigned domain, uint32_t* synd, uint32_t* det,
                               int det_words, int row0, uint32_t* fault, int cw);
