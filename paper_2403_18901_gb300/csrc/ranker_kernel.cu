@@ -28,6 +28,14 @@
 // sums per warp, then per CTA in shared memory, then add them to `grad`
 // (FP32 atomics, so the summation order and the last bits vary between
 // runs).
+//
+// What bounds the tensor-core kernel at a training minibatch (65536 records,
+// 2.4 MB): not the arithmetic but the fixed parts around it -- the launch, the
+// parameters' rounding, the reduction of 641 sums.  So one CTA of 16 warps per
+// SM takes several tiles a warp, and its warps leave their sums side by side
+// in shared memory.  512 CTAs of 8 warps with one tile each, 156 registers
+// (one CTA per SM) and shared-memory atomics (compare-and-swap loops for
+// floats) took 35.5 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -39,6 +47,7 @@ namespace rk {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kNP = 641;
+constexpr int kTcWarps = 16;  // warps of a tensor-core CTA
 
 __device__ __forceinline__ float grid_round(float x, float scale, float lim) {
   float v = rintf(x * scale);
@@ -156,15 +165,15 @@ __device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a1,
 // Tensor-core forward / backward on grid-rounded parameters (see the top of
 // the file).  Lane l of a warp: g = l / 4 (record g and g + 8 of the tile in
 // layer 1), q = l % 4 (features 2q, 2q + 1; hidden units 8t + 2q + c).
-__global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict__ params,
+__global__ void __launch_bounds__(32 * kTcWarps) ranker_tc_kernel(const float* __restrict__ params,
                                                         const RankRec* __restrict__ recs,
                                                         const uint8_t* __restrict__ labels, long long n,
                                                         float pos_weight, float scale, float* __restrict__ grad,
                                                         float* __restrict__ loss, float* __restrict__ score) {
   __shared__ float P[kNP];
-  __shared__ float G[kNP];
-  __shared__ uint32_t Bw1[8 * 32];  // B fragments of W1 for hidden units 8t..8t+7
-  const int tid = threadIdx.x, lane = tid & 31;
+  __shared__ float G[kTcWarps][kNP];  // each warp's sums
+  __shared__ uint32_t Bw1[8 * 32];    // B fragments of W1 for hidden units 8t..8t+7
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, q = lane & 3;
   for (int i = tid; i < kNP; i += blockDim.x) {
     float v = params[i];
@@ -172,7 +181,6 @@ __global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict_
     else if (i < 576) v = grid_round(v, 128.0f, 65536.0f);
     else if (i < 640) v = grid_round(v, 64.0f, 128.0f);
     P[i] = v;
-    G[i] = 0.0f;
   }
   __syncthreads();
   for (int i = tid; i < 256; i += blockDim.x) {
@@ -187,22 +195,26 @@ __global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict_
   float gb1[16] = {}, gw2[16] = {};  // units 8t + 2q + c at index 2t + c
   float gb2 = 0.0f;
   const long long n_tiles = (n + 15) / 16;
-  const long long wid = ((long long)blockIdx.x * blockDim.x + tid) >> 5;
-  const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  // tiles go to the CTAs in turn, so that few records still use many SMs
+  const long long wid = (long long)warp * gridDim.x + blockIdx.x;
+  const long long nw = (long long)gridDim.x * kTcWarps;
+  float2 xa, xb;
+  float ya = 0.0f, yb = 0.0f;
+  auto load = [&](long long tile) {
+    const long long r = tile * 16 + g;
+    if (grad || loss) {
+      ya = r < n ? (float)labels[r] : 0.0f;
+      yb = r + 8 < n ? (float)labels[r + 8] : 0.0f;
+    }
+    xa = r < n ? *(const float2*)&recs[r].x[2 * q] : make_float2(0.0f, 0.0f);
+    xb = r + 8 < n ? *(const float2*)&recs[r + 8].x[2 * q] : make_float2(0.0f, 0.0f);
+  };
+  if (wid < n_tiles) load(wid);
   for (long long tile = wid; tile < n_tiles; tile += nw) {
     const long long r0 = tile * 16 + g, r1 = r0 + 8;
     const bool v0 = r0 < n, v1 = r1 < n;
-    float x00 = 0.0f, x01 = 0.0f, x10 = 0.0f, x11 = 0.0f;
-    if (v0) {
-      const float2 x = *(const float2*)&recs[r0].x[2 * q];
-      x00 = x.x;
-      x01 = x.y;
-    }
-    if (v1) {
-      const float2 x = *(const float2*)&recs[r1].x[2 * q];
-      x10 = x.x;
-      x11 = x.y;
-    }
+    const float x00 = xa.x, x01 = xa.y, x10 = xb.x, x11 = xb.y, y0 = ya, y1 = yb;
+    if (tile + nw < n_tiles) load(tile + nw);  // the next tile's inputs, in flight during this one
     const uint32_t a0 = bf16x2_rn(x00, x01), a1 = bf16x2_rn(x10, x11);  // features are BF16 numbers
     // ---- layer 1 (exact) and layer 2 in the decoder's order ----
     float acc[8][4];
@@ -239,7 +251,7 @@ __global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict_
     for (int h = 0; h < 2; ++h) {
       const bool act = h ? v1 : v0;
       const long long r = h ? r1 : r0;
-      const float y = act ? (float)labels[r] : 0.0f;
+      const float y = h ? y1 : y0;
       const float wy = y > 0.5f ? pos_weight : 1.0f;
       const float zz = z[h];
       if (act && loss && q == 0) loss[r] = wy * (fmaxf(zz, 0.0f) + log1pf(expf(-fabsf(zz))) - y * zz);
@@ -248,34 +260,35 @@ __global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict_
     }
     if (!grad) continue;
     if (q == 0) gb2 += dz[0] + dz[1];
-    // ---- dH, dL/db1, dL/dW2; dH^T in BF16 hi / lo parts, transposed ----
-    uint32_t ah[8][2], al[8][2];  // [t][half]: (unit 8t + g, records 8 half + 2q, + 1) after the transpose
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const int u = 8 * t + 2 * q;
-      float dh[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float a = acc[t][e];
-        dh[e] = a > 0.0f ? dz[e >> 1] * W2[u + (e & 1)] : 0.0f;
-        gw2[2 * t + (e & 1)] += dz[e >> 1] * fmaxf(a, 0.0f);
-      }
-      gb1[2 * t] += dh[0] + dh[2];
-      gb1[2 * t + 1] += dh[1] + dh[3];
-      const uint32_t h0 = bf16x2_rn(dh[0], dh[1]), h1 = bf16x2_rn(dh[2], dh[3]);
-      const uint32_t l0 = bf16x2_rn(dh[0] - bf16_lo_f(h0), dh[1] - bf16_hi_f(h0));
-      const uint32_t l1 = bf16x2_rn(dh[2] - bf16_lo_f(h1), dh[3] - bf16_hi_f(h1));
-      ah[t][0] = transpose8x8(h0);
-      ah[t][1] = transpose8x8(h1);
-      al[t][0] = transpose8x8(l0);
-      al[t][1] = transpose8x8(l1);
-    }
-    // X of the tile as B (records x features): (records 2q, 2q + 1 | +8, feature g)
+    // ---- dH, dL/db1, dL/dW2; dH^T in BF16 hi / lo parts, transposed:
+    // (unit 8t + g, records 8 half + 2q, + 1); X of the tile as B (records x
+    // features): (records 2q, 2q + 1 | +8, feature g) ----
     const uint32_t xb0 = transpose8x8(a0), xb1 = transpose8x8(a1);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      mma_k16(gw1[m], ah[2 * m][0], ah[2 * m + 1][0], ah[2 * m][1], ah[2 * m + 1][1], xb0, xb1);
-      mma_k16(gw1[m], al[2 * m][0], al[2 * m + 1][0], al[2 * m][1], al[2 * m + 1][1], xb0, xb1);
+      uint32_t ah[2][2], al[2][2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int t = 2 * m + h, u = 8 * t + 2 * q;
+        float dh[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float a = acc[t][e];
+          dh[e] = a > 0.0f ? dz[e >> 1] * W2[u + (e & 1)] : 0.0f;
+          gw2[2 * t + (e & 1)] += dz[e >> 1] * fmaxf(a, 0.0f);
+        }
+        gb1[2 * t] += dh[0] + dh[2];
+        gb1[2 * t + 1] += dh[1] + dh[3];
+        const uint32_t h0 = bf16x2_rn(dh[0], dh[1]), h1 = bf16x2_rn(dh[2], dh[3]);
+        const uint32_t l0 = bf16x2_rn(dh[0] - bf16_lo_f(h0), dh[1] - bf16_hi_f(h0));
+        const uint32_t l1 = bf16x2_rn(dh[2] - bf16_lo_f(h1), dh[3] - bf16_hi_f(h1));
+        ah[h][0] = transpose8x8(h0);
+        ah[h][1] = transpose8x8(h1);
+        al[h][0] = transpose8x8(l0);
+        al[h][1] = transpose8x8(l1);
+      }
+      mma_k16(gw1[m], ah[0][0], ah[1][0], ah[0][1], ah[1][1], xb0, xb1);
+      mma_k16(gw1[m], al[0][0], al[1][0], al[0][1], al[1][1], xb0, xb1);
     }
   }
   if (!grad) return;
@@ -290,22 +303,27 @@ __global__ void __launch_bounds__(256) ranker_tc_kernel(const float* __restrict_
     }
     if (g == 0) {
       const int u = 8 * (i >> 1) + 2 * q + (i & 1);
-      atomicAdd(&G[512 + u], a);
-      atomicAdd(&G[576 + u], b);
+      G[warp][512 + u] = a;
+      G[warp][576 + u] = b;
     }
   }
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    atomicAdd(&G[(16 * m + g) * 8 + 2 * q], gw1[m][0]);
-    atomicAdd(&G[(16 * m + g) * 8 + 2 * q + 1], gw1[m][1]);
-    atomicAdd(&G[(16 * m + g + 8) * 8 + 2 * q], gw1[m][2]);
-    atomicAdd(&G[(16 * m + g + 8) * 8 + 2 * q + 1], gw1[m][3]);
+    float* w1 = &G[warp][(16 * m + g) * 8 + 2 * q];
+    w1[0] = gw1[m][0];
+    w1[1] = gw1[m][1];
+    w1[64] = gw1[m][2];
+    w1[65] = gw1[m][3];
   }
   gb2 = warp_sum(gb2);
-  if (lane == 0) atomicAdd(&G[640], gb2);
+  if (lane == 0) G[warp][640] = gb2;
   __syncthreads();
-  for (int i = tid; i < kNP; i += blockDim.x)
-    if (G[i] != 0.0f) atomicAdd(&grad[i], G[i]);
+  for (int i = tid; i < kNP; i += blockDim.x) {
+    float v = 0.0f;
+#pragma unroll
+    for (int x = 0; x < kTcWarps; ++x) v += G[x][i];
+    if (v != 0.0f) atomicAdd(&grad[i], v);
+  }
 }
 
 }  // namespace rk
@@ -319,9 +337,9 @@ cudaError_t launch_ranker(cudaStream_t st, const float* params, const RankRec* r
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   if (quantize) {  // tensor cores: 16 records per warp
-    const long long want = (n + 127) / 128;
-    const int grid = (int)(want < 4LL * sms ? want : 4LL * sms);
-    rk::ranker_tc_kernel<<<grid, 256, 0, st>>>(params, recs, labels, n, pos_weight, scale, grad, loss, score);
+    const long long tiles = (n + 15) / 16;
+    const int grid = (int)(tiles < sms ? tiles : sms);
+    rk::ranker_tc_kernel<<<grid, 32 * rk::kTcWarps, 0, st>>>(params, recs, labels, n, pos_weight, scale, grad, loss, score);
     return cudaGetLastError();
   }
   const long long want = (n + 255) / 256;
