@@ -474,23 +474,13 @@ __device__ __forceinline__ uint32_t ordkey(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-__host__ __device__ inline int lanes_per_check(int threads, int n_checks) {
-  int t = 1;
-#pragma unroll 1
-  while (t < 8 && 2 * t * n_checks <= threads) t <<= 1;
-  return t;
-}
-
-// Lanes per check of a decision path run by a whole CTA: the most (<= 8) that
-// keep the check pass within two rounds of threads / lanes checks.  Checks
-// come in descending degree, so the first round holds the heavy ones, whose
-// edges the extra lanes split (measured on [[144]] (3,1) windows, 216 checks,
-// 512 threads: 1.18 / 1.02 / 1.19 ms per window with 2 / 4 / 8 lanes).
+// Lanes per check of a decision path run by a whole CTA: two where that takes
+// one round of threads / lanes checks, else one.  A shortened graph's checks
+// have a few entries each, so more lanes mostly add reduction steps (one
+// [[144,12,12]] shot, 11 windows: 8.0 ms with up to eight lanes in two rounds,
+// 6.9 ms with four in one, 6.7 ms with two).
 __host__ __device__ inline int path_lanes_per_check(int threads, int n_checks) {
-  int t = 1;
-#pragma unroll 1
-  while (t < 8 && 2 * (threads / (2 * t)) >= n_checks) t <<= 1;
-  return t;
+  return threads / 2 >= n_checks ? 2 : 1;
 }
 
 // lexicographic (value, index) minimum over the warp
