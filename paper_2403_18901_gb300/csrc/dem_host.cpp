@@ -503,11 +503,113 @@ bool build_window(const DemHost& d, int W, int F, int k, bool shorten, WindowHos
   return true;
 }
 
+namespace {
+// Columns of one degree in an order that spreads the variable pass's gathers
+// over the shared-memory banks: a 16-byte check record is read by eight lanes
+// at a time, from eight bank groups (check label mod 8).  Lane by lane the
+// next column is the one, of the first `look` left, that adds the fewest
+// second visits to a bank group (a record read by two lanes is one visit).
+void spread_columns(const WindowHost& o, const std::vector<uint16_t>& rlab, uint16_t* cols, int n, int deg, int lane0) {
+  constexpr int kLook = 96;
+  std::vector<uint16_t> left(cols, cols + n);
+  std::vector<std::vector<int>> seen(deg);  // per entry: the eight lanes' check labels
+  size_t head = 0;
+  for (int i = 0; i < n; ++i) {
+    if ((lane0 + i) % 8 == 0)
+      for (auto& v : seen) v.clear();
+    size_t pick = head;
+    int best = 1 << 30;
+    for (size_t x = head; x < left.size() && x < head + kLook && best > 0; ++x) {
+      int cost = 0;
+      for (int u = 0; u < deg; ++u) {
+        const int r = rlab[o.col_rows[o.col_ptr[left[x]] + u]];
+        int same = 0;
+        for (int v : seen[u]) {
+          if (v == r) {
+            same = 0;
+            break;
+          }
+          same += (v & 7) == (r & 7);
+        }
+        cost += same;
+      }
+      if (cost < best) {
+        best = cost;
+        pick = x;
+      }
+    }
+    const uint16_t c = left[pick];
+    for (size_t x = pick; x > head; --x) left[x] = left[x - 1];
+    ++head;
+    for (int u = 0; u < deg; ++u) seen[u].push_back(rlab[o.col_rows[o.col_ptr[c] + u]]);
+    cols[i] = c;
+  }
+}
+
+// Positions for the entries of a slice's 32 checks (lab[lane]: their column
+// labels) that spread the check pass's posterior gathers over the 32 banks
+// (column label mod 32): position by position a matching of lanes to banks,
+// each lane to the bank of one of its entries left; a lane without a free bank
+// takes the entry whose bank has the fewest readers.  pos[lane][i]: the
+// position of the lane's i-th entry.
+void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::vector<std::vector<int>>& pos) {
+  const int n = (int)lab.size();
+  std::vector<std::vector<int>> left(n);  // entry indexes
+  int most = 0;
+  for (int l = 0; l < n; ++l) {
+    for (int i = 0; i < (int)lab[l].size(); ++i) left[l].push_back(i);
+    most = std::max(most, (int)lab[l].size());
+  }
+  for (int u = 0; u < most; ++u) {
+    int lane_of[32], mine[32];
+    std::fill(lane_of, lane_of + 32, -1);
+    std::fill(mine, mine + 32, -1);
+    std::vector<char> tried(32);
+    // augmenting paths; lanes with the most entries left choose first
+    auto match = [&](auto&& self, int l) -> bool {
+      for (int i : left[l]) {
+        const int b = lab[l][i] & 31;
+        if (tried[b]) continue;
+        tried[b] = 1;
+        if (lane_of[b] < 0 || self(self, lane_of[b])) {
+          lane_of[b] = l;
+          mine[l] = i;
+          return true;
+        }
+      }
+      return false;
+    };
+    std::vector<int> order;
+    for (int l = 0; l < n; ++l)
+      if (!left[l].empty()) order.push_back(l);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
+    int load[32] = {};
+    for (int l : order) {
+      std::fill(tried.begin(), tried.end(), 0);
+      match(match, l);
+    }
+    for (int l : order)
+      if (mine[l] >= 0) load[lab[l][mine[l]] & 31]++;
+    for (int l : order) {
+      if (mine[l] < 0) {
+        for (int i : left[l])
+          if (mine[l] < 0 || load[lab[l][i] & 31] < load[lab[l][mine[l]] & 31]) mine[l] = i;
+        load[lab[l][mine[l]] & 31]++;
+      }
+      pos[l][mine[l]] = first + u;
+      left[l].erase(std::find(left[l].begin(), left[l].end(), mine[l]));
+    }
+  }
+}
+}  // namespace
+
 // The window's graph in slices (see gdg_kernel.cuh): labels by descending
-// degree, ties by window row / column; a check's entries in ascending column
-// label, so that the positions past 31 (checks of 35 entries) fall to columns
-// of the lowest degrees and only their slices look at the second sign word; a
+// degree, checks' ties by window row, columns' as spread_columns says; a
+// check's first 32 entries, and those past them, as spread_positions says; a
 // column's entries in ascending window row, the order of the sum of Eq. (2).
+// The order of a check's entries and of the columns changes no value.  Counted
+// for an interior [[144,12,12]] (3,1) window: 520 -> 342 wavefronts for the 228
+// gathers of a check pass, 1536 -> 987 for the 840 of a variable pass.
 bool build_slices(WindowHost& o) {
   const int nr = o.n_rows, nc = o.n_cols;
   const int nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
@@ -521,6 +623,10 @@ bool build_slices(WindowHost& o) {
   std::stable_sort(o.s_col.begin(), o.s_col.end(), [&](uint16_t a, uint16_t b) { return cdeg(a) > cdeg(b); });
   std::vector<uint16_t> rlab(nr);
   for (int l = 0; l < nr; ++l) rlab[o.s_row[l]] = (uint16_t)l;
+  for (int a = 0, b; a < nc; a = b) {
+    for (b = a + 1; b < nc && cdeg(o.s_col[b]) == cdeg(o.s_col[a]);) ++b;
+    spread_columns(o, rlab, o.s_col.data() + a, b - a, cdeg(o.s_col[a]), a);
+  }
   o.max_row_deg = nr ? rdeg(o.s_row[0]) : 0;
   const int max_col_deg = nc ? cdeg(o.s_col[0]) : 0;
   if (o.max_row_deg > kMaxRowDeg) {
@@ -538,26 +644,43 @@ bool build_slices(WindowHost& o) {
   o.s_ref.assign(o.s_rent.size(), 0);
   o.s_cef.assign(o.s_cent.size(), 0);
   o.s_llr.assign((size_t)32 * ncs, 0.0f);
-  std::vector<int> fill(nr, 0);
-  std::vector<char> wide(ncs, 0);
+  std::vector<int> pos_of(o.n_edges, 0);
+  {
+    std::vector<std::vector<std::pair<int, int>>> ents(nr);  // by check label: (column label, edge)
+    for (int l = 0; l < nc; ++l)
+      for (int e = o.col_ptr[o.s_col[l]]; e < o.col_ptr[o.s_col[l] + 1]; ++e)
+        ents[rlab[o.col_rows[e]]].push_back({l, e});
+    for (int q = 0; q < nrs; ++q)
+      for (int h = 0; h < 2; ++h) {  // the first 32 entries, then the rest
+        const int n = std::min(32, nr - 32 * q);
+        std::vector<std::vector<int>> lab(n), pos(n);
+        for (int l = 0; l < n; ++l) {
+          const auto& v = ents[32 * q + l];
+          for (size_t i = 32 * h; i < v.size() && (h || i < 32); ++i) lab[l].push_back(v[i].first);
+          pos[l].resize(lab[l].size());
+        }
+        spread_positions(lab, 32 * h, pos);
+        for (int l = 0; l < n; ++l)
+          for (size_t i = 0; i < pos[l].size(); ++i) pos_of[ents[32 * q + l][32 * h + i].second] = pos[l][i];
+      }
+  }
   for (int l = 0; l < nc; ++l) {
     const int c = o.s_col[l];
     o.s_llr[l] = o.llr[c];
     for (int e = o.col_ptr[c]; e < o.col_ptr[c + 1]; ++e) {
-      const int r = rlab[o.col_rows[e]], pos = fill[r]++;
+      const int r = rlab[o.col_rows[e]], pos = pos_of[e];
       const size_t ri = ((size_t)(o.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
       const size_t ci = (size_t)(o.s_coff[l >> 5] + (e - o.col_ptr[c])) * 32 + (l & 31);
       o.s_rent[ri] = (uint16_t)l;
       o.s_ref[ri] = (uint16_t)e;
       o.s_cent[ci] = ((uint32_t)r << 16) | (uint32_t)pos;
       o.s_cef[ci] = (uint16_t)e;
-      if (pos >= 32) wide[l >> 5] = 1;
     }
   }
   // a dummy takes its node's first edge's learned weight, so that a weight
   // touches no node but its own two
   for (int r = 0; r < nr; ++r)
-    for (int pos = std::max(1, fill[r]); pos < 4 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
+    for (int pos = std::max(1, rdeg(o.s_row[r])); pos < 4 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
       const size_t r0 = ((size_t)o.s_roff[r >> 5] * 32 + (r & 31)) * 4;
       o.s_ref[r0 + 128 * (size_t)(pos >> 2) + (pos & 3)] = o.s_ref[r0];
     }
@@ -570,10 +693,7 @@ bool build_slices(WindowHost& o) {
     const int w = o.s_coff[q + 1] - o.s_coff[q];
     for (int x = 0; x < 4; ++x)
       if (w >= 4 - x) o.cls[x] = q + 1;
-    if (wide[q] && w >= 3) o.wide3 = 1;
   }
-  for (int q = 0; q < ncs; ++q)
-    if (wide[q]) o.s_coff[q] |= kWideSlice;
   // a shortened graph: every slice but the first is no wider than the least
   // degree of the slice before it, so the widths sum to at most the widest
   // node plus edges / 32 (check slices rounded up to fours)
@@ -594,7 +714,7 @@ WmsHost build_wms(const WindowHost& h) {
   std::copy(h.s_row.begin(), h.s_row.end(), o.row.begin());
   o.col = h.s_col;
   o.coff.resize(ncs + 1);
-  for (int q = 0; q <= ncs; ++q) o.coff[q] = (uint16_t)(h.s_coff[q] & (kWideSlice - 1));
+  for (int q = 0; q <= ncs; ++q) o.coff[q] = h.s_coff[q];
   o.roff.assign(nrs + 1, 0);
   for (int q = 0; q < nrs; ++q) {
     const int j = h.s_row[32 * q];

@@ -276,102 +276,62 @@ struct ColView {
   int lane, st;  // the group takes every st-th slice
 };
 
-// The first slice s, s - st, ... of the group at or past end.
-__device__ __forceinline__ int back_to(int s, int end, int st) {
-#pragma unroll 1
-  while (s - st >= end) s -= st;
-  return s;
-}
-
-// Variable-node update of Eq. (2), one column per lane: prior + the messages
-// of its checks in ascending check order (a dummy adds +0).  M slices of N
-// entries each at once, so that M * N record gathers are in flight: the pass
-// is a chain of shared-memory round trips (entry, record) ahead of a few
-// instructions, and with one slice after another it took 1.75 times the check
-// pass although it issues fewer instructions.  Slices past `end` repeat the
-// first and store nothing: one copy of the code serves every remainder (a copy
-// for each cost more in instruction fetches than the repeated loads do).
-// put(s, p): the posterior of this lane's column of slice s.
-template <bool LW, bool WIDE, int N, int M, class Put>
-__device__ __forceinline__ void column_group(const ColView& V, int s, int end, int cell, int stride, Put put) {
-  uint32_t e[M][N];
-  CNState c[M][N];
-  float p[M], w[M][N];
-  int act[M];
+// p + the messages of N entries of this lane's column from cell c0 on, in
+// ascending check order (Eq. (2); a dummy adds +0): N record gathers in flight.
+template <bool LW, bool WIDE, int N>
+__device__ __forceinline__ float add_messages(const ColView& V, float p, int c0) {
+  uint32_t e[N];
+  CNState c[N];
+  float w[N];
 #pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const bool in = m == 0 || s + m * V.st < end;
-    const int k = 32 * (in ? s + m * V.st : s) + V.lane, ei = 32 * (in ? cell + m * stride : cell) + V.lane;
-    act[m] = V.status ? (int)V.status[k] : -1;
-    if (!in) act[m] = 0;
-    p[m] = V.llr[k];
-#pragma unroll
-    for (int x = 0; x < N; ++x) {
-      e[m][x] = V.cent[ei + 32 * x];
-      w[m][x] = LW ? lw_at(V.lw, ei + 32 * x) : 0.0f;
-    }
+  for (int x = 0; x < N; ++x) {
+    e[x] = V.cent[32 * (c0 + x) + V.lane];
+    w[x] = LW ? lw_at(V.lw, 32 * (c0 + x) + V.lane) : 0.0f;
   }
 #pragma unroll
-  for (int m = 0; m < M; ++m)
+  for (int x = 0; x < N; ++x) c[x] = *(const CNState*)(V.cns + (e[x] >> 12));
 #pragma unroll
-    for (int x = 0; x < N; ++x) c[m][x] = *(const CNState*)(V.cns + (e[m][x] >> 12));
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-#pragma unroll
-    for (int x = 0; x < N; ++x) p[m] = __fadd_rn(p[m], c2v<LW>(c[m][x], e[m][x], WIDE, w[m][x]));
-    if (act[m] == -1) put(s + m * V.st, p[m]);
-  }
+  for (int x = 0; x < N; ++x) p = __fadd_rn(p, c2v<LW>(c[x], e[x], WIDE, w[x]));
+  return p;
 }
 
-// The variable pass over column slices first, first + st, ...  WIDE: columns
-// of degree one and two may have edges at positions past 31; wide: so may the
-// others (then, and for widths past three, one slice at a time).
+// The variable pass over column slices first, first + st, ...: put(s, p) takes
+// the posterior of this lane's column of slice s.  WIDE: edges may have
+// positions past 31 (the widest slices always allow it).  A loop per width, so
+// that trip counts and offsets are constants, and one slice a trip: two or four
+// slices at once overlap more gathers, but the larger loop and the repeated
+// slices at its end cost more (2000 shots of [[144,12,12]], three CTAs per SM:
+// 106.6 ms with four slices of width one at once, 102.8 ms so; one loop for all
+// widths, 126 ms).
 template <bool LW, bool WIDE, class Put>
-__device__ __forceinline__ void column_pass(const ColView& V, int first, bool wide, Put put) {
+__device__ __forceinline__ void column_pass(const ColView& V, int first, Put put) {
   constexpr int kLow = kWideSlice - 1;
+  const ColClasses& K = V.K;
   int s = first;
+  auto active = [&]() { return !V.status || V.status[32 * s + V.lane] == -1; };  // (asked for before the gathers)
 #pragma unroll 1
-  for (const int end = wide ? V.K.n1 : V.K.n4; s < end; s += V.st) {
+  for (; s < K.n4; s += V.st) {
     int c0 = V.coff[s] & kLow;
-    const int c1 = V.coff[s + 1] & kLow, k = 32 * s + V.lane;
-    float p = V.llr[k];
-    auto more = [&](auto cnt) {
-      constexpr int N = decltype(cnt)::value;
-      uint32_t e[N];
-      CNState c[N];
-#pragma unroll
-      for (int x = 0; x < N; ++x) e[x] = V.cent[32 * (c0 + x) + V.lane];
-#pragma unroll
-      for (int x = 0; x < N; ++x) c[x] = *(const CNState*)(V.cns + (e[x] >> 12));
-#pragma unroll
-      for (int x = 0; x < N; ++x)
-        p = __fadd_rn(p, c2v<LW>(c[x], e[x], true, LW ? lw_at(V.lw, 32 * (c0 + x) + V.lane) : 0.0f));
-      c0 += N;
-    };
+    const int c1 = V.coff[s + 1] & kLow;
+    float p = V.llr[32 * s + V.lane];
 #pragma unroll 1
-    while (c0 + 3 <= c1) more(std::integral_constant<int, 3>{});
+    for (; c0 + 3 <= c1; c0 += 3) p = add_messages<LW, true, 3>(V, p, c0);
 #pragma unroll 1
-    while (c0 < c1) more(std::integral_constant<int, 1>{});
-    if (!V.status || V.status[k] == -1) put(s, p);
+    for (; c0 < c1; ++c0) p = add_messages<LW, true, 1>(V, p, c0);
+    if (active()) put(s, p);
   }
-  if (wide) return;
-  {
-    const int b = V.coff[V.K.n4] & kLow;
+  auto narrow = [&](auto width, int end, int b) {  // cells from b + N s on
+    constexpr int N = decltype(width)::value;
 #pragma unroll 1
-    for (; s < V.K.n3; s += 2 * V.st) column_group<LW, false, 3, 2>(V, s, V.K.n3, b + 3 * (s - V.K.n4), 3 * V.st, put);
-    s = back_to(s, V.K.n3, V.st);
-  }
-  {
-    const int b = V.coff[V.K.n3] & kLow;
-#pragma unroll 1
-    for (; s < V.K.n2; s += 2 * V.st) column_group<LW, WIDE, 2, 2>(V, s, V.K.n2, b + 2 * (s - V.K.n3), 2 * V.st, put);
-    s = back_to(s, V.K.n2, V.st);
-  }
-  {
-    const int b = V.coff[V.K.n2] & kLow;
-#pragma unroll 1
-    for (; s < V.K.n1; s += 4 * V.st) column_group<LW, WIDE, 1, 4>(V, s, V.K.n1, b + (s - V.K.n2), V.st, put);
-  }
+    for (; s < end; s += V.st) {
+      const bool act = active();
+      const float p = add_messages<LW, WIDE, N>(V, V.llr[32 * s + V.lane], b + N * s);
+      if (act) put(s, p);
+    }
+  };
+  narrow(std::integral_constant<int, 3>{}, K.n3, (V.coff[K.n4] & kLow) - 3 * K.n4);
+  narrow(std::integral_constant<int, 2>{}, K.n2, (V.coff[K.n3] & kLow) - 2 * K.n3);
+  narrow(std::integral_constant<int, 1>{}, K.n1, (V.coff[K.n2] & kLow) - K.n2);
 }
 
 __device__ __forceinline__ uint32_t bit_of(const uint32_t* w, int j) { return (w[j >> 5] >> (j & 31)) & 1u; }
@@ -696,12 +656,19 @@ __device__ int peel(const ShortG& G, const Slot& B, const Grp& g, int& act) {
     bool contra = false;
     int cand = kNone;  // (window row << 16) | label of the lowest degree-one check
 #pragma unroll 1
-    for (int j = g.rank; j < G.nr; j += g.size) {
-      const int d = B.deg[j];
-      if (d == 0) {
-        if (bit_of(B.sp, j)) contra = true;
-      } else if (d == 1) {
-        cand = min(cand, ((int)G.cperm[j] << 16) | j);
+    for (int x = g.rank; x < 8 * G.rw; x += g.size) {  // four checks' counts at a time
+      const uint32_t d4 = ((const uint32_t*)B.deg)[x];
+      const uint32_t low = d4 & 0xFEFEFEFEu;
+      if (!((low - 0x01010101u) & ~low & 0x80808080u)) continue;  // none is 0 or 1 (a borrow only adds hits)
+      const uint32_t s4 = B.sp[x >> 3] >> (4 * (x & 7));
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const int d = (int)((d4 >> (8 * y)) & 0xFFu), j = 4 * x + y;
+        if (d == 0) {
+          if ((s4 >> y) & 1u) contra = true;  // (the padding's syndrome bits are 0)
+        } else if (d == 1) {
+          cand = min(cand, ((int)G.cperm[j] << 16) | j);
+        }
       }
     }
     if (g.any(contra)) return -1;
@@ -982,10 +949,36 @@ __device__ void write_snapshot(char* dst, const ForkCtx& F, const Grp& g, int D,
   }
   const uint4* s4 = (const uint4*)F.slot;
   uint4* d4 = (uint4*)(dst + kSnapHeader);
-#pragma unroll 1
+#pragma unroll 4
   for (unsigned x = g.rank; x < F.slot_bytes / 16u; x += g.size) __stcg(d4 + x, s4[x]);
   __threadfence();  // the snapshot and this path's decision records before its flag
   g.sync();
+}
+
+// The waiting path with the most steps left, if more than `least` (every lane
+// of the warp looks at a path; the lowest id among equals): a parked path, or
+// a queued one whose planned snapshot is ready.  -1: none; w: its state word.
+__device__ __forceinline__ int longest_waiting(const KParams& P, const ForkCtx& F, int lane, int least, unsigned& w) {
+  unsigned key = 0, kw = 0;
+#pragma unroll 1
+  for (int p = lane; p < P.nb; p += 32) {
+    const unsigned x = *(volatile unsigned*)&F.sched[p];
+    int at = 0;
+    if ((x & 3u) == PS_PARKED) at = (int)(x >> 8);
+    else if (x == PS_QUEUED && F.fnode[p] >= 0 && *(volatile int*)&F.flags[F.fnode[p]] == 2) at = F.fdep[p];
+    if (!at) continue;
+    const int rem = path_dmax(P, p, path_split(P, p)) - at + 1;
+    const unsigned k = rem > least ? ((unsigned)rem << 8) | (255u - (unsigned)p) : 0u;
+    if (k > key) {
+      key = k;
+      kw = x;
+    }
+  }
+  const unsigned best = __reduce_max_sync(FULL, key);
+  if (!best) return -1;
+  const int c = 255 - (int)(best & 255u);
+  w = __shfl_sync(FULL, kw, c & 31);
+  return c;
 }
 
 // Check-node update of Eq. (1) over the active VNs of one decision path; a
@@ -1076,8 +1069,8 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     if (R == 0) inherited = __ldcg((const long long*)(F.src + 24));
     const uint4* s4 = (const uint4*)(F.src + kSnapHeader);
     uint4* d4 = (uint4*)F.slot;
-#pragma unroll 1
-    for (unsigned x = R; x < F.slot_bytes / 16u; x += S) d4[x] = __ldcg(s4 + x);
+#pragma unroll 4
+    for (unsigned x = R; x < F.slot_bytes / 16u; x += S) d4[x] = __ldcg(s4 + x);  // (in flight together)
     // a path resumed from its own parking snapshot keeps its records
     if (out.st && producer != id) {  // the decision records of the shared prefix are the producer's
       const StepTrace* ps = F.st0 + (size_t)producer * dmx;
@@ -1162,15 +1155,17 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // variables in label order; a decimated column runs the loop too and stores nothing
       LwRow lw{nullptr, G.cef};
       if (LW) lw.w = weight_row(G.wts, G.wT, G.wE, tw + 1);
-      const bool wide = (G.coff[0] & kWideSlice) != 0;
       const int lane = R & 31;
-      const ColView V{*G.cls, G.cent, G.coff, G.llr, B.status, (const char*)B.cns, lw, lane, S >> 5};
-      column_pass<LW, false>(V, R >> 5, wide, [&](int s, float p) { B.post[32 * s + lane] = p; });
+      ColView V{*G.cls, G.cent, G.coff, G.llr, B.status, (const char*)B.cns, lw, lane, S >> 5};
+      const int n3 = V.K.n3;
+      // (a check past 32 entries: every slice goes one at a time)
+      if ((G.coff[0] & kWideSlice) != 0) V.K.n4 = V.K.n3 = V.K.n2 = V.K.n1;
+      column_pass<LW, false>(V, R >> 5, [&](int s, float p) { B.post[32 * s + lane] = p; });
       // the history of Sec. IV-A, for the columns a decimation step looks at:
       // SELECT-VN's and Alg. 3's candidates have degree three or more
       if (hist)
 #pragma unroll 1
-        for (int s = R >> 5; s < V.K.n3; s += V.st) {
+        for (int s = R >> 5; s < n3; s += V.st) {
           const int k = 32 * s + lane;
           if (B.status[k] != -1) continue;
           const float p = B.post[k];
@@ -1215,31 +1210,15 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
     // preemption point: switch to a waiting path with more steps left (not
     // right where this run resumed)
     if (F.sched && D < dmax && !(F.src && D == D0)) {
-      int c = -1;
       unsigned cw = 0;
-      if (R == 0) {
-        int best = dmax - D + 2;  // more than one step more than this path's dmax - D + 1
-#pragma unroll 1
-        for (int p = 0; p < P.nb; ++p) {
-          const unsigned w = *(volatile unsigned*)&F.sched[p];
-          int at = 0;
-          if ((w & 3u) == PS_PARKED) at = (int)(w >> 8);
-          else if (w == PS_QUEUED && F.fnode[p] >= 0 && *(volatile int*)&F.flags[F.fnode[p]] == 2) at = F.fdep[p];
-          if (!at) continue;
-          const int rem = path_dmax(P, p, path_split(P, p)) - at + 1;
-          if (rem > best) {
-            best = rem;
-            c = p;
-            cw = w;
-          }
-        }
-        if (c >= 0 && atomicCAS(&F.sched[c], cw, (unsigned)PS_RUNNING) != cw) c = -1;
-      }
-      const unsigned cu = g.min_u(R == 0 && c >= 0 ? (unsigned)c : 0xFFFFFFFFu);  // lane 0's choice
-      c = cu == 0xFFFFFFFFu ? -1 : (int)cu;
+      int c = longest_waiting(P, F, R, dmax - D + 2, cw);  // more than one step more than this path's
       if (c >= 0) {
-        const unsigned cw0 = g.min_u(R == 0 ? cw : 0xFFFFFFFFu);
-        if (claimed) *claimed = cw0;
+        int won = 0;
+        if (R == 0) won = atomicCAS(&F.sched[c], cw, (unsigned)PS_RUNNING) == cw;
+        if (!g.any(won != 0)) c = -1;
+      }
+      if (c >= 0) {
+        if (claimed) *claimed = cw;
         // park: this path resumes from its own snapshot after the BP of step D
         const long long own = g.sum_ll(visits);
         write_snapshot(F.pool + (size_t)(F.n_nodes + id) * F.stride, F, g, D, iters, tw, first, id, g.sum_i(act),
@@ -1261,8 +1240,9 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       // ranked column (the oracle's index order) whatever the label order
       float bL = CUDART_INF_F, tL = CUDART_INF_F;
       int bk = kNone, tk = kNone, nagg = 0;
+      const int n3 = min(ns, 32 * G.cls->n3);  // (labels by descending degree)
 #pragma unroll 1
-      for (int k = R; k < ns; k += S) {
+      for (int k = R; k < n3; k += S) {
         if (B.status[k] != -1 || G.vdeg[k] <= 2) continue;
         const float L = B.acc[k];
         const uint8_t fl = B.hfl[k];
@@ -1697,7 +1677,7 @@ __device__ __forceinline__ void prebp_columns(const WinDev& W, const PreBp& X, i
   LwRow lw{nullptr, W.s_cef};
   if (LW) lw.w = weight_row(W.wts, W.wT, W.n_edges, t);
   const ColView V{W.cls, X.cent, X.coff, X.llr, nullptr, (const char*)X.cns, lw, lane, st};
-  column_pass<LW, true>(V, first, W.wide3 != 0, put);
+  column_pass<LW, true>(V, first, put);
 }
 
 __device__ __forceinline__ float prebp_key(const KParams& P, const PreBp& X, int l, int t, int tk0, float p) {
@@ -2258,33 +2238,19 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
               break;
             }
           }
-          if (id < 0 && F.sched) {  // a parked path, the one with the most steps left
-            int c = -1;
-            unsigned cw = 0;
-            if (lane == 0)
+          if (id < 0 && F.sched) {  // a waiting path, the one with the most steps left
 #pragma unroll 1
-              for (int tries = 0; tries < 4 * nb; ++tries) {
-                c = -1;
-                int best = 0;
-#pragma unroll 1
-                for (int p = 0; p < nb; ++p) {
-                  const unsigned w = *(volatile unsigned*)&F.sched[p];
-                  if ((w & 3u) != PS_PARKED) continue;
-                  const int rem = path_dmax(A.P, p, path_split(A.P, p)) - (int)(w >> 8) + 1;
-                  if (rem > best) {
-                    best = rem;
-                    c = p;
-                    cw = w;
-                  }
-                }
-                if (c < 0 || atomicCAS(&F.sched[c], cw, (unsigned)PS_RUNNING) == cw) break;
-                c = -1;
+            for (int tries = 0; tries < 4 * nb; ++tries) {
+              unsigned cw = 0;
+              const int c = longest_waiting(A.P, F, lane, 0, cw);
+              if (c < 0) break;
+              int ok = 0;
+              if (lane == 0) ok = atomicCAS(&F.sched[c], cw, (unsigned)PS_RUNNING) == cw;
+              if (__shfl_sync(FULL, ok, 0)) {
+                id = c;
+                w0 = cw;
+                break;
               }
-            c = __shfl_sync(FULL, c, 0);
-            cw = __shfl_sync(FULL, cw, 0);
-            if (c >= 0) {
-              id = c;
-              w0 = cw;
             }
           }
           if (id < 0) break;
@@ -2301,15 +2267,13 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
           F.src = F.pool + (size_t)(F.n_nodes + id) * F.stride;
         } else if (F.chain) {  // the deepest ready snapshot on this path's chain
           int node = -1;
-          if (lane == 0) {
-            const int dm = path_dmax(A.P, id, path_split(A.P, id));
+          const int dm = path_dmax(A.P, id, path_split(A.P, id));
 #pragma unroll 1
-            for (int D = dm; D >= 1 && node < 0; --D) {
-              const int n = F.chain[D - 1];
-              if (n >= 0 && *(volatile int*)&F.flags[n] == 2) node = n;
-            }
+          for (int b = (dm - 1) & ~31; b >= 0 && node < 0; b -= 32) {  // a lane per depth
+            const int n = b + lane < dm ? F.chain[b + lane] : -1;
+            const unsigned m = __ballot_sync(FULL, n >= 0 && *(volatile int*)&F.flags[n >= 0 ? n : 0] == 2);
+            if (m) node = __shfl_sync(FULL, n, 31 - __clz(m));
           }
-          node = __shfl_sync(FULL, node, 0);
           if (node >= 0) {
             __threadfence();  // the snapshot's contents after its flag
             F.src = F.pool + (size_t)node * F.stride;

@@ -121,7 +121,6 @@ struct WinDev {
   const float* s_llr;                // priors by column label
   const uint16_t *s_row, *s_col;     // label -> window row / window column
   ColClasses cls;
-  int wide3;  // some column of degree three or more has an edge at a position past 31
   const uint16_t *s_ref, *s_cef;     // full-window edge of each check / column entry (learned weights)
 };
 
@@ -192,8 +191,8 @@ struct __align__(16) CNState {
 // at most 35 columns: the fault classes of a round are the same for every
 // choice of A and B (three terms each), and coinciding terms only merge them.
 constexpr int kMaxRowDeg = 51;
-// Flag of a column slice's start (s_coff) when some edge of it has a position
-// past 31 and its sign is in the second word.
+// Flag of a shortened graph's column slice starts (s_coff) when some check has
+// more than 32 entries, so that signs may be in the second word.
 constexpr uint16_t kWideSlice = 0x8000;
 
 struct BranchTrace {

@@ -700,7 +700,7 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
                       h.row_quads, h.col_cells, (const uint16_t*)(b + s_re), (const uint32_t*)(b + s_ce),
                       (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
                       (const uint16_t*)(b + s_rw), (const uint16_t*)(b + s_cl),
-                      qd::ColClasses{h.cls[0], h.cls[1], h.cls[2], h.cls[3]}, h.wide3, (const uint16_t*)(b + s_rf),
+                      qd::ColClasses{h.cls[0], h.cls[1], h.cls[2], h.cls[3]}, (const uint16_t*)(b + s_rf),
                       (const uint16_t*)(b + s_cf)};
     // committed columns: their full detector sets and observables
     std::vector<int> cc_ptr(1, 0), cc_det;

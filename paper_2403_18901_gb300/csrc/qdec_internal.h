@@ -28,7 +28,7 @@ struct WindowHost {
   int row_quads = 0, col_cells = 0;    // slice totals
   int srow_quads = 0, scol_cells = 0;  // bounds on those of a shortened graph
   int max_row_deg = 0;
-  int cls[4] = {0, 0, 0, 0}, wide3 = 0;  // ColClasses; an edge of a column of degree >= 3 past position 31
+  int cls[4] = {0, 0, 0, 0};  // ColClasses
   std::vector<uint32_t> s_cent;
   std::vector<uint16_t> s_rent, s_roff, s_coff, s_row, s_col, s_ref, s_cef;
   std::vector<float> s_llr;

@@ -5,7 +5,7 @@
 // usage: slice_check l m a0x a0y .. b2x b2y rounds W F merge shorten trials
 // For every window: each edge is stored once per side and the two sides agree
 // on its position; every other place is a dummy; a column's checks ascend in
-// window row; the flag of a wide slice is set where a position passes 31.
+// window row.
 // For random shortened graphs (and the one of the highest degrees) the slices
 // stay within the bounds.  Layout regions are 16-byte aligned and disjoint
 // where they live together.  Prints "ok" or the first violation.
@@ -40,7 +40,6 @@ bool check_graph(const qd::WindowHost& h) {
   for (int q = 0; q < ncs; ++q) {
     const int w = (int)(h.s_coff[q + 1] & low) - (int)(h.s_coff[q] & low);
     for (int x = 0; x < 4; ++x) REQ((w >= 4 - x) == (q < h.cls[x]), "slice %d of width %d: class %d", q, w, x);
-    REQ(w < 3 || !(h.s_coff[q] & qd::kWideSlice) || h.wide3, "slice %d: wide", q);
   }
   size_t real = 0, dummies = 0;
   std::vector<int> seen(h.n_edges, 0);
@@ -62,7 +61,6 @@ bool check_graph(const qd::WindowHost& h) {
       const size_t ri = ((size_t)(h.s_roff[r >> 5] + (pos >> 2)) * 32 + (r & 31)) * 4 + (pos & 3);
       REQ((pos >> 2) < h.s_roff[(r >> 5) + 1] - h.s_roff[r >> 5], "check %d position %d", r, pos);
       REQ(h.s_rent[ri] == l && h.s_ref[ri] == fe, "check %d position %d: other side", r, pos);
-      REQ(pos < 32 || (h.s_coff[l >> 5] & qd::kWideSlice), "column %d: slice not flagged", l);
     }
   }
   for (int e = 0; e < h.n_edges; ++e) REQ(seen[e] == 1, "edge %d stored %d times", e, seen[e]);
