@@ -6,8 +6,8 @@
 //       (Eq. (1)-(4)); a check node by one lane (shot mode) or a lane group
 //       (path mode), a variable node by one thread; early stop when H e = s
 //       (Sec. II-A), tested inside the next check pass
-//   a3  ranking key ((h0+h1)+h2)+h3 of the last four posteriors, bitonic sort
-//       of (key, column) ascending, first 2w' columns kept (Sec. III); the
+//   a3  ranking key ((h0+h1)+h2)+h3 of the last four posteriors, the 2w'
+//       columns of least (key, column) selected and sorted (Sec. III); the
 //       shortened matrix is rebuilt in shared memory with its checks and
 //       columns numbered in processing order (descending degree)
 //   a4-a7 GDG decision paths (Alg. 2 on the 2^k tree and the side branches of
@@ -1927,9 +1927,59 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   // ---- a3: rank by the four-iteration sum, keep the first n_short ----
   const int n_short = W.n_short, nsp = 32 * L.sw;
   unsigned long long* sortb = (unsigned long long*)(U + L.p_sort);
+  auto sort_key = [&](int l, uint32_t k) {  // ties by window column
+    return ((unsigned long long)k << 32) | ((unsigned)W.s_col[l] << 16) | (unsigned)l;
+  };
+  if (L.sortn >= nc) {
 #pragma unroll 1
-  for (int l = tid; l < L.sortn; l += NT)  // ties by window column
-    sortb[l] = l < nc ? (((unsigned long long)ordkey(key[l]) << 32) | ((unsigned)W.s_col[l] << 16) | (unsigned)l) : ~0ull;
+    for (int l = tid; l < L.sortn; l += NT) sortb[l] = l < nc ? sort_key(l, ordkey(key[l])) : ~0ull;
+  } else {
+    // select before sorting: bisection for the n_short-th smallest key, then
+    // (equal keys) for the column up to which its equals are taken
+    uint32_t* uk = (uint32_t*)key;
+    // (the sort buffer follows the keys, over the dead check records; the
+    // posteriors before them are dead too)
+    const CtaGrp cta{tid, NT, (char*)post};
+    auto count = [&](auto&& in) {
+      int n = 0;
+#pragma unroll 4
+      for (int l = tid; l < nc; l += NT) n += in(l) ? 1 : 0;
+      return cta.sum_i(n);
+    };
+#pragma unroll 1
+    for (int l = tid; l < nc; l += NT) uk[l] = ordkey(key[l]);
+    uint32_t lo = 0u, hi = 0xFFFFFFFFu;
+    int most = nc;  // keys <= hi
+#pragma unroll 1
+    while (lo < hi) {
+      const uint32_t mid = lo + (hi - lo) / 2;
+      const int n = count([&](int l) { return uk[l] <= mid; });
+      if (n >= n_short) {
+        hi = mid;
+        most = n;
+      } else {
+        lo = mid + 1;
+      }
+    }
+    int c_lo = 0, c_hi = most == n_short ? 0x7fff : nc - 1;
+    if (most > n_short) {
+#pragma unroll 1
+      while (c_lo < c_hi) {
+        const int mid = (c_lo + c_hi) / 2;
+        const int n = count([&](int l) { return uk[l] < hi || (uk[l] == hi && (int)W.s_col[l] <= mid); });
+        if (n >= n_short) c_hi = mid;
+        else c_lo = mid + 1;
+      }
+    }
+    int* next = (int*)(sm + L.misc) + 5;
+    if (tid == 0) *next = 0;
+#pragma unroll 1
+    for (int l = n_short + tid; l < L.sortn; l += NT) sortb[l] = ~0ull;
+    __syncthreads();
+#pragma unroll 1
+    for (int l = tid; l < nc; l += NT)
+      if (uk[l] < hi || (uk[l] == hi && (int)W.s_col[l] <= c_hi)) sortb[atomicAdd(next, 1)] = sort_key(l, uk[l]);
+  }
   __syncthreads();
   block_sort_u64(sortb, L.sortn);
   // (from here on the pre-BP's arrays are dead: the shortened graph takes their place)

@@ -306,8 +306,9 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.rw = (nr + 31) / 32;
   L.cw = (nc + 31) / 32;
   L.sw = (ns + 31) / 32;
+  // keys sorted: the kept columns', selected first, or all when that takes as many
   int sn = 1;
-  while (sn < nc) sn <<= 1;
+  while (sn < ns) sn <<= 1;
   L.sortn = sn;
   L.hist = ranker ? 4u : 0u;
   L.lwe = lw ? 1u : 0u;

@@ -162,7 +162,7 @@ bool check_layout(const qd::WindowHost& h, int nb, unsigned budget, bool ranker,
   if (!disjoint(pre, base, hi, "pre-BP")) return false;
   // the sort: filled from the keys; then read while the shortened graph is written
   const unsigned need = 8u * (unsigned)L.sortn, scr = 4u * (nsp + 2u * nrp);
-  REQ(L.sortn >= nc && !(L.sortn & (L.sortn - 1)), "sort size");
+  REQ(L.sortn >= ns && !(L.sortn & (L.sortn - 1)), "sort size");
   if (!disjoint({{"key", L.p_key + base, 4u * ncp}, {"sort", L.p_sort + base, need}}, base, hi, "ranking")) return false;
   if (!disjoint({{"scratch", L.p_scr + base, scr}}, base, hi, "scratch")) return false;
   if (!glob) {
