@@ -155,17 +155,37 @@ __device__ __forceinline__ CNState check_record(const CheckAcc& A, uint32_t sg0,
   return CNState{flip_sign(m1, par), flip_sign(m2, par), sg0, (sg1 & ~63u) | A.am};
 }
 
-// Learned weights' view of one iteration: its row of w, and the full-window
-// edge of each entry.
-struct LwRow {
+// Learned weights' view of one iteration: entry i's weight is w[ef[i]] (its row
+// of the weights, the entries' full-window edges), or w[i] where the weights
+// have been put in entry order (ef = nullptr; a type of its own, so that each
+// loop is compiled for one of the two).
+struct LwEdge {
   const float* w;
   const uint16_t* ef;
+  __device__ __forceinline__ float one(int i) const { return w[ef[i]]; }
+  __device__ __forceinline__ void four(int i, float (&x)[4]) const {
+    const uint2 e = *(const uint2*)(ef + i);
+    x[0] = w[e.x & 0xFFFFu];
+    x[1] = w[e.x >> 16];
+    x[2] = w[e.y & 0xFFFFu];
+    x[3] = w[e.y >> 16];
+  }
 };
-__device__ __forceinline__ float lw_at(const LwRow& r, int i) { return r.w[r.ef[i]]; }
-template <bool LW>
-__device__ __forceinline__ void lw_four(const LwRow& r, int i, bool first, float (&w)[4]) {
-#pragma unroll
-  for (int x = 0; x < 4; ++x) w[x] = LW && !first ? lw_at(r, i + x) : 0.0f;
+struct LwOrdered {
+  const float* w;
+  __device__ __forceinline__ float one(int i) const { return w[i]; }
+  __device__ __forceinline__ void four(int i, float (&x)[4]) const {
+    const float4 v = *(const float4*)(w + i);
+    x[0] = v.x;
+    x[1] = v.y;
+    x[2] = v.z;
+    x[3] = v.w;
+  }
+};
+template <bool LW, class Lw>
+__device__ __forceinline__ void lw_four(const Lw& r, int i, bool first, float (&w)[4]) {
+  w[0] = w[1] = w[2] = w[3] = 0.0f;
+  if (LW && !first) r.four(i, w);
 }
 
 // Check-node update of Eq. (1) of one check by one lane.  ent: the lane's
@@ -180,9 +200,9 @@ __device__ __forceinline__ void lw_four(const LwRow& r, int i, bool first, float
 // and the clip on every input and ragged rows, 5000 shots of [[144,12,12]]
 // took 450 ms; in slices, with the signs as bits of the record and the clip on
 // the two minima, 354 ms.
-template <bool LW, class E>
+template <bool LW, class E, class Lw>
 __device__ __forceinline__ uint32_t check_lane(const E* ent, int nq, const char* post, CNState* rec, uint32_t sbit,
-                                               float alpha, float clip, const LwRow& lw, int ei, bool first) {
+                                               float alpha, float clip, const Lw& lw, int ei, bool first) {
   CNState oc = *rec;
   if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
   const uint32_t oam = oc.am & 63u;
@@ -213,9 +233,9 @@ __device__ __forceinline__ uint32_t check_lane(const E* ent, int nq, const char*
 
 // The same by tpc neighbouring lanes (fours sub, sub + tpc, ...); every lane
 // of the group ends with the record.
-template <bool LW, class E>
+template <bool LW, class E, class Lw>
 __device__ __forceinline__ CNState check_group(const E* ent, int nq, const char* post, CNState oc, uint32_t sbit,
-                                               float alpha, float clip, bool first, const LwRow& lw, int ei, int sub,
+                                               float alpha, float clip, bool first, const Lw& lw, int ei, int sub,
                                                int tpc, bool wide, uint32_t& unsat) {
   if (first) oc = CNState{0.0f, 0.0f, 0u, 0u};
   const uint32_t oam = oc.am & 63u;
@@ -265,6 +285,7 @@ __device__ __forceinline__ uint32_t check_parity(const E* ent, int nq, const cha
 }
 
 // What the variable pass walks: this lane's view of the column slices.
+template <class Lw>
 struct ColView {
   ColClasses K;
   const uint32_t* cent;
@@ -272,21 +293,21 @@ struct ColView {
   const float* llr;
   const int8_t* status;  // nullptr: every column is active
   const char* cns;
-  LwRow lw;
+  Lw lw;
   int lane, st;  // the group takes every st-th slice
 };
 
 // p + the messages of N entries of this lane's column from cell c0 on, in
 // ascending check order (Eq. (2); a dummy adds +0): N record gathers in flight.
-template <bool LW, bool WIDE, int N>
-__device__ __forceinline__ float add_messages(const ColView& V, float p, int c0) {
+template <bool LW, bool WIDE, int N, class Lw>
+__device__ __forceinline__ float add_messages(const ColView<Lw>& V, float p, int c0) {
   uint32_t e[N];
   CNState c[N];
   float w[N];
 #pragma unroll
   for (int x = 0; x < N; ++x) {
     e[x] = V.cent[32 * (c0 + x) + V.lane];
-    w[x] = LW ? lw_at(V.lw, 32 * (c0 + x) + V.lane) : 0.0f;
+    w[x] = LW ? V.lw.one(32 * (c0 + x) + V.lane) : 0.0f;
   }
 #pragma unroll
   for (int x = 0; x < N; ++x) c[x] = *(const CNState*)(V.cns + (e[x] >> 12));
@@ -303,8 +324,8 @@ __device__ __forceinline__ float add_messages(const ColView& V, float p, int c0)
 // slices at its end cost more (2000 shots of [[144,12,12]], three CTAs per SM:
 // 106.6 ms with four slices of width one at once, 102.8 ms so; one loop for all
 // widths, 126 ms).
-template <bool LW, bool WIDE, class Put>
-__device__ __forceinline__ void column_pass(const ColView& V, int first, Put put) {
+template <bool LW, bool WIDE, class Lw, class Put>
+__device__ __forceinline__ void column_pass(const ColView<Lw>& V, int first, Put put) {
   constexpr int kLow = kWideSlice - 1;
   const ColClasses& K = V.K;
   int s = first;
@@ -990,7 +1011,7 @@ __device__ __forceinline__ int longest_waiting(const KParams& P, const ForkCtx& 
 template <bool LW>
 __device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& G, const Slot& B, int lane, bool first,
                                                 int tw) {
-  LwRow lw{nullptr, G.ref};
+  LwEdge lw{nullptr, G.ref};
   if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
   uint32_t unsat = 0u;
   int r0 = 0;
@@ -1010,7 +1031,7 @@ __device__ __forceinline__ bool check_pass_warp(const KParams& P, const ShortG& 
 template <bool LW>
 __device__ __forceinline__ bool check_pass_cta(const KParams& P, const ShortG& G, const Slot& B, int R, int S, int tpc,
                                                bool first, int tw) {
-  LwRow lw{nullptr, G.ref};
+  LwEdge lw{nullptr, G.ref};
   if (LW && !first) lw.w = weight_row(G.wts, G.wT, G.wE, tw);
   const int nrp = 32 * G.rwz, per = S / tpc, sub = R & (tpc - 1);
   uint32_t unsat = 0u;
@@ -1153,10 +1174,10 @@ __device__ int run_path(const KParams& P, const ShortG& G, const Slot& B, int id
       const bool hist = it > ips - 4;
       const bool hist0 = it == ips - 3;
       // variables in label order; a decimated column runs the loop too and stores nothing
-      LwRow lw{nullptr, G.cef};
+      LwEdge lw{nullptr, G.cef};
       if (LW) lw.w = weight_row(G.wts, G.wT, G.wE, tw + 1);
       const int lane = R & 31;
-      ColView V{*G.cls, G.cent, G.coff, G.llr, B.status, (const char*)B.cns, lw, lane, S >> 5};
+      ColView<LwEdge> V{*G.cls, G.cent, G.coff, G.llr, B.status, (const char*)B.cns, lw, lane, S >> 5};
       const int n3 = V.K.n3;
       // (a check past 32 entries: every slice goes one at a time)
       if ((G.coff[0] & kWideSlice) != 0) V.K.n4 = V.K.n3 = V.K.n2 = V.K.n1;
@@ -1674,9 +1695,9 @@ struct PreBp {
 template <bool LW, class Put>
 __device__ __forceinline__ void prebp_columns(const WinDev& W, const PreBp& X, int t, int first, int st, int lane,
                                               Put put) {
-  LwRow lw{nullptr, W.s_cef};
-  if (LW) lw.w = weight_row(W.wts, W.wT, W.n_edges, t);
-  const ColView V{W.cls, X.cent, X.coff, X.llr, nullptr, (const char*)X.cns, lw, lane, st};
+  LwOrdered lw{nullptr};
+  if (LW) lw.w = weight_row(W.w_col, W.wT, 32 * W.col_cells, t);
+  const ColView<LwOrdered> V{W.cls, X.cent, X.coff, X.llr, nullptr, (const char*)X.cns, lw, lane, st};
   column_pass<LW, true>(V, first, put);
 }
 
@@ -1723,8 +1744,8 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
   cl_sync();  // every CTA of the cluster runs and has set up its arrays
   int t;
   for (t = 1; t <= P.n_pre; ++t) {
-    LwRow lw{nullptr, W.s_ref};
-    if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
+    LwOrdered lw{nullptr};
+    if (LW && t > 1) lw.w = weight_row(W.w_row, W.wT, 128 * W.row_quads, t - 1);
     uint32_t unsat = 0u;
     for (int b = jb; b < je; b += per) {
       const int j0 = b + tid / tpc;
@@ -1749,8 +1770,8 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       t_conv = t - 1;
       break;
     }
-    LwRow lc{nullptr, W.s_cef};
-    if (LW) lc.w = weight_row(W.wts, W.wT, W.n_edges, t);
+    LwOrdered lc{nullptr};
+    if (LW) lc.w = weight_row(W.w_col, W.wT, 32 * W.col_cells, t);
     for (int i = ib + tid; i < ie; i += NT) {
       const int q = i >> 5, c0 = X.coff[q] & (kWideSlice - 1), n = (int)(X.coff[q + 1] & (kWideSlice - 1)) - c0;
       const int ei = c0 * 32 + (i & 31);
@@ -1759,7 +1780,7 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
       for (int u = 0; u < n; ++u) {
         const uint32_t e = X.cent[ei + 32 * u];
         p = __fadd_rn(p, c2v<LW>(*(const CNState*)((const char*)X.cns + (e >> 12)), e, true,
-                                 LW ? lw_at(lc, ei + 32 * u) : 0.0f));
+                                 LW ? lc.one(ei + 32 * u) : 0.0f));
       }
       for (unsigned c = 0; c < C; ++c)  // every CTA reads the whole posterior in its check pass
         cl_st_f32(cl_map(&X.post[i], c), p);
@@ -1875,8 +1896,8 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     for (t = 1; t <= P.n_pre; ++t) {
       // check nodes; each check also takes the parity of the hard decisions it
       // reads, so for t >= 2 the pass is the convergence test of iteration t-1
-      LwRow lw{nullptr, W.s_ref};
-      if (LW && t > 1) lw.w = weight_row(W.wts, W.wT, W.n_edges, t - 1);
+      LwOrdered lw{nullptr};
+      if (LW && t > 1) lw.w = weight_row(W.w_row, W.wT, 128 * W.row_quads, t - 1);
       uint32_t unsat = 0u;
 #pragma unroll 1
       for (int s = warp; s < rw; s += nw) {
@@ -2413,7 +2434,9 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
     // no snapshot yet, every path queued
     if (A.F.pool && threadIdx.x < 2 * kMaxForkNodes) ((int*)(sm + A.L.red))[threadIdx.x] = 0;
     __syncthreads();
-    shot_body<LW, false>(A, shot, sm, stg);
+    // (members without learned weights may share the launch with others)
+    if (LW && A.W.wts) shot_body<true, false>(A, shot, sm, stg);
+    else shot_body<false, false>(A, shot, sm, stg);
   }
 }
 
@@ -2492,6 +2515,20 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   if (A.keep) keep_for_next(A, sm, shot, A.kpath + ((size_t)shot * nb + outp) * A.ns_max, n_short);
   __syncthreads();
   write_outputs(A, sm, shot, false, winner, n_short, t_run, tr);
+}
+
+// Learned weights of a window in the order in which the pre-BP's passes walk its
+// edges, [T][check entries] and [T][column entries], so that they load them
+// side by side instead of through edge ids.  Runs before every decode of the
+// window (the caller may change the weights in between): 1.4 MB for
+// [[144,12,12]] (3,1) windows and T = 25.
+__global__ void __launch_bounds__(256) order_weights_kernel(const float* __restrict__ w, const uint16_t* __restrict__ ref,
+                                                            const uint16_t* __restrict__ cef, int T, int ne, int nrow,
+                                                            int ncol, float* __restrict__ w_row,
+                                                            float* __restrict__ w_col) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
+  if (i < nrow) w_row[(size_t)t * nrow + i] = w[(size_t)t * ne + ref[i]];
+  else if (i < nrow + ncol) w_col[(size_t)t * ncol + (i - nrow)] = w[(size_t)t * ne + cef[i - nrow]];
 }
 
 // ---- Philox4x32-10 (Salmon et al., SC'11) ----
@@ -2778,6 +2815,17 @@ cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem
       if (lw) dev::decode_shot_kernel<true, false, 2><<<grid, threads, smem, st>>>(A);
       else dev::decode_shot_kernel<false, false, 2><<<grid, threads, smem, st>>>(A);
     }
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_order_weights(cudaStream_t st, const WinDev& W) {
+  const int nrow = 128 * W.row_quads, ncol = 32 * W.col_cells;
+  for (int t0 = 0; t0 < W.wT; t0 += 65535) {  // (the grid's y limit)
+    const int T = W.wT - t0 < 65535 ? W.wT - t0 : 65535;
+    dev::order_weights_kernel<<<dim3((unsigned)((nrow + ncol + 255) / 256), (unsigned)T), 256, 0, st>>>(
+        W.wts + (size_t)t0 * W.n_edges, W.s_ref, W.s_cef, T, W.n_edges, nrow, ncol, W.w_row + (size_t)t0 * nrow,
+        W.w_col + (size_t)t0 * ncol);
   }
   return cudaGetLastError();
 }

@@ -112,6 +112,7 @@ struct WinDev {
   // alpha at iteration t (counted from message initialisation); NULL = alpha
   const float* wts;
   int wT;
+  float *w_row, *w_col;  // the same in the order of s_rent / s_cent (order_weights_kernel)
   int n_commit_rows;      // rows [0, n_commit_rows) are the ones the window commits
   // the graph in slices (see the top of the file), checks and columns by label
   int row_quads, col_cells;    // slice totals per lane: check entries in fours, column entries

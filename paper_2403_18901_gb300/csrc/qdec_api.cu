@@ -95,6 +95,8 @@ struct WinGpu {
   // message reuse: this window's column -> the previous window's column of
   // the same DEM column (-1: none); nullptr for the first window
   int16_t* d_prev = nullptr;
+  float* d_wts = nullptr;  // learned weights in the pre-BP's order, room for wts_T iterations
+  int wts_T = 0;
 };
 
 template <class T>
@@ -444,6 +446,27 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   return QD_OK;
 }
 
+// Room for T iterations' learned weights of window k in the pre-BP's order; the
+// first call makes room in every window, so that a decoder's weights are
+// installed window by window without further allocations.
+qd_status ensure_weight_space(qd_decoder* dec, int k, int T) {
+  for (int i = 0; i < (int)dec->wins.size(); ++i) {
+    WinGpu& g = dec->wins[i];
+    if (g.wts_T >= T || (i != k && g.wts_T > 0)) continue;
+    float* p = nullptr;
+    const size_t per = 128 * (size_t)g.dv.row_quads + 32 * (size_t)g.dv.col_cells;
+    QD_CK(cudaMalloc(&p, sizeof(float) * std::max<size_t>(per * T, 4)));
+    cudaFree(g.d_wts);
+    g.d_wts = p;
+    g.wts_T = T;
+    if (g.dv.wts) {  // (its weights are ordered again before every decode)
+      g.dv.w_row = p;
+      g.dv.w_col = p + (size_t)g.dv.wT * 128 * g.dv.row_quads;
+    }
+  }
+  return QD_OK;
+}
+
 // Lay the windows out again when the need for the quantised history changes.
 qd_status update_hist(qd_decoder* dec, const char* who) {
   const bool want = dec->kp.rkq != nullptr || dec->kp.dump != nullptr;
@@ -593,6 +616,7 @@ qd_status qd_decoder_destroy(qd_decoder* dec) {
     cudaFree(w.d_wthr);
     cudaFree(w.d_fork);
     cudaFree(w.d_prev);
+    cudaFree(w.d_wts);
   }
   cudaFree(dec->d_snap);
   cudaFree(dec->d_keep);
@@ -695,7 +719,7 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     char* b = g.d_graph;
     g.dv = qd::WinDev{h.n_rows, h.n_cols, h.n_edges, h.row0, h.n_short, h.short_edges_max, h.n_rows / h.n_blocks,
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
-                      (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0,
+                      (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0, nullptr, nullptr,
                       h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks)),
                       h.row_quads, h.col_cells, (const uint16_t*)(b + s_re), (const uint32_t*)(b + s_ce),
                       (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
@@ -849,6 +873,7 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
     path_mode = false;
   const qd::ForkDev fk = fork_dev(dec, g);
   const qd::ReuseDev ru = reuse_dev(dec, g);
+  if (g.dv.wts) QD_CK(qd::launch_order_weights(st, g.dv));
   if (global) {
     QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
     const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * g.grid_g);
@@ -939,10 +964,13 @@ qd_status qd_decoder_set_weights(qd_decoder* dec, int k, const float* w, int T) 
   QD_REQ(dec, "null argument");
   QD_REQ(k >= 0 && k < (int)dec->wins.size(), "qd_decoder_set_weights: window out of range");
   QD_REQ(w == nullptr || T >= 1, "qd_decoder_set_weights: T must be >= 1");
-  const float* old_w = dec->wins[k].dv.wts;
-  const int old_t = dec->wins[k].dv.wT;
-  dec->wins[k].dv.wts = w;
-  dec->wins[k].dv.wT = w ? T : 0;
+  if (w) QD_CK_ST(ensure_weight_space(dec, k, T));
+  const qd::WinDev old = dec->wins[k].dv;
+  WinGpu& g = dec->wins[k];
+  g.dv.wts = w;
+  g.dv.wT = w ? T : 0;
+  g.dv.w_row = w ? g.d_wts : nullptr;
+  g.dv.w_col = w ? g.d_wts + (size_t)T * 128 * g.dv.row_quads : nullptr;
   // the layouts keep the shortened edges' full-window ids only while some
   // window has learned weights
   bool want = false;
@@ -950,8 +978,7 @@ qd_status qd_decoder_set_weights(qd_decoder* dec, int k, const float* w, int T) 
   if (want != dec->lw_on) {
     dec->lw_on = want;
     if (qd_status st = configure_layouts(dec, dec->hist_on, "qd_decoder_set_weights")) {
-      dec->wins[k].dv.wts = old_w;
-      dec->wins[k].dv.wT = old_t;
+      g.dv = old;
       dec->lw_on = !want;
       return st;
     }
@@ -1138,6 +1165,7 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
     if (dec->launch_mode == 0) path_mode = n_shots * 4 <= dec->sm_count;
     if (path_mode && (n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.path_fits || global))
       path_mode = false;
+    if (g.dv.wts) QD_CK(qd::launch_order_weights(st, g.dv));
     if (path_mode) {
       const int cps = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
       QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
@@ -1174,6 +1202,7 @@ struct qd_batch {
     size_t budget = 0, smem = 0;
     unsigned q_off = 0;
     std::vector<qd::Layout> L;  // per member (unused where the member has no such window)
+    std::vector<int> form;      // per member: what its layout was made for (member_form)
   };
   std::vector<Step> steps;
   int* d_work = nullptr;  // one counter per step
@@ -1181,11 +1210,15 @@ struct qd_batch {
 };
 
 namespace {
+// The member's state its layouts depend on: learned weights, quantised history.
+int member_form(const qd_decoder* d) { return (d->lw_on ? 1 : 0) | (d->hist_on ? 2 : 0); }
+
 // CTAs of `warps` warps with at most `budget` bytes of dynamic shared memory:
 // each member's layout takes as many path slots (<= warps) as fit.
 qd_status batch_plan(qd_batch* b, int j, int warps, size_t budget) {
   qd_batch::Step S;
   S.L.assign(b->mem.size(), qd::Layout{});
+  for (const qd_decoder* d : b->mem) S.form.push_back(member_form(d));
   unsigned mx = 0;
   for (size_t i = 0; i < b->mem.size(); ++i) {
     const qd_decoder* d = b->mem[i];
@@ -1268,6 +1301,8 @@ qd_status batch_decode(qd_batch* b, int j, const std::vector<qd::BatchMember>& a
   long long tot = 0;
   for (const auto& x : m) tot += x.n;
   QD_CK(cudaMemsetAsync(b->d_work + j, 0, sizeof(int), st));
+  for (const auto& x : m)
+    if (x.W->wts) QD_CK(qd::launch_order_weights(st, *x.W));
   const long long grid = std::min<long long>(tot, (long long)b->sm_count * S.blocks);
   QD_CK(qd::launch_decode_batch(st, (int)grid, 32 * S.warps, S.smem, S.q_off, b->d_work + j, m.data(),
                                 (int)m.size()));
@@ -1360,6 +1395,14 @@ qd_status qd_batch_step(qd_batch* b, int step, uint32_t* const* det_bits, const 
     QD_REQ(n_shots[i] == 0 || (det_bits[i] && obs_pred[i] && residue_fail[i]),
            "qd_batch_step: null buffer of member " + std::to_string(i));
   }
+  // weights or a ranker installed (or removed) since the step was planned
+  for (size_t i = 0; i < b->mem.size(); ++i)
+    if (b->steps[step].form[i] != member_form(b->mem[i])) {
+      const int warps = b->steps[step].warps;
+      const size_t budget = b->steps[step].budget;
+      QD_CK_ST(batch_plan(b, step, warps, budget));
+      break;
+    }
   std::vector<qd::BatchMember> m;
   if (!batch_members(b, step, det_bits, n_shots, obs_pred, residue_fail, m)) return QD_OK;
   cudaStream_t st = (cudaStream_t)stream;

@@ -108,6 +108,8 @@ cudaError_t batch_occupancy(int threads, size_t smem, int* blocks);
 cudaError_t launch_decode_batch(cudaStream_t st, int grid, int threads, size_t smem, unsigned q_off, int* work,
                                 const BatchMember* m, int n);
 cudaError_t launch_commit_batch(cudaStream_t st, const BatchMember* m, int n);
+// Puts the window's learned weights in the pre-BP's order (w_row, w_col).
+cudaError_t launch_order_weights(cudaStream_t st, const WinDev& W);
 cudaError_t launch_sample(cudaStream_t st, int n_cols, const uint32_t* thr, const int* cptr,
                           const int* cdet, const uint32_t* cobs, int det_words,
                           unsigned long long seed, unsigned long long off, long long n, uint32_t* det,
