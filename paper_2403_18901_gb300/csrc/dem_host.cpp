@@ -511,25 +511,29 @@ namespace {
 // second visits to a bank group (a record read by two lanes is one visit).
 void spread_columns(const WindowHost& o, const std::vector<uint16_t>& rlab, uint16_t* cols, int n, int deg, int lane0) {
   constexpr int kLook = 96;
-  std::vector<uint16_t> left(cols, cols + n);
-  std::vector<std::vector<int>> seen(deg);  // per entry: the eight lanes' check labels
-  size_t head = 0;
+  std::vector<uint16_t> rows((size_t)n * deg);  // check labels of the columns, in `cols`' order
+  std::vector<int> left(n);
   for (int i = 0; i < n; ++i) {
-    if ((lane0 + i) % 8 == 0)
-      for (auto& v : seen) v.clear();
-    size_t pick = head;
-    int best = 1 << 30;
-    for (size_t x = head; x < left.size() && x < head + kLook && best > 0; ++x) {
+    left[i] = i;
+    for (int u = 0; u < deg; ++u) rows[(size_t)i * deg + u] = rlab[o.col_rows[o.col_ptr[cols[i]] + u]];
+  }
+  std::vector<uint16_t> seen((size_t)deg * 8), out(n);  // per entry: the eight lanes' check labels
+  int have = 0;
+  for (int i = 0; i < n; ++i) {
+    if ((lane0 + i) % 8 == 0) have = 0;
+    int pick = i, best = 1 << 30;
+    for (int x = i; x < n && x < i + kLook && best > 0; ++x) {
+      const uint16_t* r = rows.data() + (size_t)left[x] * deg;
       int cost = 0;
-      for (int u = 0; u < deg; ++u) {
-        const int r = rlab[o.col_rows[o.col_ptr[left[x]] + u]];
+      for (int u = 0; u < deg && cost < best; ++u) {
+        const uint16_t* v = seen.data() + 8 * u;
         int same = 0;
-        for (int v : seen[u]) {
-          if (v == r) {
+        for (int y = 0; y < have; ++y) {
+          if (v[y] == r[u]) {
             same = 0;
             break;
           }
-          same += (v & 7) == (r & 7);
+          same += ((v[y] ^ r[u]) & 7) == 0;
         }
         cost += same;
       }
@@ -538,12 +542,14 @@ void spread_columns(const WindowHost& o, const std::vector<uint16_t>& rlab, uint
         pick = x;
       }
     }
-    const uint16_t c = left[pick];
-    for (size_t x = pick; x > head; --x) left[x] = left[x - 1];
-    ++head;
-    for (int u = 0; u < deg; ++u) seen[u].push_back(rlab[o.col_rows[o.col_ptr[c] + u]]);
-    cols[i] = c;
+    const int c = left[pick];
+    for (int x = pick; x > i; --x) left[x] = left[x - 1];
+    left[i] = c;
+    for (int u = 0; u < deg; ++u) seen[8 * u + have] = rows[(size_t)c * deg + u];
+    ++have;
+    out[i] = cols[c];
   }
+  std::copy(out.begin(), out.end(), cols);
 }
 
 // Positions for the entries of a slice's 32 checks (lab[lane]: their column
@@ -554,24 +560,40 @@ void spread_columns(const WindowHost& o, const std::vector<uint16_t>& rlab, uint
 // position of the lane's i-th entry.
 void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::vector<std::vector<int>>& pos) {
   const int n = (int)lab.size();
-  std::vector<std::vector<int>> left(n);  // entry indexes
+  struct Lane {
+    uint8_t bank[kMaxRowDeg], ent[kMaxRowDeg];  // the entries left: bank, index
+    int k;
+  };
+  std::vector<Lane> left(n);
   int most = 0;
   for (int l = 0; l < n; ++l) {
-    for (int i = 0; i < (int)lab[l].size(); ++i) left[l].push_back(i);
-    most = std::max(most, (int)lab[l].size());
+    left[l].k = (int)lab[l].size();
+    for (int i = 0; i < left[l].k; ++i) {
+      left[l].bank[i] = (uint8_t)(lab[l][i] & 31);
+      left[l].ent[i] = (uint8_t)i;
+    }
+    most = std::max(most, left[l].k);
   }
   for (int u = 0; u < most; ++u) {
     int lane_of[32], mine[32];
     std::fill(lane_of, lane_of + 32, -1);
     std::fill(mine, mine + 32, -1);
-    std::vector<char> tried(32);
+    uint32_t tried = 0;
     // augmenting paths; lanes with the most entries left choose first
     auto match = [&](auto&& self, int l) -> bool {
-      for (int i : left[l]) {
-        const int b = lab[l][i] & 31;
-        if (tried[b]) continue;
-        tried[b] = 1;
-        if (lane_of[b] < 0 || self(self, lane_of[b])) {
+      for (int i = 0; i < left[l].k; ++i) {  // a free bank, if there is one
+        const int b = left[l].bank[i];
+        if (lane_of[b] < 0) {
+          lane_of[b] = l;
+          mine[l] = i;
+          return true;
+        }
+      }
+      for (int i = 0; i < left[l].k; ++i) {
+        const int b = left[l].bank[i];
+        if (tried >> b & 1u) continue;
+        tried |= 1u << b;
+        if (self(self, lane_of[b])) {
           lane_of[b] = l;
           mine[l] = i;
           return true;
@@ -579,25 +601,29 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
       }
       return false;
     };
-    std::vector<int> order;
+    int order[32], m = 0, load[32] = {};
     for (int l = 0; l < n; ++l)
-      if (!left[l].empty()) order.push_back(l);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
-    int load[32] = {};
-    for (int l : order) {
-      std::fill(tried.begin(), tried.end(), 0);
-      match(match, l);
+      if (left[l].k) order[m++] = l;
+    std::stable_sort(order, order + m, [&](int a, int b) { return left[a].k > left[b].k; });
+    for (int x = 0; x < m; ++x) {
+      tried = 0;
+      match(match, order[x]);
     }
-    for (int l : order)
-      if (mine[l] >= 0) load[lab[l][mine[l]] & 31]++;
-    for (int l : order) {
-      if (mine[l] < 0) {
-        for (int i : left[l])
-          if (mine[l] < 0 || load[lab[l][i] & 31] < load[lab[l][mine[l]] & 31]) mine[l] = i;
-        load[lab[l][mine[l]] & 31]++;
+    for (int x = 0; x < m; ++x)
+      if (mine[order[x]] >= 0) load[left[order[x]].bank[mine[order[x]]]]++;
+    for (int x = 0; x < m; ++x) {
+      Lane& a = left[order[x]];
+      int& i = mine[order[x]];
+      if (i < 0) {
+        i = 0;
+        for (int y = 1; y < a.k; ++y)
+          if (load[a.bank[y]] < load[a.bank[i]]) i = y;
+        load[a.bank[i]]++;
       }
-      pos[l][mine[l]] = first + u;
-      left[l].erase(std::find(left[l].begin(), left[l].end(), mine[l]));
+      pos[order[x]][a.ent[i]] = first + u;
+      --a.k;
+      a.bank[i] = a.bank[a.k];
+      a.ent[i] = a.ent[a.k];
     }
   }
 }
@@ -610,8 +636,31 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
 // The order of a check's entries and of the columns changes no value.  Counted
 // for an interior [[144,12,12]] (3,1) window: 520 -> 342 wavefronts for the 228
 // gathers of a check pass, 1536 -> 987 for the 840 of a variable pass.
-bool build_slices(WindowHost& o) {
+// Building them takes 1.3 ms there and a stream has three distinct matrices
+// (first, interior, last), so a window takes the slices of the one before it
+// where the matrix is the same: seven built anew cost a decoder 20 ms.
+bool build_slices(WindowHost& o, const WindowHost* like) {
   const int nr = o.n_rows, nc = o.n_cols;
+  if (like && like->n_rows == nr && like->col_ptr == o.col_ptr && like->col_rows == o.col_rows &&
+      like->n_short == o.n_short && like->short_edges_max == o.short_edges_max) {  // the interior windows share one graph
+    o.row_quads = like->row_quads;
+    o.col_cells = like->col_cells;
+    o.srow_quads = like->srow_quads;
+    o.scol_cells = like->scol_cells;
+    o.max_row_deg = like->max_row_deg;
+    std::copy(like->cls, like->cls + 4, o.cls);
+    o.s_rent = like->s_rent;
+    o.s_cent = like->s_cent;
+    o.s_roff = like->s_roff;
+    o.s_coff = like->s_coff;
+    o.s_row = like->s_row;
+    o.s_col = like->s_col;
+    o.s_ref = like->s_ref;
+    o.s_cef = like->s_cef;
+    o.s_llr.assign(like->s_llr.size(), 0.0f);
+    for (int l = 0; l < nc; ++l) o.s_llr[l] = o.llr[o.s_col[l]];
+    return true;
+  }
   const int nrs = (nr + 31) / 32, ncs = (nc + 31) / 32;
   auto cdeg = [&](int c) { return o.col_ptr[c + 1] - o.col_ptr[c]; };
   auto rdeg = [&](int j) { return o.row_ptr[j + 1] - o.row_ptr[j]; };

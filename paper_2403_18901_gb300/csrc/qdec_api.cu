@@ -708,7 +708,7 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     dec->corr_words = std::max(dec->corr_words, (h.n_cols + 31) / 32);
     dec->ns_max = std::max(dec->ns_max, h.n_short);
     dec->sw_max = std::max(dec->sw_max, (h.n_short + 31) / 32);
-    if (!qd::build_slices(g.h)) return QD_EUNSUPPORTED;
+    if (!qd::build_slices(g.h, w ? &dec->wins[w - 1].h : nullptr)) return QD_EUNSUPPORTED;
     Blob blob;
     auto put = [&](const auto& v) { return blob.put(v); };
     const size_t o_cp = put(h.col_ptr), o_cr = put(h.col_rows), o_rp = put(h.row_ptr), o_re = put(h.row_ent),

@@ -69,8 +69,10 @@ struct WmsHost {
 };
 WmsHost build_wms(const WindowHost& h);
 
-// The graph in slices (s_* of WindowHost) and the bounds for its shortened graphs.
-bool build_slices(WindowHost& o);
+// The graph in slices (s_* of WindowHost) and the bounds for its shortened
+// graphs; taken from `like` (a window whose slices are built) when its matrix is
+// the same.
+bool build_slices(WindowHost& o, const WindowHost* like = nullptr);
 
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max);
 cudaError_t set_decode_smem(size_t bytes);

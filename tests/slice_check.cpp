@@ -194,6 +194,16 @@ int main(int argc, char** argv) {
       return std::printf("window %d: %s\n", k, qd::last.c_str()), 1;
     if (h.n_cols == 0) continue;
     if (!check_graph(h)) return 1;
+    qd::WindowHost same = h, next;  // a window with the same matrix and other priors takes its slices
+    for (float& l : same.llr) l *= 1.5f;
+    same.s_rent.clear();
+    same.s_col.clear();
+    if (!qd::build_slices(same, &h) || !check_graph(same)) return 1;
+    if (same.s_rent != h.s_rent) return std::printf("window %d: slices not taken\n", k), 1;
+    if (qd::build_window(d, W, F, k ? k - 1 : 0, shorten != 0, next, merge) && next.n_cols) {
+      qd::build_slices(next, &h);  // whatever its matrix
+      if (!check_graph(next)) return 1;
+    }
     std::vector<int> cols(h.n_cols);
     for (int c = 0; c < h.n_cols; ++c) cols[c] = h.s_col[c];  // the highest degrees first
     for (int t = 0; t < trials; ++t) {
