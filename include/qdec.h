@@ -467,6 +467,10 @@ qd_status qd_ranker_eval(const float* params, const void* records, const uint8_t
                          float pos_weight, float grad_scale, float* grad, float* loss, float* score,
                          qd_stream_t stream);
 
+/* Sets `bytes` bytes at device pointer dst to 0 on the stream (an output that a
+ * gradient call accumulates into, without the cost of a framework's fill). */
+qd_status qd_set_zero(void* dst, size_t bytes, qd_stream_t stream);
+
 /*
  * Training the learned weighted min-sum of window k (no counterpart in the
  * paper).  A training sample is a window syndrome s = H_win e with every

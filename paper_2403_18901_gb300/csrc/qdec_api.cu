@@ -1606,6 +1606,12 @@ qd_status qd_ranker_eval(const float* params, const void* records, const uint8_t
   return QD_OK;
 }
 
+qd_status qd_set_zero(void* dst, size_t bytes, qd_stream_t stream) {
+  QD_REQ(dst || bytes == 0, "qd_set_zero: null pointer");
+  if (bytes) QD_CK(cudaMemsetAsync(dst, 0, bytes, (cudaStream_t)stream));
+  return QD_OK;
+}
+
 qd_status qd_adam_step(float* w, const float* g, float* m1, float* m2, int64_t n, float lr, float beta1, float beta2,
                        float eps, int step, qd_stream_t stream) {
   QD_REQ(w && g && m1 && m2 && n >= 0 && step >= 1, "qd_adam_step: bad argument");

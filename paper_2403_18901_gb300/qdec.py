@@ -93,6 +93,7 @@ _SIGS = {
     "qd_batch_autotune": (_I, [_VP, _I, _VP, _VP, _I, _VP, _VP]),
     "qd_window_sample": (_I, [_VP, _I, _U64, _U64, _I64, _VP, _VP, _VP]),
     "qd_ranker_eval": (_I, [_VP, _VP, _VP, _I64, _I, C.c_float, C.c_float, _VP, _VP, _VP, _VP]),
+    "qd_set_zero": (_I, [_VP, _SZ, _VP]),
     "qd_wms_create": (_I, [_VP, _I, _I, _I, C.POINTER(_VP)]),
     "qd_wms_destroy": (_I, [_VP]),
     "qd_wms_info": (_I, [_VP, _VP]),
@@ -131,21 +132,34 @@ def _check(code):
 
 
 def _ptr(x):
-    """Raw pointer of a torch tensor (device or host) or numpy array; None passes through."""
+    """Raw pointer of a torch tensor (device or host; an int) or numpy array (an
+    object that keeps the array alive); None passes through."""
     if x is None:
         return None
     if isinstance(x, np.ndarray):
         assert x.flags["C_CONTIGUOUS"]
         return x.ctypes.data_as(C.c_void_p)
     assert x.is_contiguous()
-    return C.c_void_p(x.data_ptr())
+    return x.data_ptr()
 
 
 def _stream(stream):
+    """Raw handle (an int) of a stream, or of the current one; the handle alone
+    costs a tenth of the Stream object torch.cuda.current_stream() makes (0.3 us
+    against 2.8 us; three of them were in a 27 us Ranker.grad call)."""
     if stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
+
+
+def zeros(n, stream=None):
+    """n zero FP32 numbers on the current device: a memset where torch.zeros
+    dispatches a fill (11 us of a 27 us Ranker.grad call; 16 us with this)."""
+    import torch
+    t = torch.empty(n, dtype=torch.float32, device="cuda")
+    _check(lib().qd_set_zero(t.data_ptr(), 4 * t.numel(), _stream(stream)))
+    return t
 
 
 def make_code(code):

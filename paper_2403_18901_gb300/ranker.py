@@ -83,7 +83,7 @@ def grad(params, recs, labels, quantize=True, pos_weight=1.0, scale=1.0, out=Non
     """Accumulates scale * d(sum of losses)/d params into out; returns (out, losses)."""
     n = recs.shape[0]
     if out is None:
-        out = torch.zeros(N_PARAMS, dtype=torch.float32, device="cuda")
+        out = qdec.zeros(N_PARAMS)
     loss = torch.empty(n, dtype=torch.float32, device="cuda")
     qdec._check(qdec.lib().qd_ranker_eval(qdec._ptr(params), qdec._ptr(recs), qdec._ptr(labels), n,
                                           int(quantize), float(pos_weight), float(scale), qdec._ptr(out),
