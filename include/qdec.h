@@ -509,21 +509,22 @@ qd_status qd_adam_step(float* w, const float* g, float* m1, float* m2, int64_t n
                        float eps, int step, qd_stream_t stream);
 
 /* Launch shape of qd_decode_windows (results are identical in every shape):
- * 0 automatic (default): path mode for batches that leave most SMs idle,
- * otherwise shot mode; 1 shot mode: persistent CTAs, one warp per decision
- * path; 2 path mode: one CTA per (shot, decision path) for the lowest
- * latency, the path CTAs of a shot launched as a thread-block cluster (up to
- * 8 CTAs, padded with idle CTAs to whole clusters) that splits the shot's
- * pre-BP, at most 64 shots per call (larger batches fall back to shot mode);
+ * 0 automatic (default): path mode for batches of at most half as many shots as
+ * there are SMs, otherwise shot mode; 1 shot mode: persistent CTAs, one warp per
+ * decision path, one to three CTAs per SM by the batch's size; 2 path mode: one
+ * CTA of 512, 256 or 128 threads (by the batch's size) per (shot, decision path)
+ * for the lowest latency, the path CTAs of a shot launched as a thread-block
+ * cluster (up to 8 CTAs, padded with idle CTAs to whole clusters) that splits the
+ * shot's pre-BP, at most 64 shots per call (larger batches fall back to shot mode);
  * 3 shot mode with every CTA's pre-BP scratch and path states in global
  * memory (L2 / HBM) instead of shared memory -- the shape a window too large
  * for shared memory always uses (chosen at decoder creation, which allocates
  * those regions; mode 3 allocates them for every window here). */
 qd_status qd_decoder_set_launch(qd_decoder* dec, int mode);
 
-/* Launch plan of window k: out[0] shared bytes per CTA in shot mode,
- * out[1] its threads, out[2] its CTAs per SM, out[3] shared bytes per CTA in
- * path mode, out[4] its threads, out[5] SM count, out[6] CTAs per cluster in
+/* Launch plan of window k: out[0] shared bytes per CTA in shot mode (for large
+ * batches), out[1] its threads, out[2] its CTAs per SM, out[3] shared bytes per
+ * CTA in path mode (with the most threads), out[4] its threads, out[5] SM count, out[6] CTAs per cluster in
  * path mode (they split each shot's pre-BP; 1: every path CTA runs it whole),
  * out[7] path-mode CTAs per shot (the paths rounded up to whole clusters). */
 qd_status qd_decoder_launch_info(const qd_decoder* dec, int k, int out[8]);

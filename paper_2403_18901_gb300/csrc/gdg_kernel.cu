@@ -29,7 +29,8 @@
 //     paths, and at every step boundary a warp parks its path for a waiting
 //     one with more steps left (snapshots in a per-CTA pool in global memory;
 //     see ForkCtx);
-//   path mode (latency, small batches): one CTA per (shot, path); the path
+//   path mode (latency, small batches): one CTA per (shot, path), of fewer
+//     threads and more to an SM the more there are; the path
 //     CTAs of a shot form a thread-block cluster that splits the pre-BP over
 //     distributed shared memory, each CTA then ranks, shortens and runs its
 //     one path with all its threads, stores the result in global scratch,

@@ -62,36 +62,49 @@ constexpr int kShotWarps = 8;
 // [[144,12,12]] run 4 % faster so than with two and 128 registers (the paper
 // preset 5 %); with learned weights or a ranker 3 and 6 % slower.
 constexpr int kShotCtas = 3;
+// Path mode's CTAs: 512 threads, one per SM; 256, two; 128, four (the same 128
+// registers a thread), see path_shape.
+constexpr int kPathShapes = 3;
 constexpr int kPathThreads = 512;
 constexpr long long kPathModeMaxShots = 64;
 constexpr int kCounters = 8;
 
+// Shot mode on up to `ctas` CTAs per SM, and its snapshot plan (qd::ForkDev):
+// queue order [nb], then the node chain [nb][dmx]; fork_nodes = 0: none.
+struct ShotShape {
+  qd::Layout L{};
+  int ctas = 2;         // CTAs per SM planned
+  int grid_per_sm = 1;  // and resident
+  int wave = 1;         // path slots of a typical shot
+  const int16_t* d_fork = nullptr;  // in WinGpu::d_fork
+  int fork_nodes = 0;
+  bool fork_on = false;
+};
+
+struct PathShape {
+  qd::Layout L{};
+  bool fits = false;
+  int pcl = 1;  // CTAs per cluster sharing a shot's pre-BP
+};
+
 struct WinGpu {
   qd::WindowHost h;
   qd::WinDev dv{};
-  qd::Layout L{};   // shot mode
-  qd::Layout Lp{};  // path mode
+  ShotShape sh[kShotCtas];  // shot mode, by CTAs per SM
+  int best = 0;             // the one for large batches
+  int16_t* d_fork = nullptr;  // the shapes' snapshot plans
+  PathShape pa[kPathShapes];  // path mode, kPathThreads >> i threads
   char* d_graph = nullptr;
   int* d_ccptr = nullptr;  // committed columns: CSR of their global detector ids
   int* d_ccdet = nullptr;
   uint32_t* d_ccobs = nullptr;
-  int grid_per_sm = 1;
-  int shot_warps = kShotWarps;
-  int wave = 1;  // path slots of a typical shot
-  int ctas = 2;  // CTAs per SM planned
   uint32_t* d_wthr = nullptr;  // window-local sampling thresholds (on first use)
   // union region in global memory (windows too large for shared memory, or
   // launch mode 3): layout, CTAs per SM, and whether the shared-memory
   // layouts fit at all
   qd::Layout Lg{};
   int grid_g = 1;
-  bool fits = true, path_fits = true;
-  int pcl = 1;  // path mode: CTAs per cluster sharing a shot's pre-BP
-  // shot mode's snapshot plan (qd::ForkDev): queue order [nb], then the
-  // node chain [nb][dmx]; fork_nodes = 0: none
-  int16_t* d_fork = nullptr;
-  int fork_nodes = 0;
-  bool fork_on = false;
+  bool fits = true;
   // message reuse: this window's column -> the previous window's column of
   // the same DEM column (-1: none); nullptr for the first window
   int16_t* d_prev = nullptr;
@@ -306,9 +319,11 @@ int typical_slots(const qd::Layout& L, const qd::WindowHost& h, int most) {
 
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   struct Conf {
-    qd::Layout L, Lp, Lg;
-    int shot_warps, wave, ctas, grid_per_sm, grid_g, pcl;
-    bool fits, path_fits;
+    ShotShape sh[kShotCtas];
+    PathShape pa[kPathShapes];
+    qd::Layout Lg;
+    int best, grid_g;
+    bool fits;
   };
   const int optin = dec->smem_optin;
   const int nb = dec->kp.nb;
@@ -316,33 +331,31 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   std::vector<Conf> cf(dec->wins.size());
   for (size_t w = 0; w < cf.size(); ++w) {
     Conf& c = cf[w];
-    c.pcl = 1;
     const auto& h = dec->wins[w].h;
     auto lay = [&](unsigned budget, bool glob = false) {
       return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob);
     };
-    // CTAs per SM: the most resident decision-path warps (CTAs x slots a
-    // typical shot gets); ties to fewer CTAs, which have room to stage more of
-    // the window graph
+    // CTAs per SM: for large batches the most resident decision-path warps
+    // (CTAs x slots a typical shot gets); ties to fewer CTAs, which have room to
+    // stage more of the window graph.  Smaller batches: see shot_shape.
     int best = 0;
     c.fits = false;
-    c.ctas = 2;
-    c.shot_warps = kShotWarps;
-    c.wave = 1;
+    c.best = 0;
     for (int n = 1; n <= (dec->lw_on || hist ? 2 : kShotCtas); ++n) {
       const unsigned budget = smem_budget(dec, n);
-      qd::Layout Ls = lay(budget);
-      if (Ls.total > budget) continue;
-      Ls.total = budget;  // the slots take what the budget holds
+      ShotShape& s = c.sh[n - 1];
+      s.L = lay(budget);
+      if (s.L.total > budget) break;  // (the budgets fall)
+      s.L.total = budget;  // the slots take what the budget holds
       int blocks = 0;
-      QD_CK(qd::decode_occupancy(0, n, 32 * kShotWarps, Ls.total, &blocks));
-      const int sl = typical_slots(Ls, h, kShotWarps);
-      if (std::min(blocks, n) * sl > best) {
-        best = std::min(blocks, n) * sl;
-        c.L = Ls;
+      QD_CK(qd::decode_occupancy(0, n, 32 * kShotWarps, s.L.total, &blocks));
+      s.ctas = n;
+      s.grid_per_sm = std::max(1, blocks);
+      s.wave = typical_slots(s.L, h, kShotWarps);
+      if (std::min(blocks, n) * s.wave > best) {
+        best = std::min(blocks, n) * s.wave;
+        c.best = n - 1;
         c.fits = true;
-        c.ctas = n;
-        c.wave = sl;
       }
     }
     // the union region in global memory: eight path slots, shared memory for
@@ -358,65 +371,72 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     QD_CK(qd::decode_occupancy(3, 2, 32 * kShotWarps, c.Lg.U, &bg));
     c.grid_g = std::max(1, bg);
     if (!c.fits) {  // shot mode streams the path state through L2 / HBM
-      c.L = c.Lg;
-      c.wave = kShotWarps;
+      c.sh[0] = ShotShape{};
+      c.sh[0].L = c.Lg;
+      c.sh[0].wave = kShotWarps;
+      c.sh[0].grid_per_sm = c.grid_g;
     }
-    c.Lp = lay((unsigned)optin);
-    c.path_fits = c.Lp.total <= (unsigned)optin;
-    // path mode: the largest cluster (8, 4 or 2 CTAs, at most the number of
-    // paths) that can be resident, its CTAs splitting the pre-BP of a shot
-    c.pcl = 1;
-    for (int C = 8; C >= 2 && c.path_fits; C >>= 1) {
-      if (C > nb || h.n_rows < 2 * C || h.n_cols < 2 * C) continue;
-      int ncl = 0;
-      if (qd::path_cluster_occupancy(kPathThreads, c.Lp.total, C, &ncl) != cudaSuccess) {
-        (void)cudaGetLastError();
-        continue;
-      }
-      if (ncl >= 1) {
-        c.pcl = C;
-        break;
+    smem_max = std::max<size_t>(smem_max, c.fits ? 0u : c.Lg.U);
+    for (int i = 0; i <= c.best && c.fits; ++i) smem_max = std::max<size_t>(smem_max, c.sh[i].L.total);
+    for (int i = 0; i < kPathShapes; ++i) {
+      PathShape& s = c.pa[i];
+      const unsigned budget = smem_budget(dec, 1 << i);
+      s.L = lay(budget);
+      s.fits = s.L.total <= budget;
+      if (!s.fits) break;
+      smem_max = std::max<size_t>(smem_max, s.L.total);
+      // the largest cluster (8, 4 or 2 CTAs, at most the number of paths) that
+      // can be resident, its CTAs splitting the pre-BP of a shot
+      for (int C = 8; C >= 2; C >>= 1) {
+        if (C > nb || h.n_rows < 2 * C || h.n_cols < 2 * C) continue;
+        int ncl = 0;
+        if (qd::path_cluster_occupancy(kPathThreads >> i, s.L.total, C, &ncl) != cudaSuccess) {
+          (void)cudaGetLastError();
+          continue;
+        }
+        if (ncl >= 1) {
+          s.pcl = C;
+          break;
+        }
       }
     }
-    smem_max = std::max<size_t>(smem_max, std::max(c.fits ? c.L.total : c.Lg.U, c.path_fits ? c.Lp.total : 0u));
-    int blocks = 0;
-    QD_CK(qd::decode_occupancy(c.fits ? 0 : 3, c.ctas, 32 * c.shot_warps, c.fits ? c.L.total : c.Lg.U,
-                               &blocks));
-    c.grid_per_sm = std::max(1, blocks);
   }
   for (size_t w = 0; w < cf.size(); ++w) {
     WinGpu& g = dec->wins[w];
-    g.L = cf[w].L;
-    g.Lp = cf[w].Lp;
+    std::copy(cf[w].sh, cf[w].sh + kShotCtas, g.sh);
+    std::copy(cf[w].pa, cf[w].pa + kPathShapes, g.pa);
+    g.best = cf[w].best;
     g.Lg = cf[w].Lg;
     g.grid_g = cf[w].grid_g;
     g.fits = cf[w].fits;
-    g.path_fits = cf[w].path_fits;
-    g.pcl = cf[w].pcl;
-    g.shot_warps = cf[w].shot_warps;
-    g.wave = cf[w].wave;
-    g.ctas = cf[w].ctas;
-    g.grid_per_sm = cf[w].grid_per_sm;
   }
   QD_CK_ST(ensure_uscratch(dec, dec->launch_mode == 3));
-  // shot mode's snapshot plans (one per window: the first wave is a typical
-  // shot's slot count) and one snapshot pool per resident CTA
+  // shot mode's snapshot plans (one per window and shape: the first wave is a
+  // typical shot's slot count) and one snapshot pool per resident CTA
   size_t cta_bytes = 0;
   int ctas = 0;
+  const size_t plan = (size_t)dec->kp.nb * (3 + dec->dmx);
   for (WinGpu& g : dec->wins) {
-    const ForkPlan F = fork_plan(dec->kp, dec->dmx, g.wave);
-    g.fork_on = F.on;
-    g.fork_nodes = F.n_nodes;
-    if (!F.on) continue;
-    std::vector<int16_t> v(F.order);
-    v.insert(v.end(), F.chain.begin(), F.chain.end());
-    v.insert(v.end(), F.fnode.begin(), F.fnode.end());
-    v.insert(v.end(), F.fdep.begin(), F.fdep.end());
-    if (!g.d_fork) QD_CK(cudaMalloc(&g.d_fork, sizeof(int16_t) * (size_t)dec->kp.nb * (3 + dec->dmx)));
+    std::vector<int16_t> v;
+    for (int i = 0; i <= g.best; ++i) {
+      ShotShape& s = g.sh[i];
+      const ForkPlan F = fork_plan(dec->kp, dec->dmx, s.wave);
+      s.fork_on = F.on;
+      s.fork_nodes = F.n_nodes;
+      if (!F.on) continue;
+      v.resize(plan * i);
+      v.insert(v.end(), F.order.begin(), F.order.end());
+      v.insert(v.end(), F.chain.begin(), F.chain.end());
+      v.insert(v.end(), F.fnode.begin(), F.fnode.end());
+      v.insert(v.end(), F.fdep.begin(), F.fdep.end());
+      // node snapshots, then one parking snapshot per path
+      cta_bytes = std::max(cta_bytes, (size_t)(F.n_nodes + dec->kp.nb) * (qd::kSnapHeaderBytes + s.L.b_size));
+      ctas = std::max(ctas, dec->sm_count * std::max(s.grid_per_sm, g.grid_g));
+    }
+    if (v.empty()) continue;
+    if (!g.d_fork) QD_CK(cudaMalloc(&g.d_fork, sizeof(int16_t) * plan * kShotCtas));
     QD_CK(cudaMemcpy(g.d_fork, v.data(), sizeof(int16_t) * v.size(), cudaMemcpyHostToDevice));
-    // node snapshots, then one parking snapshot per path
-    cta_bytes = std::max(cta_bytes, (size_t)(F.n_nodes + dec->kp.nb) * (qd::kSnapHeaderBytes + g.L.b_size));
-    ctas = std::max(ctas, dec->sm_count * std::max(g.grid_per_sm, g.grid_g));
+    for (int i = 0; i <= g.best; ++i) g.sh[i].d_fork = g.d_fork + plan * i;
   }
   if (cta_bytes > dec->snap_cta_bytes || ctas > dec->snap_ctas) {
     const size_t cb = std::max(cta_bytes, dec->snap_cta_bytes);
@@ -431,7 +451,8 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   }
   if (dec->P.reuse_msgs) {  // candidate paths' kept values: one set per resident CTA, or per path-mode shot
     int cmax = 0;
-    for (const WinGpu& g : dec->wins) cmax = std::max(cmax, dec->sm_count * std::max(g.grid_per_sm, g.grid_g));
+    for (const WinGpu& g : dec->wins)
+      for (int i = 0; i <= g.best; ++i) cmax = std::max(cmax, dec->sm_count * std::max(g.sh[i].grid_per_sm, g.grid_g));
     const size_t slots = std::max<size_t>(cmax, (size_t)std::min<long long>(dec->max_shots, kPathModeMaxShots));
     if (slots > dec->kpath_slots) {
       cudaFree(dec->d_kpath);
@@ -828,8 +849,43 @@ qd::ReuseDev reuse_dev(const qd_decoder* dec, const WinGpu& g) {
   return R;
 }
 
-// shot mode's snapshot plan of window g (pool = nullptr: none, or turned off)
-qd::ForkDev fork_dev(const qd_decoder* dec, const WinGpu& g) {
+// Path mode's CTA for n_shots shots of window g, as an index into g.pa; -1: shot
+// mode.  Path mode runs batches of up to 64 shots.  A path's serial chain is
+// what takes the time and 512 threads shorten it most, but only one such CTA
+// fits an SM; a batch of several CTAs per SM is faster with smaller ones side by
+// side.  Four CTAs of 128 threads pay from three per SM, and a window of at most
+// 128 checks gains nothing from more than 256 threads (two lanes per check).
+// All windows of a pass, ms, with 512 x 1 / 256 x 2 / 128 x 4 and in shot mode:
+// [[144,12,12]] configured, 2 shots 6.4 / 6.4 / 8.2 / 15.2, 19 shots 16.1 / 9.8 /
+// 11.2 / 20.9, 38 shots 26.2 / 15.8 / 12.6 / 18.0, 64 shots 40.3 / 24.4 / 19.6 /
+// 18.4; paper preset, 25 shots 6.1 / 4.5 / 5.0 / 11.1, 64 shots 12.5 / 7.8 / 7.0 /
+// 12.2; [[72,12,6]], 2 shots 2.45 / 2.26 / 2.47 / 3.9, 64 shots 6.5 / 4.5 / 3.7 /
+// 5.0.
+int path_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
+  bool path_mode = dec->launch_mode == 2;
+  if (dec->launch_mode == 0) path_mode = n_shots * 2 <= dec->sm_count;
+  if (!path_mode || n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.fits || !g.pa[0].fits)
+    return -1;
+  int i = 0;
+  const long long ctas = n_shots * dec->kp.nb;
+  if (g.pa[1].fits && (g.h.n_rows <= 128 || ctas > dec->sm_count)) i = 1;
+  if (g.pa[2].fits && ctas > 3LL * dec->sm_count) i = 2;
+  return i;
+}
+
+// Shot mode for n_shots shots: the fewest CTAs per SM that hold them at once
+// (more shared memory, so more path slots and staged graph, and more registers),
+// else the large batches'.  150 shots of [[144,12,12]], all windows: configured
+// 22.0 ms in the large batches' shape, 18.9 with one CTA per SM; paper preset 14.0
+// and 12.6.
+const ShotShape& shot_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
+  int i = 0;
+  while (i < g.best && n_shots > (int64_t)(i + 1) * dec->sm_count) ++i;
+  return g.sh[i];
+}
+
+// shot mode's snapshot plan (pool = nullptr: none, or turned off)
+qd::ForkDev fork_dev(const qd_decoder* dec, const ShotShape& g) {
   qd::ForkDev F{};
   // the candidate dump records path 0's every step, so path 0 runs from the root
   if (!dec->fork_on || !g.fork_on || !dec->d_snap || dec->kp.dump) return F;
@@ -865,13 +921,11 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
     return QD_OK;
   }
   // the path state in global memory when the window does not fit shared memory
-  // (or on request); otherwise path mode while a batch leaves most SMs idle
+  // (or on request)
   const bool global = !g.fits || dec->launch_mode == 3;
-  bool path_mode = dec->launch_mode == 2;
-  if (dec->launch_mode == 0) path_mode = n_shots * 4 <= dec->sm_count;
-  if (path_mode && (n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.path_fits || global))
-    path_mode = false;
-  const qd::ForkDev fk = fork_dev(dec, g);
+  const int ps = path_shape(dec, g, n_shots);
+  const ShotShape& s = shot_shape(dec, g, global ? INT64_MAX : n_shots);
+  const qd::ForkDev fk = fork_dev(dec, s);
   const qd::ReuseDev ru = reuse_dev(dec, g);
   if (g.dv.wts) QD_CK(qd::launch_order_weights(st, g.dv));
   if (global) {
@@ -883,17 +937,18 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
                             dec->d_uscratch, g.Lg.total - g.Lg.U, 1, 1, &fk, &ru));
     return QD_OK;
   }
-  if (path_mode) {
-    const int cps = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
-    QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
-                            dw, n_shots, win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes,
-                            dec->dmx, dec->ns_max, nullptr, dec->d_counters, dec->d_path_res, dec->d_arrive,
-                            dec->sw_max, nullptr, 0, cps, g.pcl, nullptr, &ru));
+  if (ps >= 0) {
+    const PathShape& p = g.pa[ps];
+    const int cps = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
+    QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads >> ps, p.L.total, st, dec->kp, g.dv, p.L,
+                            det_bits, dw, n_shots, win_correction, dec->corr_words, status, (char*)trace,
+                            dec->trace_bytes, dec->dmx, dec->ns_max, nullptr, dec->d_counters, dec->d_path_res,
+                            dec->d_arrive, dec->sw_max, nullptr, 0, cps, p.pcl, nullptr, &ru));
     return QD_OK;
   }
   QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
-  const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * g.grid_per_sm);
-  QD_CK(qd::launch_decode(0, g.ctas, (int)grid, 32 * g.shot_warps, g.L.total, st, dec->kp, g.dv, g.L, det_bits, dw,
+  const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * s.grid_per_sm);
+  QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * kShotWarps, s.L.total, st, dec->kp, g.dv, s.L, det_bits, dw,
                           n_shots, win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes,
                           dec->dmx, dec->ns_max, dec->d_work + k, dec->d_counters, nullptr, nullptr, dec->sw_max,
                           nullptr, 0, 1, 1, &fk, &ru));
@@ -1049,14 +1104,16 @@ qd_status qd_decoder_launch_info(const qd_decoder* dec, int k, int out[8]) {
   QD_REQ(dec && out, "null argument");
   QD_REQ(k >= 0 && k < (int)dec->wins.size(), "qd_decoder_launch_info: window out of range");
   const WinGpu& g = dec->wins[k];
-  out[0] = (int)g.L.total;
-  out[1] = 32 * g.shot_warps;
-  out[2] = g.grid_per_sm;
-  out[3] = (int)g.Lp.total;
+  const ShotShape& s = g.sh[g.best];
+  const PathShape& p = g.pa[0];
+  out[0] = (int)s.L.total;
+  out[1] = 32 * kShotWarps;
+  out[2] = s.grid_per_sm;
+  out[3] = (int)p.L.total;
   out[4] = kPathThreads;
   out[5] = dec->sm_count;
-  out[6] = g.pcl;
-  out[7] = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
+  out[6] = p.pcl;
+  out[7] = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
   return QD_OK;
 }
 
@@ -1161,25 +1218,24 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
     // decoder (path results and arrival counters, global union regions), and
     // the work counters go to the decoder's own (qd_decoder_counters)
     const bool global = !g.fits || dec->launch_mode == 3;
-    bool path_mode = dec->launch_mode == 2;
-    if (dec->launch_mode == 0) path_mode = n_shots * 4 <= dec->sm_count;
-    if (path_mode && (n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.path_fits || global))
-      path_mode = false;
+    const int ps = path_shape(dec, g, n_shots);
     if (g.dv.wts) QD_CK(qd::launch_order_weights(st, g.dv));
-    if (path_mode) {
-      const int cps = (dec->kp.nb + g.pcl - 1) / g.pcl * g.pcl;
-      QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads, g.Lp.total, st, dec->kp, g.dv, g.Lp, det_bits,
-                              dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0, dec->dmx, dec->ns_max, nullptr,
-                              dec->d_counters, dec->d_path_res, dec->d_arrive, dec->sw_max, nullptr, 0, cps, g.pcl,
-                              nullptr, &ru));
+    if (ps >= 0) {
+      const PathShape& p = g.pa[ps];
+      const int cps = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
+      QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads >> ps, p.L.total, st, dec->kp, g.dv, p.L,
+                              det_bits, dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0, dec->dmx, dec->ns_max,
+                              nullptr, dec->d_counters, dec->d_path_res, dec->d_arrive, dec->sw_max, nullptr, 0, cps,
+                              p.pcl, nullptr, &ru));
     } else {
       // the array keeps the previous call's contents: the work counter restarts at 0
       QD_CK(cudaMemsetAsync(work, 0, sizeof(int), st));
-      const qd::ForkDev fk = fork_dev(dec, g);
-      const qd::Layout& L = global ? g.Lg : g.L;
+      const ShotShape& s = shot_shape(dec, g, global ? INT64_MAX : n_shots);
+      const qd::ForkDev fk = fork_dev(dec, s);
+      const qd::Layout& L = global ? g.Lg : s.L;
       const long long grid =
-          std::min<long long>(n_shots, (long long)dec->sm_count * (global ? g.grid_g : g.grid_per_sm));
-      QD_CK(qd::launch_decode(0, g.ctas, (int)grid, 32 * (global ? kShotWarps : g.shot_warps), global ? L.U : L.total, st,
+          std::min<long long>(n_shots, (long long)dec->sm_count * (global ? g.grid_g : s.grid_per_sm));
+      QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * kShotWarps, global ? L.U : L.total, st,
                               dec->kp, g.dv, L, det_bits, dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0,
                               dec->dmx, dec->ns_max, work, dec->d_counters, nullptr, nullptr, dec->sw_max,
                               global ? dec->d_uscratch : nullptr, global ? L.total - L.U : 0, 1, 1, &fk, &ru));
@@ -1284,7 +1340,7 @@ int batch_members(qd_batch* b, int j, uint32_t* const* det, const int64_t* n, ui
     m.b0 = g.h.r0 * w;
     m.b1 = g.h.commit_b1 * w;
     b->forks.resize(b->mem.size());
-    b->forks[i] = fork_dev(d, g);
+    b->forks[i] = fork_dev(d, g.sh[g.best]);
     m.fork = &b->forks[i];
     out.push_back(m);
   }
