@@ -317,6 +317,12 @@ int typical_slots(const qd::Layout& L, const qd::WindowHost& h, int most) {
   return std::max(1, S.nslots);
 }
 
+bool same_dims(const qd::WindowHost& a, const qd::WindowHost& b) {  // one layout for both
+  return a.n_rows == b.n_rows && a.n_cols == b.n_cols && a.n_short == b.n_short && a.n_edges == b.n_edges &&
+         a.row_quads == b.row_quads && a.col_cells == b.col_cells && a.srow_quads == b.srow_quads &&
+         a.scol_cells == b.scol_cells;
+}
+
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   struct Conf {
     ShotShape sh[kShotCtas];
@@ -331,6 +337,10 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   std::vector<Conf> cf(dec->wins.size());
   for (size_t w = 0; w < cf.size(); ++w) {
     Conf& c = cf[w];
+    if (w && same_dims(dec->wins[w - 1].h, dec->wins[w].h)) {  // interior windows
+      c = cf[w - 1];
+      continue;
+    }
     const auto& h = dec->wins[w].h;
     auto lay = [&](unsigned budget, bool glob = false) {
       return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob);
@@ -416,11 +426,15 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   size_t cta_bytes = 0;
   int ctas = 0;
   const size_t plan = (size_t)dec->kp.nb * (3 + dec->dmx);
+  ForkPlan plans[kShotWarps + 1];  // by wave
+  bool have[kShotWarps + 1] = {};
   for (WinGpu& g : dec->wins) {
     std::vector<int16_t> v;
     for (int i = 0; i <= g.best; ++i) {
       ShotShape& s = g.sh[i];
-      const ForkPlan F = fork_plan(dec->kp, dec->dmx, s.wave);
+      ForkPlan& F = plans[s.wave];
+      if (!have[s.wave]) F = fork_plan(dec->kp, dec->dmx, s.wave);
+      have[s.wave] = true;
       s.fork_on = F.on;
       s.fork_nodes = F.n_nodes;
       if (!F.on) continue;
