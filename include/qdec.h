@@ -390,7 +390,10 @@ qd_status qd_batch_autotune(qd_batch* b, int step, uint32_t* const* det_bits, co
  * CSC edge order; iteration t (counted from message initialisation, in the
  * pre-BP and in every decision path) uses row min(t, T) - 1, and an edge of
  * the shortened matrix uses the weights of its full-window edge.  The caller
- * owns w and keeps it valid while the decoder uses it; NULL restores alpha.
+ * owns w and keeps it valid while the decoder uses it (it is read at every
+ * decode, so changes made in place take effect); NULL restores alpha.  The
+ * first call allocates room for the weights in the pre-BP's order in every
+ * window, later ones only for a larger T.
  */
 qd_status qd_decoder_set_weights(qd_decoder* dec, int k, const float* w, int T);
 
@@ -481,9 +484,11 @@ qd_status qd_set_zero(void* dst, size_t bytes, qd_stream_t stream);
  * soft-syndrome binary cross entropy at t = T: P(check j odd) =
  * (1 - prod_{i in N(j)} tanh(Lambda_i^(T) / 2)) / 2 against s_j, averaged over
  * the window's checks.  Gradients come from a hand-written adjoint of the
- * unrolled iterations, recomputed from message checkpoints every `ckpt`
- * iterations.
- *   qd_wms_create  allocates per-CTA scratch; T, ckpt as above
+ * unrolled iterations, from the check records that the forward pass keeps for
+ * every iteration.
+ *   qd_wms_create  allocates per-CTA scratch for T iterations; 1 <= ckpt <= T
+ *                  (a spacing of checkpoints; results do not depend on it, and
+ *                  none are needed now that every iteration is kept)
  *   qd_wms_info    out[6] = rows, columns, edges, T, ckpt, syndrome words
  *   qd_wms_sample  synd: device [n][syndrome words]; counter-based like
  *                  qd_sample_shots, with word 3 of the counter = 1 + k

@@ -22,7 +22,7 @@
 //       its first VN->CN messages from them
 //
 // Two launch shapes run the same path code:
-//   shot mode (throughput): persistent CTAs of up to 8 warps take shots from
+//   shot mode (throughput): persistent CTAs of 8 or 12 warps take shots from
 //     a work counter; after the CTA-wide pre-BP the warps take decision paths
 //     from a shared-memory queue in a host-planned order, one warp per path;
 //     paths resume from snapshots of the prefixes they share with earlier
@@ -2244,7 +2244,7 @@ __device__ void keep_for_next(const DecodeArgs& A, char* sm, long long shot, con
   for (int k = tid; k < n_short; k += NT) out[sel[vperm[k]]] = __ldcg(kp + k);
 }
 
-// ---- shot mode: persistent CTAs of up to 8 warps, one warp per decision path ----
+// ---- shot mode: persistent CTAs of up to 12 warps, one warp per decision path ----
 // One shot of one window by the whole CTA (every thread calls).  misc[2], the
 // decision-path queue, must be 0 on entry.
 template <bool LW, bool UG>
@@ -2388,7 +2388,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
 
 // CTAS: CTAs per SM (register budget), see configure_layouts.
 template <bool LW, bool UG, int CTAS>
-__global__ void __launch_bounds__(256, CTAS) decode_shot_kernel(DecodeArgs A) {
+__global__ void __launch_bounds__(CTAS == 1 ? 384 : 256, CTAS) decode_shot_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
   int* misc = (int*)(sm + A.L.misc);
   Stager stg = stager_init((char*)(misc + 8), &A.counters[4]);
@@ -2696,6 +2696,7 @@ size_t trace_bytes_per_shot(int nb, int dmx, int ns_max) { return dev::trace_byt
 cudaError_t set_decode_smem(size_t bytes) {
   const void* f[] = {(const void*)dev::decode_shot_kernel<false, false, 2>, (const void*)dev::decode_shot_kernel<true, false, 2>,
                      (const void*)dev::decode_shot_kernel<false, true, 2>,  (const void*)dev::decode_shot_kernel<true, true, 2>,
+                     (const void*)dev::decode_shot_kernel<false, false, 1>, (const void*)dev::decode_shot_kernel<true, false, 1>,
                      (const void*)dev::decode_shot_kernel<false, false, 3>, (const void*)dev::decode_path_kernel<false>,
                      (const void*)dev::decode_path_kernel<true>,            (const void*)dev::decode_batch_kernel<false>,
                      (const void*)dev::decode_batch_kernel<true>};
@@ -2755,6 +2756,8 @@ cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* 
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_path_kernel<false>, threads, smem);
   if (mode == 3)  // shot mode with the union region in global memory
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, true, 2>, threads, smem);
+  if (ctas == 1)
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 1>, threads, smem);
   if (ctas >= 3)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 3>, threads, smem);
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 2>, threads, smem);
@@ -2810,6 +2813,9 @@ cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem
     if (uglob) {
       if (lw) dev::decode_shot_kernel<true, true, 2><<<grid, threads, smem, st>>>(A);
       else dev::decode_shot_kernel<false, true, 2><<<grid, threads, smem, st>>>(A);
+    } else if (ctas == 1) {
+      if (lw) dev::decode_shot_kernel<true, false, 1><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, false, 1><<<grid, threads, smem, st>>>(A);
     } else if (ctas >= 3 && !lw) {
       dev::decode_shot_kernel<false, false, 3><<<grid, threads, smem, st>>>(A);
     } else {

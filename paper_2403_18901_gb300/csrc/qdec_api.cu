@@ -62,6 +62,11 @@ constexpr int kShotWarps = 8;
 // [[144,12,12]] run 4 % faster so than with two and 128 registers (the paper
 // preset 5 %); with learned weights or a ranker 3 and 6 % slower.
 constexpr int kShotCtas = 3;
+// Warps of a CTA that has its SM for itself: 150 shots of [[144,12,12]] with the
+// paper preset's 22 paths, all windows, 12.7 ms with 8, 11.2 with 12, 11.6 with 16;
+// [[288,12,18]] 34.4, 32.4 and 34.1 ms (configured, 16 paths); the configured preset
+// of [[144,12,12]] 18.9, 18.8 and 19.5.
+constexpr int kWideWarps = 12;
 // Path mode's CTAs: 512 threads, one per SM; 256, two; 128, four (the same 128
 // registers a thread), see path_shape.
 constexpr int kPathShapes = 3;
@@ -73,6 +78,7 @@ constexpr int kCounters = 8;
 // queue order [nb], then the node chain [nb][dmx]; fork_nodes = 0: none.
 struct ShotShape {
   qd::Layout L{};
+  int warps = kShotWarps;
   int ctas = 2;         // CTAs per SM planned
   int grid_per_sm = 1;  // and resident
   int wave = 1;         // path slots of a typical shot
@@ -358,12 +364,14 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       if (s.L.total > budget) break;  // (the budgets fall)
       s.L.total = budget;  // the slots take what the budget holds
       int blocks = 0;
-      QD_CK(qd::decode_occupancy(0, n, 32 * kShotWarps, s.L.total, &blocks));
+      s.warps = n == 1 ? kWideWarps : kShotWarps;
+      QD_CK(qd::decode_occupancy(0, n, 32 * s.warps, s.L.total, &blocks));
       s.ctas = n;
       s.grid_per_sm = std::max(1, blocks);
-      s.wave = typical_slots(s.L, h, kShotWarps);
-      if (std::min(blocks, n) * s.wave > best) {
-        best = std::min(blocks, n) * s.wave;
+      s.wave = typical_slots(s.L, h, s.warps);
+      const int resident = std::min(blocks, n) * std::min(s.wave, kShotWarps);
+      if (resident > best) {
+        best = resident;
         c.best = n - 1;
         c.fits = true;
       }
@@ -426,8 +434,8 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   size_t cta_bytes = 0;
   int ctas = 0;
   const size_t plan = (size_t)dec->kp.nb * (3 + dec->dmx);
-  ForkPlan plans[kShotWarps + 1];  // by wave
-  bool have[kShotWarps + 1] = {};
+  ForkPlan plans[kWideWarps + 1];  // by wave
+  bool have[kWideWarps + 1] = {};
   for (WinGpu& g : dec->wins) {
     std::vector<int16_t> v;
     for (int i = 0; i <= g.best; ++i) {
@@ -890,8 +898,8 @@ int path_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
 // Shot mode for n_shots shots: the fewest CTAs per SM that hold them at once
 // (more shared memory, so more path slots and staged graph, and more registers),
 // else the large batches'.  150 shots of [[144,12,12]], all windows: configured
-// 22.0 ms in the large batches' shape, 18.9 with one CTA per SM; paper preset 14.0
-// and 12.6.
+// 22.0 ms in the large batches' shape, 18.8 with one CTA per SM; paper preset 14.0
+// and 11.2.
 const ShotShape& shot_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
   int i = 0;
   while (i < g.best && n_shots > (int64_t)(i + 1) * dec->sm_count) ++i;
@@ -962,7 +970,7 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   }
   QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
   const long long grid = std::min<long long>(n_shots, (long long)dec->sm_count * s.grid_per_sm);
-  QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * kShotWarps, s.L.total, st, dec->kp, g.dv, s.L, det_bits, dw,
+  QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * s.warps, s.L.total, st, dec->kp, g.dv, s.L, det_bits, dw,
                           n_shots, win_correction, dec->corr_words, status, (char*)trace, dec->trace_bytes,
                           dec->dmx, dec->ns_max, dec->d_work + k, dec->d_counters, nullptr, nullptr, dec->sw_max,
                           nullptr, 0, 1, 1, &fk, &ru));
@@ -1121,7 +1129,7 @@ qd_status qd_decoder_launch_info(const qd_decoder* dec, int k, int out[8]) {
   const ShotShape& s = g.sh[g.best];
   const PathShape& p = g.pa[0];
   out[0] = (int)s.L.total;
-  out[1] = 32 * kShotWarps;
+  out[1] = 32 * s.warps;
   out[2] = s.grid_per_sm;
   out[3] = (int)p.L.total;
   out[4] = kPathThreads;
@@ -1249,7 +1257,7 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
       const qd::Layout& L = global ? g.Lg : s.L;
       const long long grid =
           std::min<long long>(n_shots, (long long)dec->sm_count * (global ? g.grid_g : s.grid_per_sm));
-      QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * kShotWarps, global ? L.U : L.total, st,
+      QD_CK(qd::launch_decode(0, s.ctas, (int)grid, 32 * (global ? kShotWarps : s.warps), global ? L.U : L.total, st,
                               dec->kp, g.dv, L, det_bits, dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0,
                               dec->dmx, dec->ns_max, work, dec->d_counters, nullptr, nullptr, dec->sw_max,
                               global ? dec->d_uscratch : nullptr, global ? L.total - L.U : 0, 1, 1, &fk, &ru));
