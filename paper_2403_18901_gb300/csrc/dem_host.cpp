@@ -634,7 +634,7 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
 // check's first 32 entries, and those past them, as spread_positions says; a
 // column's entries in ascending window row, the order of the sum of Eq. (2).
 // The order of a check's entries and of the columns changes no value.  Counted
-// for an interior [[144,12,12]] (3,1) window: 520 -> 342 wavefronts for the 228
+// for an interior [[144,12,12]] (3,1) window: 520 -> 352 wavefronts for the 228
 // gathers of a check pass, 1536 -> 987 for the 840 of a variable pass.
 // Building them takes 1.3 ms there and a stream has three distinct matrices
 // (first, interior, last), so a window takes the slices of the one before it
@@ -642,7 +642,7 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
 bool build_slices(WindowHost& o, const WindowHost* like) {
   const int nr = o.n_rows, nc = o.n_cols;
   if (like && like->n_rows == nr && like->col_ptr == o.col_ptr && like->col_rows == o.col_rows &&
-      like->n_short == o.n_short && like->short_edges_max == o.short_edges_max) {  // the interior windows share one graph
+      like->n_short == o.n_short && like->short_edges_max == o.short_edges_max) {  // interior windows
     o.row_quads = like->row_quads;
     o.col_cells = like->col_cells;
     o.srow_quads = like->srow_quads;

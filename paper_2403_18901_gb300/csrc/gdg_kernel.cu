@@ -200,7 +200,7 @@ __device__ __forceinline__ void lw_four(const Lw& r, int i, bool first, float (&
 // conflicts come next.  With a sign byte and an edge id per edge, a NaN test
 // and the clip on every input and ragged rows, 5000 shots of [[144,12,12]]
 // took 450 ms; in slices, with the signs as bits of the record and the clip on
-// the two minima, 354 ms.
+// the two minima, 354 ms (with all that followed, 231).
 template <bool LW, class E, class Lw>
 __device__ __forceinline__ uint32_t check_lane(const E* ent, int nq, const char* post, CNState* rec, uint32_t sbit,
                                                float alpha, float clip, const Lw& lw, int ei, bool first) {
@@ -1957,7 +1957,9 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     for (int l = tid; l < L.sortn; l += NT) sortb[l] = l < nc ? sort_key(l, ordkey(key[l])) : ~0ull;
   } else {
     // select before sorting: bisection for the n_short-th smallest key, then
-    // (equal keys) for the column up to which its equals are taken
+    // (equal keys) for the column up to which its equals are taken.  Sorting all
+    // 4096 places was a tenth of a window of the paper preset (3000 shots of
+    // [[144,12,12]] 44.5 ms; 42.4 with the 512 selected ones).
     uint32_t* uk = (uint32_t*)key;
     // (the sort buffer follows the keys, over the dead check records; the
     // posteriors before them are dead too)
@@ -2386,7 +2388,12 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
   write_outputs(A, sm, shot, conv, winner, n_short, t_run, tr);
 }
 
-// CTAS: CTAs per SM (register budget), see configure_layouts.
+// CTAS: CTAs per SM (register budget), see configure_layouts.  What bounds it with
+// three: instruction issue (73 % of the cycles), the ALU pipe (65 % of its peak)
+// and shared-memory wavefronts (69 %, 29 % of them bank conflicts), at 22.6 warps
+// per SM; HBM is idle.  One warp per path keeps every barrier of a path a warp's;
+// 5000 shots of [[144,12,12]], all windows, took 450 ms with two CTAs per SM and
+// the graph in CSR, 231 ms so; 9001 of the paper preset 200 and 104 ms.
 template <bool LW, bool UG, int CTAS>
 __global__ void __launch_bounds__(CTAS == 1 ? 384 : 256, CTAS) decode_shot_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
@@ -2442,6 +2449,11 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
 }
 
 // ---- path mode: one CTA per (shot, path); the last CTA of a shot decides ----
+// What bounds it: one path's serial chain (250 iterations of two passes with a
+// barrier each) after the cluster's pre-BP; 16 CTAs of 512 threads for one
+// [[144,12,12]] shot issue in 34 % of the cycles, half of the stalls are barriers.
+// One shot, all windows: 7.7 ms with eight lanes per check and remote reads in the
+// pre-BP, 5.4 ms so.  The threads per CTA follow the batch (path_shape).
 template <bool LW>
 __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
@@ -2522,7 +2534,8 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
 // edges, [T][check entries] and [T][column entries], so that they load them
 // side by side instead of through edge ids.  Runs before every decode of the
 // window (the caller may change the weights in between): 1.4 MB for
-// [[144,12,12]] (3,1) windows and T = 25.
+// [[144,12,12]] (3,1) windows and T = 25, a few microseconds at L2 rates.  2000
+// shots took 181 ms with gathers through edge ids, 147 ms so.
 __global__ void __launch_bounds__(256) order_weights_kernel(const float* __restrict__ w, const uint16_t* __restrict__ ref,
                                                             const uint16_t* __restrict__ cef, int T, int ne, int nrow,
                                                             int ncol, float* __restrict__ w_row,
@@ -2550,8 +2563,9 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 // column per lane, so that the loads of a column's detectors wait for one
 // another once per list and not once per fault.  What bounds it: the integer
 // instructions of Philox (ten rounds, two wide multiplications and two
-// three-way xors each).  100000 shots of [[144,12,12]], 12 rounds, took
-// 1061 us with scalar threshold loads and every fault worked off on the spot.
+// three-way xors each; the multiplier is what warps wait for).  100000 shots of
+// [[144,12,12]], 12 rounds, took 1061 us with scalar threshold loads and every
+// fault worked off on the spot, 726 us so.
 constexpr int kFireList = 160;  // at most 31 waiting and 128 new ones a trip
 __global__ void __launch_bounds__(256) sample_kernel(int n_cols, const uint4* __restrict__ thr,
                                                      const int* __restrict__ cptr, const int* __restrict__ cdet,
