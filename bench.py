@@ -39,14 +39,15 @@ BYTES_PER_EDGE_ITER = 16  # explicit-message shared-memory bytes per edge and it
 # capture of the current kernel (dram__bytes_read.sum + dram__bytes_write.sum;
 # see profiles/decode_shot_kernel_bb144_w3_p3e-3_configured.md).  Reported
 # only for that workload; per launch, like "achieved".
-TRAFFIC_PER_LAUNCH = {("configured", 20000, 2): 6414336 + 3036823040}
-# Unit utilisation of the same kernel from one ncu --set full capture of a
-# 4000-shot launch of this workload (same profile file): the shared-memory
-# data pipe (l1tex__data_pipe_lsu_wavefronts_mem_shared, % of peak) and the
-# ALU pipe (sm__pipe_alu_cycles_active, % of peak), as fractions.  What bounds
+TRAFFIC_PER_LAUNCH = {("configured", 20000, 2): 5175808 + 699499008}
+# Unit utilisation of the same kernel from one ncu capture of a 1824-shot
+# launch of this workload (same profile file): instruction issue
+# (smsp__issue_active), the shared-memory data pipe
+# (l1tex__data_pipe_lsu_wavefronts_mem_shared) and the ALU pipe
+# (sm__inst_executed_pipe_alu), % of peak, as fractions.  What bounds
 # the kernel in hardware terms; the algorithmic fractions above count only
 # the method's arithmetic and message bytes.
-PIPES_PER_LAUNCH = {("configured", 2): {"shared_data_pipe": 0.695, "alu_pipe": 0.574}}
+PIPES_PER_LAUNCH = {("configured", 2): {"issue": 0.732, "shared_data_pipe": 0.691, "alu_pipe": 0.649}}
 
 
 FALLBACK_NAMES = {0: "path 0's estimate", 1: "fewest unsatisfied checks",
