@@ -515,7 +515,8 @@ qd_status qd_adam_step(float* w, const float* g, float* m1, float* m2, int64_t n
 
 /* Launch shape of qd_decode_windows (results are identical in every shape):
  * 0 automatic (default): path mode for batches of at most half as many shots as
- * there are SMs, otherwise shot mode; 1 shot mode: persistent CTAs, one warp per
+ * there are SMs (and, with 32 or more pre-BP iterations, at most nine paths per
+ * SM), otherwise shot mode; 1 shot mode: persistent CTAs, one warp per
  * decision path, one to three CTAs per SM by the batch's size; 2 path mode: one
  * CTA of 512, 256 or 128 threads (by the batch's size) per (shot, decision path)
  * for the lowest latency, the path CTAs of a shot launched as a thread-block

@@ -877,6 +877,10 @@ qd::ReuseDev reuse_dev(const qd_decoder* dec, const WinGpu& g) {
 // fits an SM; a batch of several CTAs per SM is faster with smaller ones side by
 // side.  Four CTAs of 128 threads pay from three per SM, and a window of at most
 // 128 checks gains nothing from more than 256 threads (two lanes per check).
+// Every cluster of a shot repeats the pre-BP, so a long one with more than nine
+// paths per SM is left to shot mode (32 paths, configured: [[144]] W = 4, 38 shots
+// 22.9 ms against 28.1 in shot mode, 45 28.6 / 28.6, 64 36.3 / 29.0; 22 paths of the
+// paper preset on [[288]] W = 4, 64 shots 13.5 / 23.3).
 // All windows of a pass, ms, with 512 x 1 / 256 x 2 / 128 x 4 and in shot mode:
 // [[144,12,12]] configured, 2 shots 6.4 / 6.4 / 8.2 / 15.2, 19 shots 16.1 / 9.8 /
 // 11.2 / 20.9, 38 shots 26.2 / 15.8 / 12.6 / 18.0, 64 shots 40.3 / 24.4 / 19.6 /
@@ -885,7 +889,9 @@ qd::ReuseDev reuse_dev(const qd_decoder* dec, const WinGpu& g) {
 // 5.0.
 int path_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
   bool path_mode = dec->launch_mode == 2;
-  if (dec->launch_mode == 0) path_mode = n_shots * 2 <= dec->sm_count;
+  if (dec->launch_mode == 0)
+    path_mode = n_shots * 2 <= dec->sm_count &&
+                (dec->kp.n_pre < 32 || n_shots * dec->kp.nb <= 9LL * dec->sm_count);
   if (!path_mode || n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.fits || !g.pa[0].fits)
     return -1;
   int i = 0;

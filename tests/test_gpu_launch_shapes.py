@@ -47,7 +47,7 @@ def _static(dec, det0, n):
 @pytest.mark.parametrize("key,R,W,pre,k,form", [
     ("72", 6, 3, "configured", 3, ""), ("144", 4, 3, "configured", 4, ""), ("144", 4, 3, "paper", 4, ""),
     ("108", 4, 2, "paper", 3, "ranker"), ("90", 4, 3, "configured", 3, "weights"), ("144", 4, 3, "paper", 3, "reuse"),
-    ("288", 4, 3, "configured", 4, "")])
+    ("288", 4, 3, "configured", 4, ""), ("72", 6, 3, "configured", 5, "")])
 def test_batch_sizes(key, R, W, pre, k, form):
     dem = qdec.Dem(CODES[key], 0.003, R)
     over = dict(W=W, F=1, **({"reuse_msgs": 1} if form == "reuse" else {}))
@@ -63,8 +63,8 @@ def test_batch_sizes(key, R, W, pre, k, form):
     sms, nb = info["sms"], 2 ** k + (6 if pre == "paper" else 0)
     det0, _ = dem.sample(91, 0, most)
     want = _windows(dec, det0, most, 1)
-    edges = {1, sms // nb, sms // nb + 1, 3 * sms // nb, 3 * sms // nb + 1, 64, 65, sms // 2, sms // 2 + 1, sms, sms + 1,
-             2 * sms, 2 * sms + 1}
+    edges = {1, sms // nb, sms // nb + 1, 3 * sms // nb, 3 * sms // nb + 1, 9 * sms // nb,
+             9 * sms // nb + 1, 64, 65, sms // 2, sms // 2 + 1, sms, sms + 1, 2 * sms, 2 * sms + 1}
     for n in sorted(e for e in edges if 1 <= e <= most):
         for mode in (0, 2) if n <= 64 else (0,):
             for a, b in zip(_windows(dec, det0, n, mode), want):
