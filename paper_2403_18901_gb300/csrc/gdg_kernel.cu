@@ -883,8 +883,9 @@ __device__ double path_metric(const ShortG& G, const Slot& B, const Grp& g) {
 }
 
 // H e = s for the current decisions (Eq. (4), decimated VNs through s'):
-// writes every check's unsatisfied bit to B.unsat and returns whether any is
-// unsatisfied.  Checks in label order, one per lane.
+// writes every check's unsatisfied bit to B.unsat, for every lane of the group
+// to read once it has returned, and returns whether any is unsatisfied.  Checks
+// in label order, one per lane.
 template <class Grp>
 __device__ bool parity_pass(const ShortG& G, const Slot& B, const Grp& g) {
   bool any = false;
@@ -904,6 +905,7 @@ __device__ bool parity_pass(const ShortG& G, const Slot& B, const Grp& g) {
     if (lane == 0) B.unsat[s] = m;
     any |= m != 0u;
   }
+  if constexpr (Grp::kWarp) __syncwarp();  // (a warp's vote orders no memory, a CTA's is a barrier)
   return g.any(any);
 }
 
