@@ -2441,8 +2441,9 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
     const DecodeArgs& A = B.seg[m];
     const long long shot = g - (m ? B.seg_end[m - 1] : 0);
     if (threadIdx.x == 0) ((int*)(sm + A.L.misc))[2] = 0;
-    // no snapshot yet, every path queued
-    if (A.F.pool && threadIdx.x < 2 * kMaxForkNodes) ((int*)(sm + A.L.red))[threadIdx.x] = 0;
+    if (A.F.pool)  // no snapshot yet, every path queued (a CTA may have fewer threads than there are words)
+#pragma unroll 1
+      for (int x = threadIdx.x; x < 2 * kMaxForkNodes; x += blockDim.x) ((int*)(sm + A.L.red))[x] = 0;
     __syncthreads();
     // (members without learned weights may share the launch with others)
     if (LW && A.W.wts) shot_body<true, false>(A, shot, sm, stg);
