@@ -690,8 +690,8 @@ bool build_slices(WindowHost& o, const WindowHost* like) {
   o.col_cells = o.s_coff[ncs];
   o.s_rent.assign((size_t)128 * o.row_quads, (uint16_t)(32 * ncs));  // the dummy column
   o.s_cent.assign((size_t)32 * o.col_cells, (uint32_t)(32 * nrs) << 16);  // the dummy check
-  o.s_ref.assign(o.s_rent.size(), 0);
-  o.s_cef.assign(o.s_cent.size(), 0);
+  o.s_ref.assign(o.s_rent.size(), kNoEdge);
+  o.s_cef.assign(o.s_cent.size(), kNoEdge);
   o.s_llr.assign((size_t)32 * ncs, 0.0f);
   std::vector<int> pos_of(o.n_edges, 0);
   {
@@ -726,18 +726,6 @@ bool build_slices(WindowHost& o, const WindowHost* like) {
       o.s_cef[ci] = (uint16_t)e;
     }
   }
-  // a dummy takes its node's first edge's learned weight, so that a weight
-  // touches no node but its own two
-  for (int r = 0; r < nr; ++r)
-    for (int pos = std::max(1, rdeg(o.s_row[r])); pos < 4 * (o.s_roff[(r >> 5) + 1] - o.s_roff[r >> 5]); ++pos) {
-      const size_t r0 = ((size_t)o.s_roff[r >> 5] * 32 + (r & 31)) * 4;
-      o.s_ref[r0 + 128 * (size_t)(pos >> 2) + (pos & 3)] = o.s_ref[r0];
-    }
-  for (int l = 0; l < nc; ++l)
-    for (int u = cdeg(o.s_col[l]); u < o.s_coff[(l >> 5) + 1] - o.s_coff[l >> 5]; ++u) {
-      const size_t c0 = (size_t)o.s_coff[l >> 5] * 32 + (l & 31);
-      o.s_cef[c0 + 32 * (size_t)u] = o.s_cef[c0];
-    }
   for (int q = 0; q < ncs; ++q) {
     const int w = o.s_coff[q + 1] - o.s_coff[q];
     for (int x = 0; x < 4; ++x)

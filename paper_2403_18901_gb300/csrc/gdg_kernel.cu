@@ -77,6 +77,13 @@ __device__ __forceinline__ float c2v(const CNState& c, uint32_t e, bool wide, fl
   return LW ? __fmul_rn(w, m) : m;
 }
 
+// The maximum, NaN if an operand is NaN (fmaxf returns the other operand then).
+__device__ __forceinline__ float max_or_nan(float x, float y) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(x), "f"(y));
+  return m;
+}
+
 // The inputs a check has seen: two smallest magnitudes, the position of the
 // smallest, the parity of the hard decisions it read (bit 31).  The two
 // smallest and so every message do not depend on the order of the inputs.
@@ -102,9 +109,13 @@ __device__ __forceinline__ uint32_t check_input(CheckAcc& A, float pv, uint32_t 
   // (an infinite weight: no message before the first iteration, and a dead
   // input stays one)
   if (LW && (first || pv == CUDART_INF_F)) v = pv;
+  // (v is NaN where an infinite message met an infinite posterior -- no clip, or
+  // learned weights that are not finite.  Such an input counts as +inf: the
+  // comparison does not hold, the maximum is NaN and fminf returns its other
+  // operand.)
   const float a = fabsf(v);
   A.am = a < A.m1 ? u : A.am;
-  A.m2 = fminf(A.m2, fmaxf(A.m1, a));
+  A.m2 = fminf(A.m2, max_or_nan(A.m1, a));
   A.m1 = fminf(A.m1, a);
   A.hp ^= __float_as_uint(pv) - 1u;
   return __float_as_uint(v);
@@ -159,11 +170,16 @@ __device__ __forceinline__ CNState check_record(const CheckAcc& A, uint32_t sg0,
 // Learned weights' view of one iteration: entry i's weight is w[ef[i]] (its row
 // of the weights, the entries' full-window edges), or w[i] where the weights
 // have been put in entry order (ef = nullptr; a type of its own, so that each
-// loop is compiled for one of the two).
+// loop is compiled for one of the two).  A column's dummy has no edge and the
+// weight 0 (its message has to be +0, which an infinite weight would not give);
+// a check's dummies are dead inputs, whatever their weight.
 struct LwEdge {
   const float* w;
   const uint16_t* ef;
-  __device__ __forceinline__ float one(int i) const { return w[ef[i]]; }
+  __device__ __forceinline__ float one(int i) const {
+    const uint32_t e = ef[i];
+    return e == kNoEdge ? 0.0f : w[e];
+  }
   __device__ __forceinline__ void four(int i, float (&x)[4]) const {
     const uint2 e = *(const uint2*)(ef + i);
     x[0] = w[e.x & 0xFFFFu];
@@ -2127,7 +2143,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
 #pragma unroll 1
       for (int x = tid; x < 128 * nq; x += NT) sref[x] = 0;
 #pragma unroll 1
-      for (int x = tid; x < 32 * ncell; x += NT) scef[x] = 0;
+      for (int x = tid; x < 32 * ncell; x += NT) scef[x] = kNoEdge;
     }
 #pragma unroll 1
     for (int l = tid; l < nr; l += NT) cinv[cperm[l]] = l;
@@ -2155,10 +2171,6 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
         scef[ci + 32 * u] = (uint16_t)(e0 + u);
       }
     }
-    if (LW)  // a dummy takes its column's first edge's weight (a check's dummies are dead inputs)
-#pragma unroll 1
-      for (int u = d; u < (int)(coff[(k >> 5) + 1] & (kWideSlice - 1)) - (coff[k >> 5] & (kWideSlice - 1)); ++u)
-        scef[ci + 32 * u] = (uint16_t)e0;
   }
   __syncthreads();
   return false;
@@ -2544,8 +2556,11 @@ __global__ void __launch_bounds__(256) order_weights_kernel(const float* __restr
                                                             int ncol, float* __restrict__ w_row,
                                                             float* __restrict__ w_col) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
-  if (i < nrow) w_row[(size_t)t * nrow + i] = w[(size_t)t * ne + ref[i]];
-  else if (i < nrow + ncol) w_col[(size_t)t * ncol + (i - nrow)] = w[(size_t)t * ne + cef[i - nrow]];
+  if (i >= nrow + ncol) return;
+  const uint32_t e = i < nrow ? ref[i] : cef[i - nrow];
+  const float x = e == kNoEdge ? 0.0f : w[(size_t)t * ne + e];
+  if (i < nrow) w_row[(size_t)t * nrow + i] = x;
+  else w_col[(size_t)t * ncol + (i - nrow)] = x;
 }
 
 // ---- Philox4x32-10 (Salmon et al., SC'11) ----

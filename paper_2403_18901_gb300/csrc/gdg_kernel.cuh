@@ -192,6 +192,8 @@ struct __align__(16) CNState {
 // at most 35 columns: the fault classes of a round are the same for every
 // choice of A and B (three terms each), and coinciding terms only merge them.
 constexpr int kMaxRowDeg = 51;
+// Edge id of a dummy (a window has fewer than 65535 edges).
+constexpr uint16_t kNoEdge = 0xFFFF;
 // Flag of a shortened graph's column slice starts (s_coff) when some check has
 // more than 32 entries, so that signs may be in the second word.
 constexpr uint16_t kWideSlice = 0x8000;
