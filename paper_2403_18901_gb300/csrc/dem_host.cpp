@@ -762,10 +762,7 @@ WmsHost build_wms(const WindowHost& h) {
   o.rcol.assign(nre, (uint16_t)(32 * ncs));
   o.reid.assign(nre, 0);
   o.cent.assign(cells, (uint32_t)(32 * nrs) << 16);
-  o.ceid.assign(cells, 0);
-  for (int l = 0; l < nc; ++l)  // a dummy takes its column's first edge's weight
-    for (int u = 0; u < o.coff[(l >> 5) + 1] - o.coff[l >> 5]; ++u)
-      o.ceid[(size_t)(o.coff[l >> 5] + u) * 32 + (l & 31)] = h.col_ptr[h.s_col[l]];
+  o.ceid.assign(cells, kNoEdge);
   for (int j = 0; j < nr; ++j) {
     const int r = rlab[j];
     for (int q = h.row_ptr[j]; q < h.row_ptr[j + 1]; ++q) {

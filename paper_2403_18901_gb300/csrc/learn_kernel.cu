@@ -81,7 +81,7 @@ __device__ __forceinline__ WRec check_forward(const uint16_t* cell, int n, const
       const bool l1 = a < m1, l2 = a < m2;  // the first of equal magnitudes stays
       p2 = l1 ? p1 : (l2 ? (uint32_t)u : p2);
       p1 = l1 ? (uint32_t)u : p1;
-      m2 = fminf(m2, fmaxf(m1, a));
+      m2 = l1 ? m1 : (l2 ? a : m2);  // (a NaN, inf - inf, is neither)
       m1 = fminf(m1, a);
       s = s + s + (x < 0.0f ? 1u : 0u);
     }
@@ -91,6 +91,10 @@ __device__ __forceinline__ WRec check_forward(const uint16_t* cell, int n, const
   const uint32_t all = 0u - par;  // message sign = parity xor s_j xor the own sign
   return WRec{m1, m2, sg[0] ^ all, ((sg[1] ^ all) & 0xFFFFE000u) | (par << 12) | (p2 << 6) | p1};
 }
+
+// The weight of a column entry; a dummy has no edge, and its message has to be
+// +0 (an infinite weight would make it NaN).
+__device__ __forceinline__ float entry_weight(const float* wt, uint32_t id) { return id == kNoEdge ? 0.0f : wt[id]; }
 
 // Message of Eq. (1) with weight w for the edge at position p.
 __device__ __forceinline__ float message(const WRec& r, uint32_t p, float w) {
@@ -150,7 +154,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
           for (int u = 0; u < N; ++u) {
             const int c = 32 * (c0 + u) + lane;
             const uint32_t e = G.cent[c];
-            m[u] = message(rec[e >> 16], e & 0xFFFFu, wt[G.ceid[c]]);
+            m[u] = message(rec[e >> 16], e & 0xFFFFu, entry_weight(wt, G.ceid[c]));
           }
 #pragma unroll
           for (int u = 0; u < N; ++u) p = __fadd_rn(p, m[u]);  // ascending check order
@@ -169,7 +173,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
               for (int u = 0; u < d; ++u) {
                 const int c = 32 * (c0 + u) + lane;
                 const uint32_t e = G.cent[c];
-                const float m = message(rec[e >> 16], e & 0xFFFFu, wt[G.ceid[c]]);
+                const float m = message(rec[e >> 16], e & 0xFFFFu, entry_weight(wt, G.ceid[c]));
                 if (pass == 0) p = __fadd_rn(p, m);
                 else v2c[c] = clipf(__fsub_rn(p, m), G.clip);
               }
