@@ -2873,7 +2873,10 @@ cudaError_t launch_sample(cudaStream_t st, int n_cols, const uint32_t* thr, cons
                           const uint32_t* cobs, int det_words, unsigned long long seed, unsigned long long off,
                           long long n, uint32_t* det, uint32_t* obs) {
   if (n <= 0) return cudaSuccess;
-  const int wpb = 8;
+  // eight warps per CTA, fewer where their rows and fire lists would not fit the
+  // shared memory that any kernel may have (more than 1376 detector words)
+  int wpb = 8;
+  while (wpb > 1 && sizeof(uint32_t) * wpb * (det_words + dev::kFireList) > (48u << 10)) wpb >>= 1;
   const long long blocks = (n + wpb - 1) / wpb;
   dev::sample_kernel<<<(unsigned)blocks, 32 * wpb, sizeof(uint32_t) * wpb * (det_words + dev::kFireList), st>>>(
       n_cols, (const uint4*)thr, cptr, cdet, cobs, det_words, seed, off, n, det, obs);
