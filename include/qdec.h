@@ -393,7 +393,8 @@ qd_status qd_batch_autotune(qd_batch* b, int step, uint32_t* const* det_bits, co
  * owns w and keeps it valid while the decoder uses it (it is read at every
  * decode, so changes made in place take effect); NULL restores alpha.  The
  * first call allocates room for the weights in the pre-BP's order in every
- * window, later ones only for a larger T.
+ * window (for min(T, n_pre) iterations), later ones only for more of them.  A
+ * CUDA graph captured before goes on with the weights it was captured with.
  */
 qd_status qd_decoder_set_weights(qd_decoder* dec, int k, const float* w, int T);
 

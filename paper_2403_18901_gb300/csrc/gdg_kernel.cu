@@ -2860,8 +2860,8 @@ cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem
 
 cudaError_t launch_order_weights(cudaStream_t st, const WinDev& W) {
   const int nrow = 128 * W.row_quads, ncol = 32 * W.col_cells;
-  for (int t0 = 0; t0 < W.wT; t0 += 65535) {  // (the grid's y limit)
-    const int T = W.wT - t0 < 65535 ? W.wT - t0 : 65535;
+  for (int t0 = 0; t0 < W.w_rows; t0 += 65535) {  // (the grid's y limit)
+    const int T = W.w_rows - t0 < 65535 ? W.w_rows - t0 : 65535;
     dev::order_weights_kernel<<<dim3((unsigned)((nrow + ncol + 255) / 256), (unsigned)T), 256, 0, st>>>(
         W.wts + (size_t)t0 * W.n_edges, W.s_ref, W.s_cef, T, W.n_edges, nrow, ncol, W.w_row + (size_t)t0 * nrow,
         W.w_col + (size_t)t0 * ncol);

@@ -112,7 +112,10 @@ struct WinDev {
   // alpha at iteration t (counted from message initialisation); NULL = alpha
   const float* wts;
   int wT;
-  float *w_row, *w_col;  // the same in the order of s_rent / s_cent (order_weights_kernel)
+  // the first w_rows iterations' (all that the pre-BP reads) in the order of
+  // s_rent / s_cent (order_weights_kernel)
+  int w_rows;
+  float *w_row, *w_col;
   int n_commit_rows;      // rows [0, n_commit_rows) are the ones the window commits
   // the graph in slices (see the top of the file), checks and columns by label
   int row_quads, col_cells;    // slice totals per lane: check entries in fours, column entries

@@ -114,8 +114,8 @@ struct WinGpu {
   // message reuse: this window's column -> the previous window's column of
   // the same DEM column (-1: none); nullptr for the first window
   int16_t* d_prev = nullptr;
-  float* d_wts = nullptr;  // learned weights in the pre-BP's order, room for wts_T iterations
-  int wts_T = 0;
+  float* d_wts = nullptr;  // learned weights in the pre-BP's order, room for wts_rows iterations
+  int wts_rows = 0;
 };
 
 template <class T>
@@ -193,6 +193,9 @@ struct qd_decoder {
   size_t kpath_slots = 0;
   uint32_t *d_det = nullptr, *d_obs = nullptr, *d_pred = nullptr, *d_fail = nullptr, *d_resid = nullptr;
   long long* d_nfail = nullptr;
+  // buffers that larger ones have replaced: a CUDA graph captured before may
+  // still write to them, so they stay until the decoder goes
+  std::vector<void*> retired;
 };
 
 namespace {
@@ -489,23 +492,23 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   return QD_OK;
 }
 
-// Room for T iterations' learned weights of window k in the pre-BP's order; the
-// first call makes room in every window, so that a decoder's weights are
-// installed window by window without further allocations.
-qd_status ensure_weight_space(qd_decoder* dec, int k, int T) {
+// Room for `rows` iterations' learned weights of window k in the pre-BP's order;
+// the first call makes room in every window, so that a decoder's weights are
+// installed window by window without further allocations.  A window that needs
+// more later gets at least twice as much (n_pre rows at most, which is all the
+// pre-BP reads), so that the replaced buffers together are no larger than the
+// last.
+qd_status ensure_weight_space(qd_decoder* dec, int k, int rows) {
   for (int i = 0; i < (int)dec->wins.size(); ++i) {
     WinGpu& g = dec->wins[i];
-    if (g.wts_T >= T || (i != k && g.wts_T > 0)) continue;
+    if (g.wts_rows >= rows || (i != k && g.wts_rows > 0)) continue;
+    const int room = std::max(rows, std::min(2 * g.wts_rows, dec->kp.n_pre));
     float* p = nullptr;
     const size_t per = 128 * (size_t)g.dv.row_quads + 32 * (size_t)g.dv.col_cells;
-    QD_CK(cudaMalloc(&p, sizeof(float) * std::max<size_t>(per * T, 4)));
-    cudaFree(g.d_wts);
+    QD_CK(cudaMalloc(&p, sizeof(float) * std::max<size_t>(per * room, 4)));
+    if (g.d_wts) dec->retired.push_back(g.d_wts);
     g.d_wts = p;
-    g.wts_T = T;
-    if (g.dv.wts) {  // (its weights are ordered again before every decode)
-      g.dv.w_row = p;
-      g.dv.w_col = p + (size_t)g.dv.wT * 128 * g.dv.row_quads;
-    }
+    g.wts_rows = room;
   }
   return QD_OK;
 }
@@ -677,6 +680,7 @@ qd_status qd_decoder_destroy(qd_decoder* dec) {
   cudaFree(dec->d_fail);
   cudaFree(dec->d_resid);
   cudaFree(dec->d_nfail);
+  for (void* p : dec->retired) cudaFree(p);
   delete dec;
   return QD_OK;
 }
@@ -762,7 +766,7 @@ qd_status qd_decoder_create(const qd_dem* dem, const qd_gdg_params* p, int64_t m
     char* b = g.d_graph;
     g.dv = qd::WinDev{h.n_rows, h.n_cols, h.n_edges, h.row0, h.n_short, h.short_edges_max, h.n_rows / h.n_blocks,
                       (const uint16_t*)(b + o_cp), (const uint16_t*)(b + o_cr), (const uint16_t*)(b + o_rp),
-                      (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0, nullptr, nullptr,
+                      (const uint32_t*)(b + o_re), (const float*)(b + o_ll), nullptr, 0, 0, nullptr, nullptr,
                       h.last ? h.n_rows : std::min(h.n_rows, dec->P.F * (h.n_rows / h.n_blocks)),
                       h.row_quads, h.col_cells, (const uint16_t*)(b + s_re), (const uint32_t*)(b + s_ce),
                       (const uint16_t*)(b + s_ro), (const uint16_t*)(b + s_co), (const float*)(b + s_ll),
@@ -1047,13 +1051,15 @@ qd_status qd_decoder_set_weights(qd_decoder* dec, int k, const float* w, int T) 
   QD_REQ(dec, "null argument");
   QD_REQ(k >= 0 && k < (int)dec->wins.size(), "qd_decoder_set_weights: window out of range");
   QD_REQ(w == nullptr || T >= 1, "qd_decoder_set_weights: T must be >= 1");
-  if (w) QD_CK_ST(ensure_weight_space(dec, k, T));
+  const int rows = std::min(T, dec->kp.n_pre);  // that the pre-BP reads
+  if (w) QD_CK_ST(ensure_weight_space(dec, k, rows));
   const qd::WinDev old = dec->wins[k].dv;
   WinGpu& g = dec->wins[k];
   g.dv.wts = w;
   g.dv.wT = w ? T : 0;
+  g.dv.w_rows = w ? rows : 0;
   g.dv.w_row = w ? g.d_wts : nullptr;
-  g.dv.w_col = w ? g.d_wts + (size_t)T * 128 * g.dv.row_quads : nullptr;
+  g.dv.w_col = w ? g.d_wts + (size_t)rows * 128 * g.dv.row_quads : nullptr;
   // the layouts keep the shortened edges' full-window ids only while some
   // window has learned weights
   bool want = false;
