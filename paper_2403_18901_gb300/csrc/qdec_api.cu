@@ -82,7 +82,7 @@ struct ShotShape {
   int ctas = 2;         // CTAs per SM planned
   int grid_per_sm = 1;  // and resident
   int wave = 1;         // path slots of a typical shot
-  const int16_t* d_fork = nullptr;  // in WinGpu::d_fork
+  const int16_t* d_fork = nullptr;  // in one of WinGpu::d_fork
   int fork_nodes = 0;
   bool fork_on = false;
 };
@@ -98,7 +98,7 @@ struct WinGpu {
   qd::WinDev dv{};
   ShotShape sh[kShotCtas];  // shot mode, by CTAs per SM
   int best = 0;             // the one for large batches
-  int16_t* d_fork = nullptr;  // the shapes' snapshot plans
+  int16_t* d_fork[4] = {};  // the shapes' snapshot plans, by layout_form
   PathShape pa[kPathShapes];  // path mode, kPathThreads >> i threads
   char* d_graph = nullptr;
   int* d_ccptr = nullptr;  // committed columns: CSR of their global detector ids
@@ -199,6 +199,19 @@ struct qd_decoder {
 };
 
 namespace {
+// A larger buffer in the place of *p, which is kept (qd_decoder::retired).
+template <class T>
+qd_status replace_buffer(qd_decoder* dec, T** p, size_t bytes) {
+  T* q = nullptr;
+  QD_CK(cudaMalloc((void**)&q, bytes));
+  if (*p) dec->retired.push_back(*p);
+  *p = q;
+  return QD_OK;
+}
+
+// What the decoder's layouts are made for: learned weights, quantised history.
+int layout_form(bool lw, bool hist) { return (lw ? 1 : 0) | (hist ? 2 : 0); }
+
 // Shared-memory layouts of every window: as many decision-path slots (warps)
 // as fit in shot mode, then the path-mode layout with the window graph staged
 // in shared memory when it fits too.  The ranker and the candidate dump add
@@ -211,10 +224,7 @@ qd_status ensure_uscratch(qd_decoder* dec, bool all) {
     if (all || !g.fits)
       need = std::max(need, (size_t)dec->sm_count * g.grid_g * (size_t)(g.Lg.total - g.Lg.U));
   if (need <= dec->uscratch_bytes) return QD_OK;
-  cudaFree(dec->d_uscratch);
-  dec->d_uscratch = nullptr;
-  dec->uscratch_bytes = 0;
-  QD_CK(cudaMalloc(&dec->d_uscratch, need));
+  QD_CK_ST(replace_buffer(dec, &dec->d_uscratch, need));
   dec->uscratch_bytes = need;
   return QD_OK;
 }
@@ -459,18 +469,19 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       ctas = std::max(ctas, dec->sm_count * std::max(s.grid_per_sm, g.grid_g));
     }
     if (v.empty()) continue;
-    if (!g.d_fork) QD_CK(cudaMalloc(&g.d_fork, sizeof(int16_t) * plan * kShotCtas));
-    QD_CK(cudaMemcpy(g.d_fork, v.data(), sizeof(int16_t) * v.size(), cudaMemcpyHostToDevice));
-    for (int i = 0; i <= g.best; ++i) g.sh[i].d_fork = g.d_fork + plan * i;
+    // a plan follows from the form, and one that a captured graph may read is
+    // never written again
+    int16_t*& d = g.d_fork[layout_form(dec->lw_on, hist)];
+    if (!d) {
+      QD_CK(cudaMalloc(&d, sizeof(int16_t) * plan * kShotCtas));
+      QD_CK(cudaMemcpy(d, v.data(), sizeof(int16_t) * v.size(), cudaMemcpyHostToDevice));
+    }
+    for (int i = 0; i <= g.best; ++i) g.sh[i].d_fork = d + plan * i;
   }
   if (cta_bytes > dec->snap_cta_bytes || ctas > dec->snap_ctas) {
     const size_t cb = std::max(cta_bytes, dec->snap_cta_bytes);
     const int nc = std::max(ctas, dec->snap_ctas);
-    cudaFree(dec->d_snap);
-    dec->d_snap = nullptr;
-    dec->snap_cta_bytes = 0;
-    dec->snap_ctas = 0;
-    QD_CK(cudaMalloc(&dec->d_snap, cb * nc));
+    QD_CK_ST(replace_buffer(dec, &dec->d_snap, cb * nc));
     dec->snap_cta_bytes = cb;
     dec->snap_ctas = nc;
   }
@@ -480,10 +491,7 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       for (int i = 0; i <= g.best; ++i) cmax = std::max(cmax, dec->sm_count * std::max(g.sh[i].grid_per_sm, g.grid_g));
     const size_t slots = std::max<size_t>(cmax, (size_t)std::min<long long>(dec->max_shots, kPathModeMaxShots));
     if (slots > dec->kpath_slots) {
-      cudaFree(dec->d_kpath);
-      dec->d_kpath = nullptr;
-      dec->kpath_slots = 0;
-      QD_CK(cudaMalloc(&dec->d_kpath, sizeof(float) * slots * dec->kp.nb * std::max(1, dec->ns_max)));
+      QD_CK_ST(replace_buffer(dec, &dec->d_kpath, sizeof(float) * slots * dec->kp.nb * std::max(1, dec->ns_max)));
       dec->kpath_slots = slots;
     }
   }
@@ -503,11 +511,8 @@ qd_status ensure_weight_space(qd_decoder* dec, int k, int rows) {
     WinGpu& g = dec->wins[i];
     if (g.wts_rows >= rows || (i != k && g.wts_rows > 0)) continue;
     const int room = std::max(rows, std::min(2 * g.wts_rows, dec->kp.n_pre));
-    float* p = nullptr;
     const size_t per = 128 * (size_t)g.dv.row_quads + 32 * (size_t)g.dv.col_cells;
-    QD_CK(cudaMalloc(&p, sizeof(float) * std::max<size_t>(per * room, 4)));
-    if (g.d_wts) dec->retired.push_back(g.d_wts);
-    g.d_wts = p;
+    QD_CK_ST(replace_buffer(dec, &g.d_wts, sizeof(float) * std::max<size_t>(per * room, 4)));
     g.wts_rows = room;
   }
   return QD_OK;
@@ -660,7 +665,7 @@ qd_status qd_decoder_destroy(qd_decoder* dec) {
     cudaFree(w.d_ccdet);
     cudaFree(w.d_ccobs);
     cudaFree(w.d_wthr);
-    cudaFree(w.d_fork);
+    for (int16_t* p : w.d_fork) cudaFree(p);
     cudaFree(w.d_prev);
     cudaFree(w.d_wts);
   }
@@ -1300,8 +1305,7 @@ struct qd_batch {
 };
 
 namespace {
-// The member's state its layouts depend on: learned weights, quantised history.
-int member_form(const qd_decoder* d) { return (d->lw_on ? 1 : 0) | (d->hist_on ? 2 : 0); }
+int member_form(const qd_decoder* d) { return layout_form(d->lw_on, d->hist_on); }
 
 // CTAs of `warps` warps with at most `budget` bytes of dynamic shared memory:
 // each member's layout takes as many path slots (<= warps) as fit.
