@@ -1468,15 +1468,21 @@ struct DecodeArgs {
 };
 
 // UG (a template parameter, so that shared-memory kernels keep shared-memory
-// instructions for every union access): the region lives in global memory.
-template <bool UG>
+// instructions for every union access): 1: the region lives in global memory;
+// 2: the shortened graph's entries as well, at its start (Layout::gg).
+template <int UG>
 __device__ __forceinline__ char* union_base(const DecodeArgs& A, char* sm, const SlotPlan& S) {
-  if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
+  if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes + (UG == 2 ? S.U : 0u);
   return sm + S.U;
+}
+// What the entries' offsets (SlotPlan::rent, cent, ref, cef) are relative to.
+template <int UG>
+__device__ __forceinline__ char* graph_base(const DecodeArgs& A, char* sm) {
+  return UG == 2 ? A.uglob + (size_t)blockIdx.x * A.ubytes : sm;
 }
 // The pre-BP scratch: the union region in global memory, else the bytes of the
 // shortened graph and the path slots, which do not exist yet.
-template <bool UG>
+template <int UG>
 __device__ __forceinline__ char* prebp_base(const DecodeArgs& A, char* sm) {
   if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
   return sm + A.L.V;
@@ -1815,7 +1821,7 @@ __device__ int prebp_cluster(const DecodeArgs& A, const WinDev& W, const PreBp& 
 
 // a1 + a2 (+ a3 when not converged): the shared prefix of both launch shapes.
 // Returns true when the pre-BP converged (cbits then hold its decision).
-template <bool LW, bool WIDE, bool UG>
+template <bool LW, bool WIDE, int UG>
 __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, long long shot, int* t_run_out,
                               Stager& stg) {
   const KParams& P = A.P;
@@ -2128,10 +2134,11 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
                   UG ? (unsigned)A.ubytes : L.total, UG, nw);
     if (tid == 0) *(SlotPlan*)(sm + L.plan) = S;
   }
-  uint32_t* rent = (uint32_t*)(sm + S.rent);
-  uint32_t* cent = (uint32_t*)(sm + S.cent);
-  uint16_t* sref = (uint16_t*)(sm + S.ref);
-  uint16_t* scef = (uint16_t*)(sm + S.cef);
+  char* ents = graph_base<UG>(A, sm);
+  uint32_t* rent = (uint32_t*)(ents + S.rent);
+  uint32_t* cent = (uint32_t*)(ents + S.cent);
+  uint16_t* sref = (uint16_t*)(ents + S.ref);
+  uint16_t* scef = (uint16_t*)(ents + S.cef);
   // every place a dummy, then the edges
   {
     const int nq = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
@@ -2176,12 +2183,14 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   return false;
 }
 
-__device__ __forceinline__ ShortG short_graph(char* sm, const Layout& L, const SlotPlan& S, const WinDev& W, int ns) {
+// ents: see graph_base
+__device__ __forceinline__ ShortG short_graph(char* sm, char* ents, const Layout& L, const SlotPlan& S, const WinDev& W,
+                                              int ns) {
   return ShortG{W.n_rows, ns, L.rw, L.sw, S.rwz,
-                (const uint32_t*)(sm + S.rent),   (const uint32_t*)(sm + S.cent),
+                (const uint32_t*)(ents + S.rent), (const uint32_t*)(ents + S.cent),
                 (const uint16_t*)(sm + L.s_roff), (const uint16_t*)(sm + L.s_coff),
                 (const float*)(sm + L.s_llr),     (const uint8_t*)(sm + L.s_vdeg),
-                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(sm + S.ref), (const uint16_t*)(sm + S.cef),
+                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(ents + S.ref), (const uint16_t*)(ents + S.cef),
                 (const ColClasses*)(sm + L.s_cls), W.wts, W.wT, W.n_edges, W.rows_per_block,
                 (const uint16_t*)(sm + L.sel),
                 (const uint16_t*)(sm + L.s_cperm), (const uint16_t*)(sm + L.s_vperm), W.n_commit_rows};
@@ -2263,7 +2272,7 @@ __device__ void keep_for_next(const DecodeArgs& A, char* sm, long long shot, con
 // ---- shot mode: persistent CTAs of up to 12 warps, one warp per decision path ----
 // One shot of one window by the whole CTA (every thread calls).  misc[2], the
 // decision-path queue, must be 0 on entry.
-template <bool LW, bool UG>
+template <bool LW, int UG>
 __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager& stg) {
   const Layout& L = A.L;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -2282,7 +2291,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
     // warps beyond the shot's path slots sit out the paths
     const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
     if (warp < S.nslots) {
-      const ShortG G = short_graph(sm, L, S, A.W, n_short);
+      const ShortG G = short_graph(sm, graph_base<UG>(A, sm), L, S, A.W, n_short);
       char* slot = union_base<UG>(A, sm, S) + (size_t)warp * S.b_size;
       const Slot B = make_slot(slot, S);
       const WarpGrp g{lane};
@@ -2408,7 +2417,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
 // per SM; HBM is idle.  One warp per path keeps every barrier of a path a warp's;
 // 5000 shots of [[144,12,12]], all windows, took 450 ms with two CTAs per SM and
 // the graph in CSR, 231 ms so; 9001 of the paper preset 200 and 104 ms.
-template <bool LW, bool UG, int CTAS>
+template <bool LW, int UG, int CTAS>
 __global__ void __launch_bounds__(CTAS == 1 ? 384 : 256, CTAS) decode_shot_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
   int* misc = (int*)(sm + A.L.misc);
@@ -2458,8 +2467,8 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
       for (int x = threadIdx.x; x < 2 * kMaxForkNodes; x += blockDim.x) ((int*)(sm + A.L.red))[x] = 0;
     __syncthreads();
     // (members without learned weights may share the launch with others)
-    if (LW && A.W.wts) shot_body<true, false>(A, shot, sm, stg);
-    else shot_body<false, false>(A, shot, sm, stg);
+    if (LW && A.W.wts) shot_body<true, 0>(A, shot, sm, stg);
+    else shot_body<false, 0>(A, shot, sm, stg);
   }
 }
 
@@ -2481,19 +2490,19 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   char* tr = A.trace ? A.trace + (size_t)shot * A.tr_bytes : nullptr;
   Stager stg = stager_init((char*)(misc + 8), &A.counters[4]);
   int t_run = 0;
-  const bool conv = window_prefix<LW, true, false>(A, A.W, sm, shot, &t_run, stg);
+  const bool conv = window_prefix<LW, true, 0>(A, A.W, sm, shot, &t_run, stg);
   if (id >= nb) return;  // a CTA that only shared the pre-BP of its cluster
   if (conv) {
     if (id == 0) {
       write_outputs(A, sm, shot, true, -1, 0, t_run, tr);
-      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<false>(A, sm) + L.p_post));
+      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<0>(A, sm) + L.p_post));
     }
     return;
   }
   const int n_short = A.W.n_short;
   const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
-  const ShortG G = short_graph(sm, L, S, A.W, n_short);
-  const Slot B = make_slot(union_base<false>(A, sm, S), S);
+  const ShortG G = short_graph(sm, sm, L, S, A.W, n_short);
+  const Slot B = make_slot(union_base<0>(A, sm, S), S);
   const CtaGrp g{tid, (int)blockDim.x, sm + L.red};
   const size_t rb = path_result_bytes(A.sw_max);
   char* mine = A.path_res + ((size_t)shot * nb + id) * rb;
@@ -2726,10 +2735,11 @@ __global__ void evaluate_kernel(const uint32_t* __restrict__ pred, const uint32_
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max) { return dev::trace_bytes(nb, dmx, ns_max); }
 
 cudaError_t set_decode_smem(size_t bytes) {
-  const void* f[] = {(const void*)dev::decode_shot_kernel<false, false, 2>, (const void*)dev::decode_shot_kernel<true, false, 2>,
-                     (const void*)dev::decode_shot_kernel<false, true, 2>,  (const void*)dev::decode_shot_kernel<true, true, 2>,
-                     (const void*)dev::decode_shot_kernel<false, false, 1>, (const void*)dev::decode_shot_kernel<true, false, 1>,
-                     (const void*)dev::decode_shot_kernel<false, false, 3>, (const void*)dev::decode_path_kernel<false>,
+  const void* f[] = {(const void*)dev::decode_shot_kernel<false, 0, 2>, (const void*)dev::decode_shot_kernel<true, 0, 2>,
+                     (const void*)dev::decode_shot_kernel<false, 1, 2>,  (const void*)dev::decode_shot_kernel<true, 1, 2>,
+                     (const void*)dev::decode_shot_kernel<false, 2, 2>, (const void*)dev::decode_shot_kernel<true, 2, 2>,
+                     (const void*)dev::decode_shot_kernel<false, 0, 1>, (const void*)dev::decode_shot_kernel<true, 0, 1>,
+                     (const void*)dev::decode_shot_kernel<false, 0, 3>, (const void*)dev::decode_path_kernel<false>,
                      (const void*)dev::decode_path_kernel<true>,            (const void*)dev::decode_batch_kernel<false>,
                      (const void*)dev::decode_batch_kernel<true>};
   for (const void* k : f)
@@ -2786,13 +2796,15 @@ cudaError_t launch_commit_batch(cudaStream_t st, const BatchMember* m, int n) {
 cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* blocks) {
   if (mode == 1)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_path_kernel<false>, threads, smem);
+  if (mode == 4)  // shot mode with the shortened graph's entries in global memory as well
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 2, 2>, threads, smem);
   if (mode == 3)  // shot mode with the union region in global memory
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, true, 2>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 1, 2>, threads, smem);
   if (ctas == 1)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 1>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 0, 1>, threads, smem);
   if (ctas >= 3)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 3>, threads, smem);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, false, 2>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 0, 3>, threads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 0, 2>, threads, smem);
 }
 
 cudaError_t path_cluster_occupancy(int threads, size_t smem, int cluster, int* clusters) {
@@ -2842,17 +2854,20 @@ cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem
     if (lw) return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<true>, A);
     return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<false>, A);
   } else {
-    if (uglob) {
-      if (lw) dev::decode_shot_kernel<true, true, 2><<<grid, threads, smem, st>>>(A);
-      else dev::decode_shot_kernel<false, true, 2><<<grid, threads, smem, st>>>(A);
+    if (uglob && L.gg) {
+      if (lw) dev::decode_shot_kernel<true, 2, 2><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, 2, 2><<<grid, threads, smem, st>>>(A);
+    } else if (uglob) {
+      if (lw) dev::decode_shot_kernel<true, 1, 2><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, 1, 2><<<grid, threads, smem, st>>>(A);
     } else if (ctas == 1) {
-      if (lw) dev::decode_shot_kernel<true, false, 1><<<grid, threads, smem, st>>>(A);
-      else dev::decode_shot_kernel<false, false, 1><<<grid, threads, smem, st>>>(A);
+      if (lw) dev::decode_shot_kernel<true, 0, 1><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, 0, 1><<<grid, threads, smem, st>>>(A);
     } else if (ctas >= 3 && !lw) {
-      dev::decode_shot_kernel<false, false, 3><<<grid, threads, smem, st>>>(A);
+      dev::decode_shot_kernel<false, 0, 3><<<grid, threads, smem, st>>>(A);
     } else {
-      if (lw) dev::decode_shot_kernel<true, false, 2><<<grid, threads, smem, st>>>(A);
-      else dev::decode_shot_kernel<false, false, 2><<<grid, threads, smem, st>>>(A);
+      if (lw) dev::decode_shot_kernel<true, 0, 2><<<grid, threads, smem, st>>>(A);
+      else dev::decode_shot_kernel<false, 0, 2><<<grid, threads, smem, st>>>(A);
     }
   }
   return cudaGetLastError();

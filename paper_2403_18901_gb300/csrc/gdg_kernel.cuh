@@ -249,6 +249,7 @@ struct Layout {
   // The pre-BP's arrays start at V, where the shortened graph and the path
   // slots begin: neither exists before the pre-BP has ended.
   unsigned V;
+  unsigned gg;  // 1: the entries too lie in the union region in global memory (s_dyn, SlotPlan::U relative to it)
   unsigned hist, lwe;  // bytes of quantised history per column of degree >= 3; 1: learned weights' edge ids
 };
 enum { kStageRent = 1, kStageCent = 2, kStageLlr = 4, kStageOff = 8 };
@@ -288,7 +289,8 @@ __host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell
   S.b_unsat = b; b = al16(b + 4u * L.rw);
   S.b_hq = b; b = al16(b + 32u * L.hist * n3);
   S.b_size = b;
-  const unsigned room = glob ? end : (end > S.U ? end - S.U : 0u);
+  const unsigned from = glob && !L.gg ? 0u : S.U;  // the slots' start
+  const unsigned room = end > from ? end - from : 0u;
   const int n = (int)(room / b);
   S.nslots = n < most ? n : most;
   S.rwz = rwz;
@@ -305,10 +307,17 @@ __host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell
 // total: what the window needs at least (one slot), or with what is staged;
 // past the budget the window does not fit.  ub_glob: pre-BP scratch and slots
 // live in a region of global memory (eight slots), the shortened graph stays
-// in shared memory, total - U is the region's size.
+// in shared memory, total - U is the region's size.  graph_glob (with ub_glob):
+// the shortened graph's entries start that region, the pre-BP scratch and, once
+// it is dead, the slots follow; for windows whose entries at their largest do
+// not fit shared memory (padded to slices they take up to twice the bytes of
+// plain CSC and CSR arrays: an unshortened [[144,12,12]] window of nine rounds,
+// or one of 17 rounds with learned weights).
 __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, int nc, int ns, int nb, unsigned budget,
-                                                    bool ranker, bool lw, bool ub_glob) {
+                                                    bool ranker, bool lw, bool ub_glob,
+                                                    bool graph_glob = false) {
   Layout L{};
+  L.gg = graph_glob ? 1u : 0u;
   L.rw = (nr + 31) / 32;
   L.cw = (nc + 31) / 32;
   L.sw = (ns + 31) / 32;
@@ -337,12 +346,12 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.s_vdeg = o; o = al16(o + nsp);
   L.s_cperm = o; o = al16(o + 2u * nr);
   L.s_vperm = o; o = al16(o + 2u * ns);
-  L.s_dyn = o;
+  L.s_dyn = graph_glob ? 0u : o;
   const SlotPlan S = slot_plan(L, D.srow_quads, D.scol_cells, L.rw, L.sw, 0u, ub_glob, 0);  // the largest
-  L.U = S.U;
+  L.U = graph_glob ? o : S.U;
   L.b_size = S.b_size;
   const unsigned p0 = ub_glob ? 0u : L.V;  // where the pre-BP scratch starts
-  unsigned u = 0;                          // relative to it
+  unsigned u = graph_glob ? S.U : 0u;      // relative to it
   L.p_post = u; u = al16(u + 4u * (ncp + 1));
   L.p_key = u; u = al16(u + 4u * ncp);
   L.p_cns = u; u = al16(u + 16u * (nrp + 1));
@@ -359,7 +368,8 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.p_end = own > sort_end ? own : sort_end;
   if (scr_end > L.p_end) L.p_end = scr_end;
   if (ub_glob) {
-    L.total = L.U + (8u * L.b_size > L.p_end ? 8u * L.b_size : L.p_end);
+    const unsigned slots = (graph_glob ? S.U : 0u) + 8u * L.b_size;
+    L.total = L.U + (slots > L.p_end ? slots : L.p_end);
     return L;
   }
   unsigned end = L.U + L.b_size > p0 + L.p_end ? L.U + L.b_size : p0 + L.p_end;

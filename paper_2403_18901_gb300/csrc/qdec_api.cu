@@ -361,8 +361,9 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       continue;
     }
     const auto& h = dec->wins[w].h;
-    auto lay = [&](unsigned budget, bool glob = false) {
-      return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob);
+    auto lay = [&](unsigned budget, bool glob = false, bool graph_glob = false) {
+      return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob,
+                                   graph_glob);
     };
     // CTAs per SM: for large batches the most resident decision-path warps
     // (CTAs x slots a typical shot gets); ties to fewer CTAs, which have room to
@@ -390,8 +391,10 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       }
     }
     // the union region in global memory: eight path slots, shared memory for
-    // the persistent part only, no pre-BP staging (its copies need shared memory)
+    // the persistent part only, no pre-BP staging (its copies need shared memory);
+    // a shortened graph too large for that goes to the region as well
     c.Lg = lay(0, true);
+    if (c.Lg.U > (unsigned)optin) c.Lg = lay(0, true, true);
     if (c.Lg.U > (unsigned)optin) {
       set_error(std::string(who) + ": window " + std::to_string(w) + " needs " + std::to_string(c.Lg.U) +
                 " B of shared memory even with its path state in global memory (limit " +
@@ -399,7 +402,7 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       return QD_EUNSUPPORTED;
     }
     int bg = 0;
-    QD_CK(qd::decode_occupancy(3, 2, 32 * kShotWarps, c.Lg.U, &bg));
+    QD_CK(qd::decode_occupancy(c.Lg.gg ? 4 : 3, 2, 32 * kShotWarps, c.Lg.U, &bg));
     c.grid_g = std::max(1, bg);
     if (!c.fits) {  // shot mode streams the path state through L2 / HBM
       c.sh[0] = ShotShape{};

@@ -77,7 +77,7 @@ bool build_slices(WindowHost& o, const WindowHost* like = nullptr);
 size_t trace_bytes_per_shot(int nb, int dmx, int ns_max);
 cudaError_t set_decode_smem(size_t bytes);
 // CTAs per SM of the decode kernel: mode 0 shot mode, 1 path mode, 3 shot
-// mode with the union region in global memory; ctas: the CTAs per SM the kernel
+// mode with the union region in global memory, 4 with the shortened graph too; ctas: the CTAs per SM the kernel
 // is compiled for (2, or 3 with fewer registers).
 cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* blocks);
 cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
