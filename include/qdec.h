@@ -357,7 +357,9 @@ qd_status qd_batch_n_steps(const qd_batch* b, int* n_steps);
  *   residue_fail[i] [n_shots[i]], |= the Eq. (11) residue flag
  * Members without window `step`, or with n_shots[i] = 0, are skipped.
  * Asynchronous on `stream`; capturable in a CUDA graph (it launches a memset
- * and two kernels).
+ * and two kernels; a member whose window fits the step's shape as plain arrays
+ * but not in slices -- an unshortened one with learned weights -- is decoded by
+ * qd_decode_windows in their place).
  */
 qd_status qd_batch_step(qd_batch* b, int step, uint32_t* const* det_bits, const int64_t* n_shots,
                         uint32_t* const* obs_pred, uint32_t* const* residue_fail, qd_stream_t stream);

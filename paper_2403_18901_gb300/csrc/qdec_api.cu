@@ -1301,6 +1301,7 @@ struct qd_batch {
     unsigned q_off = 0;
     std::vector<qd::Layout> L;  // per member (unused where the member has no such window)
     std::vector<int> form;      // per member: what its layout was made for (member_form)
+    std::vector<char> own;      // per member: decoded by a launch of its own (see batch_plan)
   };
   std::vector<Step> steps;
   int* d_work = nullptr;  // one counter per step
@@ -1311,10 +1312,15 @@ namespace {
 int member_form(const qd_decoder* d) { return layout_form(d->lw_on, d->hist_on); }
 
 // CTAs of `warps` warps with at most `budget` bytes of dynamic shared memory:
-// each member's layout takes as many path slots (<= warps) as fit.
+// each member's layout takes as many path slots (<= warps) as fit.  A shape is
+// for windows whose plain CSC and CSR arrays leave room for a slot (make_layout);
+// in slices a few of those do not fit (unshortened windows with learned weights,
+// one size per code: [[72,12,6]] (5,1) on half an SM), and such a member is
+// decoded by its own launch in the same step.
 qd_status batch_plan(qd_batch* b, int j, int warps, size_t budget) {
   qd_batch::Step S;
   S.L.assign(b->mem.size(), qd::Layout{});
+  S.own.assign(b->mem.size(), 0);
   for (const qd_decoder* d : b->mem) S.form.push_back(member_form(d));
   unsigned mx = 0;
   for (size_t i = 0; i < b->mem.size(); ++i) {
@@ -1325,6 +1331,12 @@ qd_status batch_plan(qd_batch* b, int j, int warps, size_t budget) {
     S.L[i] = qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, d->kp.nb, room, d->hist_on, d->lw_on,
                                    false);
     if (S.L[i].total > room) {
+      const unsigned plain = qd::make_layout(h.n_rows, h.n_cols, h.n_edges, h.n_short, h.short_edges_max, d->kp.nb, 1,
+                                             false, d->hist_on, d->lw_on).total;
+      if (qd::al16(plain) + 32 <= budget) {
+        S.own[i] = 1;
+        continue;
+      }
       set_error("qd_batch: member " + std::to_string(i) + " window " + std::to_string(j) + " needs " +
                 std::to_string(S.L[i].total + 32) + " B of shared memory with one path slot (budget " +
                 std::to_string(budget) + ")");
@@ -1383,6 +1395,7 @@ int batch_members(qd_batch* b, int j, uint32_t* const* det, const int64_t* n, ui
     b->forks.resize(b->mem.size());
     b->forks[i] = fork_dev(d, g.sh[g.best]);
     m.fork = &b->forks[i];
+    m.who = i;
     out.push_back(m);
   }
   return (int)out.size();
@@ -1392,8 +1405,11 @@ qd_status batch_decode(qd_batch* b, int j, const std::vector<qd::BatchMember>& a
   const qd_batch::Step& S = b->steps[j];
   // windows without columns decide nothing; their commits still test the residue
   std::vector<qd::BatchMember> m;
-  for (const auto& x : all)
-    if (x.W->n_cols > 0) m.push_back(x);
+  for (const auto& x : all) {
+    if (x.W->n_cols == 0) continue;
+    if (S.own[x.who]) QD_CK_ST(qd_decode_windows(b->mem[x.who], j, x.det, x.n, x.corr, nullptr, nullptr, st));
+    else m.push_back(x);
+  }
   if (m.empty()) return QD_OK;
   long long tot = 0;
   for (const auto& x : m) tot += x.n;
@@ -1497,7 +1513,7 @@ qd_status qd_batch_step(qd_batch* b, int step, uint32_t* const* det_bits, const 
     if (b->steps[step].form[i] != member_form(b->mem[i])) {
       const int warps = b->steps[step].warps;
       const size_t budget = b->steps[step].budget;
-      QD_CK_ST(batch_plan(b, step, warps, budget));
+      if (batch_plan(b, step, warps, budget) != QD_OK) QD_CK_ST(batch_plan(b, step, warps, (size_t)b->optin));
       break;
     }
   std::vector<qd::BatchMember> m;
