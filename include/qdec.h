@@ -487,11 +487,13 @@ qd_status qd_set_zero(void* dst, size_t bytes, qd_stream_t stream);
  * soft-syndrome binary cross entropy at t = T: P(check j odd) =
  * (1 - prod_{i in N(j)} tanh(Lambda_i^(T) / 2)) / 2 against s_j, averaged over
  * the window's checks.  Gradients come from a hand-written adjoint of the
- * unrolled iterations, from the check records that the forward pass keeps for
- * every iteration.
- *   qd_wms_create  allocates per-CTA scratch for T iterations; 1 <= ckpt <= T
- *                  (a spacing of checkpoints; results do not depend on it, and
- *                  none are needed now that every iteration is kept)
+ * unrolled iterations, from the check records that the forward pass keeps.
+ *   qd_wms_create  allocates scratch for the check records: all T iterations'
+ *                  where that takes at most 256 MB (16 bytes per check and
+ *                  iteration for every resident CTA), else every ckpt-th one's
+ *                  and those of one segment of ckpt iterations, the others
+ *                  being computed again; 1 <= ckpt <= T, and results do not
+ *                  depend on it
  *   qd_wms_info    out[6] = rows, columns, edges, T, ckpt, syndrome words
  *   qd_wms_sample  synd: device [n][syndrome words]; counter-based like
  *                  qd_sample_shots, with word 3 of the counter = 1 + k

@@ -180,6 +180,19 @@ struct WmsSlices {
   const float* llr;              // by column label
   const uint16_t *row, *col;     // label -> window row (0 for the padding), window column
   float clip;
+  // check records kept for the backward pass: every iteration's (0), or every
+  // seg-th iteration's and those of one segment of seg iterations at a time
+  int seg;
+  __host__ __device__ int segs() const { return (T + seg - 1) / seg; }
+  __host__ __device__ int records() const { return seg ? segs() - 1 + seg : T; }  // iterations there is room for
+  // where iteration t's record goes in the forward pass, -1: it is not kept
+  __host__ __device__ int slot_forward(int t) const {
+    if (!seg) return t - 1;
+    const int n = segs();
+    return t > (n - 1) * seg ? slot_backward(t) : (t % seg ? -1 : t / seg - 1);
+  }
+  // where it is when its segment is gone through backwards
+  __host__ __device__ int slot_backward(int t) const { return seg ? segs() - 1 + (t - 1) % seg : t - 1; }
 };
 
 // Compressed state of one check node: its two smallest |input| (bounded by the

@@ -21,7 +21,11 @@
 // records of iterations t and t + 1: the two smallest magnitudes and their
 // positions and the messages' signs; an input is within the clip exactly when
 // its magnitude is below it.  So the forward pass keeps 16 bytes per check and
-// iteration in global scratch and nothing is computed twice.  The gradient
+// iteration in global scratch and nothing is computed twice -- or, where that
+// would take too much memory (kWmsKeepBytes), every `ckpt`-th iteration's, and
+// the backward pass computes the records of one segment at a time again from
+// the one before it (a record and its iteration's weights give every message,
+// so what it computes is what the forward pass computed).  The gradient
 // into the inputs of an iteration is non-zero at two edges per check only:
 // their cells are written, the columns sum theirs in ascending order (float
 // atomics on the columns would be quicker by a tenth, but make a sample's
@@ -102,7 +106,48 @@ __device__ __forceinline__ float message(const WRec& r, uint32_t p, float w) {
   return with_sign(__fmul_rn(w, m), rec_sign(r, (int)p));
 }
 
-__global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const float* __restrict__ w,
+// The records of iterations t0 + 1 .. t1 into out, from that of t0 (unused for
+// t0 = 0), by the whole CTA with the forward pass's operations; v2c is zero
+// before and after.  Apart from the kernel, whose registers it would take.
+__device__ __noinline__ void recompute_records(const WmsSlices& G, const float* w, const uint32_t* sb, float* v2c,
+                                               const WRec* from, int t0, int t1, WRec* out) {
+  const int NT = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = NT >> 5, nrp = 32 * G.nrs;
+  auto columns = [&](const WRec* rec, const float* wt) {  // the inputs of the iteration after rec's
+    for (int s = warp; s < G.ncs; s += nw) {
+      const int c0 = 32 * G.coff[s] + lane, c1 = 32 * G.coff[s + 1];
+      auto input = [&](int c) {
+        const uint32_t e = G.cent[c], l = e >> 16;
+        if ((int)l >= nrp) return 0.0f;  // the dummy check's message
+        return message(rec[l], e & 0xFFFFu, entry_weight(wt, G.ceid[c]));
+      };
+      float p = G.llr[32 * s + lane];
+      for (int c = c0; c < c1; c += 32) p = __fadd_rn(p, input(c));  // ascending check order
+      for (int c = c0; c < c1; c += 32) v2c[c] = clipf(__fsub_rn(p, input(c)), G.clip);
+    }
+  };
+  __syncthreads();
+  if (t0 > 0) {
+    columns(from, w + (size_t)(t0 - 1) * G.ne);
+  } else {
+    for (int s = warp; s < G.ncs; s += nw)
+      for (int c = 32 * G.coff[s] + lane; c < 32 * G.coff[s + 1]; c += 32) v2c[c] = G.llr[32 * s + lane];
+  }
+  __syncthreads();
+  for (int t = t0 + 1; t <= t1; ++t) {
+    WRec* o = out + (size_t)(t - t0 - 1) * nrp;
+    for (int s = warp; s < G.nrs; s += nw) {
+      const int r0 = G.roff[s], l = 32 * s + lane, j = G.row[l];
+      o[l] = check_forward(G.rcell + 32 * r0 + lane, G.roff[s + 1] - r0, v2c, (sb[j >> 5] >> (j & 31)) & 1u);
+    }
+    __syncthreads();
+    if (t < t1) columns(o, w + (size_t)(t - 1) * G.ne);
+    __syncthreads();
+  }
+  for (int c = threadIdx.x; c < 32 * G.col_cells; c += NT) v2c[c] = 0.0f;
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ WmsSlices G, const float* __restrict__ w,
                                                      const uint32_t* __restrict__ synd, long long n, int backward,
                                                      float grad_scale, float* __restrict__ grad_w,
                                                      float* __restrict__ loss_out, float* __restrict__ post_out,
@@ -116,7 +161,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
   uint32_t* sb = (uint32_t*)(rec + nrp + 1);       // window syndrome by row
   double* red = (double*)(sb + ((G.rw + 3) & ~3));  // [32]
   int* sh_sample = (int*)(red + 32);
-  WRec* hist = scratch + (size_t)blockIdx.x * G.T * nrp;  // records by iteration
+  WRec* hist = scratch + (size_t)blockIdx.x * G.records() * nrp;  // records by iteration (slot_forward)
   while (true) {
     __syncthreads();
     if (tid == 0) *sh_sample = atomicAdd(work, 1);
@@ -135,12 +180,13 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
     __syncthreads();
     // ---- forward ----
     for (int t = 1; t <= G.T; ++t) {
+      const int slot = backward ? G.slot_forward(t) : -1;
       for (int s = warp; s < G.nrs; s += nw) {
         const int r0 = G.roff[s], l = 32 * s + lane;
         const int j = G.row[l];  // window row (0 for the padding, whose inputs are dummies)
         const WRec r = check_forward(G.rcell + 32 * r0 + lane, G.roff[s + 1] - r0, v2c, (sb[j >> 5] >> (j & 31)) & 1u);
         rec[l] = r;
-        if (backward) hist[(size_t)(t - 1) * nrp + l] = r;
+        if (slot >= 0) hist[(size_t)slot * nrp + l] = r;
       }
       __syncthreads();
       const float* wt = w + (size_t)(t - 1) * G.ne;
@@ -244,6 +290,9 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
     // sends: gA, gB; their cells; the positions and whether the clip passes ----
     for (int t = G.T; t >= 1; --t) {
       if (t < G.T) {
+        if (G.seg && t % G.seg == 0)  // the last iteration of a segment gone through next
+          recompute_records(G, w, sb, v2c, hist + (size_t)max(t / G.seg - 2, 0) * nrp, t - G.seg, t,
+                            hist + (size_t)(G.segs() - 1) * nrp);
         __syncthreads();
         for (int s = warp; s < G.nrs; s += nw) {
           const WRec a = rec[32 * s + lane];
@@ -269,7 +318,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const WmsSlices G, const fl
       for (int s = warp; s < G.nrs; s += nw) {
         const int r0 = G.roff[s], d = G.roff[s + 1] - r0, l = 32 * s + lane;
         const uint16_t *col = G.rcol + 32 * r0 + lane, *eid = G.reid + 32 * r0 + lane, *cell = G.rcell + 32 * r0 + lane;
-        const WRec r = hist[(size_t)(t - 1) * nrp + l];
+        const WRec r = hist[(size_t)G.slot_backward(t) * nrp + l];
         WRec a{0.0f, 0.0f, 0u, 0u};
         if (t < G.T) a = rec[l];
         const int q1 = a.pw & 0x1000u ? (int)(a.pw & 63u) : -1, q2 = a.pw & 0x2000u ? (int)((a.pw >> 6) & 63u) : -1;
@@ -390,7 +439,7 @@ size_t wms_smem_bytes(const WmsSlices& G) {
          sizeof(lrn::WRec) * (32 * (size_t)G.nrs + 1) + 4 * (size_t)((G.rw + 3) & ~3) + 32 * sizeof(double) + 16;
 }
 
-size_t wms_scratch_per_cta(const WmsSlices& G) { return sizeof(lrn::WRec) * 32 * (size_t)G.nrs * G.T; }
+size_t wms_scratch_per_cta(const WmsSlices& G) { return sizeof(lrn::WRec) * 32 * (size_t)G.nrs * G.records(); }
 
 cudaError_t wms_set_smem(size_t bytes) {
   return cudaFuncSetAttribute(lrn::wms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);

@@ -1628,12 +1628,13 @@ qd_status qd_wms_create(const qd_decoder* dec, int k, int T, int ckpt, qd_wms** 
   m->S = qd::WmsSlices{m->G.nr, m->G.nc, m->G.ne, m->G.rw, T, (int)H.roff.size() - 1, (int)H.coff.size() - 1,
                        g.h.col_cells, u16(o_ro), u16(o_co), u16(o_rc), u16(o_rl), u16(o_re),
                        (const uint32_t*)(m->d_graph + o_ce), u16(o_ei), (const float*)(m->d_graph + o_ll), u16(o_rw),
-                       u16(o_cl), dec->P.clip};
+                       u16(o_cl), dec->P.clip, 0};
   m->smem = qd::wms_smem_bytes(m->S);
   QD_CK(qd::wms_set_smem((size_t)optin));  // the device limit: contexts of different sizes coexist
   int blocks = 0;
   QD_CK(qd::wms_occupancy(m->smem, &blocks));
   m->grid = dec->sm_count * std::max(1, blocks);
+  if (qd::wms_scratch_per_cta(m->S) * m->grid > qd::kWmsKeepBytes) m->S.seg = ckpt;
   QD_CK(cudaMalloc(&m->d_scratch, qd::wms_scratch_per_cta(m->S) * m->grid));
   QD_CK(cudaMalloc(&m->d_work, sizeof(int)));
   *out = m.release();

@@ -124,11 +124,17 @@ cudaError_t launch_commit(cudaStream_t st, int n_commit, const int* cptr, const 
 cudaError_t launch_evaluate(cudaStream_t st, const uint32_t* pred, const uint32_t* obs,
                             const uint32_t* resid, long long n, uint32_t* fail, long long* n_fail);
 
-// A window trains when this many bytes fit a CTA's shared memory (messages and
-// gradients of both directions; the kernel itself takes less, wms_smem_bytes).
+// A window trains when this many bytes fit a CTA's shared memory: the messages
+// and gradients of both directions, which a kernel without check records would
+// hold there.  The kernel itself takes less (wms_smem_bytes), but its check and
+// cell labels are 16-bit numbers and its grid has been measured up to this size
+// only, so that the limit stays.
 size_t wms_window_bytes(int ne, int nc, int rw);
 size_t wms_smem_bytes(const WmsSlices& G);
 size_t wms_scratch_per_cta(const WmsSlices& G);  // bytes
+// Every iteration's records are kept while a context's scratch stays within
+// this: 608 CTAs and [[144,12,12]] (3,1) windows, T <= 122.
+constexpr size_t kWmsKeepBytes = (size_t)256 << 20;
 cudaError_t wms_set_smem(size_t bytes);
 cudaError_t wms_occupancy(size_t smem, int* blocks);
 cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsSlices& G, const float* w, const uint32_t* synd,

@@ -57,8 +57,8 @@ class Wms:
 
 class WeightedMinSumLoss(torch.autograd.Function):
     """Mean soft-syndrome BCE of T unrolled weighted min-sum iterations.
-    Forward: qd_wms_loss; backward: the adjoint kernel qd_wms_grad (which
-    recomputes the unrolled iterations from message checkpoints)."""
+    Forward: qd_wms_loss; backward: the adjoint kernel qd_wms_grad (from the
+    check records that its own forward pass keeps)."""
 
     @staticmethod
     def forward(ctx, w, synd, wms):
