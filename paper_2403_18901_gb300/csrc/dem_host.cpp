@@ -511,65 +511,69 @@ namespace {
 // second visits to a bank group (a record read by two lanes is one visit).
 void spread_columns(const WindowHost& o, const std::vector<uint16_t>& rlab, uint16_t* cols, int n, int deg, int lane0) {
   constexpr int kLook = 96;
+  const size_t nr = rlab.size();
   std::vector<uint16_t> rows((size_t)n * deg);  // check labels of the columns, in `cols`' order
   std::vector<int> left(n);
   for (int i = 0; i < n; ++i) {
     left[i] = i;
     for (int u = 0; u < deg; ++u) rows[(size_t)i * deg + u] = rlab[o.col_rows[o.col_ptr[cols[i]] + u]];
   }
-  std::vector<uint16_t> seen((size_t)deg * 8), out(n);  // per entry: the eight lanes' check labels
-  int have = 0;
+  // per entry: the group's lanes by bank group, and which checks they read (the
+  // group that read one last; a group's number is never 0)
+  std::vector<int> lanes((size_t)deg * 8), read_by(deg * nr, 0);
+  std::vector<uint16_t> out(n);
+  int group = 1;
   for (int i = 0; i < n; ++i) {
-    if ((lane0 + i) % 8 == 0) have = 0;
+    if ((lane0 + i) % 8 == 0) {
+      std::fill(lanes.begin(), lanes.end(), 0);
+      ++group;
+    }
     int pick = i, best = 1 << 30;
     for (int x = i; x < n && x < i + kLook && best > 0; ++x) {
       const uint16_t* r = rows.data() + (size_t)left[x] * deg;
       int cost = 0;
-      for (int u = 0; u < deg && cost < best; ++u) {
-        const uint16_t* v = seen.data() + 8 * u;
-        int same = 0;
-        for (int y = 0; y < have; ++y) {
-          if (v[y] == r[u]) {
-            same = 0;
-            break;
-          }
-          same += ((v[y] ^ r[u]) & 7) == 0;
-        }
-        cost += same;
-      }
+      for (int u = 0; u < deg && cost < best; ++u)
+        if (read_by[u * nr + r[u]] != group) cost += lanes[8 * u + (r[u] & 7)];
       if (cost < best) {
         best = cost;
         pick = x;
       }
     }
     const int c = left[pick];
-    for (int x = pick; x > i; --x) left[x] = left[x - 1];
+    std::copy_backward(left.begin() + i, left.begin() + pick, left.begin() + pick + 1);
     left[i] = c;
-    for (int u = 0; u < deg; ++u) seen[8 * u + have] = rows[(size_t)c * deg + u];
-    ++have;
+    for (int u = 0; u < deg; ++u) {
+      const uint16_t r = rows[(size_t)c * deg + u];
+      lanes[8 * u + (r & 7)]++;
+      read_by[u * nr + r] = group;
+    }
     out[i] = cols[c];
   }
   std::copy(out.begin(), out.end(), cols);
 }
 
-// Positions for the entries of a slice's 32 checks (lab[lane]: their column
-// labels) that spread the check pass's posterior gathers over the 32 banks
-// (column label mod 32): position by position a matching of lanes to banks,
-// each lane to the bank of one of its entries left; a lane without a free bank
-// takes the entry whose bank has the fewest readers.  pos[lane][i]: the
-// position of the lane's i-th entry.
-void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::vector<std::vector<int>>& pos) {
-  const int n = (int)lab.size();
+// An entry of a check: its column label, its edge.
+struct RowEnt {
+  uint16_t col, edge;
+};
+
+// Positions for the entries of a slice's n <= 32 checks (lane l's: cnt[l] from
+// ent[l] on) that spread the check pass's posterior gathers over the 32 banks
+// (column label mod 32): position by position, from `first` on, a matching of
+// lanes to banks, each lane to the bank of one of its entries left; a lane
+// without a free bank takes the entry whose bank has the fewest readers.
+// pos[e]: the position of edge e.
+void spread_positions(const RowEnt* const* ent, const int* cnt, int n, int first, std::vector<uint8_t>& pos) {
   struct Lane {
     uint8_t bank[kMaxRowDeg], ent[kMaxRowDeg];  // the entries left: bank, index
     int k;
   };
-  std::vector<Lane> left(n);
+  Lane left[32];
   int most = 0;
   for (int l = 0; l < n; ++l) {
-    left[l].k = (int)lab[l].size();
+    left[l].k = cnt[l];
     for (int i = 0; i < left[l].k; ++i) {
-      left[l].bank[i] = (uint8_t)(lab[l][i] & 31);
+      left[l].bank[i] = (uint8_t)(ent[l][i].col & 31);
       left[l].ent[i] = (uint8_t)i;
     }
     most = std::max(most, left[l].k);
@@ -604,7 +608,12 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
     int order[32], m = 0, load[32] = {};
     for (int l = 0; l < n; ++l)
       if (left[l].k) order[m++] = l;
-    std::stable_sort(order, order + m, [&](int a, int b) { return left[a].k > left[b].k; });
+    for (int x = 1; x < m; ++x) {  // stable, and hardly ever a move: the lanes come by descending degree
+      const int l = order[x];
+      int y = x;
+      for (; y > 0 && left[order[y - 1]].k < left[l].k; --y) order[y] = order[y - 1];
+      order[y] = l;
+    }
     for (int x = 0; x < m; ++x) {
       tried = 0;
       match(match, order[x]);
@@ -620,7 +629,7 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
           if (load[a.bank[y]] < load[a.bank[i]]) i = y;
         load[a.bank[i]]++;
       }
-      pos[order[x]][a.ent[i]] = first + u;
+      pos[ent[order[x]][a.ent[i]].edge] = (uint8_t)(first + u);
       --a.k;
       a.bank[i] = a.bank[a.k];
       a.ent[i] = a.ent[a.k];
@@ -636,7 +645,7 @@ void spread_positions(const std::vector<std::vector<int>>& lab, int first, std::
 // The order of a check's entries and of the columns changes no value.  Counted
 // for an interior [[144,12,12]] (3,1) window: 520 -> 352 wavefronts for the 228
 // gathers of a check pass, 1536 -> 987 for the 840 of a variable pass.
-// Building them takes 1.3 ms there and a stream has three distinct matrices
+// Building them takes 0.8 ms there and a stream has three distinct matrices
 // (first, interior, last), so a window takes the slices of the one before it
 // where the matrix is the same: seven built anew cost a decoder 20 ms.
 bool build_slices(WindowHost& o, const WindowHost* like) {
@@ -693,24 +702,24 @@ bool build_slices(WindowHost& o, const WindowHost* like) {
   o.s_ref.assign(o.s_rent.size(), kNoEdge);
   o.s_cef.assign(o.s_cent.size(), kNoEdge);
   o.s_llr.assign((size_t)32 * ncs, 0.0f);
-  std::vector<int> pos_of(o.n_edges, 0);
+  std::vector<uint8_t> pos_of(o.n_edges, 0);
   {
-    std::vector<std::vector<std::pair<int, int>>> ents(nr);  // by check label: (column label, edge)
+    std::vector<RowEnt> ents(o.n_edges);  // by window row, ascending column label
+    std::vector<int> end(o.row_ptr.begin(), o.row_ptr.end() - 1);
     for (int l = 0; l < nc; ++l)
       for (int e = o.col_ptr[o.s_col[l]]; e < o.col_ptr[o.s_col[l] + 1]; ++e)
-        ents[rlab[o.col_rows[e]]].push_back({l, e});
+        ents[end[o.col_rows[e]]++] = RowEnt{(uint16_t)l, (uint16_t)e};
     for (int q = 0; q < nrs; ++q)
       for (int h = 0; h < 2; ++h) {  // the first 32 entries, then the rest
         const int n = std::min(32, nr - 32 * q);
-        std::vector<std::vector<int>> lab(n), pos(n);
+        const RowEnt* ent[32];
+        int cnt[32];
         for (int l = 0; l < n; ++l) {
-          const auto& v = ents[32 * q + l];
-          for (size_t i = 32 * h; i < v.size() && (h || i < 32); ++i) lab[l].push_back(v[i].first);
-          pos[l].resize(lab[l].size());
+          const int j = o.s_row[32 * q + l];
+          cnt[l] = h ? std::max(0, rdeg(j) - 32) : std::min(rdeg(j), 32);
+          ent[l] = ents.data() + o.row_ptr[j] + (cnt[l] > 0 ? 32 * h : 0);
         }
-        spread_positions(lab, 32 * h, pos);
-        for (int l = 0; l < n; ++l)
-          for (size_t i = 0; i < pos[l].size(); ++i) pos_of[ents[32 * q + l][32 * h + i].second] = pos[l][i];
+        spread_positions(ent, cnt, n, 32 * h, pos_of);
       }
   }
   for (int l = 0; l < nc; ++l) {
