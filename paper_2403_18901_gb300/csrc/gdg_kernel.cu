@@ -1469,22 +1469,27 @@ struct DecodeArgs {
 
 // UG (a template parameter, so that shared-memory kernels keep shared-memory
 // instructions for every union access): 1: the region lives in global memory;
-// 2: the shortened graph's entries as well, at its start (Layout::gg).
+// 2: the shortened graph's entries as well, at its start (kGraphGlobal); 3: only
+// the entries' edge ids (kIdsGlobal).
 template <int UG>
 __device__ __forceinline__ char* union_base(const DecodeArgs& A, char* sm, const SlotPlan& S) {
-  if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes + (UG == 2 ? S.U : 0u);
+  if (UG == 1 || UG == 2) return A.uglob + (size_t)blockIdx.x * A.ubytes + (UG == 2 ? S.U : 0u);
   return sm + S.U;
 }
-// What the entries' offsets (SlotPlan::rent, cent, ref, cef) are relative to.
+// What the entries' offsets are relative to: SlotPlan::rent and cent, and ref and cef.
 template <int UG>
 __device__ __forceinline__ char* graph_base(const DecodeArgs& A, char* sm) {
   return UG == 2 ? A.uglob + (size_t)blockIdx.x * A.ubytes : sm;
+}
+template <int UG>
+__device__ __forceinline__ char* ids_base(const DecodeArgs& A, char* sm) {
+  return UG >= 2 ? A.uglob + (size_t)blockIdx.x * A.ubytes : sm;
 }
 // The pre-BP scratch: the union region in global memory, else the bytes of the
 // shortened graph and the path slots, which do not exist yet.
 template <int UG>
 __device__ __forceinline__ char* prebp_base(const DecodeArgs& A, char* sm) {
-  if (UG) return A.uglob + (size_t)blockIdx.x * A.ubytes;
+  if (UG == 1 || UG == 2) return A.uglob + (size_t)blockIdx.x * A.ubytes;
   return sm + A.L.V;
 }
 
@@ -1914,7 +1919,7 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
     __syncthreads();
   }
   int t_conv = 0;
-  if (WIDE && !UG && P.n_pre > 0 && cl_size() > 1 && nr >= 2 * (int)cl_size() && nc >= 2 * (int)cl_size()) {
+  if (WIDE && UG != 1 && UG != 2 && P.n_pre > 0 && cl_size() > 1 && nr >= 2 * (int)cl_size() && nc >= 2 * (int)cl_size()) {
     t = prebp_cluster<LW>(A, W, X, sm, conv, t_conv);
   } else {
 #pragma unroll 1
@@ -2131,14 +2136,14 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
 #pragma unroll 1
     while (rwz < rw && roff[rwz + 1] > roff[rwz]) ++rwz;
     S = slot_plan(L, roff[rw], coff[L.sw] & (kWideSlice - 1), rwz, ((const int*)(sm + L.s_cls))[1],
-                  UG ? (unsigned)A.ubytes : L.total, UG, nw);
+                  UG == 1 || UG == 2 ? (unsigned)A.ubytes : L.total, UG == 1 || UG == 2, nw);
     if (tid == 0) *(SlotPlan*)(sm + L.plan) = S;
   }
   char* ents = graph_base<UG>(A, sm);
   uint32_t* rent = (uint32_t*)(ents + S.rent);
   uint32_t* cent = (uint32_t*)(ents + S.cent);
-  uint16_t* sref = (uint16_t*)(ents + S.ref);
-  uint16_t* scef = (uint16_t*)(ents + S.cef);
+  uint16_t* sref = (uint16_t*)(ids_base<UG>(A, sm) + S.ref);
+  uint16_t* scef = (uint16_t*)(ids_base<UG>(A, sm) + S.cef);
   // every place a dummy, then the edges
   {
     const int nq = roff[rw], ncell = coff[L.sw] & (kWideSlice - 1);
@@ -2183,14 +2188,15 @@ __device__ bool window_prefix(const DecodeArgs& A, const WinDev& W, char* sm, lo
   return false;
 }
 
-// ents: see graph_base
-__device__ __forceinline__ ShortG short_graph(char* sm, char* ents, const Layout& L, const SlotPlan& S, const WinDev& W,
-                                              int ns) {
+template <int UG>
+__device__ __forceinline__ ShortG short_graph(const DecodeArgs& A, char* sm, const Layout& L, const SlotPlan& S,
+                                              const WinDev& W, int ns) {
+  const char *ents = graph_base<UG>(A, sm), *ids = ids_base<UG>(A, sm);
   return ShortG{W.n_rows, ns, L.rw, L.sw, S.rwz,
                 (const uint32_t*)(ents + S.rent), (const uint32_t*)(ents + S.cent),
                 (const uint16_t*)(sm + L.s_roff), (const uint16_t*)(sm + L.s_coff),
                 (const float*)(sm + L.s_llr),     (const uint8_t*)(sm + L.s_vdeg),
-                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(ents + S.ref), (const uint16_t*)(ents + S.cef),
+                (const uint32_t*)(sm + L.sbits),  (const uint16_t*)(ids + S.ref),   (const uint16_t*)(ids + S.cef),
                 (const ColClasses*)(sm + L.s_cls), W.wts, W.wT, W.n_edges, W.rows_per_block,
                 (const uint16_t*)(sm + L.sel),
                 (const uint16_t*)(sm + L.s_cperm), (const uint16_t*)(sm + L.s_vperm), W.n_commit_rows};
@@ -2291,7 +2297,7 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
     // warps beyond the shot's path slots sit out the paths
     const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
     if (warp < S.nslots) {
-      const ShortG G = short_graph(sm, graph_base<UG>(A, sm), L, S, A.W, n_short);
+      const ShortG G = short_graph<UG>(A, sm, L, S, A.W, n_short);
       char* slot = union_base<UG>(A, sm, S) + (size_t)warp * S.b_size;
       const Slot B = make_slot(slot, S);
       const WarpGrp g{lane};
@@ -2478,7 +2484,7 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
 // [[144,12,12]] shot issue in 34 % of the cycles, half of the stalls are barriers.
 // One shot, all windows: 7.7 ms with eight lanes per check and remote reads in the
 // pre-BP, 5.4 ms so.  The threads per CTA follow the batch (path_shape).
-template <bool LW>
+template <bool LW, int UG>
 __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];
   const Layout& L = A.L;
@@ -2490,19 +2496,19 @@ __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   char* tr = A.trace ? A.trace + (size_t)shot * A.tr_bytes : nullptr;
   Stager stg = stager_init((char*)(misc + 8), &A.counters[4]);
   int t_run = 0;
-  const bool conv = window_prefix<LW, true, 0>(A, A.W, sm, shot, &t_run, stg);
+  const bool conv = window_prefix<LW, true, UG>(A, A.W, sm, shot, &t_run, stg);
   if (id >= nb) return;  // a CTA that only shared the pre-BP of its cluster
   if (conv) {
     if (id == 0) {
       write_outputs(A, sm, shot, true, -1, 0, t_run, tr);
-      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<0>(A, sm) + L.p_post));
+      if (A.keep) keep_for_next(A, sm, shot, nullptr, 0, (const float*)(prebp_base<UG>(A, sm) + L.p_post));
     }
     return;
   }
   const int n_short = A.W.n_short;
   const SlotPlan& S = *(const SlotPlan*)(sm + L.plan);
-  const ShortG G = short_graph(sm, sm, L, S, A.W, n_short);
-  const Slot B = make_slot(union_base<0>(A, sm, S), S);
+  const ShortG G = short_graph<UG>(A, sm, L, S, A.W, n_short);
+  const Slot B = make_slot(union_base<UG>(A, sm, S), S);
   const CtaGrp g{tid, (int)blockDim.x, sm + L.red};
   const size_t rb = path_result_bytes(A.sw_max);
   char* mine = A.path_res + ((size_t)shot * nb + id) * rb;
@@ -2739,8 +2745,9 @@ cudaError_t set_decode_smem(size_t bytes) {
                      (const void*)dev::decode_shot_kernel<false, 1, 2>,  (const void*)dev::decode_shot_kernel<true, 1, 2>,
                      (const void*)dev::decode_shot_kernel<false, 2, 2>, (const void*)dev::decode_shot_kernel<true, 2, 2>,
                      (const void*)dev::decode_shot_kernel<false, 0, 1>, (const void*)dev::decode_shot_kernel<true, 0, 1>,
-                     (const void*)dev::decode_shot_kernel<false, 0, 3>, (const void*)dev::decode_path_kernel<false>,
-                     (const void*)dev::decode_path_kernel<true>,            (const void*)dev::decode_batch_kernel<false>,
+                     (const void*)dev::decode_shot_kernel<false, 0, 3>, (const void*)dev::decode_path_kernel<false, 0>,
+                     (const void*)dev::decode_path_kernel<true, 0>,         (const void*)dev::decode_path_kernel<true, 3>,
+                     (const void*)dev::decode_batch_kernel<false>,
                      (const void*)dev::decode_batch_kernel<true>};
   for (const void* k : f)
     if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) return e;
@@ -2795,7 +2802,7 @@ cudaError_t launch_commit_batch(cudaStream_t st, const BatchMember* m, int n) {
 
 cudaError_t decode_occupancy(int mode, int ctas, int threads, size_t smem, int* blocks) {
   if (mode == 1)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_path_kernel<false>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_path_kernel<false, 0>, threads, smem);
   if (mode == 4)  // shot mode with the shortened graph's entries in global memory as well
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, dev::decode_shot_kernel<false, 2, 2>, threads, smem);
   if (mode == 3)  // shot mode with the union region in global memory
@@ -2819,7 +2826,7 @@ cudaError_t path_cluster_occupancy(int threads, size_t smem, int cluster, int* c
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(clusters, dev::decode_path_kernel<false>, &cfg);
+  return cudaOccupancyMaxActiveClusters(clusters, dev::decode_path_kernel<false, 0>, &cfg);
 }
 
 cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem, cudaStream_t st, const KParams& P,
@@ -2851,10 +2858,14 @@ cudaError_t launch_decode(int mode, int ctas, int grid, int threads, size_t smem
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (lw) return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<true>, A);
-    return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<false>, A);
+    if (lw && L.gg == kIdsGlobal) {
+      if (!uglob) return cudaErrorInvalidValue;
+      return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<true, 3>, A);
+    }
+    if (lw) return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<true, 0>, A);
+    return cudaLaunchKernelEx(&cfg, dev::decode_path_kernel<false, 0>, A);
   } else {
-    if (uglob && L.gg) {
+    if (uglob && L.gg == kGraphGlobal) {
       if (lw) dev::decode_shot_kernel<true, 2, 2><<<grid, threads, smem, st>>>(A);
       else dev::decode_shot_kernel<false, 2, 2><<<grid, threads, smem, st>>>(A);
     } else if (uglob) {

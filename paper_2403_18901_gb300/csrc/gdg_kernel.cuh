@@ -262,9 +262,15 @@ struct Layout {
   // The pre-BP's arrays start at V, where the shortened graph and the path
   // slots begin: neither exists before the pre-BP has ended.
   unsigned V;
-  unsigned gg;  // 1: the entries too lie in the union region in global memory (s_dyn, SlotPlan::U relative to it)
+  // GraphPlace; with kGraphGlobal s_dyn and SlotPlan::U are relative to the union
+  // region in global memory, with kIdsGlobal the shortened entries' edge ids take
+  // `ids` bytes of global memory
+  unsigned gg, ids;
   unsigned hist, lwe;  // bytes of quantised history per column of degree >= 3; 1: learned weights' edge ids
 };
+// Where the shortened graph's entries lie: in shared memory; with the union region
+// in global memory; in shared memory, but for the edge ids of learned weights.
+enum GraphPlace { kGraphShared = 0, kGraphGlobal = 1, kIdsGlobal = 2 };
 enum { kStageRent = 1, kStageCent = 2, kStageLlr = 4, kStageOff = 8 };
 
 // A shot's part of the layout: the entries of its shortened graph, then its
@@ -275,6 +281,7 @@ struct SlotPlan {
   unsigned rent, cent, ref, cef, U;
   unsigned b_acc, b_hfl, b_status, b_cns, b_deg, b_sp, b_unsat, b_hq, b_size;
   int nslots, rwz;  // path slots that fit; non-empty check slices
+  unsigned ids;     // kIdsGlobal: bytes of edge ids
 };
 
 
@@ -289,8 +296,9 @@ __host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell
   unsigned o = L.s_dyn;
   S.rent = o; o = al16(o + 512u * nq);
   S.cent = o; o = al16(o + 128u * ncell);
-  S.ref = o; o = al16(o + (L.lwe ? 256u * nq : 0u));
-  S.cef = o; o = al16(o + (L.lwe ? 64u * ncell : 0u));
+  unsigned& at = L.gg == kIdsGlobal ? S.ids : o;
+  S.ref = at; at = al16(at + (L.lwe ? 256u * nq : 0u));
+  S.cef = at; at = al16(at + (L.lwe ? 64u * ncell : 0u));
   S.U = o;
   unsigned b = al16(4u * (nsp + 1));  // posteriors and the dummy column's
   S.b_acc = b; b += 128u * n3;
@@ -302,7 +310,7 @@ __host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell
   S.b_unsat = b; b = al16(b + 4u * L.rw);
   S.b_hq = b; b = al16(b + 32u * L.hist * n3);
   S.b_size = b;
-  const unsigned from = glob && !L.gg ? 0u : S.U;  // the slots' start
+  const unsigned from = glob && L.gg != kGraphGlobal ? 0u : S.U;  // the slots' start
   const unsigned room = end > from ? end - from : 0u;
   const int n = (int)(room / b);
   S.nslots = n < most ? n : most;
@@ -320,17 +328,19 @@ __host__ __device__ inline SlotPlan slot_plan(const Layout& L, int nq, int ncell
 // total: what the window needs at least (one slot), or with what is staged;
 // past the budget the window does not fit.  ub_glob: pre-BP scratch and slots
 // live in a region of global memory (eight slots), the shortened graph stays
-// in shared memory, total - U is the region's size.  graph_glob (with ub_glob):
-// the shortened graph's entries start that region, the pre-BP scratch and, once
+// in shared memory, total - U is the region's size.  place = kGraphGlobal
+// (with ub_glob): the shortened graph's entries start that region, the pre-BP scratch and, once
 // it is dead, the slots follow; for windows whose entries at their largest do
 // not fit shared memory (padded to slices they take up to twice the bytes of
 // plain CSC and CSR arrays: an unshortened [[144,12,12]] window of nine rounds,
-// or one of 17 rounds with learned weights).
+// or one of 17 rounds with learned weights).  kIdsGlobal (without ub_glob): see
+// GraphPlace; for path mode, where one path has the CTA for itself.
 __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, int nc, int ns, int nb, unsigned budget,
                                                     bool ranker, bool lw, bool ub_glob,
-                                                    bool graph_glob = false) {
+                                                    GraphPlace place = kGraphShared) {
   Layout L{};
-  L.gg = graph_glob ? 1u : 0u;
+  const bool graph_glob = place == kGraphGlobal;
+  L.gg = place;
   L.rw = (nr + 31) / 32;
   L.cw = (nc + 31) / 32;
   L.sw = (ns + 31) / 32;
@@ -362,6 +372,7 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   L.s_dyn = graph_glob ? 0u : o;
   const SlotPlan S = slot_plan(L, D.srow_quads, D.scol_cells, L.rw, L.sw, 0u, ub_glob, 0);  // the largest
   L.U = graph_glob ? o : S.U;
+  L.ids = S.ids;
   L.b_size = S.b_size;
   const unsigned p0 = ub_glob ? 0u : L.V;  // where the pre-BP scratch starts
   unsigned u = graph_glob ? S.U : 0u;      // relative to it

@@ -212,6 +212,9 @@ qd_status replace_buffer(qd_decoder* dec, T** p, size_t bytes) {
 // What the decoder's layouts are made for: learned weights, quantised history.
 int layout_form(bool lw, bool hist) { return (lw ? 1 : 0) | (hist ? 2 : 0); }
 
+// Path mode's CTAs per shot: the paths, rounded up to whole clusters.
+int path_ctas(const qd_decoder* dec, const PathShape& p) { return (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl; }
+
 // Shared-memory layouts of every window: as many decision-path slots (warps)
 // as fit in shot mode, then the path-mode layout with the window graph staged
 // in shared memory when it fits too.  The ranker and the candidate dump add
@@ -223,6 +226,10 @@ qd_status ensure_uscratch(qd_decoder* dec, bool all) {
   for (const WinGpu& g : dec->wins)
     if (all || !g.fits)
       need = std::max(need, (size_t)dec->sm_count * g.grid_g * (size_t)(g.Lg.total - g.Lg.U));
+  for (const WinGpu& g : dec->wins)  // path mode's edge ids
+    if (g.pa[0].fits && g.pa[0].L.gg == qd::kIdsGlobal)
+      need = std::max(need, (size_t)std::min(dec->max_shots, kPathModeMaxShots) * path_ctas(dec, g.pa[0]) *
+                                (size_t)g.pa[0].L.ids);
   if (need <= dec->uscratch_bytes) return QD_OK;
   QD_CK_ST(replace_buffer(dec, &dec->d_uscratch, need));
   dec->uscratch_bytes = need;
@@ -361,9 +368,9 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       continue;
     }
     const auto& h = dec->wins[w].h;
-    auto lay = [&](unsigned budget, bool glob = false, bool graph_glob = false) {
+    auto lay = [&](unsigned budget, bool glob = false, qd::GraphPlace place = qd::kGraphShared) {
       return qd::make_slice_layout(slice_dims(h), h.n_rows, h.n_cols, h.n_short, nb, budget, hist, dec->lw_on, glob,
-                                   graph_glob);
+                                   place);
     };
     // CTAs per SM: for large batches the most resident decision-path warps
     // (CTAs x slots a typical shot gets); ties to fewer CTAs, which have room to
@@ -394,7 +401,7 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
     // the persistent part only, no pre-BP staging (its copies need shared memory);
     // a shortened graph too large for that goes to the region as well
     c.Lg = lay(0, true);
-    if (c.Lg.U > (unsigned)optin) c.Lg = lay(0, true, true);
+    if (c.Lg.U > (unsigned)optin) c.Lg = lay(0, true, qd::kGraphGlobal);
     if (c.Lg.U > (unsigned)optin) {
       set_error(std::string(who) + ": window " + std::to_string(w) + " needs " + std::to_string(c.Lg.U) +
                 " B of shared memory even with its path state in global memory (limit " +
@@ -402,7 +409,7 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       return QD_EUNSUPPORTED;
     }
     int bg = 0;
-    QD_CK(qd::decode_occupancy(c.Lg.gg ? 4 : 3, 2, 32 * kShotWarps, c.Lg.U, &bg));
+    QD_CK(qd::decode_occupancy(c.Lg.gg == qd::kGraphGlobal ? 4 : 3, 2, 32 * kShotWarps, c.Lg.U, &bg));
     c.grid_g = std::max(1, bg);
     if (!c.fits) {  // shot mode streams the path state through L2 / HBM
       c.sh[0] = ShotShape{};
@@ -416,6 +423,10 @@ qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
       PathShape& s = c.pa[i];
       const unsigned budget = smem_budget(dec, 1 << i);
       s.L = lay(budget);
+      // learned weights' edge ids in global memory rather than no path mode: one
+      // shot of an unshortened [[72,12,6]] (10,1) window takes 2.2 ms so, 28 in shot
+      // mode with its paths in global memory
+      if (i == 0 && s.L.total > budget && dec->lw_on) s.L = lay(budget, false, qd::kIdsGlobal);
       s.fits = s.L.total <= budget;
       if (!s.fits) break;
       smem_max = std::max<size_t>(smem_max, s.L.total);
@@ -904,7 +915,8 @@ int path_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
   if (dec->launch_mode == 0)
     path_mode = n_shots * 2 <= dec->sm_count &&
                 (dec->kp.n_pre < 32 || n_shots * dec->kp.nb <= 9LL * dec->sm_count);
-  if (!path_mode || n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.fits || !g.pa[0].fits)
+  if (!path_mode || n_shots > std::min<long long>(dec->max_shots, kPathModeMaxShots) || !g.pa[0].fits ||
+      (!g.fits && g.pa[0].L.gg != qd::kIdsGlobal))
     return -1;
   int i = 0;
   const long long ctas = n_shots * dec->kp.nb;
@@ -962,8 +974,8 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   }
   // the path state in global memory when the window does not fit shared memory
   // (or on request)
-  const bool global = !g.fits || dec->launch_mode == 3;
   const int ps = path_shape(dec, g, n_shots);
+  const bool global = ps < 0 && (!g.fits || dec->launch_mode == 3);
   const ShotShape& s = shot_shape(dec, g, global ? INT64_MAX : n_shots);
   const qd::ForkDev fk = fork_dev(dec, s);
   const qd::ReuseDev ru = reuse_dev(dec, g);
@@ -979,11 +991,12 @@ qd_status qd_decode_windows(qd_decoder* dec, int k, const uint32_t* det_bits, in
   }
   if (ps >= 0) {
     const PathShape& p = g.pa[ps];
-    const int cps = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
+    const int cps = path_ctas(dec, p);
     QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads >> ps, p.L.total, st, dec->kp, g.dv, p.L,
                             det_bits, dw, n_shots, win_correction, dec->corr_words, status, (char*)trace,
                             dec->trace_bytes, dec->dmx, dec->ns_max, nullptr, dec->d_counters, dec->d_path_res,
-                            dec->d_arrive, dec->sw_max, nullptr, 0, cps, p.pcl, nullptr, &ru));
+                            dec->d_arrive, dec->sw_max, p.L.ids ? dec->d_uscratch : nullptr, p.L.ids, cps,
+                            p.pcl, nullptr, &ru));
     return QD_OK;
   }
   QD_CK(cudaMemsetAsync(dec->d_work + k, 0, sizeof(int), st));
@@ -1155,7 +1168,7 @@ qd_status qd_decoder_launch_info(const qd_decoder* dec, int k, int out[8]) {
   out[4] = kPathThreads;
   out[5] = dec->sm_count;
   out[6] = p.pcl;
-  out[7] = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
+  out[7] = path_ctas(dec, p);
   return QD_OK;
 }
 
@@ -1264,11 +1277,11 @@ extern "C" qd_status qd_decode_commit_static(qd_decoder* dec, int k, uint32_t* d
     if (g.dv.wts) QD_CK(qd::launch_order_weights(st, g.dv));
     if (ps >= 0) {
       const PathShape& p = g.pa[ps];
-      const int cps = (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl;
+      const int cps = path_ctas(dec, p);
       QD_CK(qd::launch_decode(1, 1, (int)(n_shots * cps), kPathThreads >> ps, p.L.total, st, dec->kp, g.dv, p.L,
                               det_bits, dw, n_shots, corr, dec->corr_words, nullptr, nullptr, 0, dec->dmx, dec->ns_max,
-                              nullptr, dec->d_counters, dec->d_path_res, dec->d_arrive, dec->sw_max, nullptr, 0, cps,
-                              p.pcl, nullptr, &ru));
+                              nullptr, dec->d_counters, dec->d_path_res, dec->d_arrive, dec->sw_max,
+                              p.L.ids ? dec->d_uscratch : nullptr, p.L.ids, cps, p.pcl, nullptr, &ru));
     } else {
       // the array keeps the previous call's contents: the work counter restarts at 0
       QD_CK(cudaMemsetAsync(work, 0, sizeof(int), st));

@@ -1,11 +1,12 @@
 // Host check of the layouts for windows whose shortened graph does not fit a
-// CTA's shared memory (make_slice_layout's graph_glob), built with g++ by
+// CTA's shared memory (make_slice_layout's kGraphGlobal), built with g++ by
 // tests/test_large_windows_host.py.
 //
 // usage: large_check l m a0x a0y .. b2x b2y rounds W shorten limit
 // The kernels have a layout within `limit` bytes of shared memory wherever the
 // plain CSC and CSR arrays (make_layout) with the path state in global memory
-// had one.  In the region of global memory the entries, the pre-BP scratch and
+// had one; path mode has one with the learned weights' edge ids in global memory
+// wherever it had one with the plain arrays.  In the region of global memory the entries, the pre-BP scratch and
 // the slots of the largest and of smaller shortened graphs are disjoint where
 // they live together.  Prints "ok", with the number of layouts that needed it.
 #include <algorithm>
@@ -48,12 +49,23 @@ int main(int argc, char** argv) {
         if (qd::make_layout(h.n_rows, h.n_cols, h.n_edges, h.n_short, h.short_edges_max, nb, 8, false, ranker, lw).U > limit)
           continue;
         auto lay = [&](bool gg) {
-          return qd::make_slice_layout(D, h.n_rows, h.n_cols, h.n_short, nb, 0, ranker, lw, true, gg);
+          return qd::make_slice_layout(D, h.n_rows, h.n_cols, h.n_short, nb, 0, ranker, lw, true, gg ? qd::kGraphGlobal : qd::kGraphShared);
         };
+        if (lw) {  // path mode's, with the edge ids in global memory
+          const qd::Layout L = qd::make_slice_layout(D, h.n_rows, h.n_cols, h.n_short, nb, limit, ranker, lw, false,
+                                                     qd::kIdsGlobal);
+          const qd::Layout O = qd::make_layout(h.n_rows, h.n_cols, h.n_edges, h.n_short, h.short_edges_max, nb, 1, true,
+                                               ranker, lw);
+          REQ(O.total - O.g_bytes > limit || L.total <= limit);
+          const qd::SlotPlan S = qd::slot_plan(L, D.srow_quads, D.scol_cells, L.rw, L.sw, L.total, false, 1);
+          REQ(S.ref == 0 && S.cef >= 256u * D.srow_quads && S.ids >= S.cef + 64u * D.scol_cells && S.ids == L.ids);
+          REQ(S.cent >= S.rent + 512u * D.srow_quads && S.U >= S.cent + 128u * D.scol_cells && S.U == L.U);
+          REQ(S.U + S.b_size <= L.total && L.V + L.p_end <= L.total && S.nslots == 1 && L.ids % 16u == 0);
+        }
         if (lay(false).U <= limit) continue;
         ++used;
         const qd::Layout L = lay(true);
-        REQ(L.gg && L.U <= limit && L.U % 16u == 0 && L.total % 16u == 0 && L.U >= L.s_vperm + 2u * h.n_short);
+        REQ(L.gg == qd::kGraphGlobal && L.U <= limit && L.U % 16u == 0 && L.total % 16u == 0 && L.U >= L.s_vperm + 2u * h.n_short);
         const unsigned end = L.total - L.U, nsp = qd::up32(h.n_short), nrp = qd::up32(h.n_rows), ncp = qd::up32(h.n_cols);
         for (int part = 0; part < 3; ++part) {  // the largest graph, a half, the smallest
           const int nq = part == 0 ? D.srow_quads : (part == 1 ? D.srow_quads / 2 : 1);

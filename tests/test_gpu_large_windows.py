@@ -38,6 +38,26 @@ def test_learned_weights():
     _pipeline("72", W, 0.003, params, n=n, seed=188, trace_windows=(1,), mode=0, weights=weights)
 
 
+@pytest.mark.parametrize("ranker,mode", [(False, 0), (True, 2)])
+def test_path_mode_with_edge_ids_in_global_memory(ranker, mode):
+    """One size at which learned weights' edge ids are what does not fit a path's CTA."""
+    W, n = 10, 4
+    params = preset("configured", k_guess=3, W=W, shorten=0, n_pre=20, d_max_main=12)
+    o = oracle_dem("72", 0.003, W)
+    rng = np.random.default_rng(8)
+    weights = {k: rng.uniform(0.45, 0.9, size=(15, o.window(W, 1, k)["n_edges"])).astype(np.float32) for k in range(2)}
+    rk = None
+    if ranker:
+        rk = np.zeros(641, np.float32)
+        rk[:512] = rng.normal(0, 0.6, 512)
+        rk[576:640] = rng.normal(0, 0.5, 64)
+    dec = qdec.Decoder(qdec.Dem(CODES["72"], 0.003, W), params, max_shots=n)
+    for k, w in weights.items():
+        dec.set_weights(k, torch.from_numpy(w).cuda())
+    assert dec.launch_info(0)["path_smem"] <= 232448 < dec.launch_info(0)["shot_smem"]
+    _pipeline("72", W, 0.003, params, n=n, seed=191, trace_windows=(0, 1), mode=mode, weights=weights, ranker=rk)
+
+
 def test_removing_the_weights_brings_the_smaller_layout_back():
     W, n = 13, 4
     dem = qdec.Dem(CODES["72"], 0.003, W)

@@ -30,7 +30,8 @@ def checker(tmp_path_factory):
 @pytest.mark.parametrize("key,W,shorten,some", [("72", 17, 0, True), ("72", 11, 0, True), ("72", 52, 1, True),
                                                 ("72", 36, 1, True), ("144", 9, 0, True), ("144", 26, 1, True),
                                                 ("144", 17, 1, True), ("288", 5, 0, True), ("288", 13, 1, True),
-                                                ("144", 3, 1, False)])
+                                                ("72", 10, 0, False), ("90", 8, 0, False), ("108", 7, 0, False),
+                                                ("144", 5, 0, False), ("144", 3, 1, False)])
 def test_every_window_that_fits_plain_arrays_has_a_layout(checker, key, W, shorten, some):
     c = CODES[key]
     args = [c["l"], c["m"]] + [v for t in c["A"] + c["B"] for v in t] + [W + 1, W, shorten, LIMIT]
