@@ -147,6 +147,9 @@ __device__ __noinline__ void recompute_records(const WmsSlices& G, const float* 
   __syncthreads();
 }
 
+// SEG: G.seg > 0 (a template, so that the kernel that keeps every record has no
+// bookkeeping for the others: 1 % of its time).
+template <bool SEG>
 __global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ WmsSlices G, const float* __restrict__ w,
                                                      const uint32_t* __restrict__ synd, long long n, int backward,
                                                      float grad_scale, float* __restrict__ grad_w,
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ Wms
   uint32_t* sb = (uint32_t*)(rec + nrp + 1);       // window syndrome by row
   double* red = (double*)(sb + ((G.rw + 3) & ~3));  // [32]
   int* sh_sample = (int*)(red + 32);
-  WRec* hist = scratch + (size_t)blockIdx.x * G.records() * nrp;  // records by iteration (slot_forward)
+  WRec* hist = scratch + (size_t)blockIdx.x * (SEG ? G.records() : G.T) * nrp;  // records by iteration (slot_forward)
   while (true) {
     __syncthreads();
     if (tid == 0) *sh_sample = atomicAdd(work, 1);
@@ -180,13 +183,13 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ Wms
     __syncthreads();
     // ---- forward ----
     for (int t = 1; t <= G.T; ++t) {
-      const int slot = backward ? G.slot_forward(t) : -1;
+      const int slot = !backward ? -1 : (SEG ? G.slot_forward(t) : t - 1);
       for (int s = warp; s < G.nrs; s += nw) {
         const int r0 = G.roff[s], l = 32 * s + lane;
         const int j = G.row[l];  // window row (0 for the padding, whose inputs are dummies)
         const WRec r = check_forward(G.rcell + 32 * r0 + lane, G.roff[s + 1] - r0, v2c, (sb[j >> 5] >> (j & 31)) & 1u);
         rec[l] = r;
-        if (slot >= 0) hist[(size_t)slot * nrp + l] = r;
+        if (SEG ? slot >= 0 : backward != 0) hist[(size_t)slot * nrp + l] = r;
       }
       __syncthreads();
       const float* wt = w + (size_t)(t - 1) * G.ne;
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ Wms
     // sends: gA, gB; their cells; the positions and whether the clip passes ----
     for (int t = G.T; t >= 1; --t) {
       if (t < G.T) {
-        if (G.seg && t % G.seg == 0)  // the last iteration of a segment gone through next
+        if (SEG && t % G.seg == 0)  // the last iteration of a segment gone through next
           recompute_records(G, w, sb, v2c, hist + (size_t)max(t / G.seg - 2, 0) * nrp, t - G.seg, t,
                             hist + (size_t)(G.segs() - 1) * nrp);
         __syncthreads();
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(256, 4) wms_kernel(const __grid_constant__ Wms
       for (int s = warp; s < G.nrs; s += nw) {
         const int r0 = G.roff[s], d = G.roff[s + 1] - r0, l = 32 * s + lane;
         const uint16_t *col = G.rcol + 32 * r0 + lane, *eid = G.reid + 32 * r0 + lane, *cell = G.rcell + 32 * r0 + lane;
-        const WRec r = hist[(size_t)G.slot_backward(t) * nrp + l];
+        const WRec r = hist[(size_t)(SEG ? G.slot_backward(t) : t - 1) * nrp + l];
         WRec a{0.0f, 0.0f, 0u, 0u};
         if (t < G.T) a = rec[l];
         const int q1 = a.pw & 0x1000u ? (int)(a.pw & 63u) : -1, q2 = a.pw & 0x2000u ? (int)((a.pw >> 6) & 63u) : -1;
@@ -442,18 +445,21 @@ size_t wms_smem_bytes(const WmsSlices& G) {
 size_t wms_scratch_per_cta(const WmsSlices& G) { return sizeof(lrn::WRec) * 32 * (size_t)G.nrs * G.records(); }
 
 cudaError_t wms_set_smem(size_t bytes) {
-  return cudaFuncSetAttribute(lrn::wms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const cudaError_t e =
+      cudaFuncSetAttribute(lrn::wms_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(lrn::wms_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 cudaError_t wms_occupancy(size_t smem, int* blocks) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, lrn::wms_kernel, 256, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, lrn::wms_kernel<false>, 256, smem);
 }
 
 cudaError_t launch_wms(cudaStream_t st, int grid, size_t smem, const WmsSlices& G, const float* w, const uint32_t* synd,
                        long long n, int backward, float grad_scale, float* grad_w, float* loss, float* post,
                        char* scratch, int* work) {
-  lrn::wms_kernel<<<grid, 256, smem, st>>>(G, w, synd, n, backward, grad_scale, grad_w, loss, post,
-                                           (lrn::WRec*)scratch, work);
+  const auto kernel = G.seg ? lrn::wms_kernel<true> : lrn::wms_kernel<false>;
+  kernel<<<grid, 256, smem, st>>>(G, w, synd, n, backward, grad_scale, grad_w, loss, post, (lrn::WRec*)scratch, work);
   return cudaGetLastError();
 }
 
