@@ -475,8 +475,9 @@ __device__ __forceinline__ uint32_t ordkey(float f) {
 // Lanes per check of a decision path run by a whole CTA: two where that takes
 // one round of threads / lanes checks, else one.  A shortened graph's checks
 // have a few entries each, so more lanes mostly add reduction steps (one
-// [[144,12,12]] shot, 11 windows: 8.0 ms with up to eight lanes in two rounds,
-// 6.9 ms with four in one, 6.7 ms with two).
+// [[144,12,12]] shot, 11 windows, when this was chosen: 8.0 ms with up to eight
+// lanes in two rounds, 6.9 ms with four in one, 6.7 ms with two; 5.9 ms with the
+// steps that followed).
 __host__ __device__ inline int path_lanes_per_check(int threads, int n_checks) {
   return threads / 2 >= n_checks ? 2 : 1;
 }
@@ -2301,7 +2302,6 @@ __device__ void shot_body(const DecodeArgs& A, long long shot, char* sm, Stager&
       char* slot = union_base<UG>(A, sm, S) + (size_t)warp * S.b_size;
       const Slot B = make_slot(slot, S);
       const WarpGrp g{lane};
-      // snapshots of shared prefixes, when planned and this CTA has a pool
       // shared prefixes and preemption, when planned and this CTA has a pool
       const bool fork = A.F.pool && (int)blockIdx.x < A.F.pool_ctas;
       const int nb = A.P.nb;
@@ -2482,8 +2482,9 @@ __global__ void __launch_bounds__(256, 2) decode_batch_kernel(const __grid_const
 // What bounds it: one path's serial chain (250 iterations of two passes with a
 // barrier each) after the cluster's pre-BP; 16 CTAs of 512 threads for one
 // [[144,12,12]] shot issue in 34 % of the cycles, half of the stalls are barriers.
-// One shot, all windows: 7.7 ms with eight lanes per check and remote reads in the
-// pre-BP, 5.4 ms so.  The threads per CTA follow the batch (path_shape).
+// One shot, all windows decoded and committed: 8.2 ms with eight lanes per check,
+// remote reads in the pre-BP and the graph in CSR, 5.9 ms so.  The threads per CTA
+// follow the batch (path_shape).
 template <bool LW, int UG>
 __global__ void __launch_bounds__(512, 1) decode_path_kernel(DecodeArgs A) {
   extern __shared__ __align__(16) char sm[];

@@ -418,9 +418,9 @@ __host__ __device__ inline Layout make_slice_layout(const SliceDims& D, int nr, 
   return L;
 }
 
-// The layout with one sign byte per edge and plain CSC / CSR arrays, kept as
-// the reference the layout checks state their invariants on; the decode
-// kernels take make_slice_layout.
+// The layout with one sign byte per edge and plain CSC / CSR arrays.  No kernel
+// takes it: it says which windows a batched step accepts (batch_plan), and the
+// layout checks compare the layouts in slices with it.
 // lw: the shortened edges' full-window edge ids (s_efull) are kept, which
 // only learned weights read
 __host__ __device__ inline Layout make_layout(int nr, int nc, int ne, int ns, int es, int nb,

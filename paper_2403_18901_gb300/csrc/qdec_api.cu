@@ -215,10 +215,6 @@ int layout_form(bool lw, bool hist) { return (lw ? 1 : 0) | (hist ? 2 : 0); }
 // Path mode's CTAs per shot: the paths, rounded up to whole clusters.
 int path_ctas(const qd_decoder* dec, const PathShape& p) { return (dec->kp.nb + p.pcl - 1) / p.pcl * p.pcl; }
 
-// Shared-memory layouts of every window: as many decision-path slots (warps)
-// as fit in shot mode, then the path-mode layout with the window graph staged
-// in shared memory when it fits too.  The ranker and the candidate dump add
-// the quantised history (4 bytes per short column) to every slot.
 // Global union regions for the windows that need them (all windows when
 // `all`): one region per resident CTA, allocated once, never on a decode call.
 qd_status ensure_uscratch(qd_decoder* dec, bool all) {
@@ -349,6 +345,10 @@ bool same_dims(const qd::WindowHost& a, const qd::WindowHost& b) {  // one layou
          a.scol_cells == b.scol_cells;
 }
 
+// Shared-memory layouts of every window: shot mode's for one to kShotCtas CTAs
+// per SM, the one with its path state in global memory, path mode's.  The ranker
+// and the candidate dump (hist) add the quantised history (4 bytes per column of
+// degree three or more) to every slot, learned weights the entries' edge ids.
 qd_status configure_layouts(qd_decoder* dec, bool hist, const char* who) {
   struct Conf {
     ShotShape sh[kShotCtas];
@@ -900,8 +900,9 @@ qd::ReuseDev reuse_dev(const qd_decoder* dec, const WinGpu& g) {
 // fits an SM; a batch of several CTAs per SM is faster with smaller ones side by
 // side.  Four CTAs of 128 threads pay from three per SM, and a window of at most
 // 128 checks gains nothing from more than 256 threads (two lanes per check).
-// Every cluster of a shot repeats the pre-BP, so a long one with more than nine
-// paths per SM is left to shot mode (32 paths, configured: [[144]] W = 4, 38 shots
+// Every cluster of a shot repeats the pre-BP, so a long one (100 iterations in all
+// the figures, against 8 and 16; no preset lies between) with more than nine paths
+// per SM is left to shot mode (32 paths, configured: [[144]] W = 4, 38 shots
 // 22.9 ms against 28.1 in shot mode, 45 28.6 / 28.6, 64 36.3 / 29.0; 22 paths of the
 // paper preset on [[288]] W = 4, 64 shots 13.5 / 23.3).
 // All windows of a pass, ms, with 512 x 1 / 256 x 2 / 128 x 4 and in shot mode:
@@ -909,7 +910,8 @@ qd::ReuseDev reuse_dev(const qd_decoder* dec, const WinGpu& g) {
 // 11.2 / 20.9, 38 shots 26.2 / 15.8 / 12.6 / 18.0, 64 shots 40.3 / 24.4 / 19.6 /
 // 18.4; paper preset, 25 shots 6.1 / 4.5 / 5.0 / 11.1, 64 shots 12.5 / 7.8 / 7.0 /
 // 12.2; [[72,12,6]], 2 shots 2.45 / 2.26 / 2.47 / 3.9, 64 shots 6.5 / 4.5 / 3.7 /
-// 5.0.
+// 5.0.  (64 configured [[144,12,12]] shots, 6.7 paths per SM, would be 6 % faster
+// in shot mode, 64 of the paper preset 1.7 times as slow.)
 int path_shape(const qd_decoder* dec, const WinGpu& g, int64_t n_shots) {
   bool path_mode = dec->launch_mode == 2;
   if (dec->launch_mode == 0)
